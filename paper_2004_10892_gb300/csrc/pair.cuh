@@ -1,0 +1,79 @@
+// pair.cuh -- a fused chain of buckets as a register-tiled product of its two
+// large tensors (k_pair), optionally times a third one.
+//
+// A chain's result is out[o] = sum_K A B C prod_g g over the chain's
+// eliminated variables K (Eq. 2 applied m times, regrouped), with large
+// tensors A and B that both hold the first eliminated variable u_0, at most
+// one other large tensor C that does not, and small tensors g, each of which
+// has its variables among A's or among B's and is folded into that one.
+// With K2 = K & vars(C) and K1 = K - K2:
+//   out[o] = sum_K2 C[K2, o] (sum_K1 A[K1, K2, o] B[K1, K2, o]).
+#pragma once
+#include <cuda_runtime.h>
+
+namespace tnq {
+
+constexpr int PTB = 8;              // log2 threads per k_pair block
+constexpr int PTPB = 1 << PTB;
+constexpr int PR = 2;               // register tile: 2^PR entries along A's variables x 2^PR along B's
+constexpr int PE_MAX = 13;          // staged (u = 0, u = 1) pairs of one operand: at most 2^13
+constexpr int PF_MAX = 8;           // fold table of one operand: at most 2^8 pairs
+constexpr int PIN_MAX = 16;         // tensors a chain reads
+constexpr int PH_MAX = 32;          // tile bits
+constexpr int PK_MAX = 5;           // eliminated variables of one loop
+constexpr int PAIR_SMEM_MAX = 100 * 1024;  // dynamic shared memory of one block: two fit an SM
+
+// One tensor that the chain reads from memory.
+struct PIn {
+  const float2* ptr;
+  long long istride;            // per item (0 if item-invariant)
+  int hstride[PH_MAX];          // per tile bit
+  int meta;                     // meta row (-1: gate tensor, unit scale)
+  int dep;
+};
+
+// A staged operand. Its local entries are enumerated as pairs over its bit 0
+// by an index e (bits by increasing memory stride, so that consecutive threads
+// read consecutive memory); bit i of e adds g[i] to the global offset
+// (elements), d[i] to the shared-memory slot (16-byte units) and f[i] to the
+// fold table's index.
+struct POp {
+  int gin;
+  int ebits;
+  int g[PE_MAX], d[PE_MAX], f[PE_MAX];
+  int base;                     // first slot
+};
+
+// Small tensors folded into one operand: table of (u_0 = 0, u_0 = 1) pairs.
+struct PFold {
+  int n, nf;                    // tensors, table index bits
+  int inv;                      // 1: no folded tensor holds a tile bit
+  int gin[PIN_MAX], ustride[PIN_MAX];
+  int fs[PIN_MAX][PF_MAX];      // element stride of table index bit b
+};
+
+struct PairParams {
+  PIn gin[PIN_MAX];
+  POp a, b, c;                  // c.gin < 0: no third tensor
+  PFold fa, fb;
+  float2* out;
+  long long out_istride;
+  long long out_hstride[PH_MAX];
+  int ta[PTB], tb[PTB], tc[PTB], to[PTB];  // thread bits: slots of a, b, c; output offset
+  int xa[PR], xc[PR], xo[PR];   // register bits along A: slots of a and c, output offset (0 for a K2 bit)
+  int yb[PR], yc[PR], yo[PR];   // register bits along B
+  int n1, k1a[PK_MAX], k1b[PK_MAX];                // K1 without u_0: slots of a and b
+  int n2, k2a[PK_MAX], k2b[PK_MAX], k2c[PK_MAX];   // K2 outside the register tile
+  int nkx, nky;                 // K2 bits among the register bits along A / B (the low ones)
+  int n_h, n_gin, out_meta, out_dep, B;
+  int smem;                     // dynamic shared memory bytes
+  int* meta_e;
+  unsigned* meta_m;
+};
+
+// Blocks of k_pair that fit the device at once for this shape; 0 and *err on failure.
+int pair_grid(const PairParams& p, cudaError_t* err);
+// Launches the chain over n_tiles tiles (item, tile variables).
+void pair_launch(const PairParams& p, long long n_tiles, int grid, cudaStream_t s);
+
+}  // namespace tnq

@@ -27,7 +27,9 @@
 #include <vector>
 
 #include "../../include/tnq.h"
+#include "device_util.cuh"
 #include "gemm_tc.cuh"
+#include "pair.cuh"
 #include "plan.hpp"
 
 extern "C" const char* tnq_last_error(void);
@@ -184,30 +186,6 @@ __global__ void k_scalar_init(const LeafDev* __restrict__ sl, int n_sl, const in
   for (int i = 0; i < n_inout; ++i)
     if (bit_of(bits, h.n_words, brow, inout_q[i])) re = im = 0.0;
   item_scalar[item] = make_double2(re, im);
-}
-
-// Scale 2^-m that brings a tensor whose largest |re|,|im| has float bits
-// `mbits` into [0.5, 1); m is returned through *mexp.
-__device__ __forceinline__ float scale_of_max(unsigned mbits, int* mexp) {
-  if (mbits == 0u) {
-    *mexp = 0;
-    return 1.f;
-  }
-  int ex = (int)((mbits >> 23) & 0xffu);
-  if (ex == 0) ex = 1;
-  int m = ex - 126;
-  if (m > 126) m = 126;
-  *mexp = m;
-  return __int_as_float((127 - m) << 23);
-}
-
-__device__ __forceinline__ float2 cmul(float2 a, float2 b) {
-  return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
-
-__device__ __forceinline__ void atomic_max_pos(unsigned* p, float v) {
-  const unsigned b = __float_as_uint(v);
-  if (b > *reinterpret_cast<volatile unsigned*>(p)) atomicMax(p, b);
 }
 
 // K1: one bucket, all items. Element g of the launch = item * 2^out_bits + b'
@@ -1416,6 +1394,8 @@ struct ExecConfig {
   std::vector<GParams> gp;           // per fused-group step
   std::vector<int> gsmem;            // dynamic shared memory bytes per fused-group step
   std::vector<int> ggrid;            // persistent blocks per fused-group step (SMs x resident blocks at its gsmem)
+  std::vector<PairParams> pp;        // fused-group steps that k_pair runs
+  std::vector<int> pair_of;          // per fused-group step: its entry in pp, or -1 (k_group)
   int group_grid = 152 * 4;          // persistent blocks of k_group (SMs x resident blocks)
   std::vector<GemmBucketArgs> gb;    // per GEMM step (pointers are arena offsets)
   std::vector<GemmEpilogue> ge;
@@ -1790,6 +1770,251 @@ static GParams group_gparams(const tnq_plan& P, const Layout& L, const FusedGrou
   return G;
 }
 
+// A fused chain as k_pair runs it (pair.cuh), pointers as byte offsets from
+// the arena base; false when the chain has another shape and k_group runs it.
+// The choice depends on the plan alone, never on the batch (a slice's value
+// must not depend on it). Requirements and why:
+//  * two large tensors (rank above PAIR_SMALL) that hold the first eliminated
+//    variable, at most one other large one, without it: the product of two
+//    tensors is what the register tile shares operands over;
+//  * every other tensor has its variables among A's or among B's: it is
+//    multiplied into that operand as it is staged;
+//  * at least 2^PR register entries along variables of A alone and of B alone
+//    (eliminated variables of C count): without them nothing is shared;
+//  * 2^PTB threads times the register tile of outputs.
+constexpr int PAIR_SMALL = 4;
+static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g, PairParams& G) {
+  const Program& prog = P.prog;
+  std::memset(&G, 0, sizeof(G));
+  const PTensor& o = prog.tensors[g.output];
+  const auto& in = g.ext_inputs;
+  if ((int)in.size() > PIN_MAX || o.rank() > 30) return false;
+  auto vars = [&](int j) -> const std::vector<int>& { return prog.tensors[in[j]].vars; };
+  auto holds = [&](int j, int v) { return j >= 0 && index_in(vars(j), v) >= 0; };
+  std::vector<int> K;
+  for (int b : g.buckets) K.push_back(prog.buckets[b].u);
+  if ((int)K.size() > PK_MAX) return false;
+  const int u0 = K[0];
+  std::vector<int> large, small;
+  for (int j = 0; j < (int)in.size(); ++j) (prog.tensors[in[j]].rank() > PAIR_SMALL ? large : small).push_back(j);
+  int A = -1, B = -1, C = -1;
+  for (int j : large) {
+    int& to = !holds(j, u0) ? C : (A < 0 ? A : B);
+    if (to >= 0) return false;
+    to = j;
+  }
+  if (B < 0) return false;
+  int c0 = -1;
+  if (C >= 0) {  // C's bit 0: an eliminated variable that one of A and B holds (called B)
+    c0 = vars(C)[0];
+    if (index_in(K, c0) < 0 || holds(A, c0) == holds(B, c0)) return false;
+    if (holds(A, c0)) std::swap(A, B);
+  } else if (prog.tensors[in[A]].rank() < prog.tensors[in[B]].rank()) {
+    std::swap(A, B);  // B, the smaller one, is the one that is always scaled
+  }
+  if (vars(A)[0] != u0 || vars(B)[0] != u0) return false;
+  std::vector<int> sa, sb;
+  for (int j : small) {
+    bool ina = true, inb = true;
+    for (int v : vars(j)) {
+      ina = ina && holds(A, v);
+      inb = inb && holds(B, v);
+    }
+    if (!ina && !inb) return false;
+    (inb ? sb : sa).push_back(j);
+  }
+  // eliminated variables: K2 in C (register bits where A or B alone holds them), K1 the others
+  std::vector<int> k1, k2, xreg, yreg;
+  if (C >= 0) yreg.push_back(c0);
+  for (int v : K) {
+    if (v == u0 || v == c0) continue;
+    if (!holds(A, v) && !holds(B, v)) return false;
+    if (!holds(C, v)) k1.push_back(v);
+    else if (holds(A, v) && !holds(B, v) && (int)xreg.size() < PR) xreg.push_back(v);
+    else if (holds(B, v) && !holds(A, v) && (int)yreg.size() < PR) yreg.push_back(v);
+    else k2.push_back(v);
+  }
+  G.nkx = (int)xreg.size();
+  G.nky = (int)yreg.size();
+  // local output variables: the two earliest (the output is written in 32-byte
+  // runs), then the one that adds the fewest staged entries, as long as enough
+  // variables of A alone and of B alone stay for the register tile
+  const int need_x = PR - G.nkx, need_y = PR - G.nky, n_local = PTB + need_x + need_y;
+  if (o.rank() < n_local) return false;
+  const int ops[3] = {A, B, C};
+  int bits[3] = {0, 0, 0};
+  for (int k = 0; k < 3; ++k)
+    for (int v : K) bits[k] += holds(ops[k], v);
+  auto slots = [&](const int* b) {
+    double n = 0;
+    for (int k = 0; k < 3; ++k)
+      if (ops[k] >= 0) n += std::ldexp(1.0, b[k] - 1);
+    return n;
+  };
+  std::vector<char> local(o.vars.size(), 0);
+  int nx = 0, ny = 0;
+  for (int n = 0; n < n_local; ++n) {
+    int best = -1;
+    double best_cost = 0;
+    const int miss_x = std::max(0, need_x - nx), miss_y = std::max(0, need_y - ny);
+    for (int i = 0; i < (int)o.vars.size(); ++i) {
+      if (local[i]) continue;
+      const bool ha = holds(A, o.vars[i]), hb = holds(B, o.vars[i]);
+      if (n_local - n <= miss_x + miss_y && !(ha && !hb && miss_x) && !(hb && !ha && miss_y)) continue;
+      int b[3];
+      for (int k = 0; k < 3; ++k) b[k] = bits[k] + holds(ops[k], o.vars[i]);
+      const double c = slots(b);
+      if (best < 0 || c < best_cost) {
+        best = i;
+        best_cost = c;
+      }
+      if (i == n && n < 2) break;  // the two earliest variables first
+    }
+    if (best < 0) return false;
+    local[best] = 1;
+    for (int k = 0; k < 3; ++k) bits[k] += holds(ops[k], o.vars[best]);
+    nx += holds(A, o.vars[best]) && !holds(B, o.vars[best]);
+    ny += holds(B, o.vars[best]) && !holds(A, o.vars[best]);
+  }
+  // register bits: the latest local variables of A alone / B alone; the other
+  // local variables are thread bits, the earliest lowest
+  std::vector<char> is_reg(o.vars.size(), 0);
+  for (int side = 0; side < 2; ++side) {
+    std::vector<int>& reg = side ? yreg : xreg;
+    for (int i = (int)o.vars.size() - 1; i >= 0 && (int)reg.size() < PR; --i)
+      if (local[i] && holds(side ? B : A, o.vars[i]) && !holds(side ? A : B, o.vars[i])) {
+        reg.push_back(o.vars[i]);
+        is_reg[i] = 1;
+      }
+    if ((int)reg.size() < PR) return false;
+  }
+  std::vector<int> thr, tile;
+  for (int i = 0; i < (int)o.vars.size(); ++i) {
+    if (!local[i]) tile.push_back(o.vars[i]);
+    else if (!is_reg[i]) thr.push_back(o.vars[i]);
+  }
+  if ((int)thr.size() != PTB || (int)tile.size() >= PH_MAX) return false;
+  // fold tables
+  std::vector<int> fold_vars[2];
+  for (int side = 0; side < 2; ++side) {
+    PFold& F = side ? G.fb : G.fa;
+    const std::vector<int>& S = side ? sb : sa;
+    std::vector<int>& fv = fold_vars[side];
+    F.inv = 1;
+    for (int j : S)
+      for (int v : vars(j)) {
+        if (index_in(tile, v) >= 0) F.inv = 0;
+        else if (v != u0 && index_in(fv, v) < 0) fv.push_back(v);
+      }
+    F.nf = (int)fv.size();
+    if (F.nf > PF_MAX) return false;
+    for (int j : S) {
+      F.gin[F.n] = j;
+      for (int b = 0; b < F.nf; ++b) {
+        const int p = index_in(vars(j), fv[b]);
+        F.fs[F.n][b] = p < 0 ? 0 : 1 << p;
+      }
+      const int p = index_in(vars(j), u0);
+      F.ustride[F.n] = p < 0 ? 0 : 1 << p;
+      ++F.n;
+    }
+  }
+  // staged operands: slot = row + pitch * (its eliminated variables but bit
+  // 0), rows numbered by the thread bits it holds, then by its register
+  // outputs; the odd pitch and the lowest row bits on the lowest lanes keep
+  // both the staging stores and the register tile's loads free of conflicts
+  int base = 0;
+  std::vector<int> weight[3];  // per operand: slot weight of each of its variables
+  for (int k = 0; k < 3; ++k) {
+    POp& O = k == 0 ? G.a : (k == 1 ? G.b : G.c);
+    O.gin = ops[k];
+    if (O.gin < 0) continue;
+    const std::vector<int>& v = vars(O.gin);
+    std::vector<int>& w = weight[k];
+    w.assign(v.size(), 0);
+    int rows = 0;
+    auto row = [&](int x) {
+      const int p = index_in(v, x);
+      if (p >= 0) w[p] = 1 << rows++;
+    };
+    for (int x : thr) row(x);
+    for (int x : xreg)
+      if (index_in(K, x) < 0) row(x);
+    for (int x : yreg)
+      if (index_in(K, x) < 0) row(x);
+    const int pitch = (1 << rows) | 1;
+    int nk = 0;
+    for (size_t p = 1; p < v.size(); ++p)
+      if (index_in(K, v[p]) >= 0) w[p] = pitch << nk++;
+    O.base = base;
+    base += pitch << nk;
+    for (size_t p = 1; p < v.size(); ++p) {
+      if (index_in(tile, v[p]) >= 0) continue;
+      if (O.ebits >= PE_MAX || p > 30) return false;
+      O.g[O.ebits] = 1 << p;
+      O.d[O.ebits] = w[p];
+      const int f = k < 2 ? index_in(fold_vars[k], v[p]) : -1;
+      O.f[O.ebits] = f < 0 ? 0 : 1 << f;
+      ++O.ebits;
+    }
+  }
+  G.smem = base * 16;
+  if (G.smem > PAIR_SMEM_MAX) return false;
+  auto slot = [&](int k, int v) {
+    const int p = ops[k] < 0 ? -1 : index_in(vars(ops[k]), v);
+    return p < 0 ? 0 : weight[k][p];
+  };
+  auto out_of = [&](int v) {
+    const int p = index_in(o.vars, v);
+    return p < 0 ? 0 : 1 << p;
+  };
+  for (int i = 0; i < PTB; ++i) {
+    G.ta[i] = slot(0, thr[i]);
+    G.tb[i] = slot(1, thr[i]);
+    G.tc[i] = slot(2, thr[i]);
+    G.to[i] = out_of(thr[i]);
+  }
+  for (int i = 0; i < PR; ++i) {
+    G.xa[i] = slot(0, xreg[i]);
+    G.xc[i] = slot(2, xreg[i]);
+    G.xo[i] = out_of(xreg[i]);
+    G.yb[i] = slot(1, yreg[i]);
+    G.yc[i] = slot(2, yreg[i]);
+    G.yo[i] = out_of(yreg[i]);
+  }
+  for (int v : k1) {
+    G.k1a[G.n1] = slot(0, v);
+    G.k1b[G.n1++] = slot(1, v);
+  }
+  for (int v : k2) {
+    G.k2a[G.n2] = slot(0, v);
+    G.k2b[G.n2] = slot(1, v);
+    G.k2c[G.n2++] = slot(2, v);
+  }
+  G.n_h = (int)tile.size();
+  G.n_gin = (int)in.size();
+  G.B = L.B;
+  G.out_meta = g.output;
+  G.out_dep = L.dep[g.output];
+  G.out = reinterpret_cast<float2*>((size_t)L.off[g.output] * 8);
+  G.out_istride = 1ll << o.rank();
+  for (int i = 0; i < G.n_h; ++i) G.out_hstride[i] = out_of(tile[i]);
+  for (int j = 0; j < G.n_gin; ++j) {
+    const PTensor& x = prog.tensors[in[j]];
+    PIn& I = G.gin[j];
+    I.ptr = reinterpret_cast<const float2*>((size_t)L.off[in[j]] * 8);
+    I.dep = L.dep[in[j]];
+    I.istride = 1ll << x.rank();
+    I.meta = x.leaf_gate >= 0 ? -1 : in[j];
+    for (int i = 0; i < G.n_h; ++i) {
+      const int p = index_in(x.vars, tile[i]);
+      if (p > 30) return false;
+      I.hstride[i] = p < 0 ? 0 : 1 << p;
+    }
+  }
+  return true;
+}
+
 // GEMM-step parameters of a GEMM group, with pointers holding byte offsets
 // from the arena base (rebased per call). Host only.
 static bool gemm_params(const tnq_plan& P, const Layout& L, const FusedGroup& g, GemmBucketArgs& G,
@@ -1936,6 +2161,8 @@ static bool build_steps(const tnq_plan& P, const Layout& L, ExecConfig& C) {
   C.kshape.clear();
   C.gp.clear();
   C.gsmem.clear();
+  C.pp.clear();
+  C.pair_of.clear();
   C.steps.clear();
   C.step_group.clear();
   C.gb.clear();
@@ -1993,6 +2220,12 @@ static bool build_steps(const tnq_plan& P, const Layout& L, ExecConfig& C) {
       C.step_hoist.push_back(0);
       C.gp.push_back(g);
       C.gsmem.push_back(smem);
+      PairParams pp;
+      C.pair_of.push_back(-1);
+      if (pair_params(P, L, prog.groups[gi], pp)) {
+        C.pair_of.back() = (int)C.pp.size();
+        C.pp.push_back(pp);
+      }
       double by = tbytes(prog.groups[gi].output);
       for (int t : prog.groups[gi].ext_inputs) by += tbytes(t);
       C.step_bytes.push_back(by);
@@ -2147,6 +2380,58 @@ static std::string validate_config(const tnq_plan& P, int mode, int B) {
     if (G.lean2 && (C.gsmem[gi] < 2 * GTPB * (int)sizeof(float2) || C.gsmem[gi] < (8 << G.st[0].nbits)))
       return "group " + std::to_string(gi) + ": shared memory below the dense stage's reads";
   }
+  for (size_t si = 0; si < C.steps.size(); ++si) {  // chains that k_pair runs
+    if (C.steps[si].first != 1 || C.pair_of[C.steps[si].second] < 0) continue;
+    const PairParams& G = C.pp[C.pair_of[C.steps[si].second]];
+    const FusedGroup& g = prog.groups[C.step_group[si]];
+    const std::string name = "pair chain " + std::to_string(si);
+    const long long items = G.out_dep ? B : 1;
+    auto tile_max = [&](int j) {
+      long long m = G.gin[j].dep ? (items - 1) * G.gin[j].istride : 0;
+      for (int i = 0; i < G.n_h; ++i) m += G.gin[j].hstride[i];
+      return m;
+    };
+    if (G.smem > PAIR_SMEM_MAX) return name + ": shared memory";
+    const POp* ops[3] = {&G.a, &G.b, &G.c};
+    for (int k = 0; k < 3; ++k) {
+      const POp& O = *ops[k];
+      if (O.gin < 0) continue;
+      long long m = tile_max(O.gin) + 1;
+      int d = O.base, f = 0;
+      for (int i = 0; i < O.ebits; ++i) {
+        if (O.g[i] & 1) return name + ": odd local stride";
+        m += O.g[i];
+        d += O.d[i];
+        f += O.f[i];
+      }
+      for (int i = 0; i < G.n_h; ++i)
+        if (G.gin[O.gin].hstride[i] & 1) return name + ": odd tile stride";
+      if ((G.gin[O.gin].istride & 1) || ((size_t)G.gin[O.gin].ptr / 8) % 2) return name + ": unaligned input";
+      if (m >= alloc(g.ext_inputs[O.gin])) return name + ": staged input overflows";
+      if (d >= G.smem / 16) return name + ": staged operand outside shared memory";
+      if (k < 2 && f >= 1 << (k ? G.fb.nf : G.fa.nf)) return name + ": fold index";
+      // the register tile reads only staged slots
+      long long r = O.base;
+      for (int i = 0; i < PTB; ++i) r += k == 0 ? G.ta[i] : (k == 1 ? G.tb[i] : G.tc[i]);
+      for (int i = 0; i < PR; ++i) r += k == 0 ? G.xa[i] : (k == 1 ? G.yb[i] : G.xc[i] + (i ? G.yc[i] : 0));
+      for (int i = 0; i < G.n1; ++i) r += k == 0 ? G.k1a[i] : (k == 1 ? G.k1b[i] : 0);
+      for (int i = 0; i < G.n2; ++i) r += k == 0 ? G.k2a[i] : (k == 1 ? G.k2b[i] : G.k2c[i]);
+      if (r > d) return name + ": register tile outside the staged operand";
+    }
+    for (int side = 0; side < 2; ++side) {
+      const PFold& F = side ? G.fb : G.fa;
+      for (int j = 0; j < F.n; ++j) {
+        long long m = tile_max(F.gin[j]) + F.ustride[j];
+        for (int b = 0; b < F.nf; ++b) m += F.fs[j][b];
+        if (m >= alloc(g.ext_inputs[F.gin[j]])) return name + ": folded input overflows";
+      }
+    }
+    long long om = G.out_dep ? (items - 1) * G.out_istride : 0;
+    for (int i = 0; i < G.n_h; ++i) om += G.out_hstride[i];
+    for (int i = 0; i < PTB; ++i) om += G.to[i];
+    for (int i = 0; i < PR; ++i) om += G.xo[i] + G.yo[i];
+    if (om >= alloc(g.output)) return name + ": output overflows";
+  }
   for (size_t gi = 0; gi < C.gb.size(); ++gi) {
     const GemmBucketArgs& G = C.gb[gi];
     const GemmEpilogue& E = C.ge[gi];
@@ -2215,6 +2500,24 @@ static tnq_status group_grid_size(int* out, int smem = GROUP_SMEM_BYTES, int kin
   return TNQ_OK;
 }
 
+// Persistent grid of every fused-group step (SMs x blocks that fit one at its shared memory).
+static tnq_status chain_grids(ExecConfig& C) {
+  C.ggrid.clear();
+  for (size_t i = 0; i < C.gsmem.size(); ++i) {
+    int g = 0;
+    if (C.pair_of[i] >= 0) {
+      cudaError_t e = cudaSuccess;
+      g = pair_grid(C.pp[C.pair_of[i]], &e);
+      CU(e);
+    } else {
+      const tnq_status st = group_grid_size(&g, C.gsmem[i], C.gp[i].tail > 0 ? 1 : (C.gp[i].lean2 ? 2 : 0));
+      if (st != TNQ_OK) return st;
+    }
+    C.ggrid.push_back(g);
+  }
+  return TNQ_OK;
+}
+
 static tnq_status build_config(const tnq_plan& P, int mode, int B, ExecConfig** out) {
   CU(allow_group_smem());
   int ggrid = 0;
@@ -2260,11 +2563,7 @@ static tnq_status build_config(const tnq_plan& P, int mode, int B, ExecConfig** 
     return fail(TNQ_ECUDA);
   }
   if (!build_steps(P, C->L, *C)) return fail(TNQ_EUNSUPPORTED);
-  for (size_t i = 0; i < C->gsmem.size(); ++i) {  // chains with a register tail: more blocks may fit
-    int g = 0;
-    if ((gst = group_grid_size(&g, C->gsmem[i], C->gp[i].tail > 0 ? 1 : (C->gp[i].lean2 ? 2 : 0))) != TNQ_OK) return fail(gst);
-    C->ggrid.push_back(g);
-  }
+  if ((gst = chain_grids(*C)) != TNQ_OK) return fail(gst);
   if ((e = up((void**)&C->d_hoist, C->hoist_dev.data(), C->hoist_dev.size() * sizeof(HoistDev))) != cudaSuccess) {
     set_error(std::string("uploading plan tables: ") + cudaGetErrorString(e));
     return fail(TNQ_ECUDA);
@@ -2325,6 +2624,15 @@ static void launch_step(const ExecConfig& C, int i, float2* arena, int* me, unsi
     e.out = reinterpret_cast<float2*>(base + reinterpret_cast<size_t>(e.out));
     e.meta_m = mm;
     gemm_bucket_launch(g, e, status, s);
+  } else if (C.pair_of[st.second] >= 0) {
+    PairParams g = C.pp[C.pair_of[st.second]];
+    g.out = reinterpret_cast<float2*>(base + reinterpret_cast<size_t>(g.out));
+    for (int j = 0; j < g.n_gin; ++j)
+      g.gin[j].ptr = reinterpret_cast<const float2*>(base + reinterpret_cast<size_t>(g.gin[j].ptr));
+    g.meta_e = me;
+    g.meta_m = mm;
+    const long long tiles = (g.out_dep ? (long long)g.B : 1ll) << g.n_h;
+    pair_launch(g, tiles, C.ggrid.empty() ? C.group_grid : C.ggrid[st.second], s);
   } else {
     GParams g = C.gp[st.second];
     g.out = reinterpret_cast<float2*>(base + reinterpret_cast<size_t>(g.out));
@@ -2622,6 +2930,15 @@ int tnq_internal_group_text(const tnq_plan* plan, int mode, uint32_t batch, char
     out += "group " + std::to_string(gi) + " stages " + std::to_string(G.n_st) + " tail " + std::to_string(G.tail) +
            " n_h " + std::to_string(G.n_h) + " gin " + std::to_string(G.n_gin) + " lean2 " + std::to_string(G.lean2) +
            " smem " + std::to_string(C.gsmem[gi]) + "\n";
+    if (C.pair_of[gi] >= 0) {
+      const PairParams& Q = C.pp[C.pair_of[gi]];
+      out += "  pair: a " + std::to_string(Q.a.ebits) + " b " + std::to_string(Q.b.ebits) + " c " +
+             std::to_string(Q.c.gin < 0 ? -1 : Q.c.ebits) + " n1 " + std::to_string(Q.n1) + " n2 " +
+             std::to_string(Q.n2) + " nkx " + std::to_string(Q.nkx) + " nky " + std::to_string(Q.nky) + " n_h " +
+             std::to_string(Q.n_h) + " folds " + std::to_string(Q.fa.n) + "+" + std::to_string(Q.fb.n) + " nf " +
+             std::to_string(Q.fa.nf) + "+" + std::to_string(Q.fb.nf) + " inv " + std::to_string(Q.fa.inv && Q.fb.inv) +
+             " smem " + std::to_string(Q.smem) + "\n";
+    }
     for (int j = 0; j < G.n_gin; ++j) {
       int nh = 0;
       for (int i = 0; i < G.n_h; ++i) nh += G.gin[j].hstride[i] != 0;
@@ -3513,11 +3830,7 @@ static tnq_status get_noalloc_config(const tnq_plan& P, uint64_t cap, char* scra
   for (int g : prog.scalar_leaves) NC->scalars.push_back(make_leafdev(P, nullptr, g, nullptr, -1, &C.vals));
   for (int t : prog.finals) NC->finals.push_back(FinalDev{C.L.off[t], t, (int)C.L.dep[t]});
   if (!build_steps(P, C.L, C)) return TNQ_EUNSUPPORTED;
-  for (size_t i = 0; i < C.gsmem.size(); ++i) {  // per-chain persistent grids, as build_config sizes them
-    int g = 0;
-    if ((st = group_grid_size(&g, C.gsmem[i], C.gp[i].tail > 0 ? 1 : (C.gp[i].lean2 ? 2 : 0))) != TNQ_OK) return st;
-    C.ggrid.push_back(g);
-  }
+  if ((st = chain_grids(C)) != TNQ_OK) return st;
   size_t o = 0;
   auto take = [&](size_t bytes) {
     char* p = scratch + o;

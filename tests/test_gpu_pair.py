@@ -1,0 +1,93 @@
+"""Fused chains as register-tiled products (k_pair): every shape that the rule
+accepts, against the FP64 oracle and against the same plan run bucket by
+bucket. The shape of a chain is (C: a third large tensor, loops over summed
+variables outside the register tile n1 / n2, summed variables among the
+register bits nkx / nky, tile bits or one tile, small tensors folded into A)."""
+import ctypes
+import re
+
+import numpy as np
+import pytest
+
+from paper_2004_10892_gb300 import inputs as I
+
+# complex64 chains: products of <= 3 tensors, sums of <= 2^5 terms per chain
+# and ~50 buckets in sequence, each adding a few 2^-24 roundings
+TOL = 1e-5
+
+# (rows, cols, depth, seed, shapes that the plan's chains have)
+CASES = [
+    (4, 5, 26, 3, {("-", 1, 0, 0, 0)}),
+    (4, 5, 29, 2, {("-", 4, 0, 0, 0)}),
+    (4, 5, 32, 3, {("-", 3, 0, 0, 0)}),
+    (4, 7, 29, 5, {("-", 2, 0, 0, 0)}),
+    (4, 5, 26, 1, {("c", 0, 0, 0, 1)}),
+    (4, 7, 23, 2, {("c", 0, 0, 0, 2)}),
+    (4, 7, 23, 8, {("c", 0, 0, 1, 1)}),
+    (4, 5, 23, 5, {("c", 0, 0, 1, 2)}),
+    (5, 6, 23, 2, {("c", 0, 0, 2, 1)}),
+    (5, 5, 26, 5, {("c", 0, 0, 2, 2)}),
+    (5, 5, 20, 9, {("c", 0, 1, 1, 1)}),
+    (4, 7, 26, 1, {("c", 0, 1, 1, 2)}),
+    (5, 6, 20, 0, {("c", 0, 1, 2, 1)}),
+    (4, 5, 29, 1, {("c", 0, 2, 0, 2)}),
+    (4, 5, 26, 8, {("c", 1, 0, 1, 1)}),
+    (4, 7, 26, 3, {("c", 1, 0, 1, 2)}),
+    (4, 7, 29, 4, {("c", 1, 0, 2, 1)}),
+    (5, 5, 23, 0, {("c", 1, 1, 1, 1)}),
+    (4, 5, 26, 4, {("c", 2, 0, 1, 1)}),
+    (4, 5, 32, 9, {("c", 2, 1, 0, 1)}),
+    (4, 7, 29, 9, {("c", 3, 0, 0, 1)}),
+]
+
+
+def _plan(tnq_lib, rows, cols, depth, seed, **kw):
+    circ = I.random_grid_circuit(rows, cols, depth, seed)
+    return circ, tnq_lib.Plan(circ, max_bag_log2=20, max_p=20, reorder_every=1, **kw)
+
+
+def _shapes(tnq_lib, plan):
+    f = tnq_lib.lib().tnq_internal_group_text
+    f.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_uint32, ctypes.c_char_p, ctypes.c_size_t]
+    buf = ctypes.create_string_buffer(1 << 20)
+    assert f(plan.handle, 0, 2, buf, 1 << 20) == 0
+    out = set()
+    for line in re.findall(r"pair: (.*)", buf.value.decode()):
+        w = line.split()
+        d = dict(zip(w[::2], w[1::2]))
+        out.add(("-" if d["c"] == "-1" else "c",) + tuple(int(d[k]) for k in ("n1", "n2", "nkx", "nky")))
+    return out
+
+
+@pytest.mark.parametrize("rows,cols,depth,seed,shapes", CASES)
+def test_every_launch_stays_in_bounds(tnq_lib, rows, cols, depth, seed, shapes):
+    """Host only: the rule gives these shapes, and every staged, folded and
+    written index of both modes and several batch sizes is inside its tensor."""
+    _, plan = _plan(tnq_lib, rows, cols, depth, seed)
+    assert shapes <= _shapes(tnq_lib, plan)
+    msg = ctypes.create_string_buffer(512)
+    for mode in (0, 1):
+        for batch in (1, 2, 16):
+            assert tnq_lib.lib().tnq_internal_validate(plan.handle, mode, batch, msg, 512) == 0, msg.value
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("rows,cols,depth,seed,shapes", CASES)
+def test_chain_matches_oracle_and_separate_buckets(cuda, tnq_lib, oracle_lib, rows, cols, depth, seed, shapes):
+    circ, plan = _plan(tnq_lib, rows, cols, depth, seed)
+    assert shapes <= _shapes(tnq_lib, plan)
+    plain = _plan(tnq_lib, rows, cols, depth, seed, fuse_min_rank=0)[1]
+    n = min(plan.info()["n_slices"], 4)
+    bits = I.random_bitstring(circ.n_qubits, seed)
+    _, got = tnq_lib.contract_sliced(plan, bits, 0, n, per_slice=True)
+    _, sep = tnq_lib.contract_sliced(plain, bits, 0, n, per_slice=True)
+    ref = np.array([oracle_lib.contract(circ, bits, order=plan.order(), mu=plan.sliced(), slices=(s, s + 1))
+                    for s in range(n)])
+    scale = np.maximum(np.abs(ref), 2.0 ** (-(circ.n_qubits + plan.info()["p"]) / 2))
+    assert np.max(np.abs(got - ref) / scale) <= TOL
+    assert np.max(np.abs(got - sep) / scale) <= TOL
+    # three bitstrings at once: the item dimension carries (bitstring, slice)
+    more = [bits, I.random_bitstring(circ.n_qubits, seed + 1), I.random_bitstring(circ.n_qubits, seed + 2)]
+    if plan.info()["p"] == 0:
+        out = tnq_lib.amplitudes_batch([plan], [more])
+        assert abs(out[0] - got[0]) <= 1e-9 * abs(got[0])
