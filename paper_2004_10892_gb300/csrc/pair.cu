@@ -7,46 +7,88 @@ namespace tnq {
 
 // Fold table entry e of one operand: the product of its small tensors at u_0 =
 // 0 and 1, starting from (f, 0).
-__device__ __forceinline__ float4 fold_entry(const PFold& F, int e, const float2* const* s_ptr, float f) {
+__device__ __forceinline__ float4 fold_entry(const PairParams& P, const PFold& F, int e, long long item, float f) {
   float2 p0 = make_float2(f, 0.f), p1 = p0;
   for (int j = 0; j < F.n; ++j) {
-    int o = 0;
+    const PIn& g = P.gin[F.gin[j]];
+    const float2* q = g.ptr + (g.dep ? item * g.istride : 0ll);
 #pragma unroll
     for (int i = 0; i < PF_MAX; ++i)
-      if (i < F.nf && ((e >> i) & 1)) o += F.fs[j][i];
-    const float2* q = s_ptr[F.gin[j]] + o;
+      if (i < F.nf && ((e >> i) & 1)) q += F.fs[j][i];
     p0 = cmul(p0, __ldg(q));
     p1 = cmul(p1, __ldg(q + F.ustride[j]));
   }
   return make_float4(p0.x, p0.y, p1.x, p1.y);
 }
 
-// Persistent: a block loops over tiles (item, tile variables). Per tile the
-// block stages its part of A, B (and C) in shared memory once, A and B
-// multiplied by the fold tables on the way, then every thread computes a 4 x 4
-// register tile: per pair of summed values 4 + 4 16-byte shared loads feed 128
-// FMAs.
+__device__ __forceinline__ void cp_async16(unsigned dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+
+// r += a b over the pair's two values
+__device__ __forceinline__ void cfma2(float2& r, float4 a, float4 b) {
+  r.x = fmaf(a.x, b.x, r.x);
+  r.y = fmaf(a.x, b.y, r.y);
+  r.x = fmaf(-a.y, b.y, r.x);
+  r.y = fmaf(a.y, b.x, r.y);
+  r.x = fmaf(a.z, b.z, r.x);
+  r.y = fmaf(a.z, b.w, r.y);
+  r.x = fmaf(-a.w, b.w, r.x);
+  r.y = fmaf(a.w, b.z, r.y);
+}
+
+// Persistent: a block loops over tiles (item, tile variables), a tile over one
+// or two chunks of its summed values. Two stages: while a chunk is computed,
+// the next one's part of A, B (and C) comes in by cp.async; each thread then
+// multiplies what it copied by the fold tables in place, and after one barrier
+// every thread computes a 4 x 4 register tile: per pair of summed values 4 + 4
+// 16-byte shared loads feed 128 FMAs.
 template <int NKX, int NKY, bool HASC>
 __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairParams P, long long n_tiles) {
   extern __shared__ float4 sm[];
-  __shared__ float4 s_fa[1 << PF_MAX], s_fb[1 << PF_MAX];
-  __shared__ int4 s_it[3][1 << (PE_MAX - PTB)];  // staging iteration: global offset, slot, fold index
-  __shared__ int s_hstr[PIN_MAX][PH_MAX];
-  __shared__ const float2* s_ptr[PIN_MAX];
-  __shared__ long long s_out;
+  constexpr int NOP = HASC ? 3 : 2;
+  constexpr int RING = 4;  // a thread is at most one barrier ahead: what it writes is two tiles ahead
+  __shared__ float4 s_fa[2][1 << PF_MAX], s_fb[2][1 << PF_MAX];  // by item, alternating
+  __shared__ int4 s_it[NOP][1 << (PE_MAX - PTB)];  // staging iteration: global offset, slot, fold index
+  __shared__ int4 s_k2[1 << PK_MAX];               // K2 outside the register tile: slots of a, b, c
+  __shared__ int2 s_k1[1 << PK_MAX];               // K1 pairs of a chunk: slots of a, b
+  __shared__ int s_hstr[6][PH_MAX];
+  __shared__ const float2* s_src[RING][3];
+  __shared__ float2* s_out[RING];
+  __shared__ int s_fold[RING][2];
   __shared__ float s_sc[PIN_MAX];
-  __shared__ int s_e[PIN_MAX];
+  __shared__ int s_e[RING][PIN_MAX];
   __shared__ float s_red[PTPB / 32];
   constexpr int N = 1 << PR;
-  const int t = threadIdx.x;
-  for (int e = t; e < PIN_MAX * PH_MAX; e += PTPB) {
-    const int j = e / PH_MAX, i = e - j * PH_MAX;
-    s_hstr[j][i] = (i < P.n_h && j < P.n_gin) ? P.gin[j].hstride[i] : 0;
-  }
+  const int t = threadIdx.x, lane = t & 31;
   const POp* ops[3] = {&P.a, &P.b, &P.c};
-  int tg[3], td[3], tf[3];  // this thread's part of the staging offsets
+  // ---- tables that every tile uses
+  if (t < PH_MAX) {
+    s_hstr[0][t] = t < P.n_h ? P.a.h[t] : 0;
+    s_hstr[1][t] = t < P.n_h ? P.b.h[t] : 0;
+    s_hstr[2][t] = HASC && t < P.n_h ? P.c.h[t] : 0;
+    s_hstr[3][t] = t < P.n_h ? P.out_h[t] : 0;
+    s_hstr[4][t] = t < P.n_h ? P.a.fh[t] : 0;
+    s_hstr[5][t] = t < P.n_h ? P.b.fh[t] : 0;
+    int4 v = make_int4(0, 0, 0, 0);
+    for (int i = 0; i < P.n2; ++i)
+      if ((t >> i) & 1) {
+        v.x += P.k2a[i];
+        v.y += P.k2b[i];
+        v.z += P.k2c[i];
+      }
+    s_k2[t] = v;
+    int2 w = make_int2(0, 0);
+    for (int i = 0; i < P.n1; ++i)
+      if ((t >> i) & 1) {
+        w.x += P.k1a[i];
+        w.y += P.k1b[i];
+      }
+    s_k1[t] = w;
+  }
+  int tg[NOP], td[NOP], tf[NOP];  // this thread's part of the staging offsets
 #pragma unroll
-  for (int o = 0; o < (HASC ? 3 : 2); ++o) {
+  for (int o = 0; o < NOP; ++o) {
     const POp& O = *ops[o];
     tg[o] = tf[o] = 0;
     td[o] = O.base;
@@ -69,60 +111,39 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
       s_it[o][t] = v;
     }
   }
-  int ra = P.a.base, rb = P.b.base, rc = P.c.base, ro = 0;  // this thread's register tile
+  int ra = P.a.base, rb = P.b.base, rc = HASC ? P.c.base : 0, ro = 0;  // this thread's register tile
 #pragma unroll
   for (int i = 0; i < PTB; ++i)
     if ((t >> i) & 1) {
       ra += P.ta[i];
       rb += P.tb[i];
-      rc += P.tc[i];
+      if (HASC) rc += P.tc[i];
       ro += P.to[i];
     }
-  int pa[N], pb[N];
-#pragma unroll
-  for (int i = 0; i < N; ++i) {
-    pa[i] = ra + ((i & 1) ? P.xa[0] : 0) + ((i & 2) ? P.xa[1] : 0);
-    pb[i] = rb + ((i & 1) ? P.yb[0] : 0) + ((i & 2) ? P.yb[1] : 0);
-  }
   const bool fold_a = P.fa.n > 0;
-  const bool fold_inv = P.fa.inv && P.fb.inv;
-  long long cur_item = -1;
-  float tmax = 0.f;
-  auto flush = [&](long long item) {
-    float m = tmax;
-    for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
-    __syncthreads();
-    if ((t & 31) == 0) s_red[t >> 5] = m;
-    __syncthreads();
-    if (t == 0) {
-      float b = 0.f;
-      for (int w = 0; w < PTPB / 32; ++w) b = fmaxf(b, s_red[w]);
-      if (b > 0.f) atomic_max_pos(&P.meta_m[(long long)P.out_meta * P.B + (P.out_dep ? item : 0ll)], b);
+  const unsigned sm0 = (unsigned)__cvta_generic_to_shared(sm);
+  __syncthreads();
+
+  // pointers and fold offsets of a tile: one warp per value, lane i adds tile bit i's stride
+  auto tile_setup = [&](long long tile, int slot) {
+    const long long item = tile >> P.n_h;
+    const int h = (int)(tile & ((1ll << P.n_h) - 1ll));
+    const int w = t >> 5;
+    if (w >= 6) return;
+    const int v = __reduce_add_sync(0xffffffffu, ((h >> lane) & 1) ? s_hstr[w][lane] : 0);
+    if (lane) return;
+    if (w < NOP) {
+      const PIn& g = P.gin[w == 0 ? P.a.gin : (w == 1 ? P.b.gin : P.c.gin)];
+      s_src[slot][w] = g.ptr + (g.dep ? item * g.istride : 0ll) + v;
+    } else if (w == 3) {
+      s_out[slot] = P.out + (P.out_dep ? item * P.out_istride : 0ll) + v;
+    } else if (w >= 4) {
+      s_fold[slot][w - 4] = v;
     }
   };
-  for (long long tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-    const long long item = tile >> P.n_h;
-    const long long h = tile & ((1ll << P.n_h) - 1ll);
-    const bool new_item = item != cur_item;
-    if (new_item) {
-      if (cur_item >= 0) flush(cur_item);
-      tmax = 0.f;
-      cur_item = item;
-    }
-    __syncthreads();  // the previous tile is done with the staged operands
-    for (int j = t >> 5; j <= P.n_gin; j += PTPB / 32) {
-      const int lane = t & 31;
-      if (j < P.n_gin) {
-        const int v = __reduce_add_sync(0xffffffffu, ((h >> lane) & 1ll) ? s_hstr[j][lane] : 0);
-        if (lane == 0) s_ptr[j] = P.gin[j].ptr + (P.gin[j].dep ? item * P.gin[j].istride : 0ll) + v;
-      } else if (lane == 0) {
-        long long v = P.out_dep ? item * P.out_istride : 0ll;
-        for (int i = 0; i < P.n_h; ++i)
-          if ((h >> i) & 1ll) v += P.out_hstride[i];
-        s_out = v;
-      }
-    }
-    if (new_item && t < P.n_gin) {
+  // exponents, scales and fold tables of an item (every input's power-of-two scale goes into B's table)
+  auto item_setup = [&](long long item, int n) {
+    if (t < P.n_gin) {
       const PIn& g = P.gin[t];
       int m = 0, e = 0;
       float f = 1.f;
@@ -132,113 +153,142 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
         e = P.meta_e[row] + m;
       }
       s_sc[t] = f;
-      s_e[t] = e;
+      s_e[n % RING][t] = e;
     }
     __syncthreads();
-    if (new_item || !fold_inv) {  // small tensors and every input's power-of-two scale
+    if (t < (1 << P.fb.nf)) {
       float f = 1.f;
       for (int j = 0; j < P.n_gin; ++j) f *= s_sc[j];
-      if (t < (1 << P.fb.nf)) s_fb[t] = fold_entry(P.fb, t, s_ptr, f);
-      if (fold_a && t < (1 << P.fa.nf)) s_fa[t] = fold_entry(P.fa, t, s_ptr, 1.f);
-      __syncthreads();
+      s_fb[n & 1][t] = fold_entry(P, P.fb, t, item, f);
     }
+    if (fold_a && t < (1 << P.fa.nf)) s_fa[n & 1][t] = fold_entry(P, P.fa, t, item, 1.f);
+  };
+  auto issue = [&](int slot, int chunk, int buf) {
 #pragma unroll
-    for (int o = 0; o < (HASC ? 3 : 2); ++o) {
+    for (int o = 0; o < NOP; ++o) {
       const POp& O = *ops[o];
-      const float2* src = s_ptr[O.gin] + tg[o];
-      const float4* ft = (o == 0 ? s_fa : s_fb) + tf[o];
-      const bool fold = o == 1 || (o == 0 && fold_a);
+      const float2* src = s_src[slot][o] + tg[o] + (chunk ? O.gch : 0);
+      const unsigned dst = sm0 + 16u * (unsigned)(buf * P.stage + td[o]);
       const int nit = O.ebits > PTB ? 1 << (O.ebits - PTB) : 1;
-      if (O.ebits < PTB && t >= (1 << O.ebits)) continue;
-#pragma unroll 4
-      for (int it = 0; it < nit; ++it) {
-        const int4 k = s_it[o][it];
-        float4 v = __ldg(reinterpret_cast<const float4*>(src + k.x));
-        if (fold) {
-          const float4 f = ft[k.z];
+      if (O.ebits >= PTB || t < (1 << O.ebits))
+        for (int it = 0; it < nit; ++it) {
+          const int4 k = s_it[o][it];
+          cp_async16(dst + 16u * (unsigned)k.y, src + k.x);
+        }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  // multiplies the pairs this thread copied by the fold tables
+  auto fold = [&](int slot, int chunk, int buf, int n) {
+#pragma unroll
+    for (int o = 0; o < 2; ++o) {
+      if (o == 0 && !fold_a) continue;
+      const POp& O = *ops[o];
+      const float4* ft = (o == 0 ? s_fa[n & 1] : s_fb[n & 1]) + tf[o] + s_fold[slot][o] + (chunk ? O.fch : 0);
+      float4* dst = sm + buf * P.stage + td[o];
+      const int nit = O.ebits > PTB ? 1 << (O.ebits - PTB) : 1;
+      if (O.ebits >= PTB || t < (1 << O.ebits)) {
+#pragma unroll 2
+        for (int it = 0; it < nit; ++it) {
+          const int4 k = s_it[o][it];
+          const float4 v = dst[k.y], f = ft[k.z];
           const float2 v0 = cmul(make_float2(v.x, v.y), make_float2(f.x, f.y));
           const float2 v1 = cmul(make_float2(v.z, v.w), make_float2(f.z, f.w));
-          v = make_float4(v0.x, v0.y, v1.x, v1.y);
+          dst[k.y] = make_float4(v0.x, v0.y, v1.x, v1.y);
         }
-        sm[td[o] + k.y] = v;
       }
     }
+  };
+  float tmax = 0.f;
+  auto flush = [&](long long item) {
+    float m = tmax;
+    for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
     __syncthreads();
-    constexpr int XO = N >> NKX, YO = N >> NKY;
-    float2 acc[XO][YO];
+    if (lane == 0) s_red[t >> 5] = m;
+    __syncthreads();
+    if (t == 0) {
+      float b = 0.f;
+      for (int w = 0; w < PTPB / 32; ++w) b = fmaxf(b, s_red[w]);
+      if (b > 0.f) atomic_max_pos(&P.meta_m[(long long)P.out_meta * P.B + (P.out_dep ? item : 0ll)], b);
+    }
+    tmax = 0.f;
+  };
+
+  int n_item = 0, buf = 0;
+  tile_setup(blockIdx.x, 0);
+  item_setup((long long)blockIdx.x >> P.n_h, 0);
+  __syncthreads();
+  issue(0, 0, 0);
+  int slot = 0;
+  constexpr int XO = N >> NKX, YO = N >> NKY;
+  for (long long tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, slot = (slot + 1) % RING) {
+    const long long item = tile >> P.n_h, next = tile + gridDim.x;
+    const bool more = next < n_tiles;
+    const bool new_item = more && (next >> P.n_h) != item;
+    float2 x[N][N], acc[XO][YO];
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+      for (int j = 0; j < N; ++j) x[i][j] = make_float2(0.f, 0.f);
 #pragma unroll
     for (int i = 0; i < XO; ++i)
 #pragma unroll
       for (int j = 0; j < YO; ++j) acc[i][j] = make_float2(0.f, 0.f);
-    const int n1 = 1 << P.n1, n2 = HASC ? 1 << P.n2 : 1;
-    for (int q2 = 0; q2 < n2; ++q2) {
-      int oa = 0, ob = 0, oc = 0;
-      if (HASC)
-        for (int i = 0; i < P.n2; ++i)
-          if ((q2 >> i) & 1) {
-            oa += P.k2a[i];
-            ob += P.k2b[i];
-            oc += P.k2c[i];
-          }
-      float2 x[N][N];
-#pragma unroll
-      for (int i = 0; i < N; ++i)
-#pragma unroll
-        for (int j = 0; j < N; ++j) x[i][j] = make_float2(0.f, 0.f);
-      for (int q = 0; q < n1; ++q) {
-        int ka = oa, kb = ob;
-        for (int i = 0; i < P.n1; ++i)
-          if ((q >> i) & 1) {
-            ka += P.k1a[i];
-            kb += P.k1b[i];
-          }
-        float4 va[N], vb[N];
-#pragma unroll
-        for (int i = 0; i < N; ++i) va[i] = sm[pa[i] + ka];
-#pragma unroll
-        for (int j = 0; j < N; ++j) vb[j] = sm[pb[j] + kb];
-#pragma unroll
-        for (int i = 0; i < N; ++i)
-#pragma unroll
-          for (int j = 0; j < N; ++j) {
-            float2 r = x[i][j];
-            r.x = fmaf(va[i].x, vb[j].x, r.x);
-            r.y = fmaf(va[i].x, vb[j].y, r.y);
-            r.x = fmaf(-va[i].y, vb[j].y, r.x);
-            r.y = fmaf(va[i].y, vb[j].x, r.y);
-            r.x = fmaf(va[i].z, vb[j].z, r.x);
-            r.y = fmaf(va[i].z, vb[j].w, r.y);
-            r.x = fmaf(-va[i].w, vb[j].w, r.x);
-            r.y = fmaf(va[i].w, vb[j].z, r.y);
-            x[i][j] = r;
-          }
+    for (int c = 0; c < P.n_ch; ++c) {
+      const bool last = c + 1 == P.n_ch;
+      if (last && more) {
+        tile_setup(next, (slot + 1) % RING);
+        if (new_item) item_setup(next >> P.n_h, n_item + 1);
       }
-      if constexpr (HASC) {  // times C, summed over the K2 register bits (C's bit 0 is B's register bit 0)
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      fold(slot, c, buf, n_item);
+      __syncthreads();  // the chunk is staged, and every thread is done with the other stage
+      if (!last) issue(slot, c + 1, buf ^ 1);
+      else if (more) issue((slot + 1) % RING, 0, buf ^ 1);
+      const float4* pa = sm + buf * P.stage + ra;
+      const float4* pb = sm + buf * P.stage + rb;
+      const int n1 = 1 << P.n1;
+      auto products = [&](int oa, int ob) {
+#pragma unroll 1
+        for (int q = 0; q < n1; ++q) {
+          const int2 k = s_k1[q];
+          float4 va[N], vb[N];
 #pragma unroll
-        for (int i = 0; i < N; ++i)
+          for (int i = 0; i < N; ++i)
+            va[i] = pa[oa + k.x + ((i & 1) ? P.xa[0] : 0) + ((i & 2) ? P.xa[1] : 0)];
 #pragma unroll
-          for (int j = 0; j < N; j += 2) {
-            const float4 c = sm[rc + oc + ((i & 1) ? P.xc[0] : 0) + ((i & 2) ? P.xc[1] : 0) + ((j & 2) ? P.yc[1] : 0)];
-            float2 r = acc[i >> NKX][j >> NKY];
-            const float2 u = x[i][j], w = x[i][j + 1];
-            r.x = fmaf(u.x, c.x, r.x);
-            r.y = fmaf(u.x, c.y, r.y);
-            r.x = fmaf(-u.y, c.y, r.x);
-            r.y = fmaf(u.y, c.x, r.y);
-            r.x = fmaf(w.x, c.z, r.x);
-            r.y = fmaf(w.x, c.w, r.y);
-            r.x = fmaf(-w.y, c.w, r.x);
-            r.y = fmaf(w.y, c.z, r.y);
-            acc[i >> NKX][j >> NKY] = r;
-          }
+          for (int j = 0; j < N; ++j)
+            vb[j] = pb[ob + k.y + ((j & 1) ? P.yb[0] : 0) + ((j & 2) ? P.yb[1] : 0)];
+#pragma unroll
+          for (int i = 0; i < N; ++i)
+#pragma unroll
+            for (int j = 0; j < N; ++j) cfma2(x[i][j], va[i], vb[j]);
+        }
+      };
+      if constexpr (HASC) {
+        const int n2 = 1 << P.n2;
+#pragma unroll 1
+        for (int q2 = 0; q2 < n2; ++q2) {
+          const int4 k2 = s_k2[q2];
+          products(k2.x, k2.y);
+          // times C, summed over the K2 register bits (C's bit 0 is B's register bit 0)
+          const float4* pc = sm + buf * P.stage + rc + k2.z;
+#pragma unroll
+          for (int i = 0; i < N; ++i)
+#pragma unroll
+            for (int j = 0; j < N; j += 2) {
+              const float4 v = pc[((i & 1) ? P.xc[0] : 0) + ((i & 2) ? P.xc[1] : 0) + ((j & 2) ? P.yc[1] : 0)];
+              const float2 u = x[i][j], w = x[i][j + 1];
+              cfma2(acc[i >> NKX][j >> NKY], make_float4(u.x, u.y, w.x, w.y), v);
+              x[i][j] = x[i][j + 1] = make_float2(0.f, 0.f);
+            }
+        }
       } else {
-#pragma unroll
-        for (int i = 0; i < N; ++i)
-#pragma unroll
-          for (int j = 0; j < N; ++j) acc[i][j] = x[i][j];
+        products(0, 0);
       }
+      buf ^= 1;
     }
-    float2* dst = P.out + s_out + ro;
+    float2* dst = s_out[slot] + ro;
 #pragma unroll
     for (int i = 0; i < XO; ++i)
 #pragma unroll
@@ -246,16 +296,18 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
         const int ri = i << NKX, rj = j << NKY;
         const int o = ((ri & 1) ? P.xo[0] : 0) + ((ri & 2) ? P.xo[1] : 0) + ((rj & 1) ? P.yo[0] : 0) +
                       ((rj & 2) ? P.yo[1] : 0);
-        dst[o] = acc[i][j];
-        tmax = fmaxf(tmax, fmaxf(fabsf(acc[i][j].x), fabsf(acc[i][j].y)));
+        const float2 r = HASC ? acc[i][j] : x[i][j];
+        dst[o] = r;
+        tmax = fmaxf(tmax, fmaxf(fabsf(r.x), fabsf(r.y)));
       }
-    if (h == 0 && t == 0) {
+    if (t == 0 && (tile & ((1ll << P.n_h) - 1ll)) == 0) {
       int e = 0;
-      for (int j = 0; j < P.n_gin; ++j) e += s_e[j];
+      for (int j = 0; j < P.n_gin; ++j) e += s_e[n_item % RING][j];
       P.meta_e[(long long)P.out_meta * P.B + (P.out_dep ? item : 0ll)] = e;
     }
+    if (new_item || !more) flush(item);
+    n_item += new_item;
   }
-  if (cur_item >= 0) flush(cur_item);
 }
 
 using PairKernel = void (*)(PairParams, long long);

@@ -21,13 +21,13 @@ constexpr int PF_MAX = 8;           // fold table of one operand: at most 2^8 pa
 constexpr int PIN_MAX = 16;         // tensors a chain reads
 constexpr int PH_MAX = 32;          // tile bits
 constexpr int PK_MAX = 5;           // eliminated variables of one loop
-constexpr int PAIR_SMEM_MAX = 100 * 1024;  // dynamic shared memory of one block: two fit an SM
+constexpr int PAIR_SMEM_TWO = 88 * 1024;   // two stages of one block's operands, so that two blocks fit an SM
+constexpr int PAIR_SMEM_MAX = 200 * 1024;  // ... or one
 
 // One tensor that the chain reads from memory.
 struct PIn {
   const float2* ptr;
   long long istride;            // per item (0 if item-invariant)
-  int hstride[PH_MAX];          // per tile bit
   int meta;                     // meta row (-1: gate tensor, unit scale)
   int dep;
 };
@@ -36,18 +36,21 @@ struct PIn {
 // by an index e (bits by increasing memory stride, so that consecutive threads
 // read consecutive memory); bit i of e adds g[i] to the global offset
 // (elements), d[i] to the shared-memory slot (16-byte units) and f[i] to the
-// fold table's index.
+// fold table's index. Tile bit i adds h[i] and fh[i], chunk 1 adds gch and fch.
 struct POp {
   int gin;
   int ebits;
   int g[PE_MAX], d[PE_MAX], f[PE_MAX];
-  int base;                     // first slot
+  int h[PH_MAX], fh[PH_MAX];
+  int gch, fch;
+  int base;                     // first slot of a stage
 };
 
-// Small tensors folded into one operand: table of (u_0 = 0, u_0 = 1) pairs.
+// Small tensors folded into one operand: table of (u_0 = 0, u_0 = 1) pairs
+// over the other variables that they hold, tile variables included: it depends
+// on the item alone.
 struct PFold {
   int n, nf;                    // tensors, table index bits
-  int inv;                      // 1: no folded tensor holds a tile bit
   int gin[PIN_MAX], ustride[PIN_MAX];
   int fs[PIN_MAX][PF_MAX];      // element stride of table index bit b
 };
@@ -58,14 +61,16 @@ struct PairParams {
   PFold fa, fb;
   float2* out;
   long long out_istride;
-  long long out_hstride[PH_MAX];
+  int out_h[PH_MAX];            // per tile bit
   int ta[PTB], tb[PTB], tc[PTB], to[PTB];  // thread bits: slots of a, b, c; output offset
   int xa[PR], xc[PR], xo[PR];   // register bits along A: slots of a and c, output offset (0 for a K2 bit)
   int yb[PR], yc[PR], yo[PR];   // register bits along B
-  int n1, k1a[PK_MAX], k1b[PK_MAX];                // K1 without u_0: slots of a and b
+  int n1, k1a[PK_MAX], k1b[PK_MAX];                // K1 without u_0 and the chunk's variable: slots of a and b
   int n2, k2a[PK_MAX], k2b[PK_MAX], k2c[PK_MAX];   // K2 outside the register tile
   int nkx, nky;                 // K2 bits among the register bits along A / B (the low ones)
+  int n_ch;                     // chunks of a tile: 2 when one summed variable is split off, else 1
   int n_h, n_gin, out_meta, out_dep, B;
+  int stage;                    // slots of one stage; dynamic shared memory holds two
   int smem;                     // dynamic shared memory bytes
   int* meta_e;
   unsigned* meta_m;

@@ -1900,12 +1900,9 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
     PFold& F = side ? G.fb : G.fa;
     const std::vector<int>& S = side ? sb : sa;
     std::vector<int>& fv = fold_vars[side];
-    F.inv = 1;
     for (int j : S)
-      for (int v : vars(j)) {
-        if (index_in(tile, v) >= 0) F.inv = 0;
-        else if (v != u0 && index_in(fv, v) < 0) fv.push_back(v);
-      }
+      for (int v : vars(j))
+        if (v != u0 && index_in(fv, v) < 0) fv.push_back(v);
     F.nf = (int)fv.size();
     if (F.nf > PF_MAX) return false;
     for (int j : S) {
@@ -1919,6 +1916,22 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
       ++F.n;
     }
   }
+  // two stages that leave no room for a second block are split into two chunks
+  // by one summed variable of both operands (the one that keeps the longest
+  // runs of memory together); a chain with C keeps its sums in the register
+  // tile's order and is not split
+  int chunk = -1;
+  {
+    double total = 0;
+    for (int k = 0; k < 3; ++k)
+      if (ops[k] >= 0) total += std::ldexp(1.0, bits[k] - 1) * 1.05;
+    if (2 * 16 * total > PAIR_SMEM_TWO && C < 0) {
+      for (int v : k1)
+        if (holds(A, v) && holds(B, v) && (chunk < 0 || index_in(vars(A), v) > index_in(vars(A), chunk))) chunk = v;
+      if (chunk >= 0) k1.erase(std::find(k1.begin(), k1.end(), chunk));
+    }
+  }
+  G.n_ch = chunk < 0 ? 1 : 2;
   // staged operands: slot = row + pitch * (its eliminated variables but bit
   // 0), rows numbered by the thread bits it holds, then by its register
   // outputs; the odd pitch and the lowest row bits on the lowest lanes keep
@@ -1945,20 +1958,29 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
     const int pitch = (1 << rows) | 1;
     int nk = 0;
     for (size_t p = 1; p < v.size(); ++p)
-      if (index_in(K, v[p]) >= 0) w[p] = pitch << nk++;
+      if (v[p] != chunk && index_in(K, v[p]) >= 0) w[p] = pitch << nk++;
     O.base = base;
     base += pitch << nk;
     for (size_t p = 1; p < v.size(); ++p) {
-      if (index_in(tile, v[p]) >= 0) continue;
-      if (O.ebits >= PE_MAX || p > 30) return false;
-      O.g[O.ebits] = 1 << p;
-      O.d[O.ebits] = w[p];
-      const int f = k < 2 ? index_in(fold_vars[k], v[p]) : -1;
-      O.f[O.ebits] = f < 0 ? 0 : 1 << f;
-      ++O.ebits;
+      if (p > 30) return false;
+      const int fi = k < 2 ? index_in(fold_vars[k], v[p]) : -1, f = fi < 0 ? 0 : 1 << fi;
+      const int h = index_in(tile, v[p]);
+      if (h >= 0) {
+        O.h[h] = 1 << p;
+        O.fh[h] = f;
+      } else if (v[p] == chunk) {
+        O.gch = 1 << p;
+        O.fch = f;
+      } else {
+        if (O.ebits >= PE_MAX) return false;
+        O.g[O.ebits] = 1 << p;
+        O.d[O.ebits] = w[p];
+        O.f[O.ebits++] = f;
+      }
     }
   }
-  G.smem = base * 16;
+  G.stage = base;
+  G.smem = 2 * base * 16;
   if (G.smem > PAIR_SMEM_MAX) return false;
   auto slot = [&](int k, int v) {
     const int p = ops[k] < 0 ? -1 : index_in(vars(ops[k]), v);
@@ -1998,7 +2020,7 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
   G.out_dep = L.dep[g.output];
   G.out = reinterpret_cast<float2*>((size_t)L.off[g.output] * 8);
   G.out_istride = 1ll << o.rank();
-  for (int i = 0; i < G.n_h; ++i) G.out_hstride[i] = out_of(tile[i]);
+  for (int i = 0; i < G.n_h; ++i) G.out_h[i] = out_of(tile[i]);
   for (int j = 0; j < G.n_gin; ++j) {
     const PTensor& x = prog.tensors[in[j]];
     PIn& I = G.gin[j];
@@ -2006,11 +2028,6 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
     I.dep = L.dep[in[j]];
     I.istride = 1ll << x.rank();
     I.meta = x.leaf_gate >= 0 ? -1 : in[j];
-    for (int i = 0; i < G.n_h; ++i) {
-      const int p = index_in(x.vars, tile[i]);
-      if (p > 30) return false;
-      I.hstride[i] = p < 0 ? 0 : 1 << p;
-    }
   }
   return true;
 }
@@ -2386,29 +2403,28 @@ static std::string validate_config(const tnq_plan& P, int mode, int B) {
     const FusedGroup& g = prog.groups[C.step_group[si]];
     const std::string name = "pair chain " + std::to_string(si);
     const long long items = G.out_dep ? B : 1;
-    auto tile_max = [&](int j) {
-      long long m = G.gin[j].dep ? (items - 1) * G.gin[j].istride : 0;
-      for (int i = 0; i < G.n_h; ++i) m += G.gin[j].hstride[i];
-      return m;
-    };
-    if (G.smem > PAIR_SMEM_MAX) return name + ": shared memory";
+    auto item_max = [&](int j) { return G.gin[j].dep ? (items - 1) * G.gin[j].istride : 0ll; };
+    if (G.smem > PAIR_SMEM_MAX || G.smem != 2 * 16 * G.stage) return name + ": shared memory";
     const POp* ops[3] = {&G.a, &G.b, &G.c};
     for (int k = 0; k < 3; ++k) {
       const POp& O = *ops[k];
       if (O.gin < 0) continue;
-      long long m = tile_max(O.gin) + 1;
-      int d = O.base, f = 0;
+      long long m = item_max(O.gin) + 1 + (G.n_ch > 1 ? O.gch : 0);
+      int d = O.base, f = G.n_ch > 1 ? O.fch : 0;
+      for (int i = 0; i < G.n_h; ++i) {
+        if (O.h[i] & 1) return name + ": odd tile stride";
+        m += O.h[i];
+        f += O.fh[i];
+      }
       for (int i = 0; i < O.ebits; ++i) {
-        if (O.g[i] & 1) return name + ": odd local stride";
+        if ((O.g[i] & 1) || (O.gch & 1)) return name + ": odd local stride";
         m += O.g[i];
         d += O.d[i];
         f += O.f[i];
       }
-      for (int i = 0; i < G.n_h; ++i)
-        if (G.gin[O.gin].hstride[i] & 1) return name + ": odd tile stride";
       if ((G.gin[O.gin].istride & 1) || ((size_t)G.gin[O.gin].ptr / 8) % 2) return name + ": unaligned input";
       if (m >= alloc(g.ext_inputs[O.gin])) return name + ": staged input overflows";
-      if (d >= G.smem / 16) return name + ": staged operand outside shared memory";
+      if (d >= G.stage) return name + ": staged operand outside its stage";
       if (k < 2 && f >= 1 << (k ? G.fb.nf : G.fa.nf)) return name + ": fold index";
       // the register tile reads only staged slots
       long long r = O.base;
@@ -2420,14 +2436,15 @@ static std::string validate_config(const tnq_plan& P, int mode, int B) {
     }
     for (int side = 0; side < 2; ++side) {
       const PFold& F = side ? G.fb : G.fa;
+      if (F.nf > PF_MAX) return name + ": fold table";
       for (int j = 0; j < F.n; ++j) {
-        long long m = tile_max(F.gin[j]) + F.ustride[j];
+        long long m = item_max(F.gin[j]) + F.ustride[j];
         for (int b = 0; b < F.nf; ++b) m += F.fs[j][b];
         if (m >= alloc(g.ext_inputs[F.gin[j]])) return name + ": folded input overflows";
       }
     }
     long long om = G.out_dep ? (items - 1) * G.out_istride : 0;
-    for (int i = 0; i < G.n_h; ++i) om += G.out_hstride[i];
+    for (int i = 0; i < G.n_h; ++i) om += G.out_h[i];
     for (int i = 0; i < PTB; ++i) om += G.to[i];
     for (int i = 0; i < PR; ++i) om += G.xo[i] + G.yo[i];
     if (om >= alloc(g.output)) return name + ": output overflows";
@@ -2933,10 +2950,10 @@ int tnq_internal_group_text(const tnq_plan* plan, int mode, uint32_t batch, char
     if (C.pair_of[gi] >= 0) {
       const PairParams& Q = C.pp[C.pair_of[gi]];
       out += "  pair: a " + std::to_string(Q.a.ebits) + " b " + std::to_string(Q.b.ebits) + " c " +
-             std::to_string(Q.c.gin < 0 ? -1 : Q.c.ebits) + " n1 " + std::to_string(Q.n1) + " n2 " +
+             std::to_string(Q.c.gin < 0 ? -1 : Q.c.ebits) + " n1 " + std::to_string(Q.n1 + Q.n_ch - 1) + " n2 " +
              std::to_string(Q.n2) + " nkx " + std::to_string(Q.nkx) + " nky " + std::to_string(Q.nky) + " n_h " +
              std::to_string(Q.n_h) + " folds " + std::to_string(Q.fa.n) + "+" + std::to_string(Q.fb.n) + " nf " +
-             std::to_string(Q.fa.nf) + "+" + std::to_string(Q.fb.nf) + " inv " + std::to_string(Q.fa.inv && Q.fb.inv) +
+             std::to_string(Q.fa.nf) + "+" + std::to_string(Q.fb.nf) + " chunks " + std::to_string(Q.n_ch) +
              " smem " + std::to_string(Q.smem) + "\n";
     }
     for (int j = 0; j < G.n_gin; ++j) {
