@@ -41,9 +41,11 @@ __device__ __forceinline__ void cfma2(float2& r, float4 a, float4 b) {
 // or two chunks of its summed values. Two stages: while a chunk is computed,
 // the next one's part of A, B (and C) comes in by cp.async; each thread then
 // multiplies what it copied by the fold tables in place, and after one barrier
-// every thread computes a 4 x 4 register tile: per pair of summed values 4 + 4
-// 16-byte shared loads feed 128 FMAs.
-template <int NKX, int NKY, bool HASC>
+// every thread computes 4 x 2^RY register tiles: per pair of summed values 4 + 2^RY
+// 16-byte shared loads feed 32 x 2^RY FMAs. Shared memory delivers 128 bytes a
+// cycle to registers, so 4 x 4 needs all of it at the full FMA rate and 4 x 8
+// three quarters.
+template <int RY, int NKX, int NKY, bool HASC>
 __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairParams P, long long n_tiles) {
   extern __shared__ float4 sm[];
   constexpr int NOP = HASC ? 3 : 2;
@@ -51,6 +53,7 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
   __shared__ float4 s_fa[2][1 << PF_MAX], s_fb[2][1 << PF_MAX];  // by item, alternating
   __shared__ int4 s_it[NOP][1 << (PE_MAX - PTB)];  // staging iteration: global offset, slot, fold index
   __shared__ int4 s_k2[1 << PK_MAX];               // K2 outside the register tile: slots of a, b, c
+  __shared__ int4 s_l[1 << PL_MAX];                // a thread's loop: slots of a, b, c, output offset
   __shared__ int2 s_k1[1 << PK_MAX];               // K1 pairs of a chunk: slots of a, b
   __shared__ int s_hstr[6][PH_MAX];
   __shared__ const float2* s_src[RING][3];
@@ -59,7 +62,7 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
   __shared__ float s_sc[PIN_MAX];
   __shared__ int s_e[RING][PIN_MAX];
   __shared__ float s_red[PTPB / 32];
-  constexpr int N = 1 << PR;
+  constexpr int NX = 1 << PRX, NY = 1 << RY;
   const int t = threadIdx.x, lane = t & 31;
   const POp* ops[3] = {&P.a, &P.b, &P.c};
   // ---- tables that every tile uses
@@ -85,6 +88,17 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
         w.y += P.k1b[i];
       }
     s_k1[t] = w;
+  }
+  if (t < (1 << PL_MAX)) {
+    int4 v = make_int4(0, 0, 0, 0);
+    for (int i = 0; i < P.nl; ++i)
+      if ((t >> i) & 1) {
+        v.x += P.la[i];
+        v.y += P.lb[i];
+        v.z += P.lc[i];
+        v.w += P.lo[i];
+      }
+    s_l[t] = v;
   }
   int tg[NOP], td[NOP], tf[NOP];  // this thread's part of the staging offsets
 #pragma unroll
@@ -220,20 +234,16 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
   __syncthreads();
   issue(0, 0, 0);
   int slot = 0;
-  constexpr int XO = N >> NKX, YO = N >> NKY;
+  constexpr int XO = NX >> NKX, YO = NY >> NKY;
   for (long long tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, slot = (slot + 1) % RING) {
     const long long item = tile >> P.n_h, next = tile + gridDim.x;
     const bool more = next < n_tiles;
     const bool new_item = more && (next >> P.n_h) != item;
-    float2 x[N][N], acc[XO][YO];
+    float2 x[NX][NY];  // sums of A B
 #pragma unroll
-    for (int i = 0; i < N; ++i)
+    for (int i = 0; i < NX; ++i)
 #pragma unroll
-      for (int j = 0; j < N; ++j) x[i][j] = make_float2(0.f, 0.f);
-#pragma unroll
-    for (int i = 0; i < XO; ++i)
-#pragma unroll
-      for (int j = 0; j < YO; ++j) acc[i][j] = make_float2(0.f, 0.f);
+      for (int j = 0; j < NY; ++j) x[i][j] = make_float2(0.f, 0.f);
     for (int c = 0; c < P.n_ch; ++c) {
       const bool last = c + 1 == P.n_ch;
       if (last && more) {
@@ -247,59 +257,78 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
       else if (more) issue((slot + 1) % RING, 0, buf ^ 1);
       const float4* pa = sm + buf * P.stage + ra;
       const float4* pb = sm + buf * P.stage + rb;
+      float2* dst = s_out[slot] + ro;
       const int n1 = 1 << P.n1;
       auto products = [&](int oa, int ob) {
 #pragma unroll 1
         for (int q = 0; q < n1; ++q) {
           const int2 k = s_k1[q];
-          float4 va[N], vb[N];
+          const float4* qa = pa + (oa + k.x);
+          const float4* qb = pb + (ob + k.y);
+          float4 va[NX];
 #pragma unroll
-          for (int i = 0; i < N; ++i)
-            va[i] = pa[oa + k.x + ((i & 1) ? P.xa[0] : 0) + ((i & 2) ? P.xa[1] : 0)];
+          for (int i = 0; i < NX; ++i) va[i] = qa[((i & 1) ? P.xa[0] : 0) + ((i & 2) ? P.xa[1] : 0)];
 #pragma unroll
-          for (int j = 0; j < N; ++j)
-            vb[j] = pb[ob + k.y + ((j & 1) ? P.yb[0] : 0) + ((j & 2) ? P.yb[1] : 0)];
+          for (int j = 0; j < NY; ++j) {
+            const float4 vb =
+                qb[((j & 1) ? P.yb[0] : 0) + ((j & 2) ? P.yb[1] : 0) + (RY > 2 && (j & 4) ? P.yb[2] : 0)];
 #pragma unroll
-          for (int i = 0; i < N; ++i)
-#pragma unroll
-            for (int j = 0; j < N; ++j) cfma2(x[i][j], va[i], vb[j]);
+            for (int i = 0; i < NX; ++i) cfma2(x[i][j], va[i], vb);
+          }
         }
       };
-      if constexpr (HASC) {
-        const int n2 = 1 << P.n2;
+      auto store = [&](int i, int j, float2 r, int lo) {
+        const int ri = i << NKX, rj = j << NKY;
+        dst[lo + ((ri & 1) ? P.xo[0] : 0) + ((ri & 2) ? P.xo[1] : 0) + ((rj & 1) ? P.yo[0] : 0) +
+            ((rj & 2) ? P.yo[1] : 0) + (RY > 2 && (rj & 4) ? P.yo[2] : 0)] = r;
+        tmax = fmaxf(tmax, fmaxf(fabsf(r.x), fabsf(r.y)));
+      };
+      const int nl = 1 << P.nl;
 #pragma unroll 1
-        for (int q2 = 0; q2 < n2; ++q2) {
-          const int4 k2 = s_k2[q2];
-          products(k2.x, k2.y);
-          // times C, summed over the K2 register bits (C's bit 0 is B's register bit 0)
-          const float4* pc = sm + buf * P.stage + rc + k2.z;
+      for (int l = 0; l < nl; ++l) {
+        const int4 lv = s_l[l];
+        if constexpr (HASC) {
+          float2 acc[XO][YO];
 #pragma unroll
-          for (int i = 0; i < N; ++i)
+          for (int i = 0; i < XO; ++i)
 #pragma unroll
-            for (int j = 0; j < N; j += 2) {
-              const float4 v = pc[((i & 1) ? P.xc[0] : 0) + ((i & 2) ? P.xc[1] : 0) + ((j & 2) ? P.yc[1] : 0)];
-              const float2 u = x[i][j], w = x[i][j + 1];
-              cfma2(acc[i >> NKX][j >> NKY], make_float4(u.x, u.y, w.x, w.y), v);
-              x[i][j] = x[i][j + 1] = make_float2(0.f, 0.f);
-            }
+            for (int j = 0; j < YO; ++j) acc[i][j] = make_float2(0.f, 0.f);
+          const int n2 = 1 << P.n2;
+#pragma unroll 1
+          for (int q2 = 0; q2 < n2; ++q2) {
+            const int4 k2 = s_k2[q2];
+            products(lv.x + k2.x, lv.y + k2.y);
+            // times C, summed over the K2 register bits (C's bit 0 is B's register bit 0)
+            const float4* pc = sm + buf * P.stage + rc + lv.z + k2.z;
+#pragma unroll
+            for (int i = 0; i < NX; ++i)
+#pragma unroll
+              for (int j = 0; j < NY; j += 2) {
+                const float4 v = pc[((i & 1) ? P.xc[0] : 0) + ((i & 2) ? P.xc[1] : 0) + ((j & 2) ? P.yc[1] : 0)];
+                const float2 u = x[i][j], w = x[i][j + 1];
+                cfma2(acc[i >> NKX][j >> NKY], make_float4(u.x, u.y, w.x, w.y), v);
+                x[i][j] = x[i][j + 1] = make_float2(0.f, 0.f);
+              }
+          }
+#pragma unroll
+          for (int i = 0; i < XO; ++i)
+#pragma unroll
+            for (int j = 0; j < YO; ++j) store(i, j, acc[i][j], lv.w);
+        } else {
+          products(lv.x, lv.y);
+          if (last) {
+#pragma unroll
+            for (int i = 0; i < NX; ++i)
+#pragma unroll
+              for (int j = 0; j < NY; ++j) {
+                store(i, j, x[i][j], lv.w);
+                x[i][j] = make_float2(0.f, 0.f);
+              }
+          }
         }
-      } else {
-        products(0, 0);
       }
       buf ^= 1;
     }
-    float2* dst = s_out[slot] + ro;
-#pragma unroll
-    for (int i = 0; i < XO; ++i)
-#pragma unroll
-      for (int j = 0; j < YO; ++j) {
-        const int ri = i << NKX, rj = j << NKY;
-        const int o = ((ri & 1) ? P.xo[0] : 0) + ((ri & 2) ? P.xo[1] : 0) + ((rj & 1) ? P.yo[0] : 0) +
-                      ((rj & 2) ? P.yo[1] : 0);
-        const float2 r = HASC ? acc[i][j] : x[i][j];
-        dst[o] = r;
-        tmax = fmaxf(tmax, fmaxf(fabsf(r.x), fabsf(r.y)));
-      }
     if (t == 0 && (tile & ((1ll << P.n_h) - 1ll)) == 0) {
       int e = 0;
       for (int j = 0; j < P.n_gin; ++j) e += s_e[n_item % RING][j];
@@ -312,14 +341,14 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
 
 using PairKernel = void (*)(PairParams, long long);
 static PairKernel pair_kernel(const PairParams& p) {
-  if (p.c.gin < 0) return k_pair<0, 0, false>;
+  if (p.c.gin < 0) return p.ry > 2 ? k_pair<3, 0, 0, false> : k_pair<2, 0, 0, false>;
   switch (p.nkx * 4 + p.nky) {
-    case 1: return k_pair<0, 1, true>;
-    case 2: return k_pair<0, 2, true>;
-    case 5: return k_pair<1, 1, true>;
-    case 6: return k_pair<1, 2, true>;
-    case 9: return k_pair<2, 1, true>;
-    default: return k_pair<2, 2, true>;
+    case 1: return k_pair<2, 0, 1, true>;
+    case 2: return k_pair<2, 0, 2, true>;
+    case 5: return k_pair<2, 1, 1, true>;
+    case 6: return k_pair<2, 1, 2, true>;
+    case 9: return k_pair<2, 2, 1, true>;
+    default: return k_pair<2, 2, 2, true>;
   }
 }
 

@@ -15,13 +15,15 @@ namespace tnq {
 
 constexpr int PTB = 8;              // log2 threads per k_pair block
 constexpr int PTPB = 1 << PTB;
-constexpr int PR = 2;               // register tile: 2^PR entries along A's variables x 2^PR along B's
+constexpr int PRX = 2;              // register tile: 2^PRX entries along A's variables ...
+constexpr int PRY_MAX = 3;          // ... x 2^2 or (two large tensors) 2^3 along B's
 constexpr int PE_MAX = 13;          // staged (u = 0, u = 1) pairs of one operand: at most 2^13
-constexpr int PF_MAX = 8;           // fold table of one operand: at most 2^8 pairs
+constexpr int PF_MAX = 7;           // fold table of one operand: at most 2^8 pairs
 constexpr int PIN_MAX = 16;         // tensors a chain reads
 constexpr int PH_MAX = 32;          // tile bits
+constexpr int PL_MAX = 3;            // output variables of a thread's loop
 constexpr int PK_MAX = 5;           // eliminated variables of one loop
-constexpr int PAIR_SMEM_TWO = 88 * 1024;   // two stages of one block's operands, so that two blocks fit an SM
+constexpr int PAIR_SMEM_TWO = 98 * 1024;   // two stages of one block's operands, so that two blocks fit an SM
 constexpr int PAIR_SMEM_MAX = 200 * 1024;  // ... or one
 
 // One tensor that the chain reads from memory.
@@ -63,8 +65,10 @@ struct PairParams {
   long long out_istride;
   int out_h[PH_MAX];            // per tile bit
   int ta[PTB], tb[PTB], tc[PTB], to[PTB];  // thread bits: slots of a, b, c; output offset
-  int xa[PR], xc[PR], xo[PR];   // register bits along A: slots of a and c, output offset (0 for a K2 bit)
-  int yb[PR], yc[PR], yo[PR];   // register bits along B
+  int xa[PRX], xc[PRX], xo[PRX];               // register bits along A: slots of a and c, output offset (0 for a K2 bit)
+  int yb[PRY_MAX], yc[PRY_MAX], yo[PRY_MAX];   // register bits along B
+  int ry;                       // register bits along B
+  int nl, la[PL_MAX], lb[PL_MAX], lc[PL_MAX], lo[PL_MAX];  // a thread's loop over outputs
   int n1, k1a[PK_MAX], k1b[PK_MAX];                // K1 without u_0 and the chunk's variable: slots of a and b
   int n2, k2a[PK_MAX], k2b[PK_MAX], k2c[PK_MAX];   // K2 outside the register tile
   int nkx, nky;                 // K2 bits among the register bits along A / B (the low ones)

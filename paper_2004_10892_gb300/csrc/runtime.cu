@@ -1779,10 +1779,12 @@ static GParams group_gparams(const tnq_plan& P, const Layout& L, const FusedGrou
 //    tensors is what the register tile shares operands over;
 //  * every other tensor has its variables among A's or among B's: it is
 //    multiplied into that operand as it is staged;
-//  * at least 2^PR register entries along variables of A alone and of B alone
+//  * 2^PRX register entries along variables of A alone and 2^2 along B's
 //    (eliminated variables of C count): without them nothing is shared;
 //  * 2^PTB threads times the register tile of outputs.
 constexpr int PAIR_SMALL = 4;
+constexpr int PAIR_TILES = 5;
+constexpr int PAIR_LOOP = 4;  // a thread sums 2^PAIR_LOOP pairs per 4 x 4 outputs of a tile where the operands allow it
 static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g, PairParams& G) {
   const Program& prog = P.prog;
   std::memset(&G, 0, sizeof(G));
@@ -1830,18 +1832,27 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
     if (v == u0 || v == c0) continue;
     if (!holds(A, v) && !holds(B, v)) return false;
     if (!holds(C, v)) k1.push_back(v);
-    else if (holds(A, v) && !holds(B, v) && (int)xreg.size() < PR) xreg.push_back(v);
-    else if (holds(B, v) && !holds(A, v) && (int)yreg.size() < PR) yreg.push_back(v);
+    else if (holds(A, v) && !holds(B, v) && (int)xreg.size() < PRX) xreg.push_back(v);
+    else if (holds(B, v) && !holds(A, v) && (int)yreg.size() < 2) yreg.push_back(v);
     else k2.push_back(v);
   }
   G.nkx = (int)xreg.size();
   G.nky = (int)yreg.size();
+  // 4 x 8 register tiles for two tensors that have the variables, and outputs
+  // for 2^PAIR_TILES tiles an item (fewer leave the device idle), else 4 x 4
+  int only_b = 0;
+  for (int v : o.vars) only_b += holds(B, v) && !holds(A, v);
+  G.ry = C < 0 && only_b >= 3 && o.rank() >= PTB + PRX + 3 + PAIR_TILES ? 3 : 2;
+  const int need_x = PRX - G.nkx, need_y = G.ry - G.nky, n_one = PTB + need_x + need_y;
+  if (o.rank() < n_one) return false;
+  const int ops[3] = {A, B, C};
   // local output variables: the two earliest (the output is written in 32-byte
   // runs), then the one that adds the fewest staged entries, as long as enough
-  // variables of A alone and of B alone stay for the register tile
-  const int need_x = PR - G.nkx, need_y = PR - G.nky, n_local = PTB + need_x + need_y;
-  if (o.rank() < n_local) return false;
-  const int ops[3] = {A, B, C};
+  // variables of A alone and of B alone stay for the register tile. A tile of
+  // few sums takes more outputs, which its threads loop over, as long as two
+  // blocks fit an SM: the tile's set-up and barrier then count less.
+  std::vector<char> local(o.vars.size(), 0);
+  int nx = 0, ny = 0, n_local = n_one;
   int bits[3] = {0, 0, 0};
   for (int k = 0; k < 3; ++k)
     for (int v : K) bits[k] += holds(ops[k], v);
@@ -1851,8 +1862,7 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
       if (ops[k] >= 0) n += std::ldexp(1.0, b[k] - 1);
     return n;
   };
-  std::vector<char> local(o.vars.size(), 0);
-  int nx = 0, ny = 0;
+  std::vector<int> loop;
   for (int n = 0; n < n_local; ++n) {
     int best = -1;
     double best_cost = 0;
@@ -1871,27 +1881,36 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
       if (i == n && n < 2) break;  // the two earliest variables first
     }
     if (best < 0) return false;
+    if (n >= n_one) {
+      if (2 * 16 * 1.05 * best_cost > PAIR_SMEM_TWO) break;
+      loop.push_back(o.vars[best]);
+    }
     local[best] = 1;
     for (int k = 0; k < 3; ++k) bits[k] += holds(ops[k], o.vars[best]);
     nx += holds(A, o.vars[best]) && !holds(B, o.vars[best]);
     ny += holds(B, o.vars[best]) && !holds(A, o.vars[best]);
+    if (n + 1 == n_local && (int)loop.size() < PL_MAX && n_local + PAIR_TILES < o.rank() &&
+        (int)(k1.size() + k2.size()) + n_local - n_one + G.ry - 2 < PAIR_LOOP)
+      ++n_local;
   }
   // register bits: the latest local variables of A alone / B alone; the other
   // local variables are thread bits, the earliest lowest
   std::vector<char> is_reg(o.vars.size(), 0);
   for (int side = 0; side < 2; ++side) {
     std::vector<int>& reg = side ? yreg : xreg;
-    for (int i = (int)o.vars.size() - 1; i >= 0 && (int)reg.size() < PR; --i)
-      if (local[i] && holds(side ? B : A, o.vars[i]) && !holds(side ? A : B, o.vars[i])) {
+    const int want = side ? G.ry : PRX;
+    for (int i = (int)o.vars.size() - 1; i >= 0 && (int)reg.size() < want; --i)
+      if (local[i] && index_in(loop, o.vars[i]) < 0 && holds(side ? B : A, o.vars[i]) &&
+          !holds(side ? A : B, o.vars[i])) {
         reg.push_back(o.vars[i]);
         is_reg[i] = 1;
       }
-    if ((int)reg.size() < PR) return false;
+    if ((int)reg.size() < want) return false;
   }
   std::vector<int> thr, tile;
   for (int i = 0; i < (int)o.vars.size(); ++i) {
     if (!local[i]) tile.push_back(o.vars[i]);
-    else if (!is_reg[i]) thr.push_back(o.vars[i]);
+    else if (!is_reg[i] && index_in(loop, o.vars[i]) < 0) thr.push_back(o.vars[i]);
   }
   if ((int)thr.size() != PTB || (int)tile.size() >= PH_MAX) return false;
   // fold tables
@@ -1925,7 +1944,7 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
     double total = 0;
     for (int k = 0; k < 3; ++k)
       if (ops[k] >= 0) total += std::ldexp(1.0, bits[k] - 1) * 1.05;
-    if (2 * 16 * total > PAIR_SMEM_TWO && C < 0) {
+    if (2 * 16 * total > PAIR_SMEM_TWO && C < 0 && loop.empty()) {
       for (int v : k1)
         if (holds(A, v) && holds(B, v) && (chunk < 0 || index_in(vars(A), v) > index_in(vars(A), chunk))) chunk = v;
       if (chunk >= 0) k1.erase(std::find(k1.begin(), k1.end(), chunk));
@@ -1951,6 +1970,7 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
       if (p >= 0) w[p] = 1 << rows++;
     };
     for (int x : thr) row(x);
+    for (int x : loop) row(x);
     for (int x : xreg)
       if (index_in(K, x) < 0) row(x);
     for (int x : yreg)
@@ -1996,13 +2016,21 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
     G.tc[i] = slot(2, thr[i]);
     G.to[i] = out_of(thr[i]);
   }
-  for (int i = 0; i < PR; ++i) {
+  for (int i = 0; i < PRX; ++i) {
     G.xa[i] = slot(0, xreg[i]);
     G.xc[i] = slot(2, xreg[i]);
     G.xo[i] = out_of(xreg[i]);
+  }
+  for (int i = 0; i < G.ry; ++i) {
     G.yb[i] = slot(1, yreg[i]);
     G.yc[i] = slot(2, yreg[i]);
     G.yo[i] = out_of(yreg[i]);
+  }
+  for (int v : loop) {
+    G.la[G.nl] = slot(0, v);
+    G.lb[G.nl] = slot(1, v);
+    G.lc[G.nl] = slot(2, v);
+    G.lo[G.nl++] = out_of(v);
   }
   for (int v : k1) {
     G.k1a[G.n1] = slot(0, v);
@@ -2429,7 +2457,11 @@ static std::string validate_config(const tnq_plan& P, int mode, int B) {
       // the register tile reads only staged slots
       long long r = O.base;
       for (int i = 0; i < PTB; ++i) r += k == 0 ? G.ta[i] : (k == 1 ? G.tb[i] : G.tc[i]);
-      for (int i = 0; i < PR; ++i) r += k == 0 ? G.xa[i] : (k == 1 ? G.yb[i] : G.xc[i] + (i ? G.yc[i] : 0));
+      if (k != 1)
+        for (int i = 0; i < PRX; ++i) r += k == 0 ? G.xa[i] : G.xc[i];
+      if (k != 0)  // (C is read in pairs over B's register bit 0)
+        for (int i = k == 2; i < G.ry; ++i) r += k == 1 ? G.yb[i] : G.yc[i];
+      for (int i = 0; i < G.nl; ++i) r += k == 0 ? G.la[i] : (k == 1 ? G.lb[i] : G.lc[i]);
       for (int i = 0; i < G.n1; ++i) r += k == 0 ? G.k1a[i] : (k == 1 ? G.k1b[i] : 0);
       for (int i = 0; i < G.n2; ++i) r += k == 0 ? G.k2a[i] : (k == 1 ? G.k2b[i] : G.k2c[i]);
       if (r > d) return name + ": register tile outside the staged operand";
@@ -2446,7 +2478,9 @@ static std::string validate_config(const tnq_plan& P, int mode, int B) {
     long long om = G.out_dep ? (items - 1) * G.out_istride : 0;
     for (int i = 0; i < G.n_h; ++i) om += G.out_h[i];
     for (int i = 0; i < PTB; ++i) om += G.to[i];
-    for (int i = 0; i < PR; ++i) om += G.xo[i] + G.yo[i];
+    for (int i = 0; i < PRX; ++i) om += G.xo[i];
+    for (int i = 0; i < G.ry; ++i) om += G.yo[i];
+    for (int i = 0; i < G.nl; ++i) om += G.lo[i];
     if (om >= alloc(g.output)) return name + ": output overflows";
   }
   for (size_t gi = 0; gi < C.gb.size(); ++gi) {
@@ -2953,7 +2987,7 @@ int tnq_internal_group_text(const tnq_plan* plan, int mode, uint32_t batch, char
              std::to_string(Q.c.gin < 0 ? -1 : Q.c.ebits) + " n1 " + std::to_string(Q.n1 + Q.n_ch - 1) + " n2 " +
              std::to_string(Q.n2) + " nkx " + std::to_string(Q.nkx) + " nky " + std::to_string(Q.nky) + " n_h " +
              std::to_string(Q.n_h) + " folds " + std::to_string(Q.fa.n) + "+" + std::to_string(Q.fb.n) + " nf " +
-             std::to_string(Q.fa.nf) + "+" + std::to_string(Q.fb.nf) + " chunks " + std::to_string(Q.n_ch) +
+             std::to_string(Q.fa.nf) + "+" + std::to_string(Q.fb.nf) + " chunks " + std::to_string(Q.n_ch) + " ry " + std::to_string(Q.ry) + " loop " + std::to_string(Q.nl) +
              " smem " + std::to_string(Q.smem) + "\n";
     }
     for (int j = 0; j < G.n_gin; ++j) {
