@@ -284,6 +284,11 @@ __device__ __forceinline__ void epilogue_warps(const GemmArgs& a, uint32_t tmem_
   }
 }
 
+// Batch entries that hold valid items.
+__device__ __forceinline__ long long valid_batch(const GemmArgs& a) {
+  return a.n_items ? (long long)*a.n_items << a.item_ns : (long long)a.batch;
+}
+
 // Persistent, warp-specialised GEMM. Each block loops over output tiles
 // tile = blockIdx.x + i * gridDim.x (tile -> batch b, row tile rt, column
 // tile ct, ct fastest). Warp 0 (one thread) streams the four 16 KB operand
@@ -306,7 +311,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) k_gemm_tc(const GemmArgs a) {
   __shared__ int s_epi_stop[2];  // per tile parity: an epilogue thread's wait failed (set once, never cleared)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  const long long n_tiles = (long long)a.batch * a.row_tiles_a * a.row_tiles_b;
+  const long long n_tiles = valid_batch(a) * a.row_tiles_a * a.row_tiles_b;
   if (tid == 0) {
     for (int s = 0; s < N_STAGES; ++s) {
       mbar_init(&full_bar[s], 1);
@@ -449,7 +454,7 @@ __global__ void __launch_bounds__(GEMM_THREADS_FA, 1) k_gemm_tc_fa(const GemmArg
   __shared__ int s_epi_stop[2];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  const long long n_tiles = (long long)a.batch * a.row_tiles_a * a.row_tiles_b;
+  const long long n_tiles = valid_batch(a) * a.row_tiles_a * a.row_tiles_b;
   constexpr int HB = GT_TILE_BYTES_H;
   if (tid == 0) {
     for (int s = 0; s < N_STAGES; ++s) {
@@ -771,7 +776,8 @@ __global__ void k_gemm_pack(const GemmBucketArgs g, int side, int pack_items) {
   const int nops = side == 0 ? g.na : g.nb;
   const int nr = side == 0 ? g.nx : g.ny;
   const long long rows = side == 0 ? g.m_pad : g.n_pad;  // complex rows
-  const long long batch = (long long)pack_items << g.ns;  // 1 item when the side does not depend on it
+  // 1 item when the side does not depend on it, else the batch's valid ones
+  const long long batch = (long long)(pack_items > 1 ? min(pack_items, *g.n_items) : 1) << g.ns;
   const int kch = g.k_pad / CH;  // chunks per row (k_pad is a multiple of 64 / ES)
   const long long n = batch * rows * kch;
   constexpr int KB = HALF ? GT_KBYTES_H : GT_KBYTES;  // bytes of K per tile row
@@ -1098,6 +1104,8 @@ void gemm_bucket_launch(const GemmBucketArgs& g, const GemmEpilogue& ep, int* st
   a.batch = (int)batch;
   a.a_bmask = inv_a ? (1ll << g.ns) - 1 : -1ll;
   a.b_bmask = inv_b ? (1ll << g.ns) - 1 : -1ll;
+  a.n_items = g.items > 1 ? g.n_items : nullptr;
+  a.item_ns = g.ns;
   a.status = status;
   a.out_c = nullptr;
   a.ep = ep;

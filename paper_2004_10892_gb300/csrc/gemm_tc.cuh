@@ -69,6 +69,7 @@ struct GemmBucketArgs {
   int out_meta, out_dep, B;
   int* meta_e;
   unsigned* meta_m;
+  const int* n_items;          // valid items of the batch (device)
 };
 
 // Epilogue data of a bucket GEMM (in GemmArgs when out_c is null).
@@ -91,6 +92,9 @@ struct GemmArgs {
   int row_tiles_b;   // rows of B / 128 (columns of C / 128)
   int k_tiles;       // Kr bytes / 128
   int batch;
+  // valid items of the batch (device; null: the whole batch) and batch entries per item (log2)
+  const int* n_items;
+  int item_ns;
   // batch index of an operand's tiles: b & mask (all ones; or 2^ns - 1 when
   // the operand does not depend on the item, packed once for all items)
   long long a_bmask, b_bmask;

@@ -58,6 +58,7 @@ struct KParams {
   int B;                         // meta row length
   int* meta_e;
   unsigned* meta_m;
+  const int* n_items;            // valid items of the batch (device)
 };
 
 // One early bucket of a level launch (k_bucket_level): like KParams for an
@@ -105,7 +106,7 @@ struct BatchHdr {
   int mode;                      // 0: item = slice of bitstring 0; 1: item = (bitstring << p) | slice
   int p;
   int n_words;                   // 32-bit words per bitstring
-  int pad;
+  int n_items;                   // valid items of the batch, at most its size: the kernels leave the others out
 };
 
 __device__ __forceinline__ void item_decode(const BatchHdr& h, int item, unsigned long long* slice, int* brow,
@@ -136,7 +137,7 @@ __global__ void k_leaf_init(const LeafDev* __restrict__ leaves, int n_leaves, co
   if (idx >= (long long)n_leaves * B) return;
   const int li = (int)(idx / B), item = (int)(idx % B);
   const LeafDev L = leaves[li];
-  if (!L.dep && item) return;
+  if (item >= (L.dep ? h.n_items : 1)) return;
   unsigned long long slice;
   int brow;
   bool valid;
@@ -201,7 +202,8 @@ __global__ void __launch_bounds__(TPB, 5) k_bucket(const __grid_constant__ KPara
   __shared__ float4 sh_c[ITER];  // product of the thread-invariant inputs per iteration (pair over u)
   const int t = threadIdx.x;
   const long long g0 = (long long)blockIdx.x << LT;
-  const long long total = 1ll << P.G;
+  const long long total = P.G > P.out_bits ? (long long)*P.n_items << P.out_bits : 1ll << P.G;
+  if (g0 >= total) return;
 
   for (int e = t; e < NIN * ITER; e += TPB) {
     const int j = e / ITER, it = e - (e / ITER) * ITER;
@@ -374,7 +376,8 @@ __global__ void __launch_bounds__(TPB, 5) k_bucket(const __grid_constant__ KPara
 // the item above their output bits; their scales, exponents and maxima are
 // per item, as in k_bucket, and so is the arithmetic order.
 __global__ void __launch_bounds__(256) k_bucket_level(const HoistDev* __restrict__ hd, int n, char* arena,
-                                                     int* meta_e, unsigned* meta_m, int B) {
+                                                     int* meta_e, unsigned* meta_m, int B,
+                                                     const int* __restrict__ n_items) {
   __shared__ int s_b;
   __shared__ long long s_str[KMAX][HOIST_MAX_BITS];
   __shared__ const float2* s_in[KMAX];
@@ -396,6 +399,8 @@ __global__ void __launch_bounds__(256) k_bucket_level(const HoistDev* __restrict
   const int nin = H.nin, bits = H.bits, ob = H.obits;
   const long long g0 = (long long)(blockIdx.x - H.blk0) * 256;
   const bool uniform = ob >= 8 || ob == bits;  // one item for the whole block
+  const long long total = H.out_dep ? (long long)*n_items << ob : 1ll << bits;
+  if (g0 >= total) return;
   for (int e = t; e < nin * bits; e += 256) s_str[e / bits][e % bits] = H.stride[e / bits][e % bits];
   if (t < nin) s_in[t] = reinterpret_cast<const float2*>(arena + H.in[t]);
   if (uniform && t == 0) {  // the block's item: scales and the output exponent
@@ -417,7 +422,7 @@ __global__ void __launch_bounds__(256) k_bucket_level(const HoistDev* __restrict
   const long long g = g0 + t;
   const long long item = g >> ob;
   float mx = 0.f;
-  if (g < (1ll << bits)) {
+  if (g < total) {
     // scale of input j for this entry's item
     auto scale = [&](int j) -> float {
       if (uniform) return s_f[j];
@@ -476,7 +481,7 @@ __global__ void __launch_bounds__(256) k_bucket_level(const HoistDev* __restrict
     // items change every 2^ob entries: reduce within aligned lane groups
     const int grp = 1 << (ob < 5 ? ob : 5);
     for (int off = 1; off < grp; off <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-    if ((t & (grp - 1)) == 0 && mx > 0.f && g < (1ll << bits))
+    if ((t & (grp - 1)) == 0 && mx > 0.f && g < total)
       atomic_max_pos(&meta_m[(long long)H.out_meta * B + (H.out_dep ? item : 0ll)], mx);
   }
 }
@@ -535,6 +540,7 @@ struct GParams {
   int lean2;                   // 1: two stages, stage 1 reads stage 0 densely and writes the output (k_group<2>)
   int* meta_e;
   unsigned* meta_m;
+  const int* n_items;          // valid items of the batch (device)
 };
 
 // Stage buffers in shared memory are stored swizzled: complex entry o sits at
@@ -995,6 +1001,7 @@ __global__ void __launch_bounds__(GTPB, TK ? 5 : 4) k_group(const __grid_constan
   for (int i = 0; i < GTB && i < nb_last; ++i)
     if ((t >> i) & 1) out_lo += P.out_cstride[i];
   const int buf_elems = 1 << (GL_MAX - 1);
+  if (P.out_dep) n_tiles = (long long)*P.n_items << P.n_h;
   long long cur_item = -1;
   long long meta_item = -1;  // item whose exponents and scales s_e / s_F hold
   float tmax = 0.f;
@@ -2649,7 +2656,7 @@ static void launch_bucket(const KParams& k, int n_in, int LT, cudaStream_t s) {
 // Launches step i of the configuration (a single bucket or a fused group)
 // with its pointers rebased on the arena.
 static void launch_step(const ExecConfig& C, int i, float2* arena, int* me, unsigned* mm, int* status,
-                        cudaStream_t s) {
+                        const int* n_items, cudaStream_t s) {
   char* base = reinterpret_cast<char*>(arena);
   const auto st = C.steps[i];
   if (st.first == 0) {
@@ -2659,6 +2666,7 @@ static void launch_step(const ExecConfig& C, int i, float2* arena, int* me, unsi
       k.in[j] = reinterpret_cast<const float2*>(base + reinterpret_cast<size_t>(k.in[j]));
     k.meta_e = me;
     k.meta_m = mm;
+    k.n_items = n_items;
     launch_bucket(k, C.kshape[st.second].first, C.kshape[st.second].second, s);
   } else if (st.first == 2) {
     GemmBucketArgs g = C.gb[st.second];
@@ -2672,6 +2680,7 @@ static void launch_step(const ExecConfig& C, int i, float2* arena, int* me, unsi
     g.b_lo = base + reinterpret_cast<size_t>(g.b_lo);
     g.meta_e = me;
     g.meta_m = mm;
+    g.n_items = n_items;
     e.out = reinterpret_cast<float2*>(base + reinterpret_cast<size_t>(e.out));
     e.meta_m = mm;
     gemm_bucket_launch(g, e, status, s);
@@ -2682,6 +2691,7 @@ static void launch_step(const ExecConfig& C, int i, float2* arena, int* me, unsi
       g.gin[j].ptr = reinterpret_cast<const float2*>(base + reinterpret_cast<size_t>(g.gin[j].ptr));
     g.meta_e = me;
     g.meta_m = mm;
+    g.n_items = n_items;
     const long long tiles = (g.out_dep ? (long long)g.B : 1ll) << g.n_h;
     pair_launch(g, tiles, C.ggrid.empty() ? C.group_grid : C.ggrid[st.second], s);
   } else {
@@ -2690,6 +2700,7 @@ static void launch_step(const ExecConfig& C, int i, float2* arena, int* me, unsi
     for (int j = 0; j < g.n_gin; ++j) g.gin[j].ptr = reinterpret_cast<const float2*>(base + reinterpret_cast<size_t>(g.gin[j].ptr));
     g.meta_e = me;
     g.meta_m = mm;
+    g.n_items = n_items;
     const long long tiles = (g.out_dep ? (long long)g.B : 1ll) << g.n_h;
     const long long grid =
         std::min<long long>(tiles, (long long)(C.ggrid.empty() ? C.group_grid : C.ggrid[st.second]));
@@ -2734,10 +2745,11 @@ static void enqueue_batch(const tnq_plan& P, ExecConfig& C, char* ws, cudaStream
   for (size_t l = 0; l + 1 < C.hoist_first.size(); ++l)
     k_bucket_level<<<(unsigned)C.hoist_blocks[l], 256, 0, s>>>(C.d_hoist + C.hoist_first[l],
                                                                  C.hoist_first[l + 1] - C.hoist_first[l],
-                                                                 reinterpret_cast<char*>(arena), me, mm, B);
+                                                                 reinterpret_cast<char*>(arena), me, mm, B,
+                                                                 &hdr->n_items);
   if (!side) {
     for (size_t i = 0; i < C.steps.size(); ++i)
-      if (!C.step_hoist[i]) launch_step(C, (int)i, arena, me, mm, status, s);
+      if (!C.step_hoist[i]) launch_step(C, (int)i, arena, me, mm, status, &hdr->n_items, s);
   } else {
     cudaEventRecord(side->fork, s);
     for (int k = 0; k < N_SIDE_STREAMS; ++k) cudaStreamWaitEvent(side->st[k], side->fork, 0);
@@ -2745,7 +2757,7 @@ static void enqueue_batch(const tnq_plan& P, ExecConfig& C, char* ws, cudaStream
       const int k = C.step_stream[i];
       for (int j : C.step_deps[i])
         if (C.step_stream[j] != k) cudaStreamWaitEvent(side->st[k], side->done[j], 0);
-      if (!C.step_hoist[i]) launch_step(C, (int)i, arena, me, mm, status, side->st[k]);
+      if (!C.step_hoist[i]) launch_step(C, (int)i, arena, me, mm, status, &hdr->n_items, side->st[k]);
       cudaEventRecord(side->done[i], side->st[k]);
     }
     for (int k = 0; k < N_SIDE_STREAMS; ++k) {
@@ -3129,6 +3141,7 @@ static tnq_status profile_steps(const tnq_plan* plan, const uint8_t* bits, uint6
   std::memset(&h, 0, sizeof(h));
   h.item_base = s0;
   h.item_end = s1;
+  h.n_items = (int)std::min<uint64_t>(B, s1 - s0);
   h.p = (int)plan->mu.size();
   h.n_words = C->L.n_words;
   CU(cudaMemcpyAsync(ws + C->L.hdr_off, &h, sizeof(h), cudaMemcpyHostToDevice, s));
@@ -3149,7 +3162,7 @@ static tnq_status profile_steps(const tnq_plan* plan, const uint8_t* bits, uint6
   for (auto& e : ev) CU(cudaEventCreate(&e));
   for (int i = 0; i < nbk; ++i) {
     CU(cudaEventRecord(ev[2 * i], s));
-    launch_step(*C, i, arena, me, mm, reinterpret_cast<int*>(ws + L.status_off), s);
+    launch_step(*C, i, arena, me, mm, reinterpret_cast<int*>(ws + L.status_off), &hdr->n_items, s);
     CU(cudaEventRecord(ev[2 * i + 1], s));
   }
   CU(cudaGetLastError());
@@ -3531,6 +3544,7 @@ tnq_status tnq_contract_sliced(const tnq_plan* plan, const uint8_t* bits, uint64
     std::memset(&h, 0, sizeof(h));
     h.item_base = base;
     h.item_end = slice_end;
+    h.n_items = (int)std::min<uint64_t>(B, slice_end - base);
     h.mode = 0;
     h.p = (int)plan->mu.size();
     h.n_words = C->L.n_words;
@@ -3678,6 +3692,7 @@ tnq_status tnq_amplitudes_batch(const tnq_plan* const* plans, size_t n_plans, co
         std::memset(&h, 0, sizeof(h));
         h.item_base = base;
         h.item_end = n_items;
+        h.n_items = (int)(end - base);
         h.bstr_base = b0;
         h.mode = 1;
         h.p = p;
@@ -3953,6 +3968,7 @@ tnq_status tnq_contract_sliced_noalloc(const tnq_plan* plan, const uint8_t* bits
     std::memset(&h, 0, sizeof(h));
     h.item_base = b0;
     h.item_end = slice_end;
+    h.n_items = (int)std::min<uint64_t>(B, slice_end - b0);
     h.p = (int)plan->mu.size();
     h.n_words = C.L.n_words;
     CU(cudaMemcpyAsync(ws + C.L.hdr_off, &h, sizeof(h), cudaMemcpyHostToDevice, s));
