@@ -69,7 +69,7 @@ struct GemmBucketArgs {
   int out_meta, out_dep, B;
   int* meta_e;
   unsigned* meta_m;
-  const int* n_items;          // valid items of the batch (device)
+  const int* n_items;          // valid items of the batch (device; null: the batch is one item)
 };
 
 // Epilogue data of a bucket GEMM (in GemmArgs when out_c is null).

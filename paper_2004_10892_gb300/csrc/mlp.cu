@@ -4,8 +4,16 @@
 // W1 (H x F), b1 (H), W2 (H x H), b2 (H), W3 (H), b3 (1), weights row-major
 // (output x input). Every reduction runs in a fixed order (no atomics), so
 // a training step is deterministic.
+//
+// A backward pass is six launches: two layers forward, the head (prediction,
+// its derivative and the loss's partial sums), the hidden layer backward, and
+// every parameter's gradient over chunks of rows, added up in chunk order.
+// What bounds it: at a training batch of 1024 rows the launches (each matrix
+// has 8 to 64 tiles); at 10^5 rows the FP32 pipe, through the shared-memory
+// loads of an 8 x 8 register tile.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <string>
 
 #include "../../include/tnq.h"
@@ -14,68 +22,257 @@ namespace tnq {
 void set_error(const std::string& msg);
 
 namespace {
-constexpr int TS = 16;  // matmul tile
+constexpr int MT = 128;  // threads of a matrix tile
+constexpr int MK = 16;   // summed values per shared-memory step
 
-// C[M x P] = opA(A) . opB(B) (+ bias[P]) (ReLU if relu): opA(A) is M x K
-// (A stored M x K, or K x M when ta), opB(B) is K x P (B stored P x K when
-// tb, else K x P). FP32 accumulation over K in increasing order.
-__global__ void k_mm(const float* __restrict__ A, const float* __restrict__ B, const float* __restrict__ bias,
-                     float* __restrict__ C, int M, int K, int P, int ta, int tb, int relu) {
-  __shared__ float sa[TS][TS + 1], sb[TS][TS + 1];
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  const int row = blockIdx.y * TS + ty, col = blockIdx.x * TS + tx;
-  float acc = 0.f;
-  for (int k0 = 0; k0 < K; k0 += TS) {
-    const int ka = k0 + tx, kb = k0 + ty;
-    float va = 0.f, vb = 0.f;
-    if (row < M && ka < K) va = ta ? A[(size_t)ka * M + row] : A[(size_t)row * K + ka];
-    if (col < P && kb < K) vb = tb ? B[(size_t)col * K + kb] : B[(size_t)kb * P + col];
-    sa[ty][tx] = va;
-    sb[ty][tx] = vb;
+// acc += A B over k in [k0, k1), in increasing order, for the tile of 16 TM x
+// 8 TM results at (m0, p0); la(m, k) and lb(p, k) are the operands inside M x P.
+// LA / LB::kfast: consecutive k (else consecutive m / p) are consecutive memory.
+template <int TM, class LA, class LB>
+__device__ __forceinline__ void tile_product(const LA& la, const LB& lb, int m0, int p0, int M, int P, int k0, int k1,
+                                             float (&acc)[TM][TM], float* sh) {
+  constexpr int BM = 16 * TM, BN = 8 * TM;
+  constexpr int NA = BM * MK / MT, NB = BN * MK / MT;
+  float(*sa)[BM + 4] = reinterpret_cast<float(*)[BM + 4]>(sh);
+  float(*sb)[BN + 4] = reinterpret_cast<float(*)[BN + 4]>(sh + MK * (BM + 4));
+  const int t = threadIdx.x, tx = t & 7, ty = t >> 3;
+  float ra[NA], rb[NB];
+  auto place = [&](bool kfast, int e, int B, int* row, int* k) {
+    *k = kfast ? e % MK : e / B;
+    *row = kfast ? e / MK : e % B;
+  };
+  auto fetch = [&](int kb) {
+#pragma unroll
+    for (int i = 0; i < NA; ++i) {
+      int r, k;
+      place(LA::kfast, t + i * MT, BM, &r, &k);
+      ra[i] = m0 + r < M && kb + k < k1 ? la(m0 + r, kb + k) : 0.f;
+    }
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+      int r, k;
+      place(LB::kfast, t + i * MT, BN, &r, &k);
+      rb[i] = p0 + r < P && kb + k < k1 ? lb(p0 + r, kb + k) : 0.f;
+    }
+  };
+  fetch(k0);
+  for (int kb = k0; kb < k1; kb += MK) {
     __syncthreads();
 #pragma unroll
-    for (int k = 0; k < TS; ++k) acc += sa[ty][k] * sb[k][tx];
+    for (int i = 0; i < NA; ++i) {
+      int r, k;
+      place(LA::kfast, t + i * MT, BM, &r, &k);
+      sa[k][r] = ra[i];
+    }
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+      int r, k;
+      place(LB::kfast, t + i * MT, BN, &r, &k);
+      sb[k][r] = rb[i];
+    }
     __syncthreads();
-  }
-  if (row < M && col < P) {
-    if (bias) acc += bias[col];
-    if (relu) acc = acc > 0.f ? acc : 0.f;
-    C[(size_t)row * P + col] = acc;
+    if (kb + MK < k1) fetch(kb + MK);  // in flight while this step is computed
+#pragma unroll
+    for (int k = 0; k < MK; ++k) {
+      float a[TM], b[TM];
+#pragma unroll
+      for (int i = 0; i < TM; i += 4) {  // rows 4 ty (+ 64), columns 4 tx (+ 32)
+        const float4 va = *reinterpret_cast<const float4*>(&sa[k][4 * ty + 16 * i]);
+        const float4 vb = *reinterpret_cast<const float4*>(&sb[k][4 * tx + 8 * i]);
+        a[i] = va.x, a[i + 1] = va.y, a[i + 2] = va.z, a[i + 3] = va.w;
+        b[i] = vb.x, b[i + 1] = vb.y, b[i + 2] = vb.z, b[i + 3] = vb.w;
+      }
+#pragma unroll
+      for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < TM; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+    }
   }
 }
+template <int TM>
+constexpr int tile_floats() { return MK * (16 * TM + 4 + 8 * TM + 4); }
+// Row / column of acc[i][j] within the tile.
+__device__ __forceinline__ int tile_row(int i) { return 4 * (threadIdx.x >> 3) + 64 * (i >> 2) + (i & 3); }
+__device__ __forceinline__ int tile_col(int j) { return 4 * (threadIdx.x & 7) + 32 * (j >> 2) + (j & 3); }
 
-// g[i] *= (z[i] > 0): ReLU derivative applied to an upstream gradient.
-__global__ void k_relu_mask(float* __restrict__ g, const float* __restrict__ z, size_t n) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-    if (!(z[i] > 0.f)) g[i] = 0.f;
+struct RowMajor {  // X[row][k]
+  static constexpr bool kfast = true;
+  const float* p;
+  int ld;
+  __device__ float operator()(int r, int k) const { return p[(size_t)r * ld + k]; }
+};
+struct ColMajor {  // X[k][row]
+  static constexpr bool kfast = false;
+  const float* p;
+  int ld;
+  __device__ float operator()(int r, int k) const { return p[(size_t)k * ld + r]; }
+};
+// dZ2[i][j] = dP[i] W3[j] where H2[i][j] > 0, read by rows (kfast) or by columns
+template <bool K>
+struct HeadGrad {
+  static constexpr bool kfast = K;
+  const float *dP, *W3, *H2;
+  int H;
+  __device__ float at(int i, int j) const { return H2[(size_t)i * H + j] > 0.f ? dP[i] * W3[j] : 0.f; }
+  __device__ float operator()(int r, int k) const { return K ? at(r, k) : at(k, r); }
+};
+
+// C = relu(A W^T + b): A (M x K), W (P x K)
+template <int TM>
+__global__ void __launch_bounds__(MT) k_layer(const float* __restrict__ A, const float* __restrict__ W,
+                                              const float* __restrict__ bias, float* __restrict__ C, int M, int K,
+                                              int P) {
+  __shared__ __align__(16) float sh[tile_floats<TM>()];
+  const int m0 = blockIdx.x * 16 * TM, p0 = blockIdx.y * 8 * TM;
+  float acc[TM][TM] = {};
+  tile_product<TM>(RowMajor{A, K}, RowMajor{W, K}, m0, p0, M, P, 0, K, acc, sh);
+#pragma unroll
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < TM; ++j) {
+      const int r = m0 + tile_row(i), c = p0 + tile_col(j);
+      if (r < M && c < P) {
+        const float v = acc[i][j] + bias[c];
+        C[(size_t)r * P + c] = v > 0.f ? v : 0.f;
+      }
+    }
 }
 
-// out[c] = sum_r X[r, c] over rows in increasing order (one thread per column).
-__global__ void k_colsum(const float* __restrict__ X, float* __restrict__ out, int rows, int cols) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= cols) return;
+// dZ1 = (dZ2 W2) where H1 > 0
+template <int TM>
+__global__ void __launch_bounds__(MT) k_hidden_back(HeadGrad<true> dZ2, const float* __restrict__ W2,
+                                                    const float* __restrict__ H1, float* __restrict__ dZ1, int M,
+                                                    int H) {
+  __shared__ __align__(16) float sh[tile_floats<TM>()];
+  const int m0 = blockIdx.x * 16 * TM, p0 = blockIdx.y * 8 * TM;
+  float acc[TM][TM] = {};
+  tile_product<TM>(dZ2, ColMajor{W2, H}, m0, p0, M, H, 0, H, acc, sh);
+#pragma unroll
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < TM; ++j) {
+      const int r = m0 + tile_row(i), c = p0 + tile_col(j);
+      if (r < M && c < H) dZ1[(size_t)r * H + c] = H1[(size_t)r * H + c] > 0.f ? acc[i][j] : 0.f;
+    }
+}
+
+constexpr int HEAD_ROWS = 8;  // rows per block of k_head: one per warp
+
+// pred[i] = H2[i] . W3 + b3; with y: dP[i] = (pred[i] - y[i]) / n and the
+// block's partial sum of (pred - y)^2, else out[i] = pred[i].
+__global__ void __launch_bounds__(32 * HEAD_ROWS) k_head(const float* __restrict__ H2, const float* __restrict__ W3,
+                                                         const float* __restrict__ b3, const float* __restrict__ y,
+                                                         float* __restrict__ out, float* __restrict__ part, int n,
+                                                         int H) {
+  __shared__ float s_sq[HEAD_ROWS];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, i = blockIdx.x * HEAD_ROWS + w;
   float a = 0.f;
-  for (int r = 0; r < rows; ++r) a += X[(size_t)r * cols + c];
-  out[c] = a;
-}
-
-// d[i] = (pred[i] - y[i]) / n ; loss = sum (pred - y)^2 / (2n), summed in order by one block.
-__global__ void k_mse(const float* __restrict__ pred, const float* __restrict__ y, float* __restrict__ d,
-                      float* __restrict__ loss, int n) {
-  __shared__ float part[256];
-  float a = 0.f;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const float e = pred[i] - y[i];
-    d[i] = e / (float)n;
-    a += e * e;
+  if (i < n)
+    for (int k = lane; k < H; k += 32) a = fmaf(H2[(size_t)i * H + k], W3[k], a);
+  for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
+  a += *b3;
+  if (!y) {
+    if (i < n && lane == 0) out[i] = a;
+    return;
   }
-  part[threadIdx.x] = a;
+  const float e = i < n ? a - y[i] : 0.f;
+  if (i < n && lane == 0) out[i] = e / (float)n;
+  if (lane == 0) s_sq[w] = e * e;
   __syncthreads();
-  if (threadIdx.x == 0 && loss) {
-    float t = 0.f;
-    for (int i = 0; i < (int)blockDim.x; ++i) t += part[i];
-    *loss = t / (2.f * (float)n);
+  if (threadIdx.x == 0) {
+    float s = 0.f;
+    for (int q = 0; q < HEAD_ROWS; ++q) s += s_sq[q];
+    part[blockIdx.x] = s;
   }
+}
+
+struct GradArgs {
+  const float *x, *H1, *H2, *W3, *dP, *dZ1;
+  float* part;         // chunk c's sums at part + c * stride, laid out like the parameters
+  size_t stride;
+  int n, F, H, rows;   // rows per chunk
+  int t2, t1;          // tiles of W2 and W1
+};
+
+// One chunk's part of every gradient (blockIdx.y): blocks 0..t2-1 tiles of dW2
+// = dZ2^T H1, then t1 tiles of dW1 = dZ1^T x, then blocks of MT columns of the
+// biases' and W3's sums.
+template <int TM>
+__global__ void __launch_bounds__(MT) k_grads(const GradArgs g) {
+  __shared__ __align__(16) float sh[tile_floats<TM>()];
+  const int r0 = blockIdx.y * g.rows, r1 = min(g.n, r0 + g.rows);
+  float* W1 = g.part + blockIdx.y * g.stride;
+  float* b1 = W1 + (size_t)g.H * g.F;
+  float* W2 = b1 + g.H;
+  float* b2 = W2 + (size_t)g.H * g.H;
+  float* W3 = b2 + g.H;
+  int b = blockIdx.x;
+  const HeadGrad<false> dZ2{g.dP, g.W3, g.H2, g.H};
+  if (b < g.t2 + g.t1) {
+    const bool second = b < g.t2;
+    if (!second) b -= g.t2;
+    const int P = second ? g.H : g.F, cols = (P + 8 * TM - 1) / (8 * TM);
+    const int m0 = b / cols * 16 * TM, p0 = b % cols * 8 * TM;
+    float acc[TM][TM] = {};
+    if (second) tile_product<TM>(dZ2, ColMajor{g.H1, g.H}, m0, p0, g.H, P, r0, r1, acc, sh);
+    else tile_product<TM>(ColMajor{g.dZ1, g.H}, ColMajor{g.x, g.F}, m0, p0, g.H, P, r0, r1, acc, sh);
+    float* dst = second ? W2 : W1;
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+      for (int j = 0; j < TM; ++j) {
+        const int r = m0 + tile_row(i), c = p0 + tile_col(j);
+        if (r < g.H && c < P) dst[(size_t)r * P + c] = acc[i][j];
+      }
+    return;
+  }
+  b -= g.t2 + g.t1;
+  const int c = b * MT + threadIdx.x;
+  if (c < g.H) {
+    float s1 = 0.f, s2 = 0.f, s3 = 0.f;
+    const float w3 = g.W3[c];
+#pragma unroll 4
+    for (int r = r0; r < r1; ++r) {
+      const float h2 = g.H2[(size_t)r * g.H + c], d = g.dP[r];
+      s1 += g.dZ1[(size_t)r * g.H + c];
+      s2 += h2 > 0.f ? d * w3 : 0.f;
+      s3 = fmaf(d, h2, s3);
+    }
+    b1[c] = s1;
+    b2[c] = s2;
+    W3[c] = s3;
+  }
+  if (b == 0 && threadIdx.x < 32) {  // db3: lanes in turn, then over the lanes
+    float s = 0.f;
+    for (int r = r0 + (int)threadIdx.x; r < r1; r += 32) s += g.dP[r];
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if (threadIdx.x == 0) W3[g.H] = s;
+  }
+}
+
+// grads = the chunks' sums in chunk order (part == grads: they are there
+// already); the last block adds the loss's partial sums, in a fixed order.
+__global__ void __launch_bounds__(256) k_add_up(const float* part, size_t stride, int chunks, float* grads, size_t count,
+                                                const float* __restrict__ sq, int n_sq, float* loss, float scale) {
+  if (blockIdx.x + 1 == gridDim.x) {
+    __shared__ float s[256];
+    float a = 0.f;
+    for (int i = threadIdx.x; i < n_sq; i += 256) a += sq[i];
+    s[threadIdx.x] = a;
+    __syncthreads();
+    for (int off = 128; off > 0; off >>= 1) {
+      if ((int)threadIdx.x < off) s[threadIdx.x] += s[threadIdx.x + off];
+      __syncthreads();
+    }
+    if (threadIdx.x == 0 && loss) *loss = s[0] * scale;
+    return;
+  }
+  const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
+  if (part == grads || i >= count) return;
+  float a = 0.f;
+#pragma unroll 8
+  for (int c = 0; c < chunks; ++c) a += part[c * stride + i];
+  grads[i] = a;
 }
 
 // SGD with momentum: v = mu v + g ; w -= lr v.
@@ -86,12 +283,6 @@ __global__ void k_sgd(float* __restrict__ w, const float* __restrict__ g, float*
     v[i] = vi;
     w[i] -= lr * vi;
   }
-}
-
-void mm(const float* A, const float* B, const float* bias, float* C, int M, int K, int P, int ta, int tb, int relu,
-       cudaStream_t s) {
-  dim3 blk(TS, TS), grd((P + TS - 1) / TS, (M + TS - 1) / TS);
-  k_mm<<<grd, blk, 0, s>>>(A, B, bias, C, M, K, P, ta, tb, relu);
 }
 
 struct Views {
@@ -106,6 +297,17 @@ Views views(const float* p, int F, int H) {
   v.W3 = v.b2 + H;
   v.b3 = v.W3 + H;
   return v;
+}
+
+int up(int a, int b) { return (a + b - 1) / b; }
+
+// 128 x 64 tiles from MLP_LARGE rows up, else 64 x 32: at 1024 rows 64 small
+// tiles of a 128-wide layer keep four times as many SMs busy as 16 large ones.
+constexpr int MLP_LARGE = 16384;
+
+void layer(const float* A, const float* W, const float* bias, float* C, int M, int K, int P, cudaStream_t s) {
+  if (M >= MLP_LARGE) k_layer<8><<<dim3(up(M, 128), up(P, 64)), MT, 0, s>>>(A, W, bias, C, M, K, P);
+  else k_layer<4><<<dim3(up(M, 64), up(P, 32)), MT, 0, s>>>(A, W, bias, C, M, K, P);
 }
 }  // namespace
 }  // namespace tnq
@@ -128,9 +330,9 @@ tnq_status tnq_mlp_forward(const float* params, int32_t hidden, const float* x, 
   Views v = views(params, F, H);
   float* H1 = work;
   float* H2 = H1 + (size_t)N * H;
-  mm(x, v.W1, v.b1, H1, N, F, H, 0, 1, 1, s);
-  mm(H1, v.W2, v.b2, H2, N, H, H, 0, 1, 1, s);
-  mm(H2, v.W3, v.b3, out, N, H, 1, 0, 1, 0, s);
+  layer(x, v.W1, v.b1, H1, N, F, H, s);
+  layer(H1, v.W2, v.b2, H2, N, H, H, s);
+  k_head<<<up(N, HEAD_ROWS), 32 * HEAD_ROWS, 0, s>>>(H2, v.W3, v.b3, nullptr, out, nullptr, N, H);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) { set_error(cudaGetErrorString(e)); return TNQ_ECUDA; }
   return TNQ_OK;
@@ -144,41 +346,40 @@ tnq_status tnq_mlp_backward(const float* params, int32_t hidden, const float* x,
   const int F = tnq_learned_features(), H = hidden, N = (int)n;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   Views v = views(params, F, H);
-  float* Z1 = work;                       // N x H pre-activations, then dZ1
-  float* H1 = Z1 + (size_t)N * H;         // N x H
-  float* Z2 = H1 + (size_t)N * H;         // N x H, then dZ2
-  float* H2 = Z2 + (size_t)N * H;         // N x H
-  float* D = H2 + (size_t)N * H;          // N x H scratch (dH)
-  float* P = D + (size_t)N * H;           // N
-  float* dP = P + N;                      // N
-  float* g_W1 = grads;
-  float* g_b1 = g_W1 + (size_t)H * F;
-  float* g_W2 = g_b1 + H;
-  float* g_b2 = g_W2 + (size_t)H * H;
-  float* g_W3 = g_b2 + H;
-  float* g_b3 = g_W3 + H;
-  // forward, keeping pre-activations
-  mm(x, v.W1, v.b1, Z1, N, F, H, 0, 1, 0, s);
-  mm(x, v.W1, v.b1, H1, N, F, H, 0, 1, 1, s);
-  mm(H1, v.W2, v.b2, Z2, N, H, H, 0, 1, 0, s);
-  mm(H1, v.W2, v.b2, H2, N, H, H, 0, 1, 1, s);
-  mm(H2, v.W3, v.b3, P, N, H, 1, 0, 1, 0, s);
-  k_mse<<<1, 256, 0, s>>>(P, y, dP, loss, N);
-  // layer 3: dW3 = dP^T H2 ; db3 = sum dP ; dH2 = dP W3
-  mm(dP, H2, nullptr, g_W3, 1, N, H, 1, 0, 0, s);
-  k_colsum<<<1, 32, 0, s>>>(dP, g_b3, N, 1);
-  mm(dP, v.W3, nullptr, D, N, 1, H, 0, 0, 0, s);
-  // layer 2
-  const size_t nh = (size_t)N * H;
-  const int blocks = (int)((nh + 255) / 256 < 4096 ? (nh + 255) / 256 : 4096);
-  k_relu_mask<<<blocks, 256, 0, s>>>(D, Z2, nh);  // D = dZ2
-  mm(D, H1, nullptr, g_W2, H, N, H, 1, 0, 0, s);
-  k_colsum<<<(H + 127) / 128, 128, 0, s>>>(D, g_b2, N, H);
-  mm(D, v.W2, nullptr, Z2, N, H, H, 0, 0, 0, s);  // Z2 <- dH1
-  // layer 1
-  k_relu_mask<<<blocks, 256, 0, s>>>(Z2, Z1, nh);  // Z2 = dZ1
-  mm(Z2, x, nullptr, g_W1, H, N, F, 1, 0, 0, s);
-  k_colsum<<<(H + 127) / 128, 128, 0, s>>>(Z2, g_b1, N, H);
+  const size_t nh = (size_t)N * H, count = (size_t)H * F + H + (size_t)H * H + 2 * (size_t)H + 1;
+  float* H1 = work;         // N x H
+  float* H2 = H1 + nh;      // N x H
+  float* dZ1 = H2 + nh;     // N x H
+  float* dP = dZ1 + nh;     // N
+  float* sq = dP + N;       // N: the loss's partial sums
+  float* part = sq + N;     // the rest of the workspace, 2 N H + 2 N + 16 floats: the chunks' gradients
+  const bool large = N >= MLP_LARGE;
+  const int tm = large ? 128 : 64, tp = large ? 64 : 32;
+  layer(x, v.W1, v.b1, H1, N, F, H, s);
+  layer(H1, v.W2, v.b2, H2, N, H, H, s);
+  const int n_sq = up(N, HEAD_ROWS);
+  k_head<<<n_sq, 32 * HEAD_ROWS, 0, s>>>(H2, v.W3, v.b3, y, dP, sq, N, H);
+  const HeadGrad<true> dZ2{dP, v.W3, H2, H};
+  if (large) k_hidden_back<8><<<dim3(up(N, 128), up(H, 64)), MT, 0, s>>>(dZ2, v.W2, H1, dZ1, N, H);
+  else k_hidden_back<4><<<dim3(up(N, 64), up(H, 32)), MT, 0, s>>>(dZ2, v.W2, H1, dZ1, N, H);
+  // chunks of at least 64 rows (512 when large), as many as the workspace holds; one writes grads itself
+  const size_t room = (2 * nh + 2 * (size_t)N + 16) / count;
+  const int most = up(N, large ? 512 : 64);
+  int chunks = (int)std::min<size_t>(room, (size_t)std::min(most, 512));
+  GradArgs g;
+  g.rows = up(N, std::max(chunks, 1));
+  chunks = up(N, g.rows);
+  g.x = x, g.H1 = H1, g.H2 = H2, g.W3 = v.W3, g.dP = dP, g.dZ1 = dZ1;
+  g.part = chunks > 1 ? part : grads;
+  g.stride = count;
+  g.n = N, g.F = F, g.H = H;
+  g.t2 = up(H, tm) * up(H, tp);
+  g.t1 = up(H, tm) * up(F, tp);
+  const dim3 grid(g.t2 + g.t1 + up(H, MT), chunks);
+  if (large) k_grads<8><<<grid, MT, 0, s>>>(g);
+  else k_grads<4><<<grid, MT, 0, s>>>(g);
+  k_add_up<<<(unsigned)((count + 255) / 256) + 1, 256, 0, s>>>(g.part, count, chunks, grads, count, sq, n_sq, loss,
+                                                                1.f / (2.f * (float)N));
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) { set_error(cudaGetErrorString(e)); return TNQ_ECUDA; }
   return TNQ_OK;

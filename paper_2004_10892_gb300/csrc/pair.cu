@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
   constexpr int NX = 1 << PRX, NY = 1 << RY;
   const int t = threadIdx.x, lane = t & 31;
   const POp* ops[3] = {&P.a, &P.b, &P.c};
-  if (P.out_dep) n_tiles = (long long)*P.n_items << P.n_h;
+  if (P.out_dep && P.n_items) n_tiles = (long long)*P.n_items << P.n_h;
   if (blockIdx.x >= n_tiles) return;
   // ---- tables that every tile uses
   if (t < PH_MAX) {

@@ -78,7 +78,7 @@ struct PairParams {
   int smem;                     // dynamic shared memory bytes
   int* meta_e;
   unsigned* meta_m;
-  const int* n_items;           // valid items of the batch (device)
+  const int* n_items;           // valid items of the batch (device; null: the batch is one item)
 };
 
 // Blocks of k_pair that fit the device at once for this shape; 0 and *err on failure.

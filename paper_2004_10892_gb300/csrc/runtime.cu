@@ -58,7 +58,7 @@ struct KParams {
   int B;                         // meta row length
   int* meta_e;
   unsigned* meta_m;
-  const int* n_items;            // valid items of the batch (device)
+  const int* n_items;            // valid items of the batch (device; null: the batch is one item)
 };
 
 // One early bucket of a level launch (k_bucket_level): like KParams for an
@@ -202,8 +202,7 @@ __global__ void __launch_bounds__(TPB, 5) k_bucket(const __grid_constant__ KPara
   __shared__ float4 sh_c[ITER];  // product of the thread-invariant inputs per iteration (pair over u)
   const int t = threadIdx.x;
   const long long g0 = (long long)blockIdx.x << LT;
-  const long long total = P.G > P.out_bits ? (long long)*P.n_items << P.out_bits : 1ll << P.G;
-  if (g0 >= total) return;
+  const int n_valid = P.n_items ? __ldg(P.n_items) : 1;  // (not waited for before the tables are built)
 
   for (int e = t; e < NIN * ITER; e += TPB) {
     const int j = e / ITER, it = e - (e / ITER) * ITER;
@@ -222,6 +221,8 @@ __global__ void __launch_bounds__(TPB, 5) k_bucket(const __grid_constant__ KPara
       if (i < P.G && ((t >> i) & 1)) a += P.stride[j][i];
     tp[j] = a;
   }
+  const long long total = P.G > P.out_bits ? (long long)n_valid << P.out_bits : 1ll << P.G;
+  if (g0 >= total) return;
   __syncthreads();
 
   const int ob = P.out_bits;
@@ -385,6 +386,7 @@ __global__ void __launch_bounds__(256) k_bucket_level(const HoistDev* __restrict
   __shared__ int s_e;
   __shared__ float s_red[8];
   const int t = threadIdx.x;
+  const int n_valid = n_items ? __ldg(n_items) : 1;
   if (t == 0) {
     int lo = 0, hi = n - 1;
     while (lo < hi) {
@@ -399,7 +401,7 @@ __global__ void __launch_bounds__(256) k_bucket_level(const HoistDev* __restrict
   const int nin = H.nin, bits = H.bits, ob = H.obits;
   const long long g0 = (long long)(blockIdx.x - H.blk0) * 256;
   const bool uniform = ob >= 8 || ob == bits;  // one item for the whole block
-  const long long total = H.out_dep ? (long long)*n_items << ob : 1ll << bits;
+  const long long total = H.out_dep ? (long long)n_valid << ob : 1ll << bits;
   if (g0 >= total) return;
   for (int e = t; e < nin * bits; e += 256) s_str[e / bits][e % bits] = H.stride[e / bits][e % bits];
   if (t < nin) s_in[t] = reinterpret_cast<const float2*>(arena + H.in[t]);
@@ -540,7 +542,7 @@ struct GParams {
   int lean2;                   // 1: two stages, stage 1 reads stage 0 densely and writes the output (k_group<2>)
   int* meta_e;
   unsigned* meta_m;
-  const int* n_items;          // valid items of the batch (device)
+  const int* n_items;          // valid items of the batch (device; null: the batch is one item)
 };
 
 // Stage buffers in shared memory are stored swizzled: complex entry o sits at
@@ -967,6 +969,7 @@ __global__ void __launch_bounds__(GTPB, TK ? 5 : 4) k_group(const __grid_constan
   __shared__ float s_red[GTPB / 32];
   __shared__ float4 s_K[GM_MAX];  // register-tail stages with per-item constant pairs (kinv)
   const int t = threadIdx.x;
+  const int n_valid = P.n_items ? __ldg(P.n_items) : 1;  // (not waited for before the tables are built)
   // tables shared by every tile
   for (int e = t; e < (GIN_MAX + 1) * GH_MAX; e += GTPB) {
     const int j = e / GH_MAX, i = e - j * GH_MAX;
@@ -1001,7 +1004,7 @@ __global__ void __launch_bounds__(GTPB, TK ? 5 : 4) k_group(const __grid_constan
   for (int i = 0; i < GTB && i < nb_last; ++i)
     if ((t >> i) & 1) out_lo += P.out_cstride[i];
   const int buf_elems = 1 << (GL_MAX - 1);
-  if (P.out_dep) n_tiles = (long long)*P.n_items << P.n_h;
+  if (P.out_dep) n_tiles = (long long)n_valid << P.n_h;
   long long cur_item = -1;
   long long meta_item = -1;  // item whose exponents and scales s_e / s_F hold
   float tmax = 0.f;
@@ -2741,15 +2744,15 @@ static void enqueue_batch(const tnq_plan& P, ExecConfig& C, char* ws, cudaStream
   k_scalar_init<<<(B + 127) / 128, 128, 0, s>>>(C.d_scalars, C.n_scalars, C.d_inout, C.n_inout, hdr, bits, C.d_vals,
                                                 scal, B);
   int* status = reinterpret_cast<int*>(ws + L.status_off);
+  const int* n_items = B > 1 ? &hdr->n_items : nullptr;  // (a load that a batch of one item does not wait for)
   // early buckets first, one launch per level; their steps launch nothing below
   for (size_t l = 0; l + 1 < C.hoist_first.size(); ++l)
     k_bucket_level<<<(unsigned)C.hoist_blocks[l], 256, 0, s>>>(C.d_hoist + C.hoist_first[l],
                                                                  C.hoist_first[l + 1] - C.hoist_first[l],
-                                                                 reinterpret_cast<char*>(arena), me, mm, B,
-                                                                 &hdr->n_items);
+                                                                 reinterpret_cast<char*>(arena), me, mm, B, n_items);
   if (!side) {
     for (size_t i = 0; i < C.steps.size(); ++i)
-      if (!C.step_hoist[i]) launch_step(C, (int)i, arena, me, mm, status, &hdr->n_items, s);
+      if (!C.step_hoist[i]) launch_step(C, (int)i, arena, me, mm, status, n_items, s);
   } else {
     cudaEventRecord(side->fork, s);
     for (int k = 0; k < N_SIDE_STREAMS; ++k) cudaStreamWaitEvent(side->st[k], side->fork, 0);
@@ -2757,7 +2760,7 @@ static void enqueue_batch(const tnq_plan& P, ExecConfig& C, char* ws, cudaStream
       const int k = C.step_stream[i];
       for (int j : C.step_deps[i])
         if (C.step_stream[j] != k) cudaStreamWaitEvent(side->st[k], side->done[j], 0);
-      if (!C.step_hoist[i]) launch_step(C, (int)i, arena, me, mm, status, &hdr->n_items, side->st[k]);
+      if (!C.step_hoist[i]) launch_step(C, (int)i, arena, me, mm, status, n_items, side->st[k]);
       cudaEventRecord(side->done[i], side->st[k]);
     }
     for (int k = 0; k < N_SIDE_STREAMS; ++k) {
@@ -3162,7 +3165,7 @@ static tnq_status profile_steps(const tnq_plan* plan, const uint8_t* bits, uint6
   for (auto& e : ev) CU(cudaEventCreate(&e));
   for (int i = 0; i < nbk; ++i) {
     CU(cudaEventRecord(ev[2 * i], s));
-    launch_step(*C, i, arena, me, mm, reinterpret_cast<int*>(ws + L.status_off), &hdr->n_items, s);
+    launch_step(*C, i, arena, me, mm, reinterpret_cast<int*>(ws + L.status_off), B > 1 ? &hdr->n_items : nullptr, s);
     CU(cudaEventRecord(ev[2 * i + 1], s));
   }
   CU(cudaGetLastError());

@@ -67,6 +67,11 @@ def _dptr(t):
     return ctypes.c_void_p(t.data_ptr())
 
 
+def _at(t, i):
+    """Device pointer of element i of a contiguous FP32 tensor."""
+    return ctypes.c_void_p(t.data_ptr() + 4 * i)
+
+
 def gpu_forward(params, X, hidden: int = HIDDEN, stream=None):
     """Forward pass with the library's GPU kernels (torch CUDA tensors in/out)."""
     import torch
@@ -105,25 +110,22 @@ def train(X, y, epochs: int = 200, batch: int = 1024, lr: float = 0.05, mu: floa
     params = torch.from_numpy(init_params(seed, hidden)).cuda()
     mom = torch.zeros_like(params)
     grads = torch.empty_like(params)
-    loss = torch.zeros(1, dtype=torch.float32, device="cuda")
     n = Xd.shape[0]
     b = min(batch, n)
+    losses = torch.zeros(max(1, n // b), dtype=torch.float32, device="cuda")  # one per step, read once an epoch
     work = torch.empty(L.tnq_mlp_workspace_floats(hidden, b), dtype=torch.float32, device="cuda")
     g = torch.Generator(device="cpu").manual_seed(seed)
     hist = []
     st = tnq._stream_ptr(None)
+    pp, pg, pm, pw, count = _dptr(params), _dptr(grads), _dptr(mom), _dptr(work), params.numel()
     for ep in range(epochs):
         perm = torch.randperm(n, generator=g).cuda()
-        tot = 0.0
-        for i in range(0, n - b + 1, b):
-            idx = perm[i:i + b]
-            xb = Xd.index_select(0, idx).contiguous()
-            yb = yd.index_select(0, idx).contiguous()
-            tnq._check(L.tnq_mlp_backward(_dptr(params), hidden, _dptr(xb), _dptr(yb), b, _dptr(grads), _dptr(loss),
-                                          _dptr(work), st))
-            tnq._check(L.tnq_mlp_sgd(_dptr(params), _dptr(grads), _dptr(mom), params.numel(), lr, mu, st))
-            tot += float(loss)
-        hist.append(tot / max(1, n // b))
+        xp, yp = Xd.index_select(0, perm), yd.index_select(0, perm)  # the epoch's batches, one after the other
+        for k, i in enumerate(range(0, n - b + 1, b)):
+            tnq._check(L.tnq_mlp_backward(pp, hidden, _at(xp, i * xp.shape[1]), _at(yp, i), b, pg, _at(losses, k), pw,
+                                          st))
+            tnq._check(L.tnq_mlp_sgd(pp, pg, pm, count, lr, mu, st))
+        hist.append(sum(losses.tolist(), 0.0) / max(1, n // b))
     return params.cpu().numpy(), hist
 
 
