@@ -30,6 +30,7 @@ void rebuild_program(tnq_plan* P, int gemm_min_k_log2, int tile_low) {
   if (o.precision != TNQ_PREC_C64) find_gemm_chains(P->prog, P->order, gemm_min_k_log2, 8);
   if (o.leaf_absorb) absorb_leaves(P->prog);
   fuse_chains(P->prog, P->order, o.fuse_min_rank);
+  P->small.reset();
   reset_device_state(*P);
 }
 }  // namespace tnq

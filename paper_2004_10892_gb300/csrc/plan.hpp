@@ -11,6 +11,7 @@
 
 namespace tnq {
 struct DeviceState;  // per-device tables and cached graphs (runtime.cu)
+struct SmallPlan;    // the plan's one-kernel form (runtime.cu)
 void destroy_device_state(DeviceState* s);
 void set_error(const std::string& msg);
 }  // namespace tnq
@@ -36,6 +37,9 @@ struct tnq_plan {
   int gemm_min_k_log2 = 4;       // GEMM cut-over the program was compiled with
   mutable std::mutex layout_mu;
   mutable std::map<std::pair<int, int>, size_t> layout_bytes;  // (mode, batch) -> workspace bytes
+  mutable std::mutex small_mu;
+  mutable std::shared_ptr<tnq::SmallPlan> small;  // built on first use, dropped with the program
+  bool small_off = false;                         // internal test hook: always run step by step
   mutable std::mutex dev_mu;
   mutable tnq::DeviceState* dev = nullptr;
   ~tnq_plan() {

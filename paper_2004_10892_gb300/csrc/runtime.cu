@@ -31,6 +31,7 @@
 #include "gemm_tc.cuh"
 #include "pair.cuh"
 #include "plan.hpp"
+#include "small.cuh"
 
 extern "C" const char* tnq_last_error(void);
 
@@ -74,23 +75,6 @@ struct HoistDev {
   int blk0;                       // first block of this bucket in its level's launch
   int nvar;                       // inputs 0..nvar-1 vary with the index's low 8 bits (k_bucket's order)
 };
-
-struct LeafDev {
-  float2 val[4];      // entries when nv <= 2: (a, b) at a + 2b
-  long long tab;      // nv > 2 (general networks): element offset of the 2^nv entries in the leaf value table
-  long long off;      // element offset in the arena
-  int nv;             // tensor variables (binary; entry index sum_x a_x 2^x)
-  int n_free;         // leaf rank
-  int dep;            // item-dependent in this configuration
-  int pad;
-  signed char vkind[LEAF_VMAX];  // 0 free, 1 fixed to 0 (input wire), 2 output bit, 3 sliced
-  short varg[LEAF_VMAX];         // free: bit in the leaf; output: qubit; sliced: j
-};
-
-// Entry a of a leaf: inline for gates, from the value table for general tensors.
-__device__ __forceinline__ float2 leaf_entry(const LeafDev& L, const float2* __restrict__ vals, int a) {
-  return L.nv <= 2 ? L.val[a] : vals[L.tab + a];
-}
 
 struct FinalDev {
   long long off;
@@ -1233,6 +1217,23 @@ __global__ void k_accumulate(const double2* __restrict__ part, int n_rows, doubl
   }
 }
 
+// k_slice_sum and k_accumulate in one, for a batch of n items whose first is
+// item_base: bitstring row r's items are consecutive.
+__global__ void k_rows_add(const double2* __restrict__ res, int n, unsigned long long item_base, int p,
+                           unsigned long long bstr_base, int n_rows, double2* __restrict__ acc) {
+  const int r = blockIdx.x * blockDim.x + threadIdx.x;
+  if (r >= n_rows) return;
+  const long long first = (long long)(((bstr_base + r) << p) - item_base);
+  const long long i0 = first > 0 ? first : 0, i1 = min((long long)n, first + (1ll << p));
+  double re = 0.0, im = 0.0;
+  for (long long i = i0; i < i1; ++i) {
+    re += res[i].x;
+    im += res[i].y;
+  }
+  acc[r].x += re;
+  acc[r].y += im;
+}
+
 // ---------------------------------------------------------------------------
 // host side
 #define CU(call)                                                                  \
@@ -1243,6 +1244,12 @@ __global__ void k_accumulate(const double2* __restrict__ part, int n_rows, doubl
       return TNQ_ECUDA;                                                           \
     }                                                                             \
   } while (0)
+
+void reset_device_state(const tnq_plan& P);
+
+// The plan's one-kernel form (nullptr: it has none), defined below.
+const SmallPlan* small_plan(const tnq_plan& P);
+long long small_arena(const SmallPlan* S);
 
 namespace {
 
@@ -1260,6 +1267,14 @@ struct Layout {
 };
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
+
+constexpr size_t STATUS_OFF = 128;  // of the status word in every workspace
+static_assert(sizeof(BatchHdr) <= STATUS_OFF, "the status word overlaps the batch header");
+
+// What a batch of a small plan keeps in its workspace (below what make_layout
+// asks for): results after the status word, then the items' arenas.
+size_t small_res_off() { return 2 * STATUS_OFF; }
+size_t small_arena_off(int B) { return align_up(small_res_off() + 16 * (size_t)B, 256); }
 
 bool tensor_dep(const PTensor& t, int mode) { return t.dep_slice || (mode == 1 && t.dep_bits); }
 
@@ -1370,11 +1385,13 @@ Layout make_layout(const tnq_plan& P, int mode, int B) {
   }
   L.gemm_off = (long long)align_up((size_t)L.arena_elems, 128);
   if (gemm_elems) L.arena_elems = L.gemm_off + gemm_elems;
+  if (const SmallPlan* S = small_plan(P)) L.arena_elems = std::max(L.arena_elems, small_arena(S) * B);
   L.n_words = (P.net.n_qubits + 31) / 32;
   L.n_rows = B + 1;
   size_t o = 0;
-  L.hdr_off = o; o = align_up(o + sizeof(BatchHdr), 128);
-  L.status_off = o; o = align_up(o + 4, 256);
+  L.hdr_off = o;
+  o = L.status_off = STATUS_OFF;
+  o = align_up(o + 4, 256);
   L.bits_off = o; o = align_up(o + (size_t)L.n_rows * L.n_words * 4, 256);
   L.scalar_off = o; o = align_up(o + (size_t)B * 16, 256);
   L.res_off = o; o = align_up(o + (size_t)B * 16, 256);
@@ -1441,7 +1458,13 @@ struct DeviceState {
   std::map<std::pair<int, int>, ExecConfig*> configs;  // (mode, B)
   std::map<int, NoallocConfig*> noalloc;               // B
   std::map<uint64_t, int> noalloc_batch;               // batch cap -> largest B that fits the scratch
+  char* d_small = nullptr;                             // tables of the one-kernel form
+  int small_resident[4] = {0, 0, 0, 0};                // its clusters of 1, 2, 4, 8 blocks that run at once
+  double2* h_res = nullptr;                            // its results: pinned, written by the kernel, read under dev_mu
+  int h_res_n = 0;
   ~DeviceState() {
+    cudaFree(d_small);
+    if (h_res) cudaFreeHost(h_res);
     for (auto& kv : noalloc) delete kv.second;
     for (auto& kv : configs) {
       ExecConfig* c = kv.second;
@@ -1497,6 +1520,240 @@ static LeafDev make_leafdev(const tnq_plan& P, const PTensor* pt, int gate, cons
     d.off = L->off[tid];
   }
   return d;
+}
+
+// ---------------------------------------------------------------------------
+// One-kernel form of a small plan (k_small, small.cuh): every bucket of the
+// program -- fused chains and GEMM chains bucket by bucket -- in levels.
+//
+// Which plans: those whose whole slice is a few ten million operations. Below
+// that the launches are what a slice costs (6x6 d1+24+1, 16 slices: 36
+// dependent launches, 0.28 ms for 0.06 GFLOP); above it a cluster of eight SMs
+// is slower than a launch on all of them. The rule looks at the plan alone, so
+// that a slice has the same value in a batch of any size.
+struct SmallPlan {
+  bool ok = false;
+  SmallArgs args;          // counts and scales; pointers are set per call
+  std::vector<char> blob;  // device tables, one after the other
+  size_t tables = 0, leaves = 0, scalars = 0, inout = 0, finals = 0, vals = 0;  // offsets in it
+  int widest = 1;          // most entries of a level that the whole cluster works on
+};
+constexpr double SMALL_FLOPS = 1 << 25;      // per slice
+constexpr int SMALL_BITS = 20;               // variables of a bucket's result
+constexpr int SMALL_WIDE = 4096;             // a level of more entries is shared by the cluster
+constexpr int SMALL_TENSOR = 11;             // variables of a tensor in shared memory
+constexpr int SMALL_ELEMS = 64 * 1024 / 8;   // shared memory for tensors
+constexpr long long SMALL_ARENA = 1 << 20;   // elements per item in global memory
+
+long long small_arena(const SmallPlan* S) { return S->args.arena_elems; }
+
+static void build_small(const tnq_plan& P, SmallPlan& S) {
+  const Program& prog = P.prog;
+  const int nb = (int)prog.buckets.size(), T = (int)prog.tensors.size();
+  std::memset(&S.args, 0, sizeof(S.args));
+  if (prog.flops_per_slice > SMALL_FLOPS || nb == 0) return;
+  // levels: a bucket runs one level after the last of its inputs
+  std::vector<int> lv(nb, 0);
+  int n_lv = 0;
+  for (int b = 0; b < nb; ++b) {
+    const PBucket& B = prog.buckets[b];
+    if (B.k < 1 || B.k > KMAX || prog.tensors[B.output].rank() > SMALL_BITS) return;
+    for (int t : B.inputs)
+      if (prog.tensors[t].producer >= 0) lv[b] = std::max(lv[b], lv[prog.tensors[t].producer] + 1);
+    n_lv = std::max(n_lv, lv[b] + 1);
+  }
+  std::vector<long long> entries(n_lv, 0);
+  for (int b = 0; b < nb; ++b) entries[lv[b]] += 1ll << prog.tensors[prog.buckets[b].output].rank();
+  auto wide = [&](int l) { return entries[l] > SMALL_WIDE; };
+  for (int l = 0; l < n_lv; ++l) {
+    if (entries[l] > (1ll << 30)) return;
+    if (wide(l)) S.widest = std::max<int>(S.widest, (int)entries[l]);
+  }
+  // places: tensors that only the cluster's first block touches go to shared
+  // memory while there is room, the others to the item's part of the arena;
+  // in both, tensors with disjoint lives (in levels) share space
+  std::vector<int> lo(T, 0), hi(T, n_lv), off(T, 0);
+  std::vector<char> shared(T, 0);
+  std::vector<int> idx;
+  for (int t = 0; t < T; ++t) {
+    const PTensor& x = prog.tensors[t];
+    if (x.producer < 0 && x.leaf_gate < 0) return;
+    lo[t] = x.producer >= 0 ? lv[x.producer] : -1;
+    hi[t] = x.consumer >= 0 ? lv[x.consumer] : n_lv;
+    shared[t] = x.rank() <= SMALL_TENSOR && (x.producer < 0 || !wide(lv[x.producer])) &&
+                (x.consumer < 0 || !wide(lv[x.consumer]));
+    idx.push_back(t);
+  }
+  std::stable_sort(idx.begin(), idx.end(),
+                   [&](int a, int b) { return prog.tensors[a].rank() > prog.tensors[b].rank(); });
+  long long used[2] = {0, 0};
+  std::vector<int> placed[2];
+  auto place = [&](int t, int where) {
+    const long long size = std::max(4ll, 1ll << prog.tensors[t].rank());
+    std::vector<std::pair<long long, long long>> busy;
+    for (int o : placed[where])
+      if (lo[o] <= hi[t] && lo[t] <= hi[o])
+        busy.push_back({off[o], off[o] + std::max(4ll, 1ll << prog.tensors[o].rank())});
+    std::sort(busy.begin(), busy.end());
+    long long c = 0;
+    for (auto& iv : busy) {
+      if (c + size <= iv.first) break;
+      c = std::max(c, iv.second);
+    }
+    if (c + size > (where ? (long long)SMALL_ELEMS : SMALL_ARENA)) return false;
+    off[t] = (int)c;
+    used[where] = std::max(used[where], c + size);
+    placed[where].push_back(t);
+    return true;
+  };
+  for (int pass = 0; pass < 2; ++pass)  // the smallest tensors have the most readers per byte: shared memory first
+    for (int i = 0; i < T; ++i) {
+      const int t = pass == 0 ? idx[T - 1 - i] : idx[i];
+      if (pass == 0 && shared[t]) shared[t] = place(t, 1);
+      else if (pass == 1 && !shared[t] && !place(t, 0)) return;
+    }
+  auto where = [&](int t) { return shared[t] ? off[t] | SMALL_SHARED : off[t]; };
+  // tables
+  std::vector<SmallOp> ops;
+  std::vector<SmallIn> ins;
+  std::vector<SmallLevel> levels;
+  std::vector<int> op_of(nb, -1);
+  for (int l = 0; l < n_lv; ++l) {
+    std::vector<int> bs;
+    for (int b = 0; b < nb; ++b)
+      if (lv[b] == l) bs.push_back(b);
+    std::stable_sort(bs.begin(), bs.end(), [&](int a, int b) {
+      return prog.tensors[prog.buckets[a].output].rank() > prog.tensors[prog.buckets[b].output].rank();
+    });
+    SmallLevel V{(int)ops.size(), (int)bs.size(), 0, wide(l)};
+    for (int b : bs) {
+      const PBucket& B = prog.buckets[b];
+      const PTensor& o = prog.tensors[B.output];
+      op_of[b] = (int)ops.size();
+      ops.push_back(SmallOp{where(B.output), V.entries, o.rank(), (int)ins.size(), B.k, B.sum ? 1 : 0});
+      V.entries += 1 << o.rank();
+      for (int t : B.inputs) {
+        const PTensor& x = prog.tensors[t];
+        SmallIn in;
+        std::memset(&in, 0, sizeof(in));
+        in.off = where(t);
+        in.meta = x.leaf_gate >= 0 ? -1 : op_of[x.producer];
+        int next = B.sum ? 1 : 0;  // the output's variables must follow in the input's order
+        if (B.sum && (x.vars.empty() || x.vars[0] != B.u)) return;
+        for (int i = 0; i < o.rank(); ++i)
+          if (next < x.rank() && x.vars[next] == o.vars[i]) {
+            in.mask |= 1u << i;
+            ++next;
+          }
+        if (next != x.rank()) return;
+        // shift masks of the compression (Hacker's Delight, 7-4)
+        unsigned m = in.mask, mk = ~m << 1;
+        for (int i = 0; i < 5; ++i) {
+          unsigned mp = mk ^ (mk << 1);
+          mp ^= mp << 2;
+          mp ^= mp << 4;
+          mp ^= mp << 8;
+          mp ^= mp << 16;
+          const unsigned mv = mp & m;
+          in.mv[i] = mv;
+          m = (m ^ mv) | (mv >> (1 << i));
+          mk &= ~mp;
+        }
+        ins.push_back(in);
+      }
+    }
+    levels.push_back(V);
+  }
+  std::vector<LeafDev> leaves, scalars;
+  std::vector<SmallLeaf> small;
+  std::vector<float2> vals;
+  for (int t : prog.leaves) {
+    LeafDev d = make_leafdev(P, &prog.tensors[t], prog.tensors[t].leaf_gate, nullptr, t, &vals);
+    d.off = where(t);
+    if (d.nv > 2) {
+      leaves.push_back(d);
+      continue;
+    }
+    SmallLeaf L;
+    std::memset(&L, 0, sizeof(L));
+    for (int i = 0; i < 4; ++i) L.val[i] = d.val[i];
+    L.off = (int)d.off;
+    L.n_free = (short)d.n_free;
+    for (int x = 0; x < 2; ++x) {
+      L.kind[x] = x < d.nv ? d.vkind[x] : 1;
+      L.arg[x] = x < d.nv ? d.varg[x] : 0;
+    }
+    small.push_back(L);
+  }
+  for (int g : prog.scalar_leaves) scalars.push_back(make_leafdev(P, nullptr, g, nullptr, -1, &vals));
+  std::vector<int2> finals;
+  for (int t : prog.finals) finals.push_back(make_int2(where(t), op_of[prog.tensors[t].producer]));
+  auto put = [&](const void* p, size_t bytes) {
+    const size_t at = align_up(S.blob.size(), 16);
+    S.blob.resize(at + bytes);
+    if (bytes) std::memcpy(S.blob.data() + at, p, bytes);
+    return at;
+  };
+  S.tables = put(ins.data(), ins.size() * sizeof(SmallIn));  // the order of SmallArgs::tables
+  put(small.data(), small.size() * sizeof(SmallLeaf));
+  put(levels.data(), levels.size() * sizeof(SmallLevel));
+  put(ops.data(), ops.size() * sizeof(SmallOp));
+  S.blob.resize(align_up(S.blob.size(), 16));
+  S.leaves = put(leaves.data(), leaves.size() * sizeof(LeafDev));
+  S.scalars = put(scalars.data(), scalars.size() * sizeof(LeafDev));
+  S.inout = put(P.net.inout_qubits.data(), P.net.inout_qubits.size() * sizeof(int));
+  S.finals = put(finals.data(), finals.size() * sizeof(int2));
+  S.vals = put(vals.data(), vals.size() * sizeof(float2));
+  SmallArgs& A = S.args;
+  A.n_ops = (int)ops.size();
+  A.n_ins = (int)ins.size();
+  A.n_levels = n_lv;
+  A.n_small = (int)small.size();
+  A.n_leaves = (int)leaves.size();
+  A.n_scalars = (int)scalars.size();
+  A.n_inout = (int)P.net.inout_qubits.size();
+  A.n_finals = (int)finals.size();
+  A.smem_elems = (int)align_up((size_t)used[1], 2);
+  A.arena_elems = (long long)align_up((size_t)used[0], 32);
+  A.p = (int)P.mu.size();
+  A.n_words = (P.net.n_qubits + 31) / 32;
+  const long long le = std::max<long long>(-100000, std::min<long long>(100000, P.net.leaf_exp));
+  A.scale_exp = -(P.net.n_sqrt2 / 2) + (int)le;
+  A.scale_half = P.net.n_sqrt2 & 1;
+  S.ok = small_smem(A) <= SMALL_SMEM_MAX && A.n_words <= SMALL_WORDS;
+}
+
+const SmallPlan* small_plan(const tnq_plan& P) {
+  if (P.small_off) return nullptr;
+  std::lock_guard<std::mutex> lk(P.small_mu);
+  if (!P.small) {
+    P.small = std::make_shared<SmallPlan>();
+    build_small(P, *P.small);
+    if (!P.small->ok) P.small->blob.clear();
+  }
+  return P.small->ok ? P.small.get() : nullptr;
+}
+
+// Blocks per item: as many as the widest level feeds with two entries a thread
+// and as let all the items' clusters run at once, at most eight (the portable
+// cluster size).
+static int small_cluster(const SmallPlan& S, const int* resident, int n_items) {
+  int c = 1;
+  for (int i = 1; i < 4 && S.widest >= 2 * (1 << i) * STPB && n_items <= resident[i]; ++i) c = 1 << i;
+  return c;
+}
+
+static SmallArgs small_args(const SmallPlan& S, const char* tables, char* arena, double2* res) {
+  SmallArgs A = S.args;
+  A.tables = reinterpret_cast<const float4*>(tables + S.tables);
+  A.leaves = reinterpret_cast<const LeafDev*>(tables + S.leaves);
+  A.scalars = reinterpret_cast<const LeafDev*>(tables + S.scalars);
+  A.inout = reinterpret_cast<const int*>(tables + S.inout);
+  A.finals = reinterpret_cast<const int2*>(tables + S.finals);
+  A.vals = reinterpret_cast<const float2*>(tables + S.vals);
+  A.arena = reinterpret_cast<float2*>(arena);
+  A.res = res;
+  return A;
 }
 
 // Kernel parameters of every step of one configuration (single buckets and
@@ -2325,11 +2582,83 @@ static bool build_steps(const tnq_plan& P, const Layout& L, ExecConfig& C) {
   return true;
 }
 
+// Host-side check of the one-kernel form: level by level, every input range
+// holds what its producer wrote, no output overlaps another tensor of the
+// level or leaves its region, pair loads are aligned.
+static std::string validate_small(const tnq_plan& P, const SmallPlan& S) {
+  const SmallArgs& A = S.args;
+  auto up = [](size_t n) { return align_up(n, 16); };
+  const char* at = S.blob.data() + S.tables;
+  const SmallIn* ins = reinterpret_cast<const SmallIn*>(at);
+  const SmallLeaf* small = reinterpret_cast<const SmallLeaf*>(at += up(A.n_ins * sizeof(SmallIn)));
+  const SmallLevel* levels = reinterpret_cast<const SmallLevel*>(at += up(A.n_small * sizeof(SmallLeaf)));
+  const SmallOp* ops = reinterpret_cast<const SmallOp*>(at += up(A.n_levels * sizeof(SmallLevel)));
+  if (at + up(A.n_ops * sizeof(SmallOp)) != S.blob.data() + S.tables + small_tables_bytes(A)) return "tables";
+  const LeafDev* leaves = reinterpret_cast<const LeafDev*>(S.blob.data() + S.leaves);
+  const int n_leaves = A.n_small + A.n_leaves;
+  std::vector<int> owner[2] = {std::vector<int>(A.arena_elems, -1), std::vector<int>(A.smem_elems, -1)};
+  auto range = [&](int off, int bits, std::vector<int>** v, long long* lo) {
+    *v = &owner[off & SMALL_SHARED ? 1 : 0];
+    *lo = off & ~SMALL_SHARED;
+    return *lo + (1ll << bits) <= (long long)(*v)->size();
+  };
+  std::vector<int>* v;
+  long long lo;
+  for (int l = 0; l < n_leaves; ++l) {
+    const int off = l < A.n_small ? small[l].off : (int)leaves[l - A.n_small].off;
+    const int n_free = l < A.n_small ? small[l].n_free : leaves[l - A.n_small].n_free;
+    if (!range(off, n_free, &v, &lo)) return "leaf outside its region";
+    for (long long i = lo; i < lo + (1ll << n_free); ++i) {
+      if ((*v)[i] >= 0) return "leaves overlap";
+      (*v)[i] = l;
+    }
+  }
+  for (int l = 0; l < A.n_levels; ++l) {
+    const SmallLevel& V = levels[l];
+    std::vector<int> busy[2] = {std::vector<int>(A.arena_elems, 0), std::vector<int>(A.smem_elems, 0)};
+    int entries = 0;
+    for (int o = V.op0; o < V.op0 + V.nop; ++o) {
+      const SmallOp& op = ops[o];
+      if (op.first != entries || (op.first & ((1 << op.bits) - 1))) return "level entries";
+      entries += 1 << op.bits;
+      for (int j = 0; j < op.nin; ++j) {
+        const SmallIn& in = ins[op.in0 + j];
+        const int bits = __builtin_popcount(in.mask) + op.sum;
+        if (in.mask >> op.bits) return "input mask";
+        if (V.wide && (in.off & SMALL_SHARED)) return "wide level reads one block's memory";
+        if (!range(in.off, bits, &v, &lo)) return "input outside its region";
+        if (op.sum && (lo & 1)) return "unaligned pair";
+        for (long long i = lo; i < lo + (1ll << bits); ++i) {
+          const int who = (*v)[i];
+          if (in.meta >= 0 ? who != n_leaves + in.meta : (who < 0 || who >= n_leaves)) return "stale input";
+          busy[in.off & SMALL_SHARED ? 1 : 0][i] = 1;
+        }
+      }
+    }
+    if (entries != V.entries) return "level entries";
+    for (int o = V.op0; o < V.op0 + V.nop; ++o) {
+      if (V.wide && (ops[o].out & SMALL_SHARED)) return "wide level writes one block's memory";
+      if (!range(ops[o].out, ops[o].bits, &v, &lo)) return "output outside its region";
+      for (long long i = lo; i < lo + (1ll << ops[o].bits); ++i) {
+        int& b = busy[ops[o].out & SMALL_SHARED ? 1 : 0][i];
+        if (b) return "output overlaps the level's tensors";
+        b = 1;
+        (*v)[i] = n_leaves + o;
+      }
+    }
+  }
+  return small_smem(A) <= SMALL_SMEM_MAX ? "" : "shared memory";
+}
+
 // Host-side bounds check of every launch of configuration (mode, B): each
 // input's largest index stays inside its tensor, each output fits its
 // allocation, every tensor fits the arena and tensors live at the same time
 // do not overlap. Returns an empty string when everything holds.
 static std::string validate_config(const tnq_plan& P, int mode, int B) {
+  if (const SmallPlan* S = small_plan(P)) {
+    const std::string err = validate_small(P, *S);
+    if (!err.empty()) return "one-kernel form: " + err;
+  }
   const Layout L = make_layout(P, mode, B);
   ExecConfig C;
   C.L = L;
@@ -2845,6 +3174,80 @@ static int ilog2_floor(uint64_t x) {
   return b;
 }
 
+// The plan's state on the current device (caller holds dev_mu).
+static tnq_status device_state(const tnq_plan& P, DeviceState** out) {
+  int dev;
+  CU(cudaGetDevice(&dev));
+  if (P.dev && P.dev->device != dev) {
+    set_error("plan already bound to another CUDA device");
+    return TNQ_EINVAL;
+  }
+  if (!P.dev) {
+    P.dev = new DeviceState();
+    P.dev->device = dev;
+  }
+  *out = P.dev;
+  return TNQ_OK;
+}
+
+// How many of the one-kernel form's clusters the device holds at once, looked up on first use (caller holds dev_mu).
+static tnq_status small_occupancy(const SmallPlan& S, DeviceState& D) {
+  if (!D.small_resident[0])
+    for (int i = 3; i >= 0; --i) CU(small_resident(S.args, 1 << i, &D.small_resident[i]));
+  return TNQ_OK;
+}
+
+// Device tables of the one-kernel form, uploaded on first use (caller holds dev_mu).
+static tnq_status small_tables(const SmallPlan& S, DeviceState& D, const char** out) {
+  const tnq_status st = small_occupancy(S, D);
+  if (st != TNQ_OK) return st;
+  if (!D.d_small) {
+    char* d = nullptr;
+    CU(cudaMalloc(&d, S.blob.size()));
+    const cudaError_t e = cudaMemcpy(d, S.blob.data(), S.blob.size(), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) {
+      cudaFree(d);
+      CU(e);
+    }
+    D.d_small = d;
+  }
+  *out = D.d_small;
+  return TNQ_OK;
+}
+
+// tnq_contract_sliced of a small plan, B slices a launch: the header and the
+// bitstring go with the launch, the kernel writes each slice's value to
+// `host_res` (pinned) or, where that is null, to d_res, which is copied; the
+// slices are added here in increasing order. Caller holds dev_mu.
+static tnq_status contract_small(const SmallPlan& S, const tnq_plan& P, const uint8_t* bits, uint64_t begin,
+                                 uint64_t end, int B, const int* resident, const char* tables, char* arena,
+                                 double2* host_res, double2* d_res, cudaStream_t s, double* out_amp,
+                                 double* out_slice_amps) {
+  double2* dst = d_res;
+  if (host_res) CU(cudaHostGetDevicePointer(reinterpret_cast<void**>(&dst), host_res, 0));
+  SmallArgs A = small_args(S, tables, arena, dst);
+  for (int q = 0; q < P.net.n_qubits; ++q)
+    if (bits[q]) A.words[q >> 5] |= 1u << (q & 31);
+  std::vector<double2> copy(host_res ? 0 : B);
+  const double2* res = host_res ? host_res : copy.data();
+  double re = 0, im = 0;
+  for (uint64_t base = begin; base < end; base += B) {
+    const int n = (int)std::min<uint64_t>(B, end - base);
+    A.item_base = base;
+    CU(small_launch(A, n, small_cluster(S, resident, n), s));
+    if (!host_res) CU(cudaMemcpyAsync(copy.data(), d_res, (size_t)n * 16, cudaMemcpyDeviceToHost, s));
+    CU(cudaStreamSynchronize(s));
+    for (int i = 0; i < n; ++i) {
+      re += res[i].x;
+      im += res[i].y;
+    }
+    if (out_slice_amps) std::memcpy(out_slice_amps + 2 * (base - begin), res, (size_t)n * 16);
+  }
+  out_amp[0] = re;
+  out_amp[1] = im;
+  return TNQ_OK;
+}
+
 static tnq_status get_config(const tnq_plan& P, int mode, int B, ExecConfig** out) {
   int dev;
   CU(cudaGetDevice(&dev));
@@ -2926,6 +3329,19 @@ int tnq_internal_validate(const tnq_plan* plan, int mode, uint32_t batch, char* 
     msg[msg_len - 1] = 0;
   }
   return m.empty() ? 0 : 1;
+}
+
+// Internal test hook (not in include/tnq.h): whether the plan runs as one
+// kernel (k_small); use = 0 makes it run step by step, 1 undoes that. Before
+// the plan is shared, as tnq_plan_keep_chains.
+int tnq_internal_small(tnq_plan* plan, int use) {
+  plan->small_off = !use;
+  {
+    std::lock_guard<std::mutex> lk(plan->layout_mu);
+    plan->layout_bytes.clear();
+  }
+  reset_device_state(*plan);
+  return small_plan(*plan) ? 1 : 0;
 }
 
 // Internal hook (not in include/tnq.h; host only): the kernel kind of every
@@ -3493,6 +3909,7 @@ int tnq_internal_launches_per_batch(const tnq_plan* plan, int mode, uint32_t bat
     if (gi < 0) n += !hoist[b];
     else if (prog.groups[gi].buckets.back() == (int)b) n += prog.groups[gi].gemm ? 3 : 1;  // GEMM: 2 packs + MMA
   }
+  if (small_plan(*plan)) return mode ? 2 : 1;
   ExecConfig C;  // a GEMM in the fused-A form packs only B
   C.L = make_layout(*plan, mode, (int)batch);
   if (build_steps(*plan, C.L, C))
@@ -3530,10 +3947,25 @@ tnq_status tnq_contract_sliced(const tnq_plan* plan, const uint8_t* bits, uint64
   if (max_batch > 0) cap = std::min<uint64_t>(cap, 1ull << ilog2_floor(max_batch));
   const int B = pick_batch(*plan, 0, ws_bytes, cap);
   if (B == 0) { set_error("workspace too small for one slice"); return TNQ_ENOMEM; }
-  ExecConfig* C = nullptr;
-  if ((st = get_config(*plan, 0, B, &C)) != TNQ_OK) return st;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   char* ws = reinterpret_cast<char*>(workspace);
+  if (const SmallPlan* S = small_plan(*plan)) {
+    std::lock_guard<std::mutex> lk(plan->dev_mu);  // the result buffer is the plan's
+    DeviceState* D = nullptr;
+    const char* tables = nullptr;
+    if ((st = device_state(*plan, &D)) != TNQ_OK || (st = small_tables(*S, *D, &tables)) != TNQ_OK) return st;
+    if (D->h_res_n < B) {
+      if (D->h_res) cudaFreeHost(D->h_res);
+      D->h_res = nullptr;
+      D->h_res_n = 0;
+      CU(cudaHostAlloc(reinterpret_cast<void**>(&D->h_res), (size_t)B * 16, cudaHostAllocMapped));
+      D->h_res_n = B;
+    }
+    return contract_small(*S, *plan, bits, slice_begin, slice_end, B, D->small_resident, tables, ws, D->h_res,
+                          nullptr, s, out_amp, out_slice_amps);
+  }
+  ExecConfig* C = nullptr;
+  if ((st = get_config(*plan, 0, B, &C)) != TNQ_OK) return st;
   std::vector<unsigned> words((size_t)C->L.n_words * C->L.n_rows, 0u);
   pack_bits(bits, plan->net.n_qubits, words);
   CU(cudaMemcpyAsync(ws + C->L.bits_off, words.data(), words.size() * 4, cudaMemcpyHostToDevice, s));
@@ -3615,7 +4047,10 @@ tnq_status tnq_amplitudes_batch(const tnq_plan* const* plans, size_t n_plans, co
     size_t plan;
     uint64_t base, end;
     int B, lane, rows;
-    ExecConfig* C;
+    ExecConfig* C;           // null for a small plan
+    const SmallPlan* S;      // its one-kernel form and tables
+    const char* tables;
+    const int* resident;
   };
   std::vector<Job> jobs;
   int n_lanes = 0;
@@ -3680,17 +4115,28 @@ tnq_status tnq_amplitudes_batch(const tnq_plan* const* plans, size_t n_plans, co
       while (cap < n_items && cap < (1ull << MAX_ITEM_BITS)) cap <<= 1;
       const int B = pick_batch(P, 1, region, cap);
       ExecConfig* C = nullptr;
-      if ((st = get_config(P, 1, B, &C)) != TNQ_OK) return st;
+      const char* tables = nullptr;
+      const int* resident = nullptr;
+      const SmallPlan* S = small_plan(P);
+      if (S) {
+        std::lock_guard<std::mutex> lk(P.dev_mu);
+        DeviceState* D = nullptr;
+        if ((st = device_state(P, &D)) != TNQ_OK || (st = small_tables(*S, *D, &tables)) != TNQ_OK) return st;
+        resident = D->small_resident;
+      } else if ((st = get_config(P, 1, B, &C)) != TNQ_OK) {
+        return st;
+      }
+      const int n_words = (n + 31) / 32;
       for (uint64_t base = 0; base < n_items; base += B) {
         const uint64_t end = std::min<uint64_t>(n_items, base + B);
         const uint64_t b0 = base >> p, b1 = (end - 1) >> p;  // bitstrings touched by this batch
-        Job J{pi, base, end, B, lane_of[pi], (int)(b1 - b0 + 1), C};
+        Job J{pi, base, end, B, lane_of[pi], (int)(b1 - b0 + 1), C, S, tables, resident};
         word_off.push_back(words.size());
-        words.resize(words.size() + (size_t)C->L.n_words * C->L.n_rows, 0u);
+        words.resize(words.size() + (size_t)n_words * (B + 1), 0u);
         unsigned* w = words.data() + word_off.back();
         for (uint64_t b = b0; b <= b1; ++b)
           for (int q = 0; q < n; ++q)
-            if (pb[b * n + q]) w[(size_t)(b - b0) * C->L.n_words + (q >> 5)] |= 1u << (q & 31);
+            if (pb[b * n + q]) w[(size_t)(b - b0) * n_words + (q >> 5)] |= 1u << (q & 31);
         BatchHdr h;
         std::memset(&h, 0, sizeof(h));
         h.item_base = base;
@@ -3699,7 +4145,7 @@ tnq_status tnq_amplitudes_batch(const tnq_plan* const* plans, size_t n_plans, co
         h.bstr_base = b0;
         h.mode = 1;
         h.p = p;
-        h.n_words = C->L.n_words;
+        h.n_words = n_words;
         hdrs.push_back(h);
         jobs.push_back(J);
       }
@@ -3743,7 +4189,7 @@ tnq_status tnq_amplitudes_batch(const tnq_plan* const* plans, size_t n_plans, co
     }
   }
   for (int k = 0; k < n_lanes; ++k) {  // the lane's status word (timeouts of the tensor-core waits)
-    e = cudaMemsetAsync(ws + (size_t)k * region + jobs[0].C->L.status_off, 0, 4, ls[k]);
+    e = cudaMemsetAsync(ws + (size_t)k * region + STATUS_OFF, 0, 4, ls[k]);
     if (e != cudaSuccess) break;
   }
   for (size_t ji = 0; ji < jobs.size() && e == cudaSuccess; ++ji) {
@@ -3751,6 +4197,21 @@ tnq_status tnq_amplitudes_batch(const tnq_plan* const* plans, size_t n_plans, co
     const tnq_plan& P = *plans[J.plan];
     char* lws = ws + (size_t)J.lane * region;
     cudaStream_t q = ls[J.lane];
+    double2* sums = acc + bits_offset[J.plan] + (J.base >> hdrs[ji].p);
+    if (J.S) {
+      const int n = (int)(J.end - J.base);
+      double2* res = reinterpret_cast<double2*>(lws + small_res_off());
+      SmallArgs A = small_args(*J.S, J.tables, lws + small_arena_off(J.B), res);
+      A.bits = d_words + word_off[ji];
+      A.item_base = J.base;
+      A.bstr_base = hdrs[ji].bstr_base;
+      A.mode = 1;
+      e = small_launch(A, n, small_cluster(*J.S, J.resident, n), q);
+      if (e != cudaSuccess) break;
+      k_rows_add<<<(J.rows + 127) / 128, 128, 0, q>>>(res, n, J.base, hdrs[ji].p, hdrs[ji].bstr_base, J.rows, sums);
+      e = cudaGetLastError();
+      continue;
+    }
     ExecConfig& C = *J.C;
     std::lock_guard<std::mutex> lk(P.dev_mu);  // one capture/launch sequence per plan at a time
     e = cudaMemcpyAsync(lws + C.L.bits_off, d_words + word_off[ji], (size_t)C.L.n_words * C.L.n_rows * 4,
@@ -3761,11 +4222,11 @@ tnq_status tnq_amplitudes_batch(const tnq_plan* const* plans, size_t n_plans, co
       return st;
     }
     k_accumulate<<<(J.rows + 127) / 128, 128, 0, q>>>(reinterpret_cast<const double2*>(lws + C.L.part_off), J.rows,
-                                                      acc + bits_offset[J.plan] + (J.base >> hdrs[ji].p));
+                                                      sums);
     e = cudaGetLastError();
   }
   for (int k = 0; k < n_lanes && e == cudaSuccess; ++k) {
-    e = cudaMemcpyAsync(lane_status + k, ws + (size_t)k * region + jobs[0].C->L.status_off, 4,
+    e = cudaMemcpyAsync(lane_status + k, ws + (size_t)k * region + STATUS_OFF, 4,
                         cudaMemcpyDeviceToDevice, ls[k]);
     if (e == cudaSuccess && k > 0) e = cudaEventRecord(join[k], ls[k]);
     if (e == cudaSuccess && k > 0) e = cudaStreamWaitEvent(s, join[k], 0);
@@ -3942,6 +4403,23 @@ tnq_status tnq_contract_sliced_noalloc(const tnq_plan* plan, const uint8_t* bits
   const uint64_t n_items = slice_end - slice_begin;
   uint64_t cap = 1;
   while (cap < n_items && cap < (1ull << MAX_ITEM_BITS)) cap <<= 1;
+  if (const SmallPlan* S = small_plan(*plan)) {
+    // tables at the front of the scratch (up again on each call: every call shares it), results and arenas behind
+    std::lock_guard<std::mutex> lk(plan->dev_mu);
+    DeviceState* D = nullptr;
+    if ((st = device_state(*plan, &D)) != TNQ_OK || (st = small_occupancy(*S, *D)) != TNQ_OK) return st;
+    const size_t front = align_up(S->blob.size(), 256);
+    int B = 1;
+    while ((uint64_t)B * 2 <= cap &&
+           front + align_up(32 * (size_t)B, 256) + 16 * (size_t)S->args.arena_elems * B <= NOALLOC_SCRATCH_BYTES)
+      B *= 2;
+    char* base = reinterpret_cast<char*>(scratch);
+    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    CU(cudaMemcpyAsync(base, S->blob.data(), S->blob.size(), cudaMemcpyHostToDevice, s));
+    return contract_small(*S, *plan, bits, slice_begin, slice_end, B, D->small_resident, base,
+                          base + front + align_up(16 * (size_t)B, 256), nullptr,
+                          reinterpret_cast<double2*>(base + front), s, out_amp, out_slice_amps);
+  }
   NoallocConfig* NC = nullptr;
   if ((st = get_noalloc_config(*plan, cap, reinterpret_cast<char*>(scratch), &NC)) != TNQ_OK) return st;
   ExecConfig& C = NC->C;

@@ -43,7 +43,11 @@ CASES = [
 
 def _plan(tnq_lib, rows, cols, depth, seed, **kw):
     circ = I.random_grid_circuit(rows, cols, depth, seed)
-    return circ, tnq_lib.Plan(circ, max_bag_log2=20, max_p=20, reorder_every=1, **kw)
+    plan = tnq_lib.Plan(circ, max_bag_log2=20, max_p=20, reorder_every=1, **kw)
+    f = tnq_lib.lib().tnq_internal_small  # these plans are small: their chains are what is tested here
+    f.argtypes = [ctypes.c_void_p, ctypes.c_int]
+    f(plan.handle, 0)
+    return circ, plan
 
 
 def _shapes(tnq_lib, plan):

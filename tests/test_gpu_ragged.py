@@ -1,5 +1,7 @@
 """Batches that are not full: the kernels work on the valid items only, so a
 slice's value must be the same bits whatever range it was asked for in."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -14,6 +16,9 @@ def test_every_range_gives_the_same_slices(cuda, tnq_lib, precision, rows, cols,
     torch = cuda
     circ = I.random_grid_circuit(rows, cols, depth, seed)
     plan = tnq_lib.Plan(circ, max_bag_log2=bag, min_p=4, max_p=6, precision=precision, gemm_min_k_log2=3, reorder_every=1)
+    f = tnq_lib.lib().tnq_internal_small  # (step by step: the launches are what is tested here)
+    f.argtypes = [ctypes.c_void_p, ctypes.c_int]
+    f(plan.handle, 0)
     n = plan.info()["n_slices"]
     bits = I.random_bitstring(circ.n_qubits, seed)
     ws = torch.empty(plan.workspace_bytes(16), dtype=torch.uint8, device="cuda")
