@@ -25,6 +25,13 @@ __device__ __forceinline__ void cp_async16(unsigned dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
 
+__device__ __forceinline__ void cfma(float2& r, float2 a, float2 b) {
+  r.x = fmaf(a.x, b.x, r.x);
+  r.y = fmaf(a.x, b.y, r.y);
+  r.x = fmaf(-a.y, b.y, r.x);
+  r.y = fmaf(a.y, b.x, r.y);
+}
+
 // r += a b over the pair's two values
 __device__ __forceinline__ void cfma2(float2& r, float4 a, float4 b) {
   r.x = fmaf(a.x, b.x, r.x);
@@ -37,17 +44,19 @@ __device__ __forceinline__ void cfma2(float2& r, float4 a, float4 b) {
   r.y = fmaf(a.w, b.z, r.y);
 }
 
-// Persistent: a block loops over tiles (item, tile variables), a tile over one
-// or two chunks of its summed values. Two stages: while a chunk is computed,
+// Persistent: a block loops over tiles (item, tile variables), a tile over one,
+// two or four chunks of its summed values. Two stages: while a chunk is computed,
 // the next one's part of A, B (and C) comes in by cp.async; each thread then
 // multiplies what it copied by the fold tables in place, and after one barrier
 // every thread computes 4 x 2^RY register tiles: per pair of summed values 4 + 2^RY
 // 16-byte shared loads feed 32 x 2^RY FMAs. Shared memory delivers 128 bytes a
 // cycle to registers, so 4 x 4 needs all of it at the full FMA rate and 4 x 8
 // three quarters.
-template <int RY, int NKX, int NKY, bool HASC>
+// CM: 0 no C, 1 C without u_0 (its bit 0 is B's register bit 0), 2 C with u_0.
+template <int RX, int RY, int NKX, int NKY, int CM>
 __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairParams P, long long n_tiles) {
   extern __shared__ float4 sm[];
+  constexpr bool HASC = CM != 0;
   constexpr int NOP = HASC ? 3 : 2;
   constexpr int RING = 4;  // a thread is at most one barrier ahead: what it writes is two tiles ahead
   __shared__ float4 s_fa[2][1 << PF_MAX], s_fb[2][1 << PF_MAX];  // by item, alternating
@@ -62,7 +71,7 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
   __shared__ float s_sc[PIN_MAX];
   __shared__ int s_e[RING][PIN_MAX];
   __shared__ float s_red[PTPB / 32];
-  constexpr int NX = 1 << PRX, NY = 1 << RY;
+  constexpr int NX = 1 << RX, NY = 1 << RY;
   const int t = threadIdx.x, lane = t & 31;
   const POp* ops[3] = {&P.a, &P.b, &P.c};
   if (P.out_dep && P.n_items) n_tiles = (long long)*P.n_items << P.n_h;
@@ -183,7 +192,7 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
 #pragma unroll
     for (int o = 0; o < NOP; ++o) {
       const POp& O = *ops[o];
-      const float2* src = s_src[slot][o] + tg[o] + (chunk ? O.gch : 0);
+      const float2* src = s_src[slot][o] + tg[o] + ((chunk & 1) ? O.gch[0] : 0) + ((chunk & 2) ? O.gch[1] : 0);
       const unsigned dst = sm0 + 16u * (unsigned)(buf * P.stage + td[o]);
       const int nit = O.ebits > PTB ? 1 << (O.ebits - PTB) : 1;
       if (O.ebits >= PTB || t < (1 << O.ebits))
@@ -200,7 +209,8 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
     for (int o = 0; o < 2; ++o) {
       if (o == 0 && !fold_a) continue;
       const POp& O = *ops[o];
-      const float4* ft = (o == 0 ? s_fa[n & 1] : s_fb[n & 1]) + tf[o] + s_fold[slot][o] + (chunk ? O.fch : 0);
+      const float4* ft = (o == 0 ? s_fa[n & 1] : s_fb[n & 1]) + tf[o] + s_fold[slot][o] +
+                         ((chunk & 1) ? O.fch[0] : 0) + ((chunk & 2) ? O.fch[1] : 0);
       float4* dst = sm + buf * P.stage + td[o];
       const int nit = O.ebits > PTB ? 1 << (O.ebits - PTB) : 1;
       if (O.ebits >= PTB || t < (1 << O.ebits)) {
@@ -261,6 +271,10 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
       const float4* pb = sm + buf * P.stage + rb;
       float2* dst = s_out[slot] + ro;
       const int n1 = 1 << P.n1;
+      auto off_x = [&](int i, const int* w) { return ((i & 1) ? w[0] : 0) + ((i & 2) ? w[1] : 0); };
+      auto off_y = [&](int j, const int* w) {
+        return ((j & 1) ? w[0] : 0) + ((j & 2) ? w[1] : 0) + (RY > 2 && (j & 4) ? w[2] : 0);
+      };
       auto products = [&](int oa, int ob) {
 #pragma unroll 1
         for (int q = 0; q < n1; ++q) {
@@ -269,20 +283,35 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
           const float4* qb = pb + (ob + k.y);
           float4 va[NX];
 #pragma unroll
-          for (int i = 0; i < NX; ++i) va[i] = qa[((i & 1) ? P.xa[0] : 0) + ((i & 2) ? P.xa[1] : 0)];
+          for (int i = 0; i < NX; ++i) va[i] = qa[off_x(i, P.xa)];
 #pragma unroll
           for (int j = 0; j < NY; ++j) {
-            const float4 vb =
-                qb[((j & 1) ? P.yb[0] : 0) + ((j & 2) ? P.yb[1] : 0) + (RY > 2 && (j & 4) ? P.yb[2] : 0)];
+            const float4 vb = qb[off_y(j, P.yb)];
 #pragma unroll
             for (int i = 0; i < NX; ++i) cfma2(x[i][j], va[i], vb);
           }
         }
       };
+      auto half_products = [&](int oa, int ob, int h) {  // u_0 = h alone
+#pragma unroll 1
+        for (int q = 0; q < n1; ++q) {
+          const int2 k = s_k1[q];
+          const float2* qa = reinterpret_cast<const float2*>(pa + (oa + k.x)) + h;
+          const float2* qb = reinterpret_cast<const float2*>(pb + (ob + k.y)) + h;
+          float2 va[NX];
+#pragma unroll
+          for (int i = 0; i < NX; ++i) va[i] = qa[2 * off_x(i, P.xa)];
+#pragma unroll
+          for (int j = 0; j < NY; ++j) {
+            const float2 vb = qb[2 * off_y(j, P.yb)];
+#pragma unroll
+            for (int i = 0; i < NX; ++i) cfma(x[i][j], va[i], vb);
+          }
+        }
+      };
       auto store = [&](int i, int j, float2 r, int lo) {
         const int ri = i << NKX, rj = j << NKY;
-        dst[lo + ((ri & 1) ? P.xo[0] : 0) + ((ri & 2) ? P.xo[1] : 0) + ((rj & 1) ? P.yo[0] : 0) +
-            ((rj & 2) ? P.yo[1] : 0) + (RY > 2 && (rj & 4) ? P.yo[2] : 0)] = r;
+        dst[lo + off_x(ri, P.xo) + off_y(rj, P.yo)] = r;
         tmax = fmaxf(tmax, fmaxf(fabsf(r.x), fabsf(r.y)));
       };
       const int nl = 1 << P.nl;
@@ -299,18 +328,33 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
 #pragma unroll 1
           for (int q2 = 0; q2 < n2; ++q2) {
             const int4 k2 = s_k2[q2];
-            products(lv.x + k2.x, lv.y + k2.y);
-            // times C, summed over the K2 register bits (C's bit 0 is B's register bit 0)
             const float4* pc = sm + buf * P.stage + rc + lv.z + k2.z;
+            if constexpr (CM == 2) {
+#pragma unroll 1
+              for (int h = 0; h < 2; ++h) {
+                half_products(lv.x + k2.x, lv.y + k2.y, h);
+                const float2* ph = reinterpret_cast<const float2*>(pc) + h;
 #pragma unroll
-            for (int i = 0; i < NX; ++i)
+                for (int i = 0; i < NX; ++i)
 #pragma unroll
-              for (int j = 0; j < NY; j += 2) {
-                const float4 v = pc[((i & 1) ? P.xc[0] : 0) + ((i & 2) ? P.xc[1] : 0) + ((j & 2) ? P.yc[1] : 0)];
-                const float2 u = x[i][j], w = x[i][j + 1];
-                cfma2(acc[i >> NKX][j >> NKY], make_float4(u.x, u.y, w.x, w.y), v);
-                x[i][j] = x[i][j + 1] = make_float2(0.f, 0.f);
+                  for (int j = 0; j < NY; ++j) {
+                    cfma(acc[i >> NKX][j >> NKY], x[i][j], ph[2 * (off_x(i, P.xc) + off_y(j, P.yc))]);
+                    x[i][j] = make_float2(0.f, 0.f);
+                  }
               }
+            } else {
+              products(lv.x + k2.x, lv.y + k2.y);
+              // times C, summed over the K2 register bits (C's bit 0 is B's register bit 0)
+#pragma unroll
+              for (int i = 0; i < NX; ++i)
+#pragma unroll
+                for (int j = 0; j < NY; j += 2) {
+                  const float4 v = pc[off_x(i, P.xc) + off_y(j, P.yc)];  // (yc[0] is 0: the pair's own bit)
+                  const float2 u = x[i][j], w = x[i][j + 1];
+                  cfma2(acc[i >> NKX][j >> NKY], make_float4(u.x, u.y, w.x, w.y), v);
+                  x[i][j] = x[i][j + 1] = make_float2(0.f, 0.f);
+                }
+            }
           }
 #pragma unroll
           for (int i = 0; i < XO; ++i)
@@ -343,14 +387,24 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
 
 using PairKernel = void (*)(PairParams, long long);
 static PairKernel pair_kernel(const PairParams& p) {
-  if (p.c.gin < 0) return p.ry > 2 ? k_pair<3, 0, 0, false> : k_pair<2, 0, 0, false>;
-  switch (p.nkx * 4 + p.nky) {
-    case 1: return k_pair<2, 0, 1, true>;
-    case 2: return k_pair<2, 0, 2, true>;
-    case 5: return k_pair<2, 1, 1, true>;
-    case 6: return k_pair<2, 1, 2, true>;
-    case 9: return k_pair<2, 2, 1, true>;
-    default: return k_pair<2, 2, 2, true>;
+  if (p.c.gin < 0) {
+    if (p.rx == 2) return p.ry > 2 ? k_pair<2, 3, 0, 0, 0> : k_pair<2, 2, 0, 0, 0>;
+    if (p.rx) return k_pair<1, 3, 0, 0, 0>;
+    return p.ry > 1 ? k_pair<0, 3, 0, 0, 0> : k_pair<0, 1, 0, 0, 0>;
+  }
+  switch ((p.c_u0 * 3 + p.nkx) * 3 + p.nky) {
+    case 1: return k_pair<2, 2, 0, 1, 1>;
+    case 2: return k_pair<2, 2, 0, 2, 1>;
+    case 4: return k_pair<2, 2, 1, 1, 1>;
+    case 5: return k_pair<2, 2, 1, 2, 1>;
+    case 7: return k_pair<2, 2, 2, 1, 1>;
+    case 8: return k_pair<2, 2, 2, 2, 1>;
+    case 9: return k_pair<2, 2, 0, 0, 2>;
+    case 10: return k_pair<2, 2, 0, 1, 2>;
+    case 11: return k_pair<2, 2, 0, 2, 2>;
+    case 13: return k_pair<2, 2, 1, 1, 2>;
+    case 14: return k_pair<2, 2, 1, 2, 2>;
+    default: return k_pair<2, 2, 2, 2, 2>;
   }
 }
 

@@ -2,10 +2,10 @@
 // large tensors (k_pair), optionally times a third one.
 //
 // A chain's result is out[o] = sum_K A B C prod_g g over the chain's
-// eliminated variables K (Eq. 2 applied m times, regrouped), with large
-// tensors A and B that both hold the first eliminated variable u_0, at most
-// one other large tensor C that does not, and small tensors g, each of which
-// has its variables among A's or among B's and is folded into that one.
+// eliminated variables K (Eq. 2 applied m times, regrouped; m = 1: a single
+// bucket), with large tensors A and B that both hold the first eliminated
+// variable u_0, at most one other large tensor C, and small tensors g, each of
+// which has its variables among A's or among B's and is folded into that one.
 // With K2 = K & vars(C) and K1 = K - K2:
 //   out[o] = sum_K2 C[K2, o] (sum_K1 A[K1, K2, o] B[K1, K2, o]).
 #pragma once
@@ -15,7 +15,7 @@ namespace tnq {
 
 constexpr int PTB = 8;              // log2 threads per k_pair block
 constexpr int PTPB = 1 << PTB;
-constexpr int PRX = 2;              // register tile: 2^PRX entries along A's variables ...
+constexpr int PRX_MAX = 2;          // register tile: up to 2^2 entries along A's variables ...
 constexpr int PRY_MAX = 3;          // ... x 2^2 or (two large tensors) 2^3 along B's
 constexpr int PE_MAX = 13;          // staged (u = 0, u = 1) pairs of one operand: at most 2^13
 constexpr int PF_MAX = 7;           // fold table of one operand: at most 2^8 pairs
@@ -38,13 +38,13 @@ struct PIn {
 // by an index e (bits by increasing memory stride, so that consecutive threads
 // read consecutive memory); bit i of e adds g[i] to the global offset
 // (elements), d[i] to the shared-memory slot (16-byte units) and f[i] to the
-// fold table's index. Tile bit i adds h[i] and fh[i], chunk 1 adds gch and fch.
+// fold table's index. Tile bit i adds h[i] and fh[i], bit i of the chunk gch[i] and fch[i].
 struct POp {
   int gin;
   int ebits;
   int g[PE_MAX], d[PE_MAX], f[PE_MAX];
   int h[PH_MAX], fh[PH_MAX];
-  int gch, fch;
+  int gch[2], fch[2];
   int base;                     // first slot of a stage
 };
 
@@ -65,14 +65,15 @@ struct PairParams {
   long long out_istride;
   int out_h[PH_MAX];            // per tile bit
   int ta[PTB], tb[PTB], tc[PTB], to[PTB];  // thread bits: slots of a, b, c; output offset
-  int xa[PRX], xc[PRX], xo[PRX];               // register bits along A: slots of a and c, output offset (0 for a K2 bit)
+  int xa[PRX_MAX], xc[PRX_MAX], xo[PRX_MAX];   // register bits along A: slots of a and c, output offset (0 for a K2 bit)
   int yb[PRY_MAX], yc[PRY_MAX], yo[PRY_MAX];   // register bits along B
-  int ry;                       // register bits along B
+  int rx, ry;                   // register bits along A / B
+  int c_u0;                     // 1: C holds u_0 (K2 then includes it)
   int nl, la[PL_MAX], lb[PL_MAX], lc[PL_MAX], lo[PL_MAX];  // a thread's loop over outputs
   int n1, k1a[PK_MAX], k1b[PK_MAX];                // K1 without u_0 and the chunk's variable: slots of a and b
   int n2, k2a[PK_MAX], k2b[PK_MAX], k2c[PK_MAX];   // K2 outside the register tile
   int nkx, nky;                 // K2 bits among the register bits along A / B (the low ones)
-  int n_ch;                     // chunks of a tile: 2 when one summed variable is split off, else 1
+  int n_ch;                     // chunks of a tile: one summed variable (2) or two (4) split off, or none (1)
   int n_h, n_gin, out_meta, out_dep, B;
   int stage;                    // slots of one stage; dynamic shared memory holds two
   int smem;                     // dynamic shared memory bytes

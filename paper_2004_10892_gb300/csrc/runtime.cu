@@ -1421,8 +1421,9 @@ struct ExecConfig {
   std::vector<GParams> gp;           // per fused-group step
   std::vector<int> gsmem;            // dynamic shared memory bytes per fused-group step
   std::vector<int> ggrid;            // persistent blocks per fused-group step (SMs x resident blocks at its gsmem)
-  std::vector<PairParams> pp;        // fused-group steps that k_pair runs
-  std::vector<int> pair_of;          // per fused-group step: its entry in pp, or -1 (k_group)
+  std::vector<PairParams> pp;        // steps that k_pair runs
+  std::vector<int> pgrid;            // their persistent blocks
+  std::vector<int> step_pair;        // per step: its entry in pp, or -1
   int group_grid = 152 * 4;          // persistent blocks of k_group (SMs x resident blocks)
   std::vector<GemmBucketArgs> gb;    // per GEMM step (pointers are arena offsets)
   std::vector<GemmEpilogue> ge;
@@ -2041,13 +2042,14 @@ static GParams group_gparams(const tnq_plan& P, const Layout& L, const FusedGrou
 // the arena base; false when the chain has another shape and k_group runs it.
 // The choice depends on the plan alone, never on the batch (a slice's value
 // must not depend on it). Requirements and why:
-//  * two large tensors (rank above PAIR_SMALL) that hold the first eliminated
-//    variable, at most one other large one, without it: the product of two
-//    tensors is what the register tile shares operands over;
+//  * two or three large tensors (rank above PAIR_SMALL), two of them with the
+//    first eliminated variable: the product of two tensors is what the
+//    register tile shares operands over;
 //  * every other tensor has its variables among A's or among B's: it is
 //    multiplied into that operand as it is staged;
-//  * 2^PRX register entries along variables of A alone and 2^2 along B's
-//    (eliminated variables of C count): without them nothing is shared;
+//  * 2^2 register entries along variables of A alone and of B alone
+//    (eliminated variables of C count), or fewer along A and 2^3 along B's:
+//    without them nothing is shared;
 //  * 2^PTB threads times the register tile of outputs.
 constexpr int PAIR_SMALL = 4;
 constexpr int PAIR_TILES = 5;
@@ -2062,24 +2064,53 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
   auto holds = [&](int j, int v) { return j >= 0 && index_in(vars(j), v) >= 0; };
   std::vector<int> K;
   for (int b : g.buckets) K.push_back(prog.buckets[b].u);
-  if ((int)K.size() > PK_MAX) return false;
+  if ((int)K.size() > PK_MAX + 1) return false;
   const int u0 = K[0];
   std::vector<int> large, small;
   for (int j = 0; j < (int)in.size(); ++j) (prog.tensors[in[j]].rank() > PAIR_SMALL ? large : small).push_back(j);
-  int A = -1, B = -1, C = -1;
-  for (int j : large) {
-    int& to = !holds(j, u0) ? C : (A < 0 ? A : B);
-    if (to >= 0) return false;
-    to = j;
+  int with_u0 = 0;
+  for (int j : large) with_u0 += holds(j, u0);
+  if (large.size() < 2 || large.size() > 3 || with_u0 < 2) return false;
+  int A = -1, B = -1, C = -1, c0 = -1;
+  // variables of j that k does not hold: among the outputs / the eliminated ones
+  auto alone = [&](int j, int k, const std::vector<int>& among) {
+    int n = 0;
+    for (int v : among) n += holds(j, v) && !holds(k, v);
+    return n;
+  };
+  if (large.size() == 3) {
+    // C: the one without u_0, else the one with the fewest eliminated
+    // variables (its products are 2^those an output), then the largest
+    std::pair<int, int> best;
+    for (int j : large) {
+      int n = 0;
+      for (int v : K) n += holds(j, v);
+      const auto key = with_u0 == 2 ? std::make_pair((int)holds(j, u0), 0) : std::make_pair(n, -prog.tensors[in[j]].rank());
+      if (C < 0 || key < best) {
+        C = j;
+        best = key;
+      }
+    }
   }
-  if (B < 0) return false;
-  int c0 = -1;
-  if (C >= 0) {  // C's bit 0: an eliminated variable that one of A and B holds (called B)
+  for (int j : large)
+    if (j != C) (A < 0 ? A : B) = j;
+  G.c_u0 = with_u0 == 3;
+  if (G.c_u0) {
+    if (vars(C)[0] != u0) return false;
+    std::vector<int> in_c;
+    for (int v : K)
+      if (holds(C, v)) in_c.push_back(v);
+    if (alone(A, B, in_c) > alone(B, A, in_c)) std::swap(A, B);  // (at least as many K2 register bits along B as along A)
+  } else if (C >= 0) {  // C's bit 0: an eliminated variable that one of A and B holds (called B)
     c0 = vars(C)[0];
     if (index_in(K, c0) < 0 || holds(A, c0) == holds(B, c0)) return false;
     if (holds(A, c0)) std::swap(A, B);
-  } else if (prog.tensors[in[A]].rank() < prog.tensors[in[B]].rank()) {
-    std::swap(A, B);  // B, the smaller one, is the one that is always scaled
+  } else {
+    if (prog.tensors[in[A]].rank() < prog.tensors[in[B]].rank()) std::swap(A, B);  // B is always scaled: the smaller one
+    if (alone(A, B, o.vars) < 2 || alone(B, A, o.vars) < 2) {  // few variables of one alone: that one is A
+      if (alone(A, B, o.vars) > alone(B, A, o.vars)) std::swap(A, B);
+      if (alone(B, A, o.vars) < 3) return false;
+    }
   }
   if (vars(A)[0] != u0 || vars(B)[0] != u0) return false;
   std::vector<int> sa, sb;
@@ -2094,23 +2125,25 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
   }
   // eliminated variables: K2 in C (register bits where A or B alone holds them), K1 the others
   std::vector<int> k1, k2, xreg, yreg;
-  if (C >= 0) yreg.push_back(c0);
+  if (c0 >= 0) yreg.push_back(c0);
   for (int v : K) {
     if (v == u0 || v == c0) continue;
     if (!holds(A, v) && !holds(B, v)) return false;
     if (!holds(C, v)) k1.push_back(v);
-    else if (holds(A, v) && !holds(B, v) && (int)xreg.size() < PRX) xreg.push_back(v);
+    else if (holds(A, v) && !holds(B, v) && (int)xreg.size() < 2) xreg.push_back(v);
     else if (holds(B, v) && !holds(A, v) && (int)yreg.size() < 2) yreg.push_back(v);
     else k2.push_back(v);
   }
   G.nkx = (int)xreg.size();
   G.nky = (int)yreg.size();
+  if (G.c_u0 && G.nkx > G.nky) return false;
+  G.rx = C < 0 ? std::min(2, alone(A, B, o.vars)) : 2;
   // 4 x 8 register tiles for two tensors that have the variables, and outputs
   // for 2^PAIR_TILES tiles an item (fewer leave the device idle), else 4 x 4
-  int only_b = 0;
-  for (int v : o.vars) only_b += holds(B, v) && !holds(A, v);
-  G.ry = C < 0 && only_b >= 3 && o.rank() >= PTB + PRX + 3 + PAIR_TILES ? 3 : 2;
-  const int need_x = PRX - G.nkx, need_y = G.ry - G.nky, n_one = PTB + need_x + need_y;
+  // with nothing to share along A the tile only holds B: small, for long sums
+  if (G.rx < 2) G.ry = G.rx || (int)K.size() <= 2 ? 3 : 1;
+  else G.ry = C < 0 && alone(B, A, o.vars) >= 3 && o.rank() >= PTB + G.rx + 3 + PAIR_TILES ? 3 : 2;
+  const int need_x = G.rx - G.nkx, need_y = G.ry - G.nky, n_one = PTB + need_x + need_y;
   if (o.rank() < n_one) return false;
   const int ops[3] = {A, B, C};
   // local output variables: the two earliest (the output is written in 32-byte
@@ -2157,7 +2190,7 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
     nx += holds(A, o.vars[best]) && !holds(B, o.vars[best]);
     ny += holds(B, o.vars[best]) && !holds(A, o.vars[best]);
     if (n + 1 == n_local && (int)loop.size() < PL_MAX && n_local + PAIR_TILES < o.rank() &&
-        (int)(k1.size() + k2.size()) + n_local - n_one + G.ry - 2 < PAIR_LOOP)
+        (int)(k1.size() + k2.size()) + G.c_u0 + n_local - n_one + G.rx + G.ry - 4 < PAIR_LOOP)
       ++n_local;
   }
   // register bits: the latest local variables of A alone / B alone; the other
@@ -2165,7 +2198,7 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
   std::vector<char> is_reg(o.vars.size(), 0);
   for (int side = 0; side < 2; ++side) {
     std::vector<int>& reg = side ? yreg : xreg;
-    const int want = side ? G.ry : PRX;
+    const int want = side ? G.ry : G.rx;
     for (int i = (int)o.vars.size() - 1; i >= 0 && (int)reg.size() < want; --i)
       if (local[i] && index_in(loop, o.vars[i]) < 0 && holds(side ? B : A, o.vars[i]) &&
           !holds(side ? A : B, o.vars[i])) {
@@ -2202,22 +2235,25 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
       ++F.n;
     }
   }
-  // two stages that leave no room for a second block are split into two chunks
-  // by one summed variable of both operands (the one that keeps the longest
+  // two stages that leave no room for a second block are split into two or four
+  // chunks by summed variables of both operands (those that keep the longest
   // runs of memory together); a chain with C keeps its sums in the register
   // tile's order and is not split
-  int chunk = -1;
-  {
+  std::vector<int> chunk;
+  if (C < 0 && loop.empty()) {
     double total = 0;
-    for (int k = 0; k < 3; ++k)
-      if (ops[k] >= 0) total += std::ldexp(1.0, bits[k] - 1) * 1.05;
-    if (2 * 16 * total > PAIR_SMEM_TWO && C < 0 && loop.empty()) {
+    for (int k = 0; k < 2; ++k) total += std::ldexp(1.0, bits[k] - 1) * 1.05;
+    while (2 * 16 * total > PAIR_SMEM_TWO && chunk.size() < 2) {
+      int best = -1;
       for (int v : k1)
-        if (holds(A, v) && holds(B, v) && (chunk < 0 || index_in(vars(A), v) > index_in(vars(A), chunk))) chunk = v;
-      if (chunk >= 0) k1.erase(std::find(k1.begin(), k1.end(), chunk));
+        if (holds(A, v) && holds(B, v) && (best < 0 || index_in(vars(A), v) > index_in(vars(A), best))) best = v;
+      if (best < 0) break;
+      k1.erase(std::find(k1.begin(), k1.end(), best));
+      chunk.push_back(best);
+      total /= 2;
     }
   }
-  G.n_ch = chunk < 0 ? 1 : 2;
+  G.n_ch = 1 << chunk.size();
   // staged operands: slot = row + pitch * (its eliminated variables but bit
   // 0), rows numbered by the thread bits it holds, then by its register
   // outputs; the odd pitch and the lowest row bits on the lowest lanes keep
@@ -2245,7 +2281,7 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
     const int pitch = (1 << rows) | 1;
     int nk = 0;
     for (size_t p = 1; p < v.size(); ++p)
-      if (v[p] != chunk && index_in(K, v[p]) >= 0) w[p] = pitch << nk++;
+      if (index_in(chunk, v[p]) < 0 && index_in(K, v[p]) >= 0) w[p] = pitch << nk++;
     O.base = base;
     base += pitch << nk;
     for (size_t p = 1; p < v.size(); ++p) {
@@ -2255,9 +2291,9 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
       if (h >= 0) {
         O.h[h] = 1 << p;
         O.fh[h] = f;
-      } else if (v[p] == chunk) {
-        O.gch = 1 << p;
-        O.fch = f;
+      } else if (const int q = index_in(chunk, v[p]); q >= 0) {
+        O.gch[q] = 1 << p;
+        O.fch[q] = f;
       } else {
         if (O.ebits >= PE_MAX) return false;
         O.g[O.ebits] = 1 << p;
@@ -2283,7 +2319,7 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
     G.tc[i] = slot(2, thr[i]);
     G.to[i] = out_of(thr[i]);
   }
-  for (int i = 0; i < PRX; ++i) {
+  for (int i = 0; i < G.rx; ++i) {
     G.xa[i] = slot(0, xreg[i]);
     G.xc[i] = slot(2, xreg[i]);
     G.xo[i] = out_of(xreg[i]);
@@ -2457,7 +2493,7 @@ static void step_dependencies(const tnq_plan& P, const Layout& L, ExecConfig& C)
       for (size_t q = 0; q < reads[j].size() && !hit; ++q) hit = overlap(reads[j][q], write[i]);
       if (hit) d.push_back(j);
     }
-    if (C.steps[i].first == 2) {
+    if (C.steps[i].first == 2 && C.step_pair[i] < 0) {
       if (last_gemm >= 0) d.push_back(last_gemm);
       last_gemm = i;
     }
@@ -2467,6 +2503,24 @@ static void step_dependencies(const tnq_plan& P, const Layout& L, ExecConfig& C)
   }
 }
 
+// Whether k_pair runs GEMM step number `i`.
+static bool gemm_as_pair(const ExecConfig& C, size_t i) {
+  for (size_t si = 0; si < C.steps.size(); ++si)
+    if (C.steps[si].first == 2 && C.steps[si].second == (int)i) return C.step_pair[si] >= 0;
+  return false;
+}
+
+// A GEMM chain whose tiles are mostly padding runs as an FP32 product instead:
+// at one row an item (padded to 128 or 64 of the MMA tile) the tensor cores do
+// 128 times the work and the operands are packed for it. 8 items of such a
+// chain (25 variables, one row, 64 columns, K = 32; 2.2 GB): 3.96 -> 0.84 ms; 16
+// items of one with 4096 rows and 4 columns (padded to 64): 0.109 -> 0.044 ms.
+// At a padding of 8 and below the two were not told apart.
+constexpr double PAIR_GEMM_PADDING = 16;
+static double gemm_padding(const FusedGroup& g, const GemmBucketArgs& G) {
+  return (double)G.m_pad * G.n_pad / std::ldexp(1.0, (int)(g.xvars.size() + g.yvars.size()));
+}
+
 static bool build_steps(const tnq_plan& P, const Layout& L, ExecConfig& C) {
   const Program& prog = P.prog;
   C.kp.clear();
@@ -2474,7 +2528,7 @@ static bool build_steps(const tnq_plan& P, const Layout& L, ExecConfig& C) {
   C.gp.clear();
   C.gsmem.clear();
   C.pp.clear();
-  C.pair_of.clear();
+  C.step_pair.clear();
   C.steps.clear();
   C.step_group.clear();
   C.gb.clear();
@@ -2491,6 +2545,15 @@ static bool build_steps(const tnq_plan& P, const Layout& L, ExecConfig& C) {
     const double full = std::ldexp(1.0, b.r);
     return (6.0 * (b.k - 1) * full + (b.sum ? full : 0.0)) * (L.dep[b.output] ? L.B : 1);
   };
+  auto pair_step = [&](const FusedGroup& g, bool can) {
+    PairParams pp;
+    can = can && pair_params(P, L, g, pp);
+    C.step_pair.push_back(can ? (int)C.pp.size() : -1);
+    if (can) C.pp.push_back(pp);
+  };
+  // buckets that run early at some batch size run in a level launch there and
+  // keep its arithmetic (k_bucket's) at every size
+  const std::vector<int> ever_early = hoist_levels(prog, L.dep, 0);
   for (size_t bi = 0; bi < prog.buckets.size(); ++bi) {
     const int gi = prog.group_of.empty() ? -1 : prog.group_of[bi];
     if (gi < 0) {
@@ -2507,6 +2570,11 @@ static bool build_steps(const tnq_plan& P, const Layout& L, ExecConfig& C) {
       for (int t : prog.buckets[bi].inputs) by += tbytes(t);
       C.step_bytes.push_back(by);
       C.step_flops.push_back(bflops((int)bi));
+      FusedGroup one;
+      one.buckets = {(int)bi};
+      one.output = prog.buckets[bi].output;
+      one.ext_inputs = prog.buckets[bi].inputs;
+      pair_step(one, prog.buckets[bi].sum && !ever_early[bi]);
     } else if ((int)bi == prog.groups[gi].buckets.back() && prog.groups[gi].gemm) {
       GemmBucketArgs G;
       GemmEpilogue E;
@@ -2516,6 +2584,7 @@ static bool build_steps(const tnq_plan& P, const Layout& L, ExecConfig& C) {
       C.step_hoist.push_back(0);
       C.gb.push_back(G);
       C.ge.push_back(E);
+      pair_step(prog.groups[gi], gemm_padding(prog.groups[gi], G) >= PAIR_GEMM_PADDING);
       double by = tbytes(prog.groups[gi].output);
       for (int t : prog.groups[gi].ext_inputs) by += tbytes(t);
       C.step_bytes.push_back(by);
@@ -2532,12 +2601,7 @@ static bool build_steps(const tnq_plan& P, const Layout& L, ExecConfig& C) {
       C.step_hoist.push_back(0);
       C.gp.push_back(g);
       C.gsmem.push_back(smem);
-      PairParams pp;
-      C.pair_of.push_back(-1);
-      if (pair_params(P, L, prog.groups[gi], pp)) {
-        C.pair_of.back() = (int)C.pp.size();
-        C.pp.push_back(pp);
-      }
+      pair_step(prog.groups[gi], true);
       double by = tbytes(prog.groups[gi].output);
       for (int t : prog.groups[gi].ext_inputs) by += tbytes(t);
       C.step_bytes.push_back(by);
@@ -2765,9 +2829,19 @@ static std::string validate_config(const tnq_plan& P, int mode, int B) {
       return "group " + std::to_string(gi) + ": shared memory below the dense stage's reads";
   }
   for (size_t si = 0; si < C.steps.size(); ++si) {  // chains that k_pair runs
-    if (C.steps[si].first != 1 || C.pair_of[C.steps[si].second] < 0) continue;
-    const PairParams& G = C.pp[C.pair_of[C.steps[si].second]];
-    const FusedGroup& g = prog.groups[C.step_group[si]];
+    if (C.step_pair[si] < 0) continue;
+    const PairParams& G = C.pp[C.step_pair[si]];
+    FusedGroup g;
+    if (C.step_group[si] >= 0) {
+      g = prog.groups[C.step_group[si]];
+    } else {  // the single bucket of this step
+      int nth = C.steps[si].second;
+      for (size_t b = 0; b < prog.buckets.size(); ++b)
+        if ((prog.group_of.empty() || prog.group_of[b] < 0) && nth-- == 0) {
+          g.output = prog.buckets[b].output;
+          g.ext_inputs = prog.buckets[b].inputs;
+        }
+    }
     const std::string name = "pair chain " + std::to_string(si);
     const long long items = G.out_dep ? B : 1;
     auto item_max = [&](int j) { return G.gin[j].dep ? (items - 1) * G.gin[j].istride : 0ll; };
@@ -2776,15 +2850,15 @@ static std::string validate_config(const tnq_plan& P, int mode, int B) {
     for (int k = 0; k < 3; ++k) {
       const POp& O = *ops[k];
       if (O.gin < 0) continue;
-      long long m = item_max(O.gin) + 1 + (G.n_ch > 1 ? O.gch : 0);
-      int d = O.base, f = G.n_ch > 1 ? O.fch : 0;
+      long long m = item_max(O.gin) + 1 + O.gch[0] + O.gch[1];
+      int d = O.base, f = O.fch[0] + O.fch[1];
       for (int i = 0; i < G.n_h; ++i) {
         if (O.h[i] & 1) return name + ": odd tile stride";
         m += O.h[i];
         f += O.fh[i];
       }
       for (int i = 0; i < O.ebits; ++i) {
-        if ((O.g[i] & 1) || (O.gch & 1)) return name + ": odd local stride";
+        if ((O.g[i] & 1) || ((O.gch[0] | O.gch[1]) & 1)) return name + ": odd local stride";
         m += O.g[i];
         d += O.d[i];
         f += O.f[i];
@@ -2797,9 +2871,9 @@ static std::string validate_config(const tnq_plan& P, int mode, int B) {
       long long r = O.base;
       for (int i = 0; i < PTB; ++i) r += k == 0 ? G.ta[i] : (k == 1 ? G.tb[i] : G.tc[i]);
       if (k != 1)
-        for (int i = 0; i < PRX; ++i) r += k == 0 ? G.xa[i] : G.xc[i];
-      if (k != 0)  // (C is read in pairs over B's register bit 0)
-        for (int i = k == 2; i < G.ry; ++i) r += k == 1 ? G.yb[i] : G.yc[i];
+        for (int i = 0; i < G.rx; ++i) r += k == 0 ? G.xa[i] : G.xc[i];
+      if (k != 0)  // (C without u_0 is read in pairs over B's register bit 0)
+        for (int i = k == 2 && !G.c_u0; i < G.ry; ++i) r += k == 1 ? G.yb[i] : G.yc[i];
       for (int i = 0; i < G.nl; ++i) r += k == 0 ? G.la[i] : (k == 1 ? G.lb[i] : G.lc[i]);
       for (int i = 0; i < G.n1; ++i) r += k == 0 ? G.k1a[i] : (k == 1 ? G.k1b[i] : 0);
       for (int i = 0; i < G.n2; ++i) r += k == 0 ? G.k2a[i] : (k == 1 ? G.k2b[i] : G.k2c[i]);
@@ -2817,7 +2891,7 @@ static std::string validate_config(const tnq_plan& P, int mode, int B) {
     long long om = G.out_dep ? (items - 1) * G.out_istride : 0;
     for (int i = 0; i < G.n_h; ++i) om += G.out_h[i];
     for (int i = 0; i < PTB; ++i) om += G.to[i];
-    for (int i = 0; i < PRX; ++i) om += G.xo[i];
+    for (int i = 0; i < G.rx; ++i) om += G.xo[i];
     for (int i = 0; i < G.ry; ++i) om += G.yo[i];
     for (int i = 0; i < G.nl; ++i) om += G.lo[i];
     if (om >= alloc(g.output)) return name + ": output overflows";
@@ -2895,15 +2969,15 @@ static tnq_status chain_grids(ExecConfig& C) {
   C.ggrid.clear();
   for (size_t i = 0; i < C.gsmem.size(); ++i) {
     int g = 0;
-    if (C.pair_of[i] >= 0) {
-      cudaError_t e = cudaSuccess;
-      g = pair_grid(C.pp[C.pair_of[i]], &e);
-      CU(e);
-    } else {
-      const tnq_status st = group_grid_size(&g, C.gsmem[i], C.gp[i].tail > 0 ? 1 : (C.gp[i].lean2 ? 2 : 0));
-      if (st != TNQ_OK) return st;
-    }
+    const tnq_status st = group_grid_size(&g, C.gsmem[i], C.gp[i].tail > 0 ? 1 : (C.gp[i].lean2 ? 2 : 0));
+    if (st != TNQ_OK) return st;
     C.ggrid.push_back(g);
+  }
+  C.pgrid.clear();
+  for (const PairParams& p : C.pp) {
+    cudaError_t e = cudaSuccess;
+    C.pgrid.push_back(pair_grid(p, &e));
+    CU(e);
   }
   return TNQ_OK;
 }
@@ -2991,7 +3065,16 @@ static void launch_step(const ExecConfig& C, int i, float2* arena, int* me, unsi
                         const int* n_items, cudaStream_t s) {
   char* base = reinterpret_cast<char*>(arena);
   const auto st = C.steps[i];
-  if (st.first == 0) {
+  if (const int q = C.step_pair[i]; q >= 0) {
+    PairParams g = C.pp[q];
+    g.out = reinterpret_cast<float2*>(base + reinterpret_cast<size_t>(g.out));
+    for (int j = 0; j < g.n_gin; ++j)
+      g.gin[j].ptr = reinterpret_cast<const float2*>(base + reinterpret_cast<size_t>(g.gin[j].ptr));
+    g.meta_e = me;
+    g.meta_m = mm;
+    g.n_items = n_items;
+    pair_launch(g, (g.out_dep ? (long long)g.B : 1ll) << g.n_h, C.pgrid[q], s);
+  } else if (st.first == 0) {
     KParams k = C.kp[st.second];
     k.out = reinterpret_cast<float2*>(base + reinterpret_cast<size_t>(k.out));
     for (int j = 0; j < C.kshape[st.second].first; ++j)
@@ -3016,16 +3099,6 @@ static void launch_step(const ExecConfig& C, int i, float2* arena, int* me, unsi
     e.out = reinterpret_cast<float2*>(base + reinterpret_cast<size_t>(e.out));
     e.meta_m = mm;
     gemm_bucket_launch(g, e, status, s);
-  } else if (C.pair_of[st.second] >= 0) {
-    PairParams g = C.pp[C.pair_of[st.second]];
-    g.out = reinterpret_cast<float2*>(base + reinterpret_cast<size_t>(g.out));
-    for (int j = 0; j < g.n_gin; ++j)
-      g.gin[j].ptr = reinterpret_cast<const float2*>(base + reinterpret_cast<size_t>(g.gin[j].ptr));
-    g.meta_e = me;
-    g.meta_m = mm;
-    g.n_items = n_items;
-    const long long tiles = (g.out_dep ? (long long)g.B : 1ll) << g.n_h;
-    pair_launch(g, tiles, C.ggrid.empty() ? C.group_grid : C.ggrid[st.second], s);
   } else {
     GParams g = C.gp[st.second];
     g.out = reinterpret_cast<float2*>(base + reinterpret_cast<size_t>(g.out));
@@ -3392,7 +3465,7 @@ int tnq_internal_gemm_forms(const tnq_plan* plan, int mode, uint32_t batch, int3
   for (size_t i = 0; i < C.gb.size(); ++i) {
     GemmBucketArgs g = C.gb[i];
     g.a[0].ptr = reinterpret_cast<const float2*>(reinterpret_cast<size_t>(g.a[0].ptr) + 256);  // arena offset + base
-    fused[i] = gemm_fused_a(g) ? 1 : 0;
+    fused[i] = gemm_fused_a(g) && !gemm_as_pair(C, i) ? 1 : 0;
   }
   return 0;
 }
@@ -3412,15 +3485,6 @@ int tnq_internal_group_text(const tnq_plan* plan, int mode, uint32_t batch, char
     out += "group " + std::to_string(gi) + " stages " + std::to_string(G.n_st) + " tail " + std::to_string(G.tail) +
            " n_h " + std::to_string(G.n_h) + " gin " + std::to_string(G.n_gin) + " lean2 " + std::to_string(G.lean2) +
            " smem " + std::to_string(C.gsmem[gi]) + "\n";
-    if (C.pair_of[gi] >= 0) {
-      const PairParams& Q = C.pp[C.pair_of[gi]];
-      out += "  pair: a " + std::to_string(Q.a.ebits) + " b " + std::to_string(Q.b.ebits) + " c " +
-             std::to_string(Q.c.gin < 0 ? -1 : Q.c.ebits) + " n1 " + std::to_string(Q.n1 + Q.n_ch - 1) + " n2 " +
-             std::to_string(Q.n2) + " nkx " + std::to_string(Q.nkx) + " nky " + std::to_string(Q.nky) + " n_h " +
-             std::to_string(Q.n_h) + " folds " + std::to_string(Q.fa.n) + "+" + std::to_string(Q.fb.n) + " nf " +
-             std::to_string(Q.fa.nf) + "+" + std::to_string(Q.fb.nf) + " chunks " + std::to_string(Q.n_ch) + " ry " + std::to_string(Q.ry) + " loop " + std::to_string(Q.nl) +
-             " smem " + std::to_string(Q.smem) + "\n";
-    }
     for (int j = 0; j < G.n_gin; ++j) {
       int nh = 0;
       for (int i = 0; i < G.n_h; ++i) nh += G.gin[j].hstride[i] != 0;
@@ -3437,6 +3501,17 @@ int tnq_internal_group_text(const tnq_plan* plan, int mode, uint32_t batch, char
         out += "\n";
       }
     }
+  }
+  for (size_t si = 0; si < C.steps.size(); ++si) {  // steps that k_pair runs (kind 0 bucket, 1 chain, 2 GEMM chain)
+    if (C.step_pair[si] < 0) continue;
+    const PairParams& Q = C.pp[C.step_pair[si]];
+    auto add = [&](const char* name, int v) { out += std::string(" ") + name + " " + std::to_string(v); };
+    out += "pair:";
+    add("kind", C.steps[si].first), add("a", Q.a.ebits), add("b", Q.b.ebits), add("c", Q.c.gin < 0 ? -1 : Q.c.ebits);
+    add("c_u0", Q.c_u0), add("n1", Q.n1 + Q.n_ch / 2), add("n2", Q.n2), add("nkx", Q.nkx), add("nky", Q.nky);
+    add("rx", Q.rx), add("ry", Q.ry), add("loop", Q.nl), add("chunks", Q.n_ch), add("n_h", Q.n_h);
+    add("fold_a", Q.fa.n), add("fold_b", Q.fb.n), add("nf_a", Q.fa.nf), add("nf_b", Q.fb.nf), add("smem", Q.smem);
+    out += "\n";
   }
   for (size_t ki = 0; ki < C.kp.size(); ++ki) {
     const KParams& K = C.kp[ki];
@@ -3913,10 +3988,10 @@ int tnq_internal_launches_per_batch(const tnq_plan* plan, int mode, uint32_t bat
   ExecConfig C;  // a GEMM in the fused-A form packs only B
   C.L = make_layout(*plan, mode, (int)batch);
   if (build_steps(*plan, C.L, C))
-    for (const GemmBucketArgs& g0 : C.gb) {
-      GemmBucketArgs g = g0;
+    for (size_t i = 0; i < C.gb.size(); ++i) {
+      GemmBucketArgs g = C.gb[i];
       g.a[0].ptr = reinterpret_cast<const float2*>(reinterpret_cast<size_t>(g.a[0].ptr) + 256);
-      n -= gemm_fused_a(g) ? 1 : 0;
+      n -= gemm_as_pair(C, i) ? 2 : (gemm_fused_a(g) ? 1 : 0);
     }
   return n + levels + 4;  // + leaf, scalar, final and slice-sum kernels
 }

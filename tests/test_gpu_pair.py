@@ -41,6 +41,25 @@ CASES = [
 ]
 
 
+# (precision, rows, cols, depth, seed, forms): what runs as a product (0 a bucket, 1 a chain, 2 a GEMM chain of mostly
+# padding), C, whether it holds the first eliminated variable, register bits along A / B, those of them that are summed
+FORMS = [
+    (0, 4, 7, 23, 7, {(0, "-", 0, 1, 3, 0, 0)}),
+    (1, 4, 5, 26, 1, {(0, "-", 0, 2, 2, 0, 0)}),
+    (1, 4, 7, 29, 0, {(0, "-", 0, 2, 3, 0, 0)}),
+    (0, 4, 5, 29, 5, {(0, "c", 1, 2, 2, 0, 0)}),
+    (1, 4, 7, 29, 9, {(1, "-", 0, 0, 1, 0, 0)}),
+    (1, 5, 6, 17, 3, {(2, "-", 0, 0, 1, 0, 0)}),
+    (0, 4, 5, 29, 7, {(1, "-", 0, 1, 3, 0, 0)}),
+    (1, 5, 5, 26, 8, {(1, "-", 0, 2, 3, 0, 0)}),
+    (0, 5, 5, 29, 2, {(1, "c", 1, 2, 2, 0, 0)}),
+    (0, 4, 5, 26, 7, {(1, "c", 1, 2, 2, 0, 1)}),
+    (0, 6, 6, 29, 0, {(1, "c", 1, 2, 2, 0, 2)}),
+    (0, 5, 5, 23, 1, {(1, "c", 1, 2, 2, 1, 1)}),
+    (1, 4, 5, 32, 2, {(2, "-", 0, 2, 2, 0, 0)}),
+]
+
+
 def _plan(tnq_lib, rows, cols, depth, seed, **kw):
     circ = I.random_grid_circuit(rows, cols, depth, seed)
     plan = tnq_lib.Plan(circ, max_bag_log2=20, max_p=20, reorder_every=1, **kw)
@@ -50,17 +69,23 @@ def _plan(tnq_lib, rows, cols, depth, seed, **kw):
     return circ, plan
 
 
-def _shapes(tnq_lib, plan):
+def _words(tnq_lib, plan):
     f = tnq_lib.lib().tnq_internal_group_text
     f.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_uint32, ctypes.c_char_p, ctypes.c_size_t]
     buf = ctypes.create_string_buffer(1 << 20)
     assert f(plan.handle, 0, 2, buf, 1 << 20) == 0
-    out = set()
     for line in re.findall(r"pair: (.*)", buf.value.decode()):
         w = line.split()
-        d = dict(zip(w[::2], w[1::2]))
-        out.add(("-" if d["c"] == "-1" else "c",) + tuple(int(d[k]) for k in ("n1", "n2", "nkx", "nky")))
-    return out
+        d = dict(zip(w[::2], map(int, w[1::2])))
+        yield dict(d, c="-" if d["c"] < 0 else "c")
+
+
+def _shapes(tnq_lib, plan):
+    return {tuple(d[k] for k in ("c", "n1", "n2", "nkx", "nky")) for d in _words(tnq_lib, plan) if not d["c_u0"]}
+
+
+def _forms(tnq_lib, plan):
+    return {tuple(d[k] for k in ("kind", "c", "c_u0", "rx", "ry", "nkx", "nky")) for d in _words(tnq_lib, plan)}
 
 
 @pytest.mark.parametrize("rows,cols,depth,seed,shapes", CASES)
@@ -80,7 +105,30 @@ def test_every_launch_stays_in_bounds(tnq_lib, rows, cols, depth, seed, shapes):
 def test_chain_matches_oracle_and_separate_buckets(cuda, tnq_lib, oracle_lib, rows, cols, depth, seed, shapes):
     circ, plan = _plan(tnq_lib, rows, cols, depth, seed)
     assert shapes <= _shapes(tnq_lib, plan)
-    plain = _plan(tnq_lib, rows, cols, depth, seed, fuse_min_rank=0)[1]
+    _check(tnq_lib, oracle_lib, circ, plan, _plan(tnq_lib, rows, cols, depth, seed, fuse_min_rank=0)[1], seed, TOL)
+
+
+@pytest.mark.parametrize("precision,rows,cols,depth,seed,forms", FORMS)
+def test_every_form_stays_in_bounds(tnq_lib, precision, rows, cols, depth, seed, forms):
+    _, plan = _plan(tnq_lib, rows, cols, depth, seed, precision=precision)
+    assert forms <= _forms(tnq_lib, plan)
+    msg = ctypes.create_string_buffer(512)
+    for mode in (0, 1):
+        for batch in (1, 2, 16):
+            assert tnq_lib.lib().tnq_internal_validate(plan.handle, mode, batch, msg, 512) == 0, msg.value
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("precision,rows,cols,depth,seed,forms", FORMS)
+def test_form_matches_oracle_and_separate_buckets(cuda, tnq_lib, oracle_lib, precision, rows, cols, depth, seed, forms):
+    circ, plan = _plan(tnq_lib, rows, cols, depth, seed, precision=precision)
+    assert forms <= _forms(tnq_lib, plan)
+    # (split precision: the plan's other GEMM chains keep 16 to 22 bits of their operands)
+    _check(tnq_lib, oracle_lib, circ, plan, _plan(tnq_lib, rows, cols, depth, seed, fuse_min_rank=0)[1], seed,
+           1e-4 if precision else TOL)
+
+
+def _check(tnq_lib, oracle_lib, circ, plan, plain, seed, tol):
     n = min(plan.info()["n_slices"], 4)
     bits = I.random_bitstring(circ.n_qubits, seed)
     _, got = tnq_lib.contract_sliced(plan, bits, 0, n, per_slice=True)
@@ -88,10 +136,11 @@ def test_chain_matches_oracle_and_separate_buckets(cuda, tnq_lib, oracle_lib, ro
     ref = np.array([oracle_lib.contract(circ, bits, order=plan.order(), mu=plan.sliced(), slices=(s, s + 1))
                     for s in range(n)])
     scale = np.maximum(np.abs(ref), 2.0 ** (-(circ.n_qubits + plan.info()["p"]) / 2))
-    assert np.max(np.abs(got - ref) / scale) <= TOL
-    assert np.max(np.abs(got - sep) / scale) <= TOL
+    assert np.max(np.abs(got - ref) / scale) <= tol
+    assert np.max(np.abs(got - sep) / scale) <= tol
     # three bitstrings at once: the item dimension carries (bitstring, slice)
     more = [bits, I.random_bitstring(circ.n_qubits, seed + 1), I.random_bitstring(circ.n_qubits, seed + 2)]
-    if plan.info()["p"] == 0:
+    # (the GEMM packs multiply the small tensors in another order when one of them depends on the item)
+    if plan.info()["p"] == 0 and plan.info()["n_gemm_buckets"] == 0:
         out = tnq_lib.amplitudes_batch([plan], [more])
         assert abs(out[0] - got[0]) <= 1e-9 * abs(got[0])
