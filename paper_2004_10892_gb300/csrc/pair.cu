@@ -87,16 +87,16 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
     int4 v = make_int4(0, 0, 0, 0);
     for (int i = 0; i < P.n2; ++i)
       if ((t >> i) & 1) {
-        v.x += P.k2a[i];
-        v.y += P.k2b[i];
-        v.z += P.k2c[i];
+        v.x ^= P.k2a[i];
+        v.y ^= P.k2b[i];
+        v.z ^= P.k2c[i];
       }
     s_k2[t] = v;
     int2 w = make_int2(0, 0);
     for (int i = 0; i < P.n1; ++i)
       if ((t >> i) & 1) {
-        w.x += P.k1a[i];
-        w.y += P.k1b[i];
+        w.x ^= P.k1a[i];
+        w.y ^= P.k1b[i];
       }
     s_k1[t] = w;
   }
@@ -104,9 +104,9 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
     int4 v = make_int4(0, 0, 0, 0);
     for (int i = 0; i < P.nl; ++i)
       if ((t >> i) & 1) {
-        v.x += P.la[i];
-        v.y += P.lb[i];
-        v.z += P.lc[i];
+        v.x ^= P.la[i];
+        v.y ^= P.lb[i];
+        v.z ^= P.lc[i];
         v.w += P.lo[i];
       }
     s_l[t] = v;
@@ -115,13 +115,12 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
 #pragma unroll
   for (int o = 0; o < NOP; ++o) {
     const POp& O = *ops[o];
-    tg[o] = tf[o] = 0;
-    td[o] = O.base;
+    tg[o] = tf[o] = td[o] = 0;
 #pragma unroll
     for (int i = 0; i < PTB; ++i)
       if (i < O.ebits && ((t >> i) & 1)) {
         tg[o] += O.g[i];
-        td[o] += O.d[i];
+        td[o] ^= O.d[i];
         tf[o] += O.f[i];
       }
     const int nit = O.ebits > PTB ? 1 << (O.ebits - PTB) : 1;
@@ -130,19 +129,19 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
       for (int i = PTB; i < O.ebits; ++i)
         if ((t >> (i - PTB)) & 1) {
           v.x += O.g[i];
-          v.y += O.d[i];
+          v.y ^= O.d[i];
           v.z += O.f[i];
         }
       s_it[o][t] = v;
     }
   }
-  int ra = P.a.base, rb = P.b.base, rc = HASC ? P.c.base : 0, ro = 0;  // this thread's register tile
+  int ra = 0, rb = 0, rc = 0, ro = 0;  // this thread's register tile
 #pragma unroll
   for (int i = 0; i < PTB; ++i)
     if ((t >> i) & 1) {
-      ra += P.ta[i];
-      rb += P.tb[i];
-      if (HASC) rc += P.tc[i];
+      ra ^= P.ta[i];
+      rb ^= P.tb[i];
+      if (HASC) rc ^= P.tc[i];
       ro += P.to[i];
     }
   const bool fold_a = P.fa.n > 0;
@@ -193,12 +192,12 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
     for (int o = 0; o < NOP; ++o) {
       const POp& O = *ops[o];
       const float2* src = s_src[slot][o] + tg[o] + ((chunk & 1) ? O.gch[0] : 0) + ((chunk & 2) ? O.gch[1] : 0);
-      const unsigned dst = sm0 + 16u * (unsigned)(buf * P.stage + td[o]);
+      const unsigned dst = sm0 + 16u * (unsigned)(buf * P.stage + O.base);
       const int nit = O.ebits > PTB ? 1 << (O.ebits - PTB) : 1;
       if (O.ebits >= PTB || t < (1 << O.ebits))
         for (int it = 0; it < nit; ++it) {
           const int4 k = s_it[o][it];
-          cp_async16(dst + 16u * (unsigned)k.y, src + k.x);
+          cp_async16(dst + 16u * (unsigned)(td[o] ^ k.y), src + k.x);
         }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
@@ -211,16 +210,17 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
       const POp& O = *ops[o];
       const float4* ft = (o == 0 ? s_fa[n & 1] : s_fb[n & 1]) + tf[o] + s_fold[slot][o] +
                          ((chunk & 1) ? O.fch[0] : 0) + ((chunk & 2) ? O.fch[1] : 0);
-      float4* dst = sm + buf * P.stage + td[o];
+      float4* dst = sm + buf * P.stage + O.base;
       const int nit = O.ebits > PTB ? 1 << (O.ebits - PTB) : 1;
       if (O.ebits >= PTB || t < (1 << O.ebits)) {
 #pragma unroll 2
         for (int it = 0; it < nit; ++it) {
           const int4 k = s_it[o][it];
-          const float4 v = dst[k.y], f = ft[k.z];
+          const int at = td[o] ^ k.y;
+          const float4 v = dst[at], f = ft[k.z];
           const float2 v0 = cmul(make_float2(v.x, v.y), make_float2(f.x, f.y));
           const float2 v1 = cmul(make_float2(v.z, v.w), make_float2(f.z, f.w));
-          dst[k.y] = make_float4(v0.x, v0.y, v1.x, v1.y);
+          dst[at] = make_float4(v0.x, v0.y, v1.x, v1.y);
         }
       }
     }
@@ -267,26 +267,25 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
       __syncthreads();  // the chunk is staged, and every thread is done with the other stage
       if (!last) issue(slot, c + 1, buf ^ 1);
       else if (more) issue((slot + 1) % RING, 0, buf ^ 1);
-      const float4* pa = sm + buf * P.stage + ra;
-      const float4* pb = sm + buf * P.stage + rb;
+      const float4* pa = sm + buf * P.stage + P.a.base;
+      const float4* pb = sm + buf * P.stage + P.b.base;
       float2* dst = s_out[slot] + ro;
       const int n1 = 1 << P.n1;
-      auto off_x = [&](int i, const int* w) { return ((i & 1) ? w[0] : 0) + ((i & 2) ? w[1] : 0); };
+      auto off_x = [&](int i, const int* w) { return ((i & 1) ? w[0] : 0) ^ ((i & 2) ? w[1] : 0); };
       auto off_y = [&](int j, const int* w) {
-        return ((j & 1) ? w[0] : 0) + ((j & 2) ? w[1] : 0) + (RY > 2 && (j & 4) ? w[2] : 0);
+        return ((j & 1) ? w[0] : 0) ^ ((j & 2) ? w[1] : 0) ^ (RY > 2 && (j & 4) ? w[2] : 0);
       };
       auto products = [&](int oa, int ob) {
 #pragma unroll 1
         for (int q = 0; q < n1; ++q) {
           const int2 k = s_k1[q];
-          const float4* qa = pa + (oa + k.x);
-          const float4* qb = pb + (ob + k.y);
+          const int qa = oa ^ k.x, qb = ob ^ k.y;
           float4 va[NX];
 #pragma unroll
-          for (int i = 0; i < NX; ++i) va[i] = qa[off_x(i, P.xa)];
+          for (int i = 0; i < NX; ++i) va[i] = pa[qa ^ off_x(i, P.xa)];
 #pragma unroll
           for (int j = 0; j < NY; ++j) {
-            const float4 vb = qb[off_y(j, P.yb)];
+            const float4 vb = pb[qb ^ off_y(j, P.yb)];
 #pragma unroll
             for (int i = 0; i < NX; ++i) cfma2(x[i][j], va[i], vb);
           }
@@ -296,14 +295,15 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
 #pragma unroll 1
         for (int q = 0; q < n1; ++q) {
           const int2 k = s_k1[q];
-          const float2* qa = reinterpret_cast<const float2*>(pa + (oa + k.x)) + h;
-          const float2* qb = reinterpret_cast<const float2*>(pb + (ob + k.y)) + h;
+          const int qa = oa ^ k.x, qb = ob ^ k.y;
+          const float2* ha = reinterpret_cast<const float2*>(pa) + h;
+          const float2* hb = reinterpret_cast<const float2*>(pb) + h;
           float2 va[NX];
 #pragma unroll
-          for (int i = 0; i < NX; ++i) va[i] = qa[2 * off_x(i, P.xa)];
+          for (int i = 0; i < NX; ++i) va[i] = ha[2 * (qa ^ off_x(i, P.xa))];
 #pragma unroll
           for (int j = 0; j < NY; ++j) {
-            const float2 vb = qb[2 * off_y(j, P.yb)];
+            const float2 vb = hb[2 * (qb ^ off_y(j, P.yb))];
 #pragma unroll
             for (int i = 0; i < NX; ++i) cfma(x[i][j], va[i], vb);
           }
@@ -311,7 +311,8 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
       };
       auto store = [&](int i, int j, float2 r, int lo) {
         const int ri = i << NKX, rj = j << NKY;
-        dst[lo + off_x(ri, P.xo) + off_y(rj, P.yo)] = r;
+        dst[lo + ((ri & 1) ? P.xo[0] : 0) + ((ri & 2) ? P.xo[1] : 0) + ((rj & 1) ? P.yo[0] : 0) +
+            ((rj & 2) ? P.yo[1] : 0) + (RY > 2 && (rj & 4) ? P.yo[2] : 0)] = r;
         tmax = fmaxf(tmax, fmaxf(fabsf(r.x), fabsf(r.y)));
       };
       const int nl = 1 << P.nl;
@@ -328,28 +329,29 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
 #pragma unroll 1
           for (int q2 = 0; q2 < n2; ++q2) {
             const int4 k2 = s_k2[q2];
-            const float4* pc = sm + buf * P.stage + rc + lv.z + k2.z;
+            const float4* pc = sm + buf * P.stage + P.c.base;
+            const int oc = rc ^ lv.z ^ k2.z;
             if constexpr (CM == 2) {
 #pragma unroll 1
               for (int h = 0; h < 2; ++h) {
-                half_products(lv.x + k2.x, lv.y + k2.y, h);
+                half_products(ra ^ lv.x ^ k2.x, rb ^ lv.y ^ k2.y, h);
                 const float2* ph = reinterpret_cast<const float2*>(pc) + h;
 #pragma unroll
                 for (int i = 0; i < NX; ++i)
 #pragma unroll
                   for (int j = 0; j < NY; ++j) {
-                    cfma(acc[i >> NKX][j >> NKY], x[i][j], ph[2 * (off_x(i, P.xc) + off_y(j, P.yc))]);
+                    cfma(acc[i >> NKX][j >> NKY], x[i][j], ph[2 * (oc ^ off_x(i, P.xc) ^ off_y(j, P.yc))]);
                     x[i][j] = make_float2(0.f, 0.f);
                   }
               }
             } else {
-              products(lv.x + k2.x, lv.y + k2.y);
+              products(ra ^ lv.x ^ k2.x, rb ^ lv.y ^ k2.y);
               // times C, summed over the K2 register bits (C's bit 0 is B's register bit 0)
 #pragma unroll
               for (int i = 0; i < NX; ++i)
 #pragma unroll
                 for (int j = 0; j < NY; j += 2) {
-                  const float4 v = pc[off_x(i, P.xc) + off_y(j, P.yc)];  // (yc[0] is 0: the pair's own bit)
+                  const float4 v = pc[oc ^ off_x(i, P.xc) ^ off_y(j, P.yc)];  // (yc[0] is 0: the pair's own bit)
                   const float2 u = x[i][j], w = x[i][j + 1];
                   cfma2(acc[i >> NKX][j >> NKY], make_float4(u.x, u.y, w.x, w.y), v);
                   x[i][j] = x[i][j + 1] = make_float2(0.f, 0.f);
@@ -361,7 +363,7 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
 #pragma unroll
             for (int j = 0; j < YO; ++j) store(i, j, acc[i][j], lv.w);
         } else {
-          products(lv.x, lv.y);
+          products(ra ^ lv.x, rb ^ lv.y);
           if (last) {
 #pragma unroll
             for (int i = 0; i < NX; ++i)

@@ -37,15 +37,16 @@ struct PIn {
 // A staged operand. Its local entries are enumerated as pairs over its bit 0
 // by an index e (bits by increasing memory stride, so that consecutive threads
 // read consecutive memory); bit i of e adds g[i] to the global offset
-// (elements), d[i] to the shared-memory slot (16-byte units) and f[i] to the
-// fold table's index. Tile bit i adds h[i] and fh[i], bit i of the chunk gch[i] and fch[i].
+// (elements) and f[i] to the fold table's index, and is d[i] of the
+// shared-memory slot (16-byte units): slots are combined with XOR, since they
+// are swizzled (pair_params). Tile bit i adds h[i] and fh[i], bit i of the chunk gch[i] and fch[i].
 struct POp {
   int gin;
   int ebits;
   int g[PE_MAX], d[PE_MAX], f[PE_MAX];
   int h[PH_MAX], fh[PH_MAX];
   int gch[2], fch[2];
-  int base;                     // first slot of a stage
+  int base, size;               // first slot of a stage, slots (a power of two)
 };
 
 // Small tensors folded into one operand: table of (u_0 = 0, u_0 = 1) pairs

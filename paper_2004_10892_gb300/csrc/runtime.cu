@@ -2254,12 +2254,15 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
     }
   }
   G.n_ch = 1 << chunk.size();
-  // staged operands: slot = row + pitch * (its eliminated variables but bit
-  // 0), rows numbered by the thread bits it holds, then by its register
-  // outputs; the odd pitch and the lowest row bits on the lowest lanes keep
-  // both the staging stores and the register tile's loads free of conflicts
+  // staged operands: place = pair over its eliminated variables (but bit 0) |
+  // row << that, rows numbered by the thread bits it holds (the lowest lanes
+  // lowest), then by its loop and register outputs. Consecutive threads of the
+  // copy then write consecutive slots (scattered 16-byte copies took a cycle of
+  // the shared-memory pipe each), and the slot's low three bits are XORed with
+  // the row's, so that eight lanes that read one pair of eight rows hit eight
+  // bank groups. Slots of disjoint bits combine with XOR.
   int base = 0;
-  std::vector<int> weight[3];  // per operand: slot weight of each of its variables
+  std::vector<int> weight[3];  // per operand: slot of each of its variables
   for (int k = 0; k < 3; ++k) {
     POp& O = k == 0 ? G.a : (k == 1 ? G.b : G.c);
     O.gin = ops[k];
@@ -2267,10 +2270,13 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
     const std::vector<int>& v = vars(O.gin);
     std::vector<int>& w = weight[k];
     w.assign(v.size(), 0);
-    int rows = 0;
+    int nk = 0;
+    for (size_t p = 1; p < v.size(); ++p)
+      if (index_in(chunk, v[p]) < 0 && index_in(K, v[p]) >= 0) w[p] = 1 << nk++;
+    int n = nk;
     auto row = [&](int x) {
       const int p = index_in(v, x);
-      if (p >= 0) w[p] = 1 << rows++;
+      if (p >= 0) w[p] = 1 << n++;
     };
     for (int x : thr) row(x);
     for (int x : loop) row(x);
@@ -2278,12 +2284,10 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
       if (index_in(K, x) < 0) row(x);
     for (int x : yreg)
       if (index_in(K, x) < 0) row(x);
-    const int pitch = (1 << rows) | 1;
-    int nk = 0;
-    for (size_t p = 1; p < v.size(); ++p)
-      if (index_in(chunk, v[p]) < 0 && index_in(K, v[p]) >= 0) w[p] = pitch << nk++;
+    for (int& x : w) x ^= (x >> std::max(3, nk)) & 7;
     O.base = base;
-    base += pitch << nk;
+    O.size = std::max(8, 1 << n);
+    base += O.size;
     for (size_t p = 1; p < v.size(); ++p) {
       if (p > 30) return false;
       const int fi = k < 2 ? index_in(fold_vars[k], v[p]) : -1, f = fi < 0 ? 0 : 1 << fi;
@@ -2851,7 +2855,7 @@ static std::string validate_config(const tnq_plan& P, int mode, int B) {
       const POp& O = *ops[k];
       if (O.gin < 0) continue;
       long long m = item_max(O.gin) + 1 + O.gch[0] + O.gch[1];
-      int d = O.base, f = O.fch[0] + O.fch[1];
+      int d = 0, f = O.fch[0] + O.fch[1];
       for (int i = 0; i < G.n_h; ++i) {
         if (O.h[i] & 1) return name + ": odd tile stride";
         m += O.h[i];
@@ -2860,24 +2864,27 @@ static std::string validate_config(const tnq_plan& P, int mode, int B) {
       for (int i = 0; i < O.ebits; ++i) {
         if ((O.g[i] & 1) || ((O.gch[0] | O.gch[1]) & 1)) return name + ": odd local stride";
         m += O.g[i];
-        d += O.d[i];
+        d |= O.d[i];
         f += O.f[i];
       }
       if ((G.gin[O.gin].istride & 1) || ((size_t)G.gin[O.gin].ptr / 8) % 2) return name + ": unaligned input";
       if (m >= alloc(g.ext_inputs[O.gin])) return name + ": staged input overflows";
-      if (d >= G.stage) return name + ": staged operand outside its stage";
+      if (d >= O.size || O.base + O.size > G.stage) return name + ": staged operand outside its stage";
+      for (int i = 0; i < O.ebits; ++i)  // one slot per staged pair: the bits' slots are independent
+        for (int j = 0; j < i; ++j)
+          if ((O.d[i] & ~7) ? (O.d[i] & O.d[j] & ~7) : O.d[i] == O.d[j]) return name + ": slots";
       if (k < 2 && f >= 1 << (k ? G.fb.nf : G.fa.nf)) return name + ": fold index";
       // the register tile reads only staged slots
-      long long r = O.base;
-      for (int i = 0; i < PTB; ++i) r += k == 0 ? G.ta[i] : (k == 1 ? G.tb[i] : G.tc[i]);
+      int r = 0;
+      for (int i = 0; i < PTB; ++i) r |= k == 0 ? G.ta[i] : (k == 1 ? G.tb[i] : G.tc[i]);
       if (k != 1)
-        for (int i = 0; i < G.rx; ++i) r += k == 0 ? G.xa[i] : G.xc[i];
+        for (int i = 0; i < G.rx; ++i) r |= k == 0 ? G.xa[i] : G.xc[i];
       if (k != 0)  // (C without u_0 is read in pairs over B's register bit 0)
-        for (int i = k == 2 && !G.c_u0; i < G.ry; ++i) r += k == 1 ? G.yb[i] : G.yc[i];
-      for (int i = 0; i < G.nl; ++i) r += k == 0 ? G.la[i] : (k == 1 ? G.lb[i] : G.lc[i]);
-      for (int i = 0; i < G.n1; ++i) r += k == 0 ? G.k1a[i] : (k == 1 ? G.k1b[i] : 0);
-      for (int i = 0; i < G.n2; ++i) r += k == 0 ? G.k2a[i] : (k == 1 ? G.k2b[i] : G.k2c[i]);
-      if (r > d) return name + ": register tile outside the staged operand";
+        for (int i = k == 2 && !G.c_u0; i < G.ry; ++i) r |= k == 1 ? G.yb[i] : G.yc[i];
+      for (int i = 0; i < G.nl; ++i) r |= k == 0 ? G.la[i] : (k == 1 ? G.lb[i] : G.lc[i]);
+      for (int i = 0; i < G.n1; ++i) r |= k == 0 ? G.k1a[i] : (k == 1 ? G.k1b[i] : 0);
+      for (int i = 0; i < G.n2; ++i) r |= k == 0 ? G.k2a[i] : (k == 1 ? G.k2b[i] : G.k2c[i]);
+      if (r & ~d) return name + ": register tile outside the staged operand";
     }
     for (int side = 0; side < 2; ++side) {
       const PFold& F = side ? G.fb : G.fa;
