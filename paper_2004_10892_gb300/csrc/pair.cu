@@ -394,6 +394,14 @@ static PairKernel pair_kernel(const PairParams& p) {
     if (p.rx) return k_pair<1, 3, 0, 0, 0>;
     return p.ry > 1 ? k_pair<0, 3, 0, 0, 0> : k_pair<0, 1, 0, 0, 0>;
   }
+  if (p.ry > 2) switch (p.nkx * 3 + p.nky) {
+    case 1: return k_pair<2, 3, 0, 1, 1>;
+    case 2: return k_pair<2, 3, 0, 2, 1>;
+    case 4: return k_pair<2, 3, 1, 1, 1>;
+    case 5: return k_pair<2, 3, 1, 2, 1>;
+    case 7: return k_pair<2, 3, 2, 1, 1>;
+    default: return k_pair<2, 3, 2, 2, 1>;
+  }
   switch ((p.c_u0 * 3 + p.nkx) * 3 + p.nky) {
     case 1: return k_pair<2, 2, 0, 1, 1>;
     case 2: return k_pair<2, 2, 0, 2, 1>;

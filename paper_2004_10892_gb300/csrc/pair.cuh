@@ -16,7 +16,7 @@ namespace tnq {
 constexpr int PTB = 8;              // log2 threads per k_pair block
 constexpr int PTPB = 1 << PTB;
 constexpr int PRX_MAX = 2;          // register tile: up to 2^2 entries along A's variables ...
-constexpr int PRY_MAX = 3;          // ... x 2^2 or (two large tensors) 2^3 along B's
+constexpr int PRY_MAX = 3;          // ... x 2^2 or 2^3 along B's
 constexpr int PE_MAX = 13;          // staged (u = 0, u = 1) pairs of one operand: at most 2^13
 constexpr int PF_MAX = 7;           // fold table of one operand: at most 2^8 pairs
 constexpr int PIN_MAX = 16;         // tensors a chain reads

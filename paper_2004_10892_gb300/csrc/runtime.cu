@@ -2138,11 +2138,12 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
   G.nky = (int)yreg.size();
   if (G.c_u0 && G.nkx > G.nky) return false;
   G.rx = C < 0 ? std::min(2, alone(A, B, o.vars)) : 2;
-  // 4 x 8 register tiles for two tensors that have the variables, and outputs
-  // for 2^PAIR_TILES tiles an item (fewer leave the device idle), else 4 x 4
+  // 4 x 8 register tiles where B has the variables and there are outputs for
+  // 2^PAIR_TILES tiles an item (fewer leave the device idle), else 4 x 4
   // with nothing to share along A the tile only holds B: small, for long sums
   if (G.rx < 2) G.ry = G.rx || (int)K.size() <= 2 ? 3 : 1;
-  else G.ry = C < 0 && alone(B, A, o.vars) >= 3 && o.rank() >= PTB + G.rx + 3 + PAIR_TILES ? 3 : 2;
+  else G.ry = !G.c_u0 && alone(B, A, o.vars) + G.nky >= 3 &&
+              o.rank() >= PTB + G.rx - G.nkx + 3 - G.nky + PAIR_TILES ? 3 : 2;
   const int need_x = G.rx - G.nkx, need_y = G.ry - G.nky, n_one = PTB + need_x + need_y;
   if (o.rank() < n_one) return false;
   const int ops[3] = {A, B, C};
