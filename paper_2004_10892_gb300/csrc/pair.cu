@@ -52,12 +52,14 @@ __device__ __forceinline__ void cfma2(float2& r, float4 a, float4 b) {
 // 16-byte shared loads feed 32 x 2^RY FMAs. Shared memory delivers 128 bytes a
 // cycle to registers, so 4 x 4 needs all of it at the full FMA rate and 4 x 8
 // three quarters.
-// CM: 0 no C, 1 C without u_0 (its bit 0 is B's register bit 0), 2 C with u_0.
+// CM: 0 no C, 1 C without u_0 (its bit 0 is B's register bit 0), 2 C with u_0,
+// 3 B alone: B comes through shared memory only to be read in consecutive
+// pieces, and is multiplied by the small tensors' product as it is summed.
 template <int RX, int RY, int NKX, int NKY, int CM>
 __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairParams P, long long n_tiles) {
   extern __shared__ float4 sm[];
-  constexpr bool HASC = CM != 0;
-  constexpr int NOP = HASC ? 3 : 2;
+  constexpr bool HASC = CM == 1 || CM == 2, ONE = CM == 3;
+  constexpr int NOP = HASC ? 3 : 2, OP0 = ONE ? 1 : 0;
   constexpr int RING = 4;  // a thread is at most one barrier ahead: what it writes is two tiles ahead
   __shared__ float4 s_fa[2][1 << PF_MAX], s_fb[2][1 << PF_MAX];  // by item, alternating
   __shared__ int4 s_it[NOP][1 << (PE_MAX - PTB)];  // staging iteration: global offset, slot, fold index
@@ -78,7 +80,7 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
   if (blockIdx.x >= n_tiles) return;
   // ---- tables that every tile uses
   if (t < PH_MAX) {
-    s_hstr[0][t] = t < P.n_h ? P.a.h[t] : 0;
+    s_hstr[0][t] = !ONE && t < P.n_h ? P.a.h[t] : 0;
     s_hstr[1][t] = t < P.n_h ? P.b.h[t] : 0;
     s_hstr[2][t] = HASC && t < P.n_h ? P.c.h[t] : 0;
     s_hstr[3][t] = t < P.n_h ? P.out_h[t] : 0;
@@ -95,7 +97,7 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
     int2 w = make_int2(0, 0);
     for (int i = 0; i < P.n1; ++i)
       if ((t >> i) & 1) {
-        w.x ^= P.k1a[i];
+        w.x ^= ONE ? P.k1f[i] : P.k1a[i];
         w.y ^= P.k1b[i];
       }
     s_k1[t] = w;
@@ -113,7 +115,7 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
   }
   int tg[NOP], td[NOP], tf[NOP];  // this thread's part of the staging offsets
 #pragma unroll
-  for (int o = 0; o < NOP; ++o) {
+  for (int o = OP0; o < NOP; ++o) {
     const POp& O = *ops[o];
     tg[o] = tf[o] = td[o] = 0;
 #pragma unroll
@@ -139,7 +141,7 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
 #pragma unroll
   for (int i = 0; i < PTB; ++i)
     if ((t >> i) & 1) {
-      ra ^= P.ta[i];
+      ra ^= ONE ? P.ft[i] : P.ta[i];
       rb ^= P.tb[i];
       if (HASC) rc ^= P.tc[i];
       ro += P.to[i];
@@ -157,6 +159,7 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
     const int v = __reduce_add_sync(0xffffffffu, ((h >> lane) & 1) ? s_hstr[w][lane] : 0);
     if (lane) return;
     if (w < NOP) {
+      if (w < OP0) return;
       const PIn& g = P.gin[w == 0 ? P.a.gin : (w == 1 ? P.b.gin : P.c.gin)];
       s_src[slot][w] = g.ptr + (g.dep ? item * g.istride : 0ll) + v;
     } else if (w == 3) {
@@ -189,7 +192,7 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
   };
   auto issue = [&](int slot, int chunk, int buf) {
 #pragma unroll
-    for (int o = 0; o < NOP; ++o) {
+    for (int o = OP0; o < NOP; ++o) {
       const POp& O = *ops[o];
       const float2* src = s_src[slot][o] + tg[o] + ((chunk & 1) ? O.gch[0] : 0) + ((chunk & 2) ? O.gch[1] : 0);
       const unsigned dst = sm0 + 16u * (unsigned)(buf * P.stage + O.base);
@@ -263,11 +266,12 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
         if (new_item) item_setup(next >> P.n_h, n_item + 1);
       }
       asm volatile("cp.async.wait_all;" ::: "memory");
-      fold(slot, c, buf, n_item);
+      if constexpr (!ONE) fold(slot, c, buf, n_item);
       __syncthreads();  // the chunk is staged, and every thread is done with the other stage
       if (!last) issue(slot, c + 1, buf ^ 1);
       else if (more) issue((slot + 1) % RING, 0, buf ^ 1);
-      const float4* pa = sm + buf * P.stage + P.a.base;
+      const float4* pa = ONE ? s_fb[n_item & 1] + s_fold[slot][1] + ((c & 1) ? P.b.fch[0] : 0) + ((c & 2) ? P.b.fch[1] : 0)
+                             : sm + buf * P.stage + P.a.base;
       const float4* pb = sm + buf * P.stage + P.b.base;
       float2* dst = s_out[slot] + ro;
       const int n1 = 1 << P.n1;
@@ -282,12 +286,13 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
           const int qa = oa ^ k.x, qb = ob ^ k.y;
           float4 va[NX];
 #pragma unroll
-          for (int i = 0; i < NX; ++i) va[i] = pa[qa ^ off_x(i, P.xa)];
+          for (int i = 0; i < NX; ++i)
+            if (!ONE) va[i] = pa[qa ^ off_x(i, P.xa)];
 #pragma unroll
           for (int j = 0; j < NY; ++j) {
             const float4 vb = pb[qb ^ off_y(j, P.yb)];
 #pragma unroll
-            for (int i = 0; i < NX; ++i) cfma2(x[i][j], va[i], vb);
+            for (int i = 0; i < NX; ++i) cfma2(x[i][j], ONE ? pa[qa ^ off_y(j, P.yf)] : va[i], vb);
           }
         }
       };
@@ -389,6 +394,7 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
 
 using PairKernel = void (*)(PairParams, long long);
 static PairKernel pair_kernel(const PairParams& p) {
+  if (p.a.gin < 0) return p.ry > 1 ? k_pair<0, 3, 0, 0, 3> : k_pair<0, 1, 0, 0, 3>;
   if (p.c.gin < 0) {
     if (p.rx == 2) return p.ry > 2 ? k_pair<2, 3, 0, 0, 0> : k_pair<2, 2, 0, 0, 0>;
     if (p.rx) return k_pair<1, 3, 0, 0, 0>;

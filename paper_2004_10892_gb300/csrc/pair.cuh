@@ -8,6 +8,7 @@
 // which has its variables among A's or among B's and is folded into that one.
 // With K2 = K & vars(C) and K1 = K - K2:
 //   out[o] = sum_K2 C[K2, o] (sum_K1 A[K1, K2, o] B[K1, K2, o]).
+// With one large tensor only (B) the small tensors' product takes A's place.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -60,7 +61,7 @@ struct PFold {
 
 struct PairParams {
   PIn gin[PIN_MAX];
-  POp a, b, c;                  // c.gin < 0: no third tensor
+  POp a, b, c;                  // a.gin < 0: B alone; c.gin < 0: no third tensor
   PFold fa, fb;
   float2* out;
   long long out_istride;
@@ -71,6 +72,7 @@ struct PairParams {
   int rx, ry;                   // register bits along A / B
   int c_u0;                     // 1: C holds u_0 (K2 then includes it)
   int nl, la[PL_MAX], lb[PL_MAX], lc[PL_MAX], lo[PL_MAX];  // a thread's loop over outputs
+  int ft[PTB], yf[PRY_MAX], k1f[PK_MAX];        // B alone: the fold table's index instead of A's slots
   int n1, k1a[PK_MAX], k1b[PK_MAX];                // K1 without u_0 and the chunk's variable: slots of a and b
   int n2, k2a[PK_MAX], k2b[PK_MAX], k2c[PK_MAX];   // K2 outside the register tile
   int nkx, nky;                 // K2 bits among the register bits along A / B (the low ones)

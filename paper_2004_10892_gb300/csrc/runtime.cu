@@ -2044,7 +2044,7 @@ static GParams group_gparams(const tnq_plan& P, const Layout& L, const FusedGrou
 // must not depend on it). Requirements and why:
 //  * two or three large tensors (rank above PAIR_SMALL), two of them with the
 //    first eliminated variable: the product of two tensors is what the
-//    register tile shares operands over;
+//    register tile shares operands over; or one, which is streamed;
 //  * every other tensor has its variables among A's or among B's: it is
 //    multiplied into that operand as it is staged;
 //  * 2^2 register entries along variables of A alone and of B alone
@@ -2070,7 +2070,7 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
   for (int j = 0; j < (int)in.size(); ++j) (prog.tensors[in[j]].rank() > PAIR_SMALL ? large : small).push_back(j);
   int with_u0 = 0;
   for (int j : large) with_u0 += holds(j, u0);
-  if (large.size() < 2 || large.size() > 3 || with_u0 < 2) return false;
+  if (large.empty() || large.size() > 3 || with_u0 < std::min<int>(2, (int)large.size())) return false;
   int A = -1, B = -1, C = -1, c0 = -1;
   // variables of j that k does not hold: among the outputs / the eliminated ones
   auto alone = [&](int j, int k, const std::vector<int>& among) {
@@ -2092,10 +2092,14 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
       }
     }
   }
-  for (int j : large)
-    if (j != C) (A < 0 ? A : B) = j;
+  const bool one = large.size() == 1;
+  if (one) B = large[0];
+  else
+    for (int j : large)
+      if (j != C) (A < 0 ? A : B) = j;
   G.c_u0 = with_u0 == 3;
-  if (G.c_u0) {
+  if (one) {
+  } else if (G.c_u0) {
     if (vars(C)[0] != u0) return false;
     std::vector<int> in_c;
     for (int v : K)
@@ -2112,7 +2116,7 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
       if (alone(B, A, o.vars) < 3) return false;
     }
   }
-  if (vars(A)[0] != u0 || vars(B)[0] != u0) return false;
+  if ((!one && vars(A)[0] != u0) || vars(B)[0] != u0) return false;
   std::vector<int> sa, sb;
   for (int j : small) {
     bool ina = true, inb = true;
@@ -2137,7 +2141,7 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
   G.nkx = (int)xreg.size();
   G.nky = (int)yreg.size();
   if (G.c_u0 && G.nkx > G.nky) return false;
-  G.rx = C < 0 ? std::min(2, alone(A, B, o.vars)) : 2;
+  G.rx = one ? 0 : (C < 0 ? std::min(2, alone(A, B, o.vars)) : 2);
   // 4 x 8 register tiles where B has the variables and there are outputs for
   // 2^PAIR_TILES tiles an item (fewer leave the device idle), else 4 x 4
   // with nothing to share along A the tile only holds B: small, for long sums
@@ -2191,7 +2195,7 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
     nx += holds(A, o.vars[best]) && !holds(B, o.vars[best]);
     ny += holds(B, o.vars[best]) && !holds(A, o.vars[best]);
     if (n + 1 == n_local && (int)loop.size() < PL_MAX && n_local + PAIR_TILES < o.rank() &&
-        (int)(k1.size() + k2.size()) + G.c_u0 + n_local - n_one + G.rx + G.ry - 4 < PAIR_LOOP)
+        !one && (int)(k1.size() + k2.size()) + G.c_u0 + n_local - n_one + G.rx + G.ry - 4 < PAIR_LOOP)
       ++n_local;
   }
   // register bits: the latest local variables of A alone / B alone; the other
@@ -2243,11 +2247,11 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
   std::vector<int> chunk;
   if (C < 0 && loop.empty()) {
     double total = 0;
-    for (int k = 0; k < 2; ++k) total += std::ldexp(1.0, bits[k] - 1) * 1.05;
+    for (int k = one; k < 2; ++k) total += std::ldexp(1.0, bits[k] - 1) * 1.05;
     while (2 * 16 * total > PAIR_SMEM_TWO && chunk.size() < 2) {
       int best = -1;
       for (int v : k1)
-        if (holds(A, v) && holds(B, v) && (best < 0 || index_in(vars(A), v) > index_in(vars(A), best))) best = v;
+        if ((one || holds(A, v)) && holds(B, v) && (best < 0 || index_in(vars(B), v) > index_in(vars(B), best))) best = v;
       if (best < 0) break;
       k1.erase(std::find(k1.begin(), k1.end(), best));
       chunk.push_back(best);
@@ -2339,6 +2343,15 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
     G.lb[G.nl] = slot(1, v);
     G.lc[G.nl] = slot(2, v);
     G.lo[G.nl++] = out_of(v);
+  }
+  if (one) {  // the fold table in A's place
+    auto fold = [&](int v) {
+      const int i = index_in(fold_vars[1], v);
+      return i < 0 ? 0 : 1 << i;
+    };
+    for (int i = 0; i < PTB; ++i) G.ft[i] = fold(thr[i]);
+    for (int i = 0; i < G.ry; ++i) G.yf[i] = fold(yreg[i]);
+    for (size_t i = 0; i < k1.size(); ++i) G.k1f[i] = fold(k1[i]);
   }
   for (int v : k1) {
     G.k1a[G.n1] = slot(0, v);
@@ -2875,6 +2888,14 @@ static std::string validate_config(const tnq_plan& P, int mode, int B) {
         for (int j = 0; j < i; ++j)
           if ((O.d[i] & ~7) ? (O.d[i] & O.d[j] & ~7) : O.d[i] == O.d[j]) return name + ": slots";
       if (k < 2 && f >= 1 << (k ? G.fb.nf : G.fa.nf)) return name + ": fold index";
+      if (G.a.gin < 0) {
+        int r = O.fch[0] | O.fch[1];
+        for (int i = 0; i < G.n_h; ++i) r |= O.fh[i];
+        for (int i = 0; i < PTB; ++i) r |= G.ft[i];
+        for (int i = 0; i < G.ry; ++i) r |= G.yf[i];
+        for (int i = 0; i < G.n1; ++i) r |= G.k1f[i];
+        if (r != f) return name + ": fold index of the sum";
+      }
       // the register tile reads only staged slots
       int r = 0;
       for (int i = 0; i < PTB; ++i) r |= k == 0 ? G.ta[i] : (k == 1 ? G.tb[i] : G.tc[i]);

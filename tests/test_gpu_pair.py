@@ -42,7 +42,7 @@ CASES = [
 
 
 # (precision, rows, cols, depth, seed, forms): what runs as a product (0 a bucket, 1 a chain, 2 a GEMM chain of mostly
-# padding), C, whether it holds the first eliminated variable, register bits along A / B, those of them that are summed
+# padding), C ("B": B alone), whether it holds the first eliminated variable, register bits along A / B, those of them that are summed
 FORMS = [
     (0, 4, 7, 23, 7, {(0, "-", 0, 1, 3, 0, 0)}),
     (1, 4, 5, 26, 1, {(0, "-", 0, 2, 2, 0, 0)}),
@@ -63,6 +63,11 @@ FORMS = [
     (0, 6, 6, 29, 0, {(1, "c", 1, 2, 2, 0, 2)}),
     (0, 5, 5, 23, 1, {(1, "c", 1, 2, 2, 1, 1)}),
     (1, 4, 5, 32, 2, {(2, "-", 0, 2, 2, 0, 0)}),
+    (0, 4, 5, 29, 1, {(0, "B", 0, 0, 3, 0, 0)}),
+    (0, 4, 5, 26, 0, {(1, "B", 0, 0, 3, 0, 0)}),
+    (0, 4, 5, 32, 4, {(1, "B", 0, 0, 1, 0, 0)}),  # one chunk, 2^6 products of small tensors
+    (0, 4, 5, 32, 0, {(1, "B", 0, 0, 1, 0, 0)}),  # two chunks
+    (1, 5, 6, 29, 6, {(1, "B", 0, 0, 1, 0, 0)}),  # four
 ]
 
 
@@ -88,7 +93,7 @@ def _words(tnq_lib, plan):
     for line in re.findall(r"pair: (.*)", buf.value.decode()):
         w = line.split()
         d = dict(zip(w[::2], map(int, w[1::2])))
-        yield dict(d, c="-" if d["c"] < 0 else "c")
+        yield dict(d, c="B" if d["a"] == 0 else "-" if d["c"] < 0 else "c")
 
 
 def _shapes(tnq_lib, plan):
