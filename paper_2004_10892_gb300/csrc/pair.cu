@@ -148,6 +148,7 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
     }
   const bool fold_a = P.fa.n > 0;
   const unsigned sm0 = (unsigned)__cvta_generic_to_shared(sm);
+  char* smb = reinterpret_cast<char*>(sm);
   __syncthreads();
 
   // pointers and fold offsets of a tile: one warp per value, lane i adds tile bit i's stride
@@ -195,12 +196,12 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
     for (int o = OP0; o < NOP; ++o) {
       const POp& O = *ops[o];
       const float2* src = s_src[slot][o] + tg[o] + ((chunk & 1) ? O.gch[0] : 0) + ((chunk & 2) ? O.gch[1] : 0);
-      const unsigned dst = sm0 + 16u * (unsigned)(buf * P.stage + O.base);
+      const int at = td[o] ^ (O.base + (buf ? O.size : 0));
       const int nit = O.ebits > PTB ? 1 << (O.ebits - PTB) : 1;
       if (O.ebits >= PTB || t < (1 << O.ebits))
         for (int it = 0; it < nit; ++it) {
           const int4 k = s_it[o][it];
-          cp_async16(dst + 16u * (unsigned)(td[o] ^ k.y), src + k.x);
+          cp_async16(sm0 + (unsigned)(at ^ k.y), src + k.x);
         }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
@@ -213,17 +214,17 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
       const POp& O = *ops[o];
       const float4* ft = (o == 0 ? s_fa[n & 1] : s_fb[n & 1]) + tf[o] + s_fold[slot][o] +
                          ((chunk & 1) ? O.fch[0] : 0) + ((chunk & 2) ? O.fch[1] : 0);
-      float4* dst = sm + buf * P.stage + O.base;
+      const int at = td[o] ^ (O.base + (buf ? O.size : 0));
       const int nit = O.ebits > PTB ? 1 << (O.ebits - PTB) : 1;
       if (O.ebits >= PTB || t < (1 << O.ebits)) {
 #pragma unroll 2
         for (int it = 0; it < nit; ++it) {
           const int4 k = s_it[o][it];
-          const int at = td[o] ^ k.y;
-          const float4 v = dst[at], f = ft[k.z];
+          float4& dst = *reinterpret_cast<float4*>(smb + (at ^ k.y));
+          const float4 v = dst, f = ft[k.z];
           const float2 v0 = cmul(make_float2(v.x, v.y), make_float2(f.x, f.y));
           const float2 v1 = cmul(make_float2(v.z, v.w), make_float2(f.z, f.w));
-          dst[at] = make_float4(v0.x, v0.y, v1.x, v1.y);
+          dst = make_float4(v0.x, v0.y, v1.x, v1.y);
         }
       }
     }
@@ -255,10 +256,12 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
     const bool more = next < n_tiles;
     const bool new_item = more && (next >> P.n_h) != item;
     float2 x[NX][NY];  // sums of A B
+    auto zero = [&] {
 #pragma unroll
-    for (int i = 0; i < NX; ++i)
+      for (int i = 0; i < NX; ++i)
 #pragma unroll
-      for (int j = 0; j < NY; ++j) x[i][j] = make_float2(0.f, 0.f);
+        for (int j = 0; j < NY; ++j) x[i][j] = make_float2(0.f, 0.f);
+    };
     for (int c = 0; c < P.n_ch; ++c) {
       const bool last = c + 1 == P.n_ch;
       if (last && more) {
@@ -270,9 +273,14 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
       __syncthreads();  // the chunk is staged, and every thread is done with the other stage
       if (!last) issue(slot, c + 1, buf ^ 1);
       else if (more) issue((slot + 1) % RING, 0, buf ^ 1);
-      const float4* pa = ONE ? s_fb[n_item & 1] + s_fold[slot][1] + ((c & 1) ? P.b.fch[0] : 0) + ((c & 2) ? P.b.fch[1] : 0)
-                             : sm + buf * P.stage + P.a.base;
-      const float4* pb = sm + buf * P.stage + P.b.base;
+      // slots are byte offsets and stages aligned, so an address is one XOR
+      const char* pa = ONE ? reinterpret_cast<const char*>(s_fb[n_item & 1] + s_fold[slot][1] +
+                                                           ((c & 1) ? P.b.fch[0] : 0) + ((c & 2) ? P.b.fch[1] : 0))
+                           : smb;
+      const int ca = ONE ? ra : ra ^ (P.a.base + (buf ? P.a.size : 0)), cb = rb ^ (P.b.base + (buf ? P.b.size : 0));
+      const int cc = HASC ? rc ^ (P.c.base + (buf ? P.c.size : 0)) : 0;
+      auto quad = [](const char* p, int at) { return *reinterpret_cast<const float4*>(p + at); };
+      auto elem = [](const char* p, int at) { return *reinterpret_cast<const float2*>(p + at); };
       float2* dst = s_out[slot] + ro;
       const int n1 = 1 << P.n1;
       auto off_x = [&](int i, const int* w) { return ((i & 1) ? w[0] : 0) ^ ((i & 2) ? w[1] : 0); };
@@ -287,12 +295,12 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
           float4 va[NX];
 #pragma unroll
           for (int i = 0; i < NX; ++i)
-            if (!ONE) va[i] = pa[qa ^ off_x(i, P.xa)];
+            if (!ONE) va[i] = quad(pa, qa ^ off_x(i, P.xa));
 #pragma unroll
           for (int j = 0; j < NY; ++j) {
-            const float4 vb = pb[qb ^ off_y(j, P.yb)];
+            const float4 vb = quad(smb, qb ^ off_y(j, P.yb));
 #pragma unroll
-            for (int i = 0; i < NX; ++i) cfma2(x[i][j], ONE ? pa[qa ^ off_y(j, P.yf)] : va[i], vb);
+            for (int i = 0; i < NX; ++i) cfma2(x[i][j], ONE ? quad(pa, qa ^ off_y(j, P.yf)) : va[i], vb);
           }
         }
       };
@@ -300,15 +308,13 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
 #pragma unroll 1
         for (int q = 0; q < n1; ++q) {
           const int2 k = s_k1[q];
-          const int qa = oa ^ k.x, qb = ob ^ k.y;
-          const float2* ha = reinterpret_cast<const float2*>(pa) + h;
-          const float2* hb = reinterpret_cast<const float2*>(pb) + h;
+          const int qa = oa ^ k.x ^ 8 * h, qb = ob ^ k.y ^ 8 * h;
           float2 va[NX];
 #pragma unroll
-          for (int i = 0; i < NX; ++i) va[i] = ha[2 * (qa ^ off_x(i, P.xa))];
+          for (int i = 0; i < NX; ++i) va[i] = elem(smb, qa ^ off_x(i, P.xa));
 #pragma unroll
           for (int j = 0; j < NY; ++j) {
-            const float2 vb = hb[2 * (qb ^ off_y(j, P.yb))];
+            const float2 vb = elem(smb, qb ^ off_y(j, P.yb));
 #pragma unroll
             for (int i = 0; i < NX; ++i) cfma(x[i][j], va[i], vb);
           }
@@ -334,32 +340,29 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
 #pragma unroll 1
           for (int q2 = 0; q2 < n2; ++q2) {
             const int4 k2 = s_k2[q2];
-            const float4* pc = sm + buf * P.stage + P.c.base;
-            const int oc = rc ^ lv.z ^ k2.z;
+            const int oc = cc ^ lv.z ^ k2.z;
             if constexpr (CM == 2) {
 #pragma unroll 1
               for (int h = 0; h < 2; ++h) {
-                half_products(ra ^ lv.x ^ k2.x, rb ^ lv.y ^ k2.y, h);
-                const float2* ph = reinterpret_cast<const float2*>(pc) + h;
+                zero();
+                half_products(ca ^ lv.x ^ k2.x, cb ^ lv.y ^ k2.y, h);
 #pragma unroll
                 for (int i = 0; i < NX; ++i)
 #pragma unroll
-                  for (int j = 0; j < NY; ++j) {
-                    cfma(acc[i >> NKX][j >> NKY], x[i][j], ph[2 * (oc ^ off_x(i, P.xc) ^ off_y(j, P.yc))]);
-                    x[i][j] = make_float2(0.f, 0.f);
-                  }
+                  for (int j = 0; j < NY; ++j)
+                    cfma(acc[i >> NKX][j >> NKY], x[i][j], elem(smb, oc ^ 8 * h ^ off_x(i, P.xc) ^ off_y(j, P.yc)));
               }
             } else {
-              products(ra ^ lv.x ^ k2.x, rb ^ lv.y ^ k2.y);
+              zero();
+              products(ca ^ lv.x ^ k2.x, cb ^ lv.y ^ k2.y);
               // times C, summed over the K2 register bits (C's bit 0 is B's register bit 0)
 #pragma unroll
               for (int i = 0; i < NX; ++i)
 #pragma unroll
                 for (int j = 0; j < NY; j += 2) {
-                  const float4 v = pc[oc ^ off_x(i, P.xc) ^ off_y(j, P.yc)];  // (yc[0] is 0: the pair's own bit)
+                  const float4 v = quad(smb, oc ^ off_x(i, P.xc) ^ off_y(j, P.yc));  // (yc[0] is 0: the pair's own bit)
                   const float2 u = x[i][j], w = x[i][j + 1];
                   cfma2(acc[i >> NKX][j >> NKY], make_float4(u.x, u.y, w.x, w.y), v);
-                  x[i][j] = x[i][j + 1] = make_float2(0.f, 0.f);
                 }
             }
           }
@@ -368,15 +371,13 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
 #pragma unroll
             for (int j = 0; j < YO; ++j) store(i, j, acc[i][j], lv.w);
         } else {
-          products(ra ^ lv.x, rb ^ lv.y);
+          if (c == 0) zero();
+          products(ca ^ lv.x, cb ^ lv.y);
           if (last) {
 #pragma unroll
             for (int i = 0; i < NX; ++i)
 #pragma unroll
-              for (int j = 0; j < NY; ++j) {
-                store(i, j, x[i][j], lv.w);
-                x[i][j] = make_float2(0.f, 0.f);
-              }
+              for (int j = 0; j < NY; ++j) store(i, j, x[i][j], lv.w);
           }
         }
       }

@@ -39,7 +39,7 @@ struct PIn {
 // by an index e (bits by increasing memory stride, so that consecutive threads
 // read consecutive memory); bit i of e adds g[i] to the global offset
 // (elements) and f[i] to the fold table's index, and is d[i] of the
-// shared-memory slot (16-byte units): slots are combined with XOR, since they
+// shared-memory slot (bytes): slots are combined with XOR, since they
 // are swizzled (pair_params). Tile bit i adds h[i] and fh[i], bit i of the chunk gch[i] and fch[i].
 struct POp {
   int gin;
@@ -47,7 +47,7 @@ struct POp {
   int g[PE_MAX], d[PE_MAX], f[PE_MAX];
   int h[PH_MAX], fh[PH_MAX];
   int gch[2], fch[2];
-  int base, size;               // first slot of a stage, slots (a power of two)
+  int base, size;               // bytes: its first stage (a multiple of size; the second follows it), a stage (a power of two)
 };
 
 // Small tensors folded into one operand: table of (u_0 = 0, u_0 = 1) pairs
@@ -78,7 +78,6 @@ struct PairParams {
   int nkx, nky;                 // K2 bits among the register bits along A / B (the low ones)
   int n_ch;                     // chunks of a tile: one summed variable (2) or two (4) split off, or none (1)
   int n_h, n_gin, out_meta, out_dep, B;
-  int stage;                    // slots of one stage; dynamic shared memory holds two
   int smem;                     // dynamic shared memory bytes
   int* meta_e;
   unsigned* meta_m;

@@ -2046,7 +2046,8 @@ static GParams group_gparams(const tnq_plan& P, const Layout& L, const FusedGrou
 //    first eliminated variable: the product of two tensors is what the
 //    register tile shares operands over; or one, which is streamed;
 //  * every other tensor has its variables among A's or among B's: it is
-//    multiplied into that operand as it is staged;
+//    multiplied into that operand as it is staged (beside one large tensor
+//    it may have any: its product is indexed by the sum's variables);
 //  * 2^2 register entries along variables of A alone and of B alone
 //    (eliminated variables of C count), or fewer along A and 2^3 along B's:
 //    without them nothing is shared;
@@ -2124,8 +2125,8 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
       ina = ina && holds(A, v);
       inb = inb && holds(B, v);
     }
-    if (!ina && !inb) return false;
-    (inb ? sb : sa).push_back(j);
+    if (!one && !ina && !inb) return false;
+    (inb || one ? sb : sa).push_back(j);
   }
   // eliminated variables: K2 in C (register bits where A or B alone holds them), K1 the others
   std::vector<int> k1, k2, xreg, yreg;
@@ -2266,8 +2267,7 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
   // the shared-memory pipe each), and the slot's low three bits are XORed with
   // the row's, so that eight lanes that read one pair of eight rows hit eight
   // bank groups. Slots of disjoint bits combine with XOR.
-  int base = 0;
-  std::vector<int> weight[3];  // per operand: slot of each of its variables
+  std::vector<int> weight[3];  // per operand: slot of each of its variables, in bytes
   for (int k = 0; k < 3; ++k) {
     POp& O = k == 0 ? G.a : (k == 1 ? G.b : G.c);
     O.gin = ops[k];
@@ -2289,10 +2289,8 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
       if (index_in(K, x) < 0) row(x);
     for (int x : yreg)
       if (index_in(K, x) < 0) row(x);
-    for (int& x : w) x ^= (x >> std::max(3, nk)) & 7;
-    O.base = base;
-    O.size = std::max(8, 1 << n);
-    base += O.size;
+    for (int& x : w) x = 16 * (x ^ ((x >> std::max(3, nk)) & 7));
+    O.size = 16 * std::max(8, 1 << n);
     for (size_t p = 1; p < v.size(); ++p) {
       if (p > 30) return false;
       const int fi = k < 2 ? index_in(fold_vars[k], v[p]) : -1, f = fi < 0 ? 0 : 1 << fi;
@@ -2311,8 +2309,14 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
       }
     }
   }
-  G.stage = base;
-  G.smem = 2 * base * 16;
+  // both stages of an operand side by side, the largest operand first: every
+  // base is a multiple of its operand's size, so base and slot combine with XOR
+  POp* by_size[3] = {&G.a, &G.b, &G.c};
+  std::stable_sort(by_size, by_size + 3, [](const POp* x, const POp* y) { return x->size > y->size; });
+  for (POp* O : by_size) {
+    O->base = G.smem;
+    G.smem += 2 * O->size;
+  }
   if (G.smem > PAIR_SMEM_MAX) return false;
   auto slot = [&](int k, int v) {
     const int p = ops[k] < 0 ? -1 : index_in(vars(ops[k]), v);
@@ -2347,8 +2351,9 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
   if (one) {  // the fold table in A's place
     auto fold = [&](int v) {
       const int i = index_in(fold_vars[1], v);
-      return i < 0 ? 0 : 1 << i;
+      return i < 0 ? 0 : 16 << i;
     };
+    for (int h = 0; h < (int)tile.size(); ++h) G.b.fh[h] = fold(tile[h]) / 16;
     for (int i = 0; i < PTB; ++i) G.ft[i] = fold(thr[i]);
     for (int i = 0; i < G.ry; ++i) G.yf[i] = fold(yreg[i]);
     for (size_t i = 0; i < k1.size(); ++i) G.k1f[i] = fold(k1[i]);
@@ -2863,7 +2868,7 @@ static std::string validate_config(const tnq_plan& P, int mode, int B) {
     const std::string name = "pair chain " + std::to_string(si);
     const long long items = G.out_dep ? B : 1;
     auto item_max = [&](int j) { return G.gin[j].dep ? (items - 1) * G.gin[j].istride : 0ll; };
-    if (G.smem > PAIR_SMEM_MAX || G.smem != 2 * 16 * G.stage) return name + ": shared memory";
+    if (G.smem > PAIR_SMEM_MAX || G.smem != 2 * (G.a.size + G.b.size + G.c.size)) return name + ": shared memory";
     const POp* ops[3] = {&G.a, &G.b, &G.c};
     for (int k = 0; k < 3; ++k) {
       const POp& O = *ops[k];
@@ -2883,18 +2888,23 @@ static std::string validate_config(const tnq_plan& P, int mode, int B) {
       }
       if ((G.gin[O.gin].istride & 1) || ((size_t)G.gin[O.gin].ptr / 8) % 2) return name + ": unaligned input";
       if (m >= alloc(g.ext_inputs[O.gin])) return name + ": staged input overflows";
-      if (d >= O.size || O.base + O.size > G.stage) return name + ": staged operand outside its stage";
+      if (d >= O.size || (O.size & (O.size - 1)) || O.base % O.size || O.base + 2 * O.size > G.smem)
+        return name + ": staged operand outside its stage";
+      for (int j = 0; j < k; ++j)
+        if (ops[j]->gin >= 0 && O.base < ops[j]->base + 2 * ops[j]->size && ops[j]->base < O.base + 2 * O.size)
+          return name + ": stages overlap";
       for (int i = 0; i < O.ebits; ++i)  // one slot per staged pair: the bits' slots are independent
         for (int j = 0; j < i; ++j)
-          if ((O.d[i] & ~7) ? (O.d[i] & O.d[j] & ~7) : O.d[i] == O.d[j]) return name + ": slots";
-      if (k < 2 && f >= 1 << (k ? G.fb.nf : G.fa.nf)) return name + ": fold index";
-      if (G.a.gin < 0) {
-        int r = O.fch[0] | O.fch[1];
-        for (int i = 0; i < G.n_h; ++i) r |= O.fh[i];
-        for (int i = 0; i < PTB; ++i) r |= G.ft[i];
-        for (int i = 0; i < G.ry; ++i) r |= G.yf[i];
-        for (int i = 0; i < G.n1; ++i) r |= G.k1f[i];
-        if (r != f) return name + ": fold index of the sum";
+          if ((O.d[i] & ~127) ? (O.d[i] & O.d[j] & ~127) : O.d[i] == O.d[j]) return name + ": slots";
+      if (G.a.gin < 0) {  // the sum reads the fold table
+        f = 16 * (O.fch[0] + O.fch[1]);
+        for (int i = 0; i < G.n_h; ++i) f += 16 * O.fh[i];
+        for (int i = 0; i < PTB; ++i) f += G.ft[i];
+        for (int i = 0; i < G.ry; ++i) f += G.yf[i];
+        for (int i = 0; i < G.n1; ++i) f += G.k1f[i];
+        if (f != 16 * ((1 << G.fb.nf) - 1)) return name + ": fold index of the sum";
+      } else if (k < 2 && f >= 1 << (k ? G.fb.nf : G.fa.nf)) {
+        return name + ": fold index";
       }
       // the register tile reads only staged slots
       int r = 0;

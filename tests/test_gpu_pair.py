@@ -42,7 +42,7 @@ CASES = [
 
 
 # (precision, rows, cols, depth, seed, forms): what runs as a product (0 a bucket, 1 a chain, 2 a GEMM chain of mostly
-# padding), C ("B": B alone), whether it holds the first eliminated variable, register bits along A / B, those of them that are summed
+# padding), C ("B": B alone, "X": and small tensors with other variables), whether it holds the first eliminated variable, register bits along A / B, those of them that are summed
 FORMS = [
     (0, 4, 7, 23, 7, {(0, "-", 0, 1, 3, 0, 0)}),
     (1, 4, 5, 26, 1, {(0, "-", 0, 2, 2, 0, 0)}),
@@ -68,6 +68,9 @@ FORMS = [
     (0, 4, 5, 32, 4, {(1, "B", 0, 0, 1, 0, 0)}),  # one chunk, 2^6 products of small tensors
     (0, 4, 5, 32, 0, {(1, "B", 0, 0, 1, 0, 0)}),  # two chunks
     (1, 5, 6, 29, 6, {(1, "B", 0, 0, 1, 0, 0)}),  # four
+    (0, 5, 6, 32, 9, {(0, "X", 0, 0, 3, 0, 0)}),
+    (0, 5, 6, 32, 0, {(0, "X", 0, 0, 3, 0, 0)}),  # 2^7 products of small tensors
+    (0, 4, 5, 26, 5, {(1, "X", 0, 0, 3, 0, 0)}),
 ]
 
 
@@ -93,7 +96,8 @@ def _words(tnq_lib, plan):
     for line in re.findall(r"pair: (.*)", buf.value.decode()):
         w = line.split()
         d = dict(zip(w[::2], map(int, w[1::2])))
-        yield dict(d, c="B" if d["a"] == 0 else "-" if d["c"] < 0 else "c")
+        outside = d["b"] < 8 + d["ry"] + d["n1"] - d["chunks"] // 2  # local outputs that the large tensor lacks
+        yield dict(d, c="BX"[outside] if d["a"] == 0 else "-" if d["c"] < 0 else "c")
 
 
 def _shapes(tnq_lib, plan):
