@@ -2188,7 +2188,7 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
     }
     if (best < 0) return false;
     if (n >= n_one) {
-      if (2 * 16 * 1.05 * best_cost > PAIR_SMEM_TWO) break;
+      if (2 * 16 * best_cost > PAIR_SMEM_TWO) break;
       loop.push_back(o.vars[best]);
     }
     local[best] = 1;
@@ -2248,7 +2248,7 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
   std::vector<int> chunk;
   if (C < 0 && loop.empty()) {
     double total = 0;
-    for (int k = one; k < 2; ++k) total += std::ldexp(1.0, bits[k] - 1) * 1.05;
+    for (int k = one; k < 2; ++k) total += std::ldexp(1.0, bits[k] - 1);
     while (2 * 16 * total > PAIR_SMEM_TWO && chunk.size() < 2) {
       int best = -1;
       for (int v : k1)
