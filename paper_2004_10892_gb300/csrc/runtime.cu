@@ -41,6 +41,7 @@ constexpr int GMAX = 52;  // index bits of one bucket launch (output bits + item
 static_assert(GB_SIDE >= GEMM_SIDE_MAX + 1 && GB_BITS >= GEMM_BITS_MAX, "GEMM limits of planner and kernels differ");
 constexpr int TPB = 256;  // threads per block of the bucket kernel
 constexpr int MAX_ITEM_BITS = 16;
+constexpr int LEVEL_R = 3;          // most pieces of 256 entries a block of k_bucket_level takes: 2^LEVEL_R
 constexpr int HOIST_MAX_BITS = 24;  // largest early-bucket result (2^24 entries; see hoist_levels)
 
 // ---------------------------------------------------------------------------
@@ -72,7 +73,7 @@ struct HoistDev {
   int in_dep[KMAX];               // 1: input j's meta row is per item
   int nin, bits, sum, out_meta;   // inputs, index bits, 1: sum over bit 0 (Eq. 2), meta row of the result
   int obits, out_dep;             // output bits per item; 1: the result is per item (items above bit obits)
-  int blk0;                       // first block of this bucket in its level's launch
+  int blk0, r;                    // first block of this bucket in its level's launch; 256 << r entries a block
   int nvar;                       // inputs 0..nvar-1 vary with the index's low 8 bits (k_bucket's order)
 };
 
@@ -144,33 +145,42 @@ __global__ void k_leaf_init(const LeafDev* __restrict__ leaves, int n_leaves, co
 }
 
 // Product of the fully fixed gate tensors and the <x_q|0> factors of wires
-// without a non-diagonal gate, per item (FP64).
+// without a non-diagonal gate, per item (FP64). A warp per item: its lanes
+// fetch 32 factors at once, which are then multiplied in order: 7 us on a 7x7
+// circuit (a thread per item waited for each in turn: 21 us).
 __global__ void k_scalar_init(const LeafDev* __restrict__ sl, int n_sl, const int* __restrict__ inout_q, int n_inout,
                               const BatchHdr* __restrict__ hdr_p, const unsigned* __restrict__ bits,
                               const float2* __restrict__ vals, double2* __restrict__ item_scalar, int B) {
   const BatchHdr h = *hdr_p;
-  int item = blockIdx.x * blockDim.x + threadIdx.x;
+  const int item = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (item >= B) return;
   unsigned long long slice;
   int brow;
   bool valid;
   item_decode(h, item, &slice, &brow, &valid);
   double re = 1.0, im = 0.0;
-  for (int i = 0; i < n_sl; ++i) {
-    const LeafDev& L = sl[i];
-    int a = 0;
-    for (int x = 0; x < L.nv; ++x) {
-      if (L.vkind[x] == 2) a |= bit_of(bits, h.n_words, brow, L.varg[x]) << x;
-      else if (L.vkind[x] == 3) a |= (int)((slice >> L.varg[x]) & 1ull) << x;
+  for (int i0 = 0; i0 < n_sl; i0 += 32) {
+    float2 v = make_float2(1.f, 0.f);
+    if (i0 + lane < n_sl) {
+      const LeafDev& L = sl[i0 + lane];
+      int a = 0;
+      for (int x = 0; x < L.nv; ++x) {
+        if (L.vkind[x] == 2) a |= bit_of(bits, h.n_words, brow, L.varg[x]) << x;
+        else if (L.vkind[x] == 3) a |= (int)((slice >> L.varg[x]) & 1ull) << x;
+      }
+      v = leaf_entry(L, vals, a);
     }
-    const float2 v = leaf_entry(L, vals, a);
-    const double nr = re * v.x - im * v.y, ni = re * v.y + im * v.x;
-    re = nr;
-    im = ni;
+    for (int i = 0; i < 32 && i0 + i < n_sl; ++i) {
+      const double x = __shfl_sync(0xffffffffu, v.x, i), y = __shfl_sync(0xffffffffu, v.y, i);
+      const double nr = re * x - im * y, ni = re * y + im * x;
+      re = nr;
+      im = ni;
+    }
   }
-  for (int i = 0; i < n_inout; ++i)
-    if (bit_of(bits, h.n_words, brow, inout_q[i])) re = im = 0.0;
-  item_scalar[item] = make_double2(re, im);
+  bool zero = false;
+  for (int i = lane; i < n_inout; i += 32) zero = zero || bit_of(bits, h.n_words, brow, inout_q[i]);
+  if (__any_sync(0xffffffffu, zero)) re = im = 0.0;
+  if (lane == 0) item_scalar[item] = make_double2(re, im);
 }
 
 // K1: one bucket, all items. Element g of the launch = item * 2^out_bits + b'
@@ -356,111 +366,143 @@ __global__ void __launch_bounds__(TPB, 5) k_bucket(const __grid_constant__ KPara
 }
 
 // K1 for the early buckets of one level (see hoist_levels): every bucket of
-// the level in one launch, 256 index entries per block; block b works on the
-// bucket whose blk0 is the largest not above b. Item-dependent buckets carry
-// the item above their output bits; their scales, exponents and maxima are
-// per item, as in k_bucket, and so is the arithmetic order.
+// the level in one launch, 256 << r index entries per block (r chosen per
+// bucket, see build_steps); block b works on the bucket whose blk0 is the
+// largest not above b. Item-dependent buckets carry the item above their output
+// bits; their scales, exponents and maxima are per item, as in k_bucket, and so
+// is the arithmetic order.
+// Small levels are bound by the block's chain of dependent loads, large ones by
+// instructions per entry. So warp j prepares input j (strides, scale, exponent
+// and the offset of the block's bits, one trip to memory each), and an entry's
+// offset is its thread's part plus its piece's part. A level of 9.5 million
+// entries takes 56 us; with a loop over all bits per entry it took 208.
+template <int NC>
+__device__ __forceinline__ float level_entries(const HoistDev& H, int t, long long g0, long long total,
+                                               const float2* const* s_in, const int (*s_str)[8],
+                                               const int (*s_piece)[1 << LEVEL_R], const float* s_f, bool uniform,
+                                               const unsigned* meta_m, int B, char* arena) {
+  const int nin = H.nin, nvar = H.nvar;
+  const bool in = g0 + t < total;  // (pieces after the first are whole: r > 0 only in uniform blocks)
+  float2 a0[NC], a1[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) a0[c] = a1[c] = make_float2(1.f, 0.f);
+  if (!in) return 0.f;
+  // the arithmetic order of k_bucket (thread-invariant inputs nvar.. first,
+  // then 0..nvar-1), so that a bucket's value does not depend on which
+  // kernel runs it
+  for (int jj = 0; jj < nin; ++jj) {
+    const int j = jj < nin - nvar ? nvar + jj : jj - (nin - nvar);
+    int at = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) at += ((t >> i) & 1) ? s_str[j][i] : 0;
+    float f = 1.f;
+    if (uniform) {
+      f = s_f[j];
+    } else if (H.in_meta[j] >= 0) {
+      int m;
+      f = scale_of_max(meta_m[(long long)H.in_meta[j] * B + (H.in_dep[j] ? (g0 + t) >> H.obits : 0ll)], &m);
+    }
+    const float2* src = s_in[j] + at;
+    if (H.sum) {
+      float4 v[NC];
+#pragma unroll
+      for (int c = 0; c < NC; ++c) v[c] = __ldg(reinterpret_cast<const float4*>(src + s_piece[j][c]));
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        a0[c] = cmul(a0[c], make_float2(v[c].x * f, v[c].y * f));
+        a1[c] = cmul(a1[c], make_float2(v[c].z * f, v[c].w * f));
+      }
+    } else {
+      float2 v[NC];
+#pragma unroll
+      for (int c = 0; c < NC; ++c) v[c] = __ldg(src + s_piece[j][c]);
+#pragma unroll
+      for (int c = 0; c < NC; ++c) a0[c] = cmul(a0[c], make_float2(v[c].x * f, v[c].y * f));
+    }
+  }
+  float mx = 0.f;
+  float2* out = reinterpret_cast<float2*>(arena + H.out) + g0 + t;
+#pragma unroll
+  for (int c = 0; c < NC; ++c) {
+    const float2 r = H.sum ? make_float2(a0[c].x + a1[c].x, a0[c].y + a1[c].y) : a0[c];
+    out[256 * c] = r;
+    mx = fmaxf(mx, fmaxf(fabsf(r.x), fabsf(r.y)));
+  }
+  return mx;
+}
+
 __global__ void __launch_bounds__(256) k_bucket_level(const HoistDev* __restrict__ hd, int n, char* arena,
                                                      int* meta_e, unsigned* meta_m, int B,
                                                      const int* __restrict__ n_items) {
-  __shared__ int s_b;
-  __shared__ long long s_str[KMAX][HOIST_MAX_BITS];
+  __shared__ int s_str[KMAX][8], s_piece[KMAX][1 << LEVEL_R];
   __shared__ const float2* s_in[KMAX];
   __shared__ float s_f[KMAX];
-  __shared__ int s_e;
+  __shared__ int s_e[KMAX];
   __shared__ float s_red[8];
-  const int t = threadIdx.x;
+  static_assert(KMAX <= 8, "a warp per input");
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   const int n_valid = n_items ? __ldg(n_items) : 1;
-  if (t == 0) {
-    int lo = 0, hi = n - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (hd[mid].blk0 <= (int)blockIdx.x) lo = mid;
-      else hi = mid - 1;
-    }
-    s_b = lo;
-  }
-  __syncthreads();
-  const HoistDev& H = hd[s_b];
-  const int nin = H.nin, bits = H.bits, ob = H.obits;
-  const long long g0 = (long long)(blockIdx.x - H.blk0) * 256;
+  int nb = 0;  // buckets that start at or before this block
+  for (int i = 0; i < n; i += 256) nb += __syncthreads_count(i + t < n && hd[i + t].blk0 <= (int)blockIdx.x);
+  const HoistDev& H = hd[nb - 1];
+  const int nin = H.nin, bits = H.bits, ob = H.obits, r = H.r;
+  const long long g0 = (long long)(blockIdx.x - H.blk0) << (8 + r);
   const bool uniform = ob >= 8 || ob == bits;  // one item for the whole block
   const long long total = H.out_dep ? (long long)n_valid << ob : 1ll << bits;
   if (g0 >= total) return;
-  for (int e = t; e < nin * bits; e += 256) s_str[e / bits][e % bits] = H.stride[e / bits][e % bits];
-  if (t < nin) s_in[t] = reinterpret_cast<const float2*>(arena + H.in[t]);
-  if (uniform && t == 0) {  // the block's item: scales and the output exponent
-    const long long item = g0 >> ob;
-    int e = 0;
-    for (int j = 0; j < nin; ++j) {
-      if (H.in_meta[j] < 0) {
-        s_f[j] = 1.f;
-        continue;
-      }
-      const long long row = (long long)H.in_meta[j] * B + (H.in_dep[j] ? item : 0ll);
-      int m;
-      s_f[j] = scale_of_max(meta_m[row], &m);
-      e += meta_e[row] + m;
+  if (w < nin) {
+    const int st = lane < bits ? (int)H.stride[w][lane] : 0;  // (an early bucket's inputs are below 2^31 entries)
+    if (lane < 8) s_str[w][lane] = st;
+    const int base = __reduce_add_sync(0xffffffffu, lane >= 8 + r && ((g0 >> lane) & 1ll) ? st : 0);
+    int piece = 0;
+    for (int i = 0; i < r; ++i) {
+      const int x = __shfl_sync(0xffffffffu, st, 8 + i);
+      piece += ((lane >> i) & 1) ? x : 0;
     }
-    s_e = e;
+    if (lane < 1 << LEVEL_R) s_piece[w][lane] = piece;
+    if (lane == 0) {
+      s_in[w] = reinterpret_cast<const float2*>(arena + H.in[w]) + base;
+      float f = 1.f;
+      int e = 0;
+      if (uniform && H.in_meta[w] >= 0) {  // the block's item: scale and exponent
+        const long long row = (long long)H.in_meta[w] * B + (H.in_dep[w] ? g0 >> ob : 0ll);
+        f = scale_of_max(meta_m[row], &e);
+        e += meta_e[row];
+      }
+      s_f[w] = f;
+      s_e[w] = e;
+    }
   }
   __syncthreads();
-  const long long g = g0 + t;
-  const long long item = g >> ob;
   float mx = 0.f;
-  if (g < total) {
-    // scale of input j for this entry's item
-    auto scale = [&](int j) -> float {
-      if (uniform) return s_f[j];
-      if (H.in_meta[j] < 0) return 1.f;
-      int m;
-      return scale_of_max(meta_m[(long long)H.in_meta[j] * B + (H.in_dep[j] ? item : 0ll)], &m);
-    };
-    // the arithmetic order of k_bucket (thread-invariant inputs nvar.. first,
-    // then 0..nvar-1), so that a bucket's value does not depend on which
-    // kernel runs it
-    float2 a0 = make_float2(1.f, 0.f), a1 = make_float2(1.f, 0.f);
-    for (int jj = 0; jj < nin; ++jj) {
-      const int j = jj < nin - H.nvar ? H.nvar + jj : jj - (nin - H.nvar);
-      long long idx = 0;
-      for (int i = 0; i < bits; ++i)
-        if ((g >> i) & 1ll) idx += s_str[j][i];
-      const float fj = scale(j);
-      if (H.sum) {
-        const float4 v = __ldg(reinterpret_cast<const float4*>(s_in[j] + idx));
-        a0 = cmul(a0, make_float2(v.x * fj, v.y * fj));
-        a1 = cmul(a1, make_float2(v.z * fj, v.w * fj));
-      } else {
-        const float2 v = __ldg(s_in[j] + idx);
-        a0 = cmul(a0, make_float2(v.x * fj, v.y * fj));
-      }
-    }
-    const float2 r = H.sum ? make_float2(a0.x + a1.x, a0.y + a1.y) : a0;
-    reinterpret_cast<float2*>(arena + H.out)[g] = r;
-    mx = fmaxf(fabsf(r.x), fabsf(r.y));
-    if ((g & ((1ll << ob) - 1ll)) == 0) {  // the item's first entry writes its exponent
-      int esum = 0;
+  switch (r) {
+    case 0: mx = level_entries<1>(H, t, g0, total, s_in, s_str, s_piece, s_f, uniform, meta_m, B, arena); break;
+    case 1: mx = level_entries<2>(H, t, g0, total, s_in, s_str, s_piece, s_f, uniform, meta_m, B, arena); break;
+    case 2: mx = level_entries<4>(H, t, g0, total, s_in, s_str, s_piece, s_f, uniform, meta_m, B, arena); break;
+    default: mx = level_entries<8>(H, t, g0, total, s_in, s_str, s_piece, s_f, uniform, meta_m, B, arena);
+  }
+  const long long g = g0 + t, item = g >> ob;
+  if (g < total && (g & ((1ll << ob) - 1ll)) == 0) {  // the item's first entry writes its exponent
+    int esum = 0;
+    for (int j = 0; j < nin; ++j) {
       if (uniform) {
-        esum = s_e;
-      } else {
-        for (int j = 0; j < nin; ++j) {
-          if (H.in_meta[j] < 0) continue;
-          const long long row = (long long)H.in_meta[j] * B + (H.in_dep[j] ? item : 0ll);
-          int m;
-          scale_of_max(meta_m[row], &m);
-          esum += meta_e[row] + m;
-        }
+        esum += s_e[j];
+      } else if (H.in_meta[j] >= 0) {
+        const long long row = (long long)H.in_meta[j] * B + (H.in_dep[j] ? item : 0ll);
+        int m;
+        scale_of_max(meta_m[row], &m);
+        esum += meta_e[row] + m;
       }
-      meta_e[(long long)H.out_meta * B + (H.out_dep ? item : 0ll)] = esum;
     }
+    meta_e[(long long)H.out_meta * B + (H.out_dep ? item : 0ll)] = esum;
   }
   if (uniform) {
     for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-    if ((t & 31) == 0) s_red[t >> 5] = mx;
+    if (lane == 0) s_red[w] = mx;
     __syncthreads();
     if (t == 0) {
       float b = 0.f;
-      for (int w = 0; w < 8; ++w) b = fmaxf(b, s_red[w]);
+      for (int i = 0; i < 8; ++i) b = fmaxf(b, s_red[i]);
       if (b > 0.f) atomic_max_pos(&meta_m[(long long)H.out_meta * B + (H.out_dep ? (g0 >> ob) : 0ll)], b);
     }
   } else {
@@ -1187,23 +1229,32 @@ __global__ void k_finalize(const FinalDev* __restrict__ fin, int n_fin, const do
 }
 
 // Per-bitstring FP64 partial sums of one batch, items in increasing order.
+// A warp per row fetches 32 items at once and adds them in order (one thread
+// that fetched them in turn took 12 us for 64).
 __global__ void k_slice_sum(const double2* __restrict__ res, int B, const BatchHdr* __restrict__ hdr_p,
                             double2* __restrict__ part, int n_rows) {
   const BatchHdr h = *hdr_p;
-  int row = blockIdx.x * blockDim.x + threadIdx.x;
+  const int row = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (row >= n_rows) return;
   double re = 0.0, im = 0.0;
-  for (int item = 0; item < B; ++item) {
-    unsigned long long slice;
-    int brow;
-    bool valid;
-    item_decode(h, item, &slice, &brow, &valid);
-    if (valid && brow == row) {
-      re += res[item].x;
-      im += res[item].y;
+  for (int i0 = 0; i0 < B; i0 += 32) {
+    double2 v = make_double2(0.0, 0.0);
+    bool mine = false;
+    if (i0 + lane < B) {
+      unsigned long long slice;
+      int brow;
+      bool valid;
+      item_decode(h, i0 + lane, &slice, &brow, &valid);
+      mine = valid && brow == row;
+      if (mine) v = res[i0 + lane];
+    }
+    for (unsigned m = __ballot_sync(0xffffffffu, mine); m; m &= m - 1) {
+      const int i = __ffs(m) - 1;
+      re += __shfl_sync(0xffffffffu, v.x, i);
+      im += __shfl_sync(0xffffffffu, v.y, i);
     }
   }
-  part[row] = make_double2(re, im);
+  if (lane == 0) part[row] = make_double2(re, im);
 }
 
 // Adds one batch's per-bitstring partial sums (rows 0..n_rows-1) to the FP64
@@ -2659,7 +2710,10 @@ static bool build_steps(const tnq_plan& P, const Layout& L, ExecConfig& C) {
         h.in_dep[j] = k.in_dep[j];
         for (int b = 0; b < k.G; ++b) h.stride[j][b] = k.stride[j][b];
       }
-      blocks += (int)(((1ll << k.G) + 255) >> 8);
+      // several pieces of 256 entries a block once 512 blocks remain (three and
+      // a half for every SM), in blocks of one item
+      if (k.out_bits >= 8 + LEVEL_R || k.G == k.out_bits) h.r = std::min(LEVEL_R, std::max(0, k.G - 17));
+      blocks += (int)(((1ll << k.G) + (256ll << h.r) - 1) >> (8 + h.r));
       C.hoist_dev.push_back(h);
     }
     C.hoist_blocks.push_back(blocks);
@@ -3182,7 +3236,7 @@ static void enqueue_batch(const tnq_plan& P, ExecConfig& C, char* ws, cudaStream
     long long n = (long long)C.n_leaves * B;
     k_leaf_init<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(C.d_leaves, C.n_leaves, hdr, bits, C.d_vals, arena, B);
   }
-  k_scalar_init<<<(B + 127) / 128, 128, 0, s>>>(C.d_scalars, C.n_scalars, C.d_inout, C.n_inout, hdr, bits, C.d_vals,
+  k_scalar_init<<<(B + 3) / 4, 128, 0, s>>>(C.d_scalars, C.n_scalars, C.d_inout, C.n_inout, hdr, bits, C.d_vals,
                                                 scal, B);
   int* status = reinterpret_cast<int*>(ws + L.status_off);
   const int* n_items = B > 1 ? &hdr->n_items : nullptr;  // (a load that a batch of one item does not wait for)
@@ -3216,7 +3270,7 @@ static void enqueue_batch(const tnq_plan& P, ExecConfig& C, char* ws, cudaStream
   const int scale_exp = -(n_sqrt2 / 2) + (int)le, scale_half = n_sqrt2 & 1;
   k_finalize<<<(B + 127) / 128, 128, 0, s>>>(C.d_finals, C.n_finals, scal, arena, me, B, hdr, scale_exp, scale_half,
                                               res);
-  k_slice_sum<<<(L.n_rows + 127) / 128, 128, 0, s>>>(res, B, hdr, part, L.n_rows);
+  k_slice_sum<<<(L.n_rows + 3) / 4, 128, 0, s>>>(res, B, hdr, part, L.n_rows);
 }
 
 static bool use_graphs() {
@@ -3552,6 +3606,8 @@ int tnq_internal_group_text(const tnq_plan* plan, int mode, uint32_t batch, char
     add("fold_a", Q.fa.n), add("fold_b", Q.fb.n), add("nf_a", Q.fa.nf), add("nf_b", Q.fb.nf), add("smem", Q.smem);
     out += "\n";
   }
+  for (const HoistDev& H : C.hoist_dev)  // early buckets: index bits, output bits, pieces a block (log2)
+    out += "early: " + std::to_string(H.bits) + " " + std::to_string(H.obits) + " " + std::to_string(H.r) + "\n";
   for (size_t ki = 0; ki < C.kp.size(); ++ki) {
     const KParams& K = C.kp[ki];
     if (K.out_bits < 18) continue;
