@@ -19,8 +19,11 @@ __device__ __forceinline__ float scale_of_max(unsigned mbits, int* mexp) {
   return __int_as_float((127 - m) << 23);
 }
 
+// The roundings are spelled out: left to the compiler, which products it fuses
+// depends on the surrounding code, and kernels that share a bucket's arithmetic
+// must agree (a slice's value must not depend on the batch, to the last bit).
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
-  return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+  return make_float2(fmaf(a.x, b.x, -__fmul_rn(a.y, b.y)), fmaf(a.x, b.y, __fmul_rn(a.y, b.x)));
 }
 
 __device__ __forceinline__ void atomic_max_pos(unsigned* p, float v) {

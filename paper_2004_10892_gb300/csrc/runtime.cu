@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(TPB, 5) k_bucket(const __grid_constant__ KPara
             a0 = cmul(a0, make_float2(v.x * f[j], v.y * f[j]));
             a1 = cmul(a1, make_float2(v.z * f[j], v.w * f[j]));
           }
-          r = make_float2(a0.x + a1.x, a0.y + a1.y);
+          r = make_float2(__fadd_rn(a0.x, a1.x), __fadd_rn(a0.y, a1.y));
         } else {
           float2 a = make_float2(cc.x, cc.y);
 #pragma unroll
@@ -424,7 +424,7 @@ __device__ __forceinline__ float level_entries(const HoistDev& H, int t, long lo
   float2* out = reinterpret_cast<float2*>(arena + H.out) + g0 + t;
 #pragma unroll
   for (int c = 0; c < NC; ++c) {
-    const float2 r = H.sum ? make_float2(a0[c].x + a1[c].x, a0[c].y + a1[c].y) : a0[c];
+    const float2 r = H.sum ? make_float2(__fadd_rn(a0[c].x, a1[c].x), __fadd_rn(a0[c].y, a1[c].y)) : a0[c];
     out[256 * c] = r;
     mx = fmaxf(mx, fmaxf(fabsf(r.x), fabsf(r.y)));
   }
