@@ -10,7 +10,10 @@
 // every parameter's gradient over chunks of rows, added up in chunk order.
 // What bounds it: at a training batch of 1024 rows the launches (each matrix
 // has 8 to 64 tiles); at 10^5 rows the FP32 pipe, through the shared-memory
-// loads of an 8 x 8 register tile.
+// loads of a 4 x 4 register tile.
+// GB300, before (one thread per column for every sum over rows) and now: an
+// epoch of 8256 rows in batches of 1024, 3.0 -> 1.1 ms; the gradient over
+// 162805 rows (1.7e10 flops) 42.5 -> 1.14 ms, 15 TFLOP/s.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -24,14 +27,18 @@ void set_error(const std::string& msg);
 namespace {
 constexpr int MT = 128;  // threads of a matrix tile
 constexpr int MK = 16;   // summed values per shared-memory step
+constexpr int TM = 4;    // a thread's tile: TM x TM results
+constexpr int BM = 16 * TM, BN = 8 * TM;  // a block's
 
-// acc += A B over k in [k0, k1), in increasing order, for the tile of 16 TM x
-// 8 TM results at (m0, p0); la(m, k) and lb(p, k) are the operands inside M x P.
+// acc += A B over k in [k0, k1), in increasing order, for the tile of BM x BN
+// results at (m0, p0); la(m, k) and lb(p, k) are the operands inside M x P.
 // LA / LB::kfast: consecutive k (else consecutive m / p) are consecutive memory.
-template <int TM, class LA, class LB>
+// 4 x 4 results a thread: 64 such tiles of a 128-wide layer at 1024 rows keep
+// four times as many SMs busy as 8 x 8 would (epoch 1.1 against 2.4 ms), and at
+// 10^5 rows more blocks an SM hide the fetches better (1.14 against 1.33 ms).
+template <class LA, class LB>
 __device__ __forceinline__ void tile_product(const LA& la, const LB& lb, int m0, int p0, int M, int P, int k0, int k1,
                                              float (&acc)[TM][TM], float* sh) {
-  constexpr int BM = 16 * TM, BN = 8 * TM;
   constexpr int NA = BM * MK / MT, NB = BN * MK / MT;
   float(*sa)[BM + 4] = reinterpret_cast<float(*)[BM + 4]>(sh);
   float(*sb)[BN + 4] = reinterpret_cast<float(*)[BN + 4]>(sh + MK * (BM + 4));
@@ -74,14 +81,9 @@ __device__ __forceinline__ void tile_product(const LA& la, const LB& lb, int m0,
     if (kb + MK < k1) fetch(kb + MK);  // in flight while this step is computed
 #pragma unroll
     for (int k = 0; k < MK; ++k) {
-      float a[TM], b[TM];
-#pragma unroll
-      for (int i = 0; i < TM; i += 4) {  // rows 4 ty (+ 64), columns 4 tx (+ 32)
-        const float4 va = *reinterpret_cast<const float4*>(&sa[k][4 * ty + 16 * i]);
-        const float4 vb = *reinterpret_cast<const float4*>(&sb[k][4 * tx + 8 * i]);
-        a[i] = va.x, a[i + 1] = va.y, a[i + 2] = va.z, a[i + 3] = va.w;
-        b[i] = vb.x, b[i + 1] = vb.y, b[i + 2] = vb.z, b[i + 3] = vb.w;
-      }
+      const float4 va = *reinterpret_cast<const float4*>(&sa[k][4 * ty]);
+      const float4 vb = *reinterpret_cast<const float4*>(&sb[k][4 * tx]);
+      const float a[TM] = {va.x, va.y, va.z, va.w}, b[TM] = {vb.x, vb.y, vb.z, vb.w};
 #pragma unroll
       for (int i = 0; i < TM; ++i)
 #pragma unroll
@@ -89,11 +91,10 @@ __device__ __forceinline__ void tile_product(const LA& la, const LB& lb, int m0,
     }
   }
 }
-template <int TM>
-constexpr int tile_floats() { return MK * (16 * TM + 4 + 8 * TM + 4); }
+constexpr int TILE_FLOATS = MK * (BM + 4 + BN + 4);
 // Row / column of acc[i][j] within the tile.
-__device__ __forceinline__ int tile_row(int i) { return 4 * (threadIdx.x >> 3) + 64 * (i >> 2) + (i & 3); }
-__device__ __forceinline__ int tile_col(int j) { return 4 * (threadIdx.x & 7) + 32 * (j >> 2) + (j & 3); }
+__device__ __forceinline__ int tile_row(int i) { return 4 * (threadIdx.x >> 3) + i; }
+__device__ __forceinline__ int tile_col(int j) { return 4 * (threadIdx.x & 7) + j; }
 
 struct RowMajor {  // X[row][k]
   static constexpr bool kfast = true;
@@ -118,14 +119,13 @@ struct HeadGrad {
 };
 
 // C = relu(A W^T + b): A (M x K), W (P x K)
-template <int TM>
 __global__ void __launch_bounds__(MT) k_layer(const float* __restrict__ A, const float* __restrict__ W,
                                               const float* __restrict__ bias, float* __restrict__ C, int M, int K,
                                               int P) {
-  __shared__ __align__(16) float sh[tile_floats<TM>()];
-  const int m0 = blockIdx.x * 16 * TM, p0 = blockIdx.y * 8 * TM;
+  __shared__ __align__(16) float sh[TILE_FLOATS];
+  const int m0 = blockIdx.x * BM, p0 = blockIdx.y * BN;
   float acc[TM][TM] = {};
-  tile_product<TM>(RowMajor{A, K}, RowMajor{W, K}, m0, p0, M, P, 0, K, acc, sh);
+  tile_product(RowMajor{A, K}, RowMajor{W, K}, m0, p0, M, P, 0, K, acc, sh);
 #pragma unroll
   for (int i = 0; i < TM; ++i)
 #pragma unroll
@@ -139,14 +139,13 @@ __global__ void __launch_bounds__(MT) k_layer(const float* __restrict__ A, const
 }
 
 // dZ1 = (dZ2 W2) where H1 > 0
-template <int TM>
 __global__ void __launch_bounds__(MT) k_hidden_back(HeadGrad<true> dZ2, const float* __restrict__ W2,
                                                     const float* __restrict__ H1, float* __restrict__ dZ1, int M,
                                                     int H) {
-  __shared__ __align__(16) float sh[tile_floats<TM>()];
-  const int m0 = blockIdx.x * 16 * TM, p0 = blockIdx.y * 8 * TM;
+  __shared__ __align__(16) float sh[TILE_FLOATS];
+  const int m0 = blockIdx.x * BM, p0 = blockIdx.y * BN;
   float acc[TM][TM] = {};
-  tile_product<TM>(dZ2, ColMajor{W2, H}, m0, p0, M, H, 0, H, acc, sh);
+  tile_product(dZ2, ColMajor{W2, H}, m0, p0, M, H, 0, H, acc, sh);
 #pragma unroll
   for (int i = 0; i < TM; ++i)
 #pragma unroll
@@ -197,9 +196,8 @@ struct GradArgs {
 // One chunk's part of every gradient (blockIdx.y): blocks 0..t2-1 tiles of dW2
 // = dZ2^T H1, then t1 tiles of dW1 = dZ1^T x, then blocks of MT columns of the
 // biases' and W3's sums.
-template <int TM>
 __global__ void __launch_bounds__(MT) k_grads(const GradArgs g) {
-  __shared__ __align__(16) float sh[tile_floats<TM>()];
+  __shared__ __align__(16) float sh[TILE_FLOATS];
   const int r0 = blockIdx.y * g.rows, r1 = min(g.n, r0 + g.rows);
   float* W1 = g.part + blockIdx.y * g.stride;
   float* b1 = W1 + (size_t)g.H * g.F;
@@ -211,11 +209,11 @@ __global__ void __launch_bounds__(MT) k_grads(const GradArgs g) {
   if (b < g.t2 + g.t1) {
     const bool second = b < g.t2;
     if (!second) b -= g.t2;
-    const int P = second ? g.H : g.F, cols = (P + 8 * TM - 1) / (8 * TM);
-    const int m0 = b / cols * 16 * TM, p0 = b % cols * 8 * TM;
+    const int P = second ? g.H : g.F, cols = (P + BN - 1) / BN;
+    const int m0 = b / cols * BM, p0 = b % cols * BN;
     float acc[TM][TM] = {};
-    if (second) tile_product<TM>(dZ2, ColMajor{g.H1, g.H}, m0, p0, g.H, P, r0, r1, acc, sh);
-    else tile_product<TM>(ColMajor{g.dZ1, g.H}, ColMajor{g.x, g.F}, m0, p0, g.H, P, r0, r1, acc, sh);
+    if (second) tile_product(dZ2, ColMajor{g.H1, g.H}, m0, p0, g.H, P, r0, r1, acc, sh);
+    else tile_product(ColMajor{g.dZ1, g.H}, ColMajor{g.x, g.F}, m0, p0, g.H, P, r0, r1, acc, sh);
     float* dst = second ? W2 : W1;
 #pragma unroll
     for (int i = 0; i < TM; ++i)
@@ -301,13 +299,8 @@ Views views(const float* p, int F, int H) {
 
 int up(int a, int b) { return (a + b - 1) / b; }
 
-// 128 x 64 tiles from MLP_LARGE rows up, else 64 x 32: at 1024 rows 64 small
-// tiles of a 128-wide layer keep four times as many SMs busy as 16 large ones.
-constexpr int MLP_LARGE = 16384;
-
 void layer(const float* A, const float* W, const float* bias, float* C, int M, int K, int P, cudaStream_t s) {
-  if (M >= MLP_LARGE) k_layer<8><<<dim3(up(M, 128), up(P, 64)), MT, 0, s>>>(A, W, bias, C, M, K, P);
-  else k_layer<4><<<dim3(up(M, 64), up(P, 32)), MT, 0, s>>>(A, W, bias, C, M, K, P);
+  k_layer<<<dim3(up(M, BM), up(P, BN)), MT, 0, s>>>(A, W, bias, C, M, K, P);
 }
 }  // namespace
 }  // namespace tnq
@@ -353,18 +346,15 @@ tnq_status tnq_mlp_backward(const float* params, int32_t hidden, const float* x,
   float* dP = dZ1 + nh;     // N
   float* sq = dP + N;       // N: the loss's partial sums
   float* part = sq + N;     // the rest of the workspace, 2 N H + 2 N + 16 floats: the chunks' gradients
-  const bool large = N >= MLP_LARGE;
-  const int tm = large ? 128 : 64, tp = large ? 64 : 32;
   layer(x, v.W1, v.b1, H1, N, F, H, s);
   layer(H1, v.W2, v.b2, H2, N, H, H, s);
   const int n_sq = up(N, HEAD_ROWS);
   k_head<<<n_sq, 32 * HEAD_ROWS, 0, s>>>(H2, v.W3, v.b3, y, dP, sq, N, H);
   const HeadGrad<true> dZ2{dP, v.W3, H2, H};
-  if (large) k_hidden_back<8><<<dim3(up(N, 128), up(H, 64)), MT, 0, s>>>(dZ2, v.W2, H1, dZ1, N, H);
-  else k_hidden_back<4><<<dim3(up(N, 64), up(H, 32)), MT, 0, s>>>(dZ2, v.W2, H1, dZ1, N, H);
-  // chunks of at least 64 rows (512 when large), as many as the workspace holds; one writes grads itself
+  k_hidden_back<<<dim3(up(N, BM), up(H, BN)), MT, 0, s>>>(dZ2, v.W2, H1, dZ1, N, H);
+  // chunks of at least 64 rows, as many as the workspace holds; one writes grads itself
   const size_t room = (2 * nh + 2 * (size_t)N + 16) / count;
-  const int most = up(N, large ? 512 : 64);
+  const int most = up(N, 64);
   int chunks = (int)std::min<size_t>(room, (size_t)std::min(most, 512));
   GradArgs g;
   g.rows = up(N, std::max(chunks, 1));
@@ -373,11 +363,10 @@ tnq_status tnq_mlp_backward(const float* params, int32_t hidden, const float* x,
   g.part = chunks > 1 ? part : grads;
   g.stride = count;
   g.n = N, g.F = F, g.H = H;
-  g.t2 = up(H, tm) * up(H, tp);
-  g.t1 = up(H, tm) * up(F, tp);
+  g.t2 = up(H, BM) * up(H, BN);
+  g.t1 = up(H, BM) * up(F, BN);
   const dim3 grid(g.t2 + g.t1 + up(H, MT), chunks);
-  if (large) k_grads<8><<<grid, MT, 0, s>>>(g);
-  else k_grads<4><<<grid, MT, 0, s>>>(g);
+  k_grads<<<grid, MT, 0, s>>>(g);
   k_add_up<<<(unsigned)((count + 255) / 256) + 1, 256, 0, s>>>(g.part, count, chunks, grads, count, sq, n_sq, loss,
                                                                 1.f / (2.f * (float)N));
   cudaError_t e = cudaGetLastError();
