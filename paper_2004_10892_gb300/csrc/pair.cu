@@ -52,6 +52,19 @@ __device__ __forceinline__ void cfma2(float2& r, float4 a, float4 b) {
 // 16-byte shared loads feed 32 x 2^RY FMAs. Shared memory delivers 128 bytes a
 // cycle to registers, so 4 x 4 needs all of it at the full FMA rate and 4 x 8
 // three quarters.
+//
+// What bounds it, and GB300 figures against the bucket-by-bucket chain kernel
+// (k_group) that ran these chains:
+//  * two tensors: the FMA pipe (78 TFLOP/s measured). 5 buckets, bag 28, 32
+//    items: 12.9 -> 1.97 ms, 72 TFLOP/s.
+//  * three: issue slots (68 % busy, 62 % of them FMAs; 128 registers hold two
+//    blocks an SM) and the reads of C, each used once. 3 buckets, bag 28, 64
+//    items: 19.9 -> 5.53 ms, 36 TFLOP/s.
+//  * one: memory. A bucket of bag 23, 32 items: 4.0 -> 5.6 TB/s (k_bucket
+//    before); 5 buckets, bag 22: 3.5 -> 5.1 TB/s of a copy's 6.8.
+// Slower: register double buffering by halves of a pair (8-byte reads at a
+// 16-byte stride cost twice the cycles, 2.28 -> 2.85 ms on the first); no
+// faster: three or four stages.
 // CM: 0 no C, 1 C without u_0 (its bit 0 is B's register bit 0), 2 C with u_0,
 // 3 B alone: B comes through shared memory only to be read in consecutive
 // pieces, and is multiplied by the small tensors' product as it is summed.

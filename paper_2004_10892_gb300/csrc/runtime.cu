@@ -1590,6 +1590,12 @@ struct SmallPlan {
   size_t tables = 0, leaves = 0, scalars = 0, inout = 0, finals = 0, vals = 0;  // offsets in it
   int widest = 1;          // most entries of a level that the whole cluster works on
 };
+// The lines, GB300, twelve small plans in one call / a 6x6 network of
+// three-valued indices (642 to 654 / 303 us): plans above 2^23 flops by
+// launches 720 / 372; one kernel up to 2^27 650 / 305 (none lies between; its
+// eight SMs then need 100 us and more for the arithmetic alone). Levels above
+// 2^10 or 2^14 entries over the cluster: 639 / 298 and 653 / 314, and 160 / 163
+// / 184 us (2^10, 2^12, 2^14) for 16 slices of 6x6 depth 24.
 constexpr double SMALL_FLOPS = 1 << 25;      // per slice
 constexpr int SMALL_BITS = 20;               // variables of a bucket's result
 constexpr int SMALL_WIDE = 4096;             // a level of more entries is shared by the cluster
@@ -2103,6 +2109,11 @@ static GParams group_gparams(const tnq_plan& P, const Layout& L, const FusedGrou
 //    (eliminated variables of C count), or fewer along A and 2^3 along B's:
 //    without them nothing is shared;
 //  * 2^PTB threads times the register tile of outputs.
+// The lines, GB300, bf16x3 amplitude of 7x7 depth 32 / 37 of its 256 slices in
+// complex64 (5.147 / 5.846 ms): a rank limit for small tensors of 3 or 6 gives
+// 5.143 / 5.854 and 5.122 / 5.861 (the plans' tensors are gates or large, few
+// lie between); 2^3 or 2^7 tiles 5.137 / 5.814 and 5.163 / 5.888; 2^3 or 2^5
+// pairs a loop 5.227 / 5.888 and 5.135 / 5.870.
 constexpr int PAIR_SMALL = 4;
 constexpr int PAIR_TILES = 5;
 constexpr int PAIR_LOOP = 4;  // a thread sums 2^PAIR_LOOP pairs per 4 x 4 outputs of a tile where the operands allow it
