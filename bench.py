@@ -117,31 +117,32 @@ class ClockSampler:
 
 
 # ncu DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of every
-# k_group launch of a one-slice batch of this workload (capture command in
-# profiles/k_group_7x7_d1+32+1.md), valid only while the fused-chain kernel's
-# source (runtime.cu between the "Fused chain of buckets" and "K4: amplitude"
-# comments) hashes to `kernel_sha1` and the plan has the recorded tuning and
-# k_group launch count (reported as null otherwise). Per launch at batch B:
-# bytes_one_slice x B / k_group launches per batch (traffic scales with the
-# slices of a batch; item-invariant operands are read once per batch, so this
-# slightly overstates it).
-MEASURED_TRAFFIC = {"k_group": [
-    {"kernel_sha1": "9600051a4d6febd8fe8034590085acd1e4118364", "tuning": [4, 64], "bytes_one_slice": 106121216.0,
-     "launches": 12,
-     "capture": "ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum -k regex:k_group -s 12 -c 12 on a one-slice "
-                "batch of the tuned default plan (tuning 2^4 / 64)"},
-]}
+# k_pair and k_group launch of a one-slice batch of this workload (capture
+# command in profiles/k_pair_7x7_d1+32+1.md), valid only while the chain kernels'
+# source (pair.cu, and runtime.cu between the "Fused chain of buckets" and "K4:
+# amplitude" comments) hashes to `kernel_sha1` and the plan has the recorded
+# tuning and number of chains (reported as null otherwise). Per launch at batch
+# B: bytes_one_slice x B / launches (traffic scales with the slices of a batch;
+# item-invariant operands are read once per batch, so this slightly overstates
+# it).
+MEASURED_TRAFFIC = [
+    {"kernel_sha1": "78232f70757bcf02e3642f6750eae68851d4e32c", "tuning": [4, 64], "chains": 12,
+     "bytes_one_slice": 158943744.0, "launches": 22,
+     "capture": "ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum -k regex:k_pair|k_group, the 22 k_pair "
+                "launches of a one-slice batch of the tuned default plan (tuning 2^4 / 64; 12 chains, 10 buckets)"},
+]
 
 
 def kernel_source_sha1():
-    """SHA-1 of the fused-chain kernel's source region of runtime.cu."""
+    """SHA-1 of the chain kernels' source: pair.cu and the region of runtime.cu."""
     import hashlib
 
     with open(os.path.join(ROOT, "paper_2004_10892_gb300", "csrc", "runtime.cu")) as f:
         text = f.read()
     a = text.index("// Fused chain of buckets")
     b = text.index("// K4: amplitude")
-    return hashlib.sha1(text[a:b].encode()).hexdigest()
+    with open(os.path.join(ROOT, "paper_2004_10892_gb300", "csrc", "pair.cu")) as f:
+        return hashlib.sha1((f.read() + text[a:b]).encode()).hexdigest()
 
 
 # FP32 CUDA-core peak of GB300 from unit counts and clocks: 152 SMs x 128 FP32
@@ -202,7 +203,7 @@ def launch_roofline(L, plan, bits, ws, B, n_sl, stream, peaks, info):
         "derived: 152 SMs x 128 FP32 lanes x 2 x max SM clock"
     one_gbs = sum(by[i] for i in one) / (t_one / 1e3) / 1e9 if t_one > 0 else None
     grp_tfs = sum(fl[i] for i in grp) / (t_grp / 1e3) / 1e12 if t_grp > 0 else None
-    k_bucket = {"kernel": "k_bucket", "bound": "hbm", "achieved": one_gbs, "peak": hbm, "unit": "GB/s",
+    k_bucket = {"kernel": "k_bucket (large buckets: k_pair)", "bound": "hbm", "achieved": one_gbs, "peak": hbm, "unit": "GB/s",
                 "frac": one_gbs / hbm if one_gbs else None, "launches": len(one), "time_share": t_one / tot,
                 "bytes_per_launch": sum(by[i] for i in one) / max(len(one), 1),
                 "ms_per_launch": t_one / max(len(one), 1),
@@ -216,23 +217,24 @@ def launch_roofline(L, plan, bits, ws, B, n_sl, stream, peaks, info):
                                         "share_of_k_bucket_time": t_big1 / t_one,
                                         "each": [{"bag": bag[i], "MB": round(by[i] / 1e6, 1), "ms": round(ms[i], 4),
                                                   "gbs": round(by[i] / (ms[i] / 1e3) / 1e9, 1)} for i in big1]}
-    k_group = {"kernel": "k_group", "bound": "alu", "achieved": grp_tfs, "peak": fp32, "unit": "TFLOP/s",
+    chains = {"kernel": "k_pair (chains of other shapes: k_group)", "bound": "alu", "achieved": grp_tfs, "peak": fp32, "unit": "TFLOP/s",
                "frac": grp_tfs / fp32 if grp_tfs else None, "launches": len(grp), "time_share": t_grp / tot,
                "flops_per_launch": sum(fl[i] for i in grp) / max(len(grp), 1),
                "ms_per_launch": t_grp / max(len(grp), 1),
                "peak_source": fp32_src}
-    dom, other = (k_group, k_bucket) if t_grp >= t_one else (k_bucket, k_group)
+    # (bucket launches below 20 us are launch-bound here; the captured graph runs most of them in level launches)
+    dom, other = (chains, k_bucket) if t_grp >= sum(ms[i] for i in one if ms[i] >= 0.02) else (k_bucket, chains)
     out = dict(dom)
     out["traffic"] = None
-    if dom["kernel"] == "k_group" and grp:
+    if dom is chains and grp:
         big = max(grp, key=lambda i: ms[i])
         out["largest_launch"] = {"ms": ms[big], "flops": fl[big], "algorithmic_bytes": by[big],
                                  "achieved_tflops": fl[big] / (ms[big] / 1e3) / 1e12 if ms[big] > 0 else None}
-        for mt in MEASURED_TRAFFIC["k_group"]:
+        for mt in MEASURED_TRAFFIC:
             if (mt["kernel_sha1"] == kernel_source_sha1() and mt["tuning"] == list(plan.tuning())
-                    and mt["launches"] == len(grp) and mt["bytes_one_slice"] > 0):
-                out["traffic"] = mt["bytes_one_slice"] * b_out.value / len(grp)
-                out["traffic_source"] = mt["capture"] + ", x batch / k_group launches per batch"
+                    and mt["chains"] == len(grp)):
+                out["traffic"] = mt["bytes_one_slice"] * b_out.value / mt["launches"]
+                out["traffic_source"] = mt["capture"] + ", x batch / those launches per batch"
     out["peak_source"] = dom.get("peak_source", "measured (MEASURED_PEAKS.json hbm_gbs)")
     out["batch"] = b_out.value
     out["other_kernel"] = other
