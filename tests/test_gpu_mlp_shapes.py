@@ -1,5 +1,5 @@
 """Forward and backward kernels of the proposer at the sizes where their tiles
-end: one row, one short of / past a tile, one chunk and many, both tile sizes,
+end: one row, one short of / past a tile, one chunk and many,
 hidden widths that are no multiple of a tile."""
 import numpy as np
 import pytest
