@@ -2598,8 +2598,8 @@ static bool gemm_as_pair(const ExecConfig& C, size_t i) {
 // A GEMM chain whose tiles are mostly padding runs as an FP32 product instead:
 // at one row an item (padded to 128 or 64 of the MMA tile) the tensor cores do
 // 128 times the work and the operands are packed for it. 8 items of such a
-// chain (25 variables, one row, 64 columns, K = 32; 2.2 GB): 3.96 -> 0.84 ms; 16
-// items of one with 4096 rows and 4 columns (padded to 64): 0.109 -> 0.044 ms.
+// chain (25 variables, one row, 64 columns, K = 32; 2.2 GB): 3.96 -> 0.49 ms; 16
+// items of one with 4096 rows and 4 columns (padded to 64): 0.109 -> 0.039 ms.
 // At a padding of 8 and below the two were not told apart.
 constexpr double PAIR_GEMM_PADDING = 16;
 static double gemm_padding(const FusedGroup& g, const GemmBucketArgs& G) {
@@ -2722,7 +2722,9 @@ static bool build_steps(const tnq_plan& P, const Layout& L, ExecConfig& C) {
         for (int b = 0; b < k.G; ++b) h.stride[j][b] = k.stride[j][b];
       }
       // several pieces of 256 entries a block once 512 blocks remain (three and
-      // a half for every SM), in blocks of one item
+      // a half for every SM), in blocks of one item. 7x7 amplitude / four mixed
+      // plans on GB300: 5.14 / 92.0 ms; one piece always 5.35 / 98.0, four at
+      // most 5.16 / 92.1; once 64 blocks remain 5.12 / 92.0, 4096 5.18 / 93.5
       if (k.out_bits >= 8 + LEVEL_R || k.G == k.out_bits) h.r = std::min(LEVEL_R, std::max(0, k.G - 17));
       blocks += (int)(((1ll << k.G) + (256ll << h.r) - 1) >> (8 + h.r));
       C.hoist_dev.push_back(h);
