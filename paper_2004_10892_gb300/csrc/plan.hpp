@@ -12,6 +12,7 @@
 namespace tnq {
 struct DeviceState;  // per-device tables and cached graphs (runtime.cu)
 struct SmallPlan;    // the plan's one-kernel form (runtime.cu)
+enum SmallMode { SMALL_RULE, SMALL_OFF, SMALL_ON };  // whether a plan uses it: by the rule, never, wherever it has it
 void destroy_device_state(DeviceState* s);
 void set_error(const std::string& msg);
 }  // namespace tnq
@@ -39,7 +40,7 @@ struct tnq_plan {
   mutable std::map<std::pair<int, int>, size_t> layout_bytes;  // (mode, batch) -> workspace bytes
   mutable std::mutex small_mu;
   mutable std::shared_ptr<tnq::SmallPlan> small;  // built on first use, dropped with the program
-  bool small_off = false;                         // internal test hook: always run step by step
+  tnq::SmallMode small_mode = tnq::SMALL_RULE;    // the other two: internal test hook
   mutable std::mutex dev_mu;
   mutable tnq::DeviceState* dev = nullptr;
   ~tnq_plan() {

@@ -1781,8 +1781,17 @@ static void build_small(const tnq_plan& P, SmallPlan& S) {
   S.ok = small_smem(A) <= SMALL_SMEM_MAX && A.n_words <= SMALL_WORDS;
 }
 
+// Plans whose GEMM chains run in 3xBF16 keep their launches: a slice's value is
+// that of the precision asked for (13 such requests moved by 3e-6 to 1.6e-5
+// in FP32). 3xTF32 keeps all but two of FP32's bits: its values move by 1e-6.
+static bool small_wanted(const tnq_plan& P) {
+  if (P.small_mode != SMALL_RULE) return P.small_mode == SMALL_ON;
+  if (P.opts.precision != TNQ_PREC_SPLIT_BF16) return true;
+  return std::none_of(P.prog.groups.begin(), P.prog.groups.end(), [](const FusedGroup& g) { return g.gemm; });
+}
+
 const SmallPlan* small_plan(const tnq_plan& P) {
-  if (P.small_off) return nullptr;
+  if (!small_wanted(P)) return nullptr;
   std::lock_guard<std::mutex> lk(P.small_mu);
   if (!P.small) {
     P.small = std::make_shared<SmallPlan>();
@@ -3511,10 +3520,11 @@ int tnq_internal_validate(const tnq_plan* plan, int mode, uint32_t batch, char* 
 }
 
 // Internal test hook (not in include/tnq.h): whether the plan runs as one
-// kernel (k_small); use = 0 makes it run step by step, 1 undoes that. Before
-// the plan is shared, as tnq_plan_keep_chains.
+// kernel (k_small); use = 0 makes it run step by step, 1 as one kernel wherever
+// it has that form, 2 by the rule (as a plan without this call does). Before the
+// plan is shared, as tnq_plan_keep_chains.
 int tnq_internal_small(tnq_plan* plan, int use) {
-  plan->small_off = !use;
+  plan->small_mode = use == 0 ? SMALL_OFF : (use == 1 ? SMALL_ON : SMALL_RULE);
   {
     std::lock_guard<std::mutex> lk(plan->layout_mu);
     plan->layout_bytes.clear();

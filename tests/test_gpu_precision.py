@@ -1,0 +1,50 @@
+"""3xBF16 plans give 3xBF16 values on every route that a plan can take."""
+import ctypes
+
+import numpy as np
+import pytest
+
+from paper_2004_10892_gb300 import inputs as I
+
+# small enough for one kernel, with GEMM chains (rows, cols, depth, seed, plan options)
+SMALL = [
+    (5, 5, 22, 8835, dict(max_bag_log2=20, min_p=2, max_p=40)),
+    (6, 6, 20, 3416, dict(max_bag_log2=25, max_p=40)),
+    (5, 4, 31, 4704, dict(max_bag_log2=26, min_p=2, max_p=40)),
+]
+
+
+def _plan(tnq_lib, case, precision):
+    rows, cols, depth, seed, kw = case
+    circ = I.random_grid_circuit(rows, cols, depth, seed)
+    return circ, tnq_lib.Plan(circ, precision=precision, reorder_every=1, **kw)
+
+
+def _small(tnq_lib, plan, use):
+    f = tnq_lib.lib().tnq_internal_small
+    f.argtypes = [ctypes.c_void_p, ctypes.c_int]
+    return f(plan.handle, use)
+
+
+@pytest.mark.parametrize("case", SMALL, ids=str)
+def test_gemm_chains_in_bf16_keep_their_launches(tnq_lib, case):
+    _, plan = _plan(tnq_lib, case, tnq_lib.PREC_SPLIT_BF16)
+    assert plan.info()["n_gemm_buckets"] > 0
+    assert _small(tnq_lib, plan, 1) == 1  # it has a one-kernel form,
+    assert _small(tnq_lib, plan, 2) == 0  # which the rule does not take
+    plan.keep_chains([])  # without GEMM chains every product is FP32
+    assert plan.info()["n_gemm_buckets"] == 0 and _small(tnq_lib, plan, 2) == 1
+    _, plan = _plan(tnq_lib, case, tnq_lib.PREC_C64)
+    assert _small(tnq_lib, plan, 2) == 1
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("case", SMALL, ids=str)
+def test_small_bf16_plans_run_their_gemm_chains(cuda, tnq_lib, case):
+    circ, plan = _plan(tnq_lib, case, tnq_lib.PREC_SPLIT_BF16)
+    bits = I.random_bitstring(circ.n_qubits, 1)
+    _, got = tnq_lib.contract_sliced(plan, bits, per_slice=True)
+    _, loc = tnq_lib.contract_sliced_noalloc(plan, bits, per_slice=True)
+    _small(tnq_lib, plan, 0)
+    _, steps = tnq_lib.contract_sliced(plan, bits, per_slice=True)
+    assert np.array_equal(got, steps) and np.array_equal(loc, steps)
