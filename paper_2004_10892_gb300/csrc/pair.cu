@@ -1,5 +1,7 @@
 // pair.cu -- k_pair: a fused chain of buckets as a register-tiled contraction
 // (see pair.cuh).
+#include <cuda_bf16.h>
+
 #include "device_util.cuh"
 #include "pair.cuh"
 
@@ -44,6 +46,24 @@ __device__ __forceinline__ void cfma2(float2& r, float4 a, float4 b) {
   r.y = fmaf(a.w, b.z, r.y);
 }
 
+// 3xBF16 as the GEMM packs it: x = hi + lo, two roundings to bf16. hi + lo is a
+// float itself, so an operand is staged as that sum, and of a product a b the
+// GEMM's three terms are a b - lo(a) lo(b).
+__device__ __forceinline__ float2 bf16_lo(float2 x) {
+  const float2 h = __bfloat1622float2(__float22bfloat162_rn(x));
+  return make_float2(x.x - h.x, x.y - h.y);
+}
+__device__ __forceinline__ float2 bf16_split(float2 x) {
+  const float2 h = __bfloat1622float2(__float22bfloat162_rn(x));
+  const float2 l = __bfloat1622float2(__float22bfloat162_rn(make_float2(x.x - h.x, x.y - h.y)));
+  return make_float2(h.x + l.x, h.y + l.y);
+}
+template <class F>
+__device__ __forceinline__ float4 both(F f, float4 v, float sign = 1.f) {  // f of the pair's two values
+  const float2 a = f(make_float2(v.x, v.y)), b = f(make_float2(v.z, v.w));
+  return make_float4(sign * a.x, sign * a.y, sign * b.x, sign * b.y);
+}
+
 // Persistent: a block loops over tiles (item, tile variables), a tile over one,
 // two or four chunks of its summed values. Two stages: while a chunk is computed,
 // the next one's part of A, B (and C) comes in by cp.async; each thread then
@@ -68,7 +88,8 @@ __device__ __forceinline__ void cfma2(float2& r, float4 a, float4 b) {
 // CM: 0 no C, 1 C without u_0 (its bit 0 is B's register bit 0), 2 C with u_0,
 // 3 B alone: B comes through shared memory only to be read in consecutive
 // pieces, and is multiplied by the small tensors' product as it is summed.
-template <int RX, int RY, int NKX, int NKY, int CM>
+// SPLIT: 3xBF16 (CM 0 only).
+template <int RX, int RY, int NKX, int NKY, int CM, bool SPLIT = false>
 __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairParams P, long long n_tiles) {
   extern __shared__ float4 sm[];
   constexpr bool HASC = CM == 1 || CM == 2, ONE = CM == 3;
@@ -223,7 +244,8 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
   auto fold = [&](int slot, int chunk, int buf, int n) {
 #pragma unroll
     for (int o = 0; o < 2; ++o) {
-      if (o == 0 && !fold_a) continue;
+      const bool folded = o == 1 || fold_a;
+      if (!SPLIT && !folded) continue;
       const POp& O = *ops[o];
       const float4* ft = (o == 0 ? s_fa[n & 1] : s_fb[n & 1]) + tf[o] + s_fold[slot][o] +
                          ((chunk & 1) ? O.fch[0] : 0) + ((chunk & 2) ? O.fch[1] : 0);
@@ -234,10 +256,14 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
         for (int it = 0; it < nit; ++it) {
           const int4 k = s_it[o][it];
           float4& dst = *reinterpret_cast<float4*>(smb + (at ^ k.y));
-          const float4 v = dst, f = ft[k.z];
-          const float2 v0 = cmul(make_float2(v.x, v.y), make_float2(f.x, f.y));
-          const float2 v1 = cmul(make_float2(v.z, v.w), make_float2(f.z, f.w));
-          dst = make_float4(v0.x, v0.y, v1.x, v1.y);
+          float4 v = dst;
+          if (folded) {
+            const float4 f = ft[k.z];
+            const float2 v0 = cmul(make_float2(v.x, v.y), make_float2(f.x, f.y));
+            const float2 v1 = cmul(make_float2(v.z, v.w), make_float2(f.z, f.w));
+            v = make_float4(v0.x, v0.y, v1.x, v1.y);
+          }
+          dst = SPLIT ? both(bf16_split, v) : v;
         }
       }
     }
@@ -305,15 +331,22 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
         for (int q = 0; q < n1; ++q) {
           const int2 k = s_k1[q];
           const int qa = oa ^ k.x, qb = ob ^ k.y;
-          float4 va[NX];
+          float4 va[NX], la[SPLIT ? NX : 1];
 #pragma unroll
-          for (int i = 0; i < NX; ++i)
+          for (int i = 0; i < NX; ++i) {
             if (!ONE) va[i] = quad(pa, qa ^ off_x(i, P.xa));
+            if constexpr (SPLIT) la[i] = both(bf16_lo, va[i], -1.f);
+          }
 #pragma unroll
           for (int j = 0; j < NY; ++j) {
             const float4 vb = quad(smb, qb ^ off_y(j, P.yb));
 #pragma unroll
             for (int i = 0; i < NX; ++i) cfma2(x[i][j], ONE ? quad(pa, qa ^ off_y(j, P.yf)) : va[i], vb);
+            if constexpr (SPLIT) {
+              const float4 lb = both(bf16_lo, vb);
+#pragma unroll
+              for (int i = 0; i < NX; ++i) cfma2(x[i][j], la[i], lb);
+            }
           }
         }
       };
@@ -408,6 +441,11 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
 
 using PairKernel = void (*)(PairParams, long long);
 static PairKernel pair_kernel(const PairParams& p) {
+  if (p.split) {
+    if (p.rx == 2) return k_pair<2, 2, 0, 0, 0, true>;
+    if (p.rx) return k_pair<1, 3, 0, 0, 0, true>;
+    return p.ry > 1 ? k_pair<0, 3, 0, 0, 0, true> : k_pair<0, 1, 0, 0, 0, true>;
+  }
   if (p.a.gin < 0) return p.ry > 1 ? k_pair<0, 3, 0, 0, 3> : k_pair<0, 1, 0, 0, 3>;
   if (p.c.gin < 0) {
     if (p.rx == 2) return p.ry > 2 ? k_pair<2, 3, 0, 0, 0> : k_pair<2, 2, 0, 0, 0>;

@@ -9,6 +9,8 @@
 // With K2 = K & vars(C) and K1 = K - K2:
 //   out[o] = sum_K2 C[K2, o] (sum_K1 A[K1, K2, o] B[K1, K2, o]).
 // With one large tensor only (B) the small tensors' product takes A's place.
+// A GEMM chain of mostly padding comes here too; in 3xBF16 it keeps that
+// precision's sums (`split`).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -71,6 +73,7 @@ struct PairParams {
   int yb[PRY_MAX], yc[PRY_MAX], yo[PRY_MAX];   // register bits along B
   int rx, ry;                   // register bits along A / B
   int c_u0;                     // 1: C holds u_0 (K2 then includes it)
+  int split;                    // 1: 3xBF16 (two large tensors only): operands as bf16 hi + lo, without lo times lo
   int nl, la[PL_MAX], lb[PL_MAX], lc[PL_MAX], lo[PL_MAX];  // a thread's loop over outputs
   int ft[PTB], yf[PRY_MAX], k1f[PK_MAX];        // B alone: the fold table's index instead of A's slots
   int n1, k1a[PK_MAX], k1b[PK_MAX];                // K1 without u_0 and the chunk's variable: slots of a and b

@@ -2190,7 +2190,13 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
   }
   if ((!one && vars(A)[0] != u0) || vars(B)[0] != u0) return false;
   std::vector<int> sa, sb;
+  if (g.gemm && large.size() != 2) return false;
+  G.split = g.gemm && P.opts.precision == TNQ_PREC_SPLIT_BF16;
   for (int j : small) {
+    if (g.gemm) {  // (inputs: two operands, what is folded into the first, into the second: the products that are rounded)
+      ((j < 2 + (int)g.a_side.size() ? 0 : 1) == A ? sa : sb).push_back(j);
+      continue;
+    }
     bool ina = true, inb = true;
     for (int v : vars(j)) {
       ina = ina && holds(A, v);
@@ -2218,7 +2224,7 @@ static bool pair_params(const tnq_plan& P, const Layout& L, const FusedGroup& g,
   // 2^PAIR_TILES tiles an item (fewer leave the device idle), else 4 x 4
   // with nothing to share along A the tile only holds B: small, for long sums
   if (G.rx < 2) G.ry = G.rx || (int)K.size() <= 2 ? 3 : 1;
-  else G.ry = !G.c_u0 && alone(B, A, o.vars) + G.nky >= 3 &&
+  else G.ry = !G.c_u0 && !G.split && alone(B, A, o.vars) + G.nky >= 3 &&
               o.rank() >= PTB + G.rx - G.nkx + 3 - G.nky + PAIR_TILES ? 3 : 2;
   const int need_x = G.rx - G.nkx, need_y = G.ry - G.nky, n_one = PTB + need_x + need_y;
   if (o.rank() < n_one) return false;
@@ -2604,7 +2610,8 @@ static bool gemm_as_pair(const ExecConfig& C, size_t i) {
   return false;
 }
 
-// A GEMM chain whose tiles are mostly padding runs as an FP32 product instead:
+// A GEMM chain whose tiles are mostly padding runs in k_pair instead (3xBF16 as
+// the same sums on the FP32 pipe, 3xTF32 in FP32, which differs from it by 1e-6):
 // at one row an item (padded to 128 or 64 of the MMA tile) the tensor cores do
 // 128 times the work and the operands are packed for it. 8 items of such a
 // chain (25 variables, one row, 64 columns, K = 32; 2.2 GB): 3.96 -> 0.49 ms; 16
@@ -2678,7 +2685,7 @@ static bool build_steps(const tnq_plan& P, const Layout& L, ExecConfig& C) {
       C.step_hoist.push_back(0);
       C.gb.push_back(G);
       C.ge.push_back(E);
-      pair_step(prog.groups[gi], gemm_padding(prog.groups[gi], G) >= PAIR_GEMM_PADDING);
+      pair_step(prog.groups[gi], P.pair_gemm && gemm_padding(prog.groups[gi], G) >= PAIR_GEMM_PADDING);
       double by = tbytes(prog.groups[gi].output);
       for (int t : prog.groups[gi].ext_inputs) by += tbytes(t);
       C.step_bytes.push_back(by);
@@ -3531,6 +3538,13 @@ int tnq_internal_small(tnq_plan* plan, int use) {
   }
   reset_device_state(*plan);
   return small_plan(*plan) ? 1 : 0;
+}
+
+// Internal test hook (not in include/tnq.h): use = 0 runs GEMM chains of mostly
+// padding on the tensor cores, 1 undoes that. Before the plan is shared.
+void tnq_internal_pair_gemm(tnq_plan* plan, int use) {
+  plan->pair_gemm = use != 0;
+  reset_device_state(*plan);
 }
 
 // Internal hook (not in include/tnq.h; host only): the kernel kind of every

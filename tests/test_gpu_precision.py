@@ -48,3 +48,34 @@ def test_small_bf16_plans_run_their_gemm_chains(cuda, tnq_lib, case):
     _small(tnq_lib, plan, 0)
     _, steps = tnq_lib.contract_sliced(plan, bits, per_slice=True)
     assert np.array_equal(got, steps) and np.array_equal(loc, steps)
+
+
+# GEMM chains of mostly padding: every tile that they get, small tensors folded into either operand
+PADDED = [
+    (7, 5, 28, 2045, dict(max_bag_log2=22, max_p=40)),
+    (5, 6, 31, 2775, dict(max_bag_log2=20, max_p=40)),
+    (7, 6, 29, 6996, dict(max_bag_log2=23, max_p=40)),
+    (6, 6, 20, 3416, dict(max_bag_log2=25, max_p=40)),
+]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("case", PADDED, ids=str)
+def test_padded_bf16_chains_give_the_gemm_values(cuda, tnq_lib, case):
+    """FP32 sums in another order (2^-24 per addition, ~50 steps), and operands
+    of later splits that they move across a rounding boundary (2^-17 each, with
+    a probability of 2^-6): 5e-6 in all. FP32 products differ by up to 2e-5."""
+    circ, plan = _plan(tnq_lib, case, tnq_lib.PREC_SPLIT_BF16)
+    bits = I.random_bitstring(circ.n_qubits, 88)
+    n = min(8, plan.info()["n_slices"])
+    f = tnq_lib.lib().tnq_internal_pair_gemm
+    f.argtypes = [ctypes.c_void_p, ctypes.c_int]
+    f.restype = None
+    launches = tnq_lib.lib().tnq_internal_launches_per_batch
+    launches.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_uint32]
+    got = tnq_lib.contract_sliced(plan, bits, 0, n, per_slice=True)[1]
+    fewer = launches(plan.handle, 0, 1)
+    f(plan.handle, 0)
+    assert launches(plan.handle, 0, 1) > fewer  # (a GEMM packs its operands first)
+    gemm = tnq_lib.contract_sliced(plan, bits, 0, n, per_slice=True)[1]
+    assert np.linalg.norm(got - gemm) <= 5e-6 * np.linalg.norm(gemm)
