@@ -1574,6 +1574,52 @@ static LeafDev make_leafdev(const tnq_plan& P, const PTensor* pt, int gate, cons
   return d;
 }
 
+// A bucket's inputs in the order of k_bucket's parameters. It multiplies the
+// last ones, from *n_var on, first: the choice depends on the bucket alone (not
+// on the batch size or on which variables make an input item-dependent), so
+// every configuration and every kernel multiplies in the same order.
+static std::vector<int> bucket_inputs(const Program& prog, const PBucket& b, int* n_var) {
+  std::vector<int> ins(b.inputs.begin(), b.inputs.end());
+  const std::vector<int>& out = prog.tensors[b.output].vars;
+  auto holds = [&](int j, int i) {
+    const auto& v = prog.tensors[ins[j]].vars;
+    return std::find(v.begin(), v.end(), out[i]) != v.end();
+  };
+  const int nout = (int)out.size(), n = (int)ins.size();
+  // the input with the most distinct entries per block (then the largest)
+  // first, among those that vary with output bits 0-7: k_bucket loads input 0
+  // several iterations ahead
+  auto weight = [&](int j) {  // (-1: constant over output bits 0-7; else output bits 0-11 it varies with, rank)
+    int w8 = 0, w = 0, rank = 0;
+    for (int i = 0; i < nout; ++i) {
+      const bool nz = holds(j, i);
+      w8 += (i < 8) && nz;
+      w += (i < 12) && nz;
+      rank += nz;
+    }
+    return w8 ? std::make_pair(w, rank) : std::make_pair(-1, 0);
+  };
+  int best = 0;
+  for (int j = 1; j < n; ++j)
+    if (weight(j) > weight(best)) best = j;
+  if (best != 0 && weight(best).first >= 0) std::swap(ins[best], ins[0]);
+  // inputs that vary with the low 8 bits (a block's threads) first; the others
+  // are the same for every thread of a block's iteration (k_bucket multiplies
+  // them once per block into a constant pair)
+  // (output bits only: whether an input varies with the item bits depends on
+  // the configuration, and the arithmetic order must not)
+  auto varies = [&](int j) {
+    for (int i = 0; i < 8 && i < nout; ++i)
+      if (holds(j, i)) return true;
+    return false;
+  };
+  int nv = 0;
+  for (int j = 0; j < n; ++j)
+    if (varies(j)) std::swap(ins[j], ins[nv++]);
+  *n_var = nv;
+  return ins;
+}
+
 // ---------------------------------------------------------------------------
 // One-kernel form of a small plan (k_small, small.cuh): every bucket of the
 // program -- fused chains and GEMM chains bucket by bucket -- in levels.
@@ -1690,7 +1736,10 @@ static void build_small(const tnq_plan& P, SmallPlan& S) {
       op_of[b] = (int)ops.size();
       ops.push_back(SmallOp{where(B.output), V.entries, o.rank(), (int)ins.size(), B.k, B.sum ? 1 : 0});
       V.entries += 1 << o.rank();
-      for (int t : B.inputs) {
+      int nv = 0;
+      std::vector<int> in_order = bucket_inputs(prog, B, &nv);
+      std::rotate(in_order.begin(), in_order.begin() + nv, in_order.end());  // as k_bucket multiplies them
+      for (int t : in_order) {
         const PTensor& x = prog.tensors[t];
         SmallIn in;
         std::memset(&in, 0, sizeof(in));
@@ -1840,8 +1889,9 @@ static KParams single_kparams(const tnq_plan& P, const Layout& L, const PBucket&
   k.B = L.B;
   k.out_meta = b.output;
   k.out = reinterpret_cast<float2*>((size_t)L.off[b.output] * 8);
+  const std::vector<int> ins = bucket_inputs(prog, b, &k.n_var);
   for (int j = 0; j < b.k; ++j) {
-    const int tid = b.inputs[j];
+    const int tid = ins[j];
     const PTensor& x = prog.tensors[tid];
     k.in[j] = reinterpret_cast<const float2*>((size_t)L.off[tid] * 8);
     k.in_meta[j] = x.leaf_gate >= 0 ? -1 : tid;
@@ -1852,54 +1902,6 @@ static KParams single_kparams(const tnq_plan& P, const Layout& L, const PBucket&
     }
     for (int i = k.out_bits; i < k.G; ++i) k.stride[j][i] = L.dep[tid] ? ((1ll << x.rank()) << (i - k.out_bits)) : 0;
   }
-  // the input with the most distinct entries per block (then the largest)
-  // first, among those that vary with output bits 0-7: k_bucket loads input 0
-  // several iterations ahead. The choice depends on the bucket alone (not on
-  // the batch size or on which variables make an input item-dependent), so
-  // every configuration multiplies in the same order.
-  {
-    auto weight = [&](int j) {  // (-1: constant over output bits 0-7; else output bits 0-11 it varies with, rank)
-      int w8 = 0, w = 0, rank = 0;
-      for (int i = 0; i < k.out_bits; ++i) {
-        const bool nz = k.stride[j][i] != 0;
-        w8 += (i < 8) && nz;
-        w += (i < 12) && nz;
-        rank += nz;
-      }
-      return w8 ? std::make_pair(w, rank) : std::make_pair(-1, 0);
-    };
-    int best = 0;
-    for (int j = 1; j < b.k; ++j)
-      if (weight(j) > weight(best)) best = j;
-    if (best != 0 && weight(best).first >= 0) {
-      std::swap(k.in[best], k.in[0]);
-      std::swap(k.in_meta[best], k.in_meta[0]);
-      std::swap(k.in_dep[best], k.in_dep[0]);
-      for (int i = 0; i < GMAX; ++i) std::swap(k.stride[best][i], k.stride[0][i]);
-    }
-  }
-  // inputs that vary with the low 8 bits (a block's threads) first; the others
-  // are the same for every thread of a block's iteration (k_bucket multiplies
-  // them once per block into a constant pair)
-  // (output bits only: whether an input varies with the item bits depends on
-  // the configuration, and the arithmetic order must not)
-  auto varies = [&](int j) {
-    for (int i = 0; i < 8 && i < k.out_bits; ++i)
-      if (k.stride[j][i]) return true;
-    return false;
-  };
-  int nv = 0;
-  for (int j = 0; j < b.k; ++j)
-    if (varies(j)) {
-      if (j != nv) {
-        std::swap(k.in[j], k.in[nv]);
-        std::swap(k.in_meta[j], k.in_meta[nv]);
-        std::swap(k.in_dep[j], k.in_dep[nv]);
-        for (int i = 0; i < GMAX; ++i) std::swap(k.stride[j][i], k.stride[nv][i]);
-      }
-      ++nv;
-    }
-  k.n_var = nv;
   return k;
 }
 

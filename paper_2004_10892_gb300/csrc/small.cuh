@@ -53,7 +53,7 @@ struct SmallOp {
   int out;             // offset of the result
   int first;           // first entry within its level
   int bits;            // output variables
-  int in0, nin;        // inputs, in the order they are multiplied
+  int in0, nin;        // inputs, in the order they are multiplied (k_bucket's, so that both give the same bits)
   int sum;             // 1: sum over bit 0 of every input (Eq. 2), 0: product only
 };
 

@@ -1,0 +1,51 @@
+"""The one-kernel form of a small plan against its launches, bit by bit."""
+import ctypes
+
+import numpy as np
+import pytest
+
+from paper_2004_10892_gb300 import inputs as I
+
+# (rows, cols, depth, seed, plan options): no fused chains, so that every bucket is summed on its own
+CIRCUITS = [
+    (4, 4, 12, 4, {}),
+    (4, 4, 16, 0, dict(min_p=2, max_p=2)),
+    (5, 5, 20, 3, dict(leaf_absorb=0)),
+    (5, 6, 26, 3, dict(max_bag_log2=15, max_p=9)),
+    (6, 6, 20, 4116, dict(max_bag_log2=20, max_p=30, reorder_every=1)),
+]
+
+
+def _steps(tnq_lib, plan):
+    f = tnq_lib.lib().tnq_internal_small
+    f.argtypes = [ctypes.c_void_p, ctypes.c_int]
+    assert f(plan.handle, 2) == 1  # the rule takes the one-kernel form
+    assert f(plan.handle, 0) == 0
+
+
+def _equal(a, b):
+    """Every slice is a product of FP32 tensors in FP64, whose factors are multiplied in another order."""
+    assert np.max(np.abs(a - b)) <= 1e-14 * np.max(np.abs(b))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("case", CIRCUITS, ids=str)
+def test_circuits_have_the_launches_bits(cuda, tnq_lib, case):
+    rows, cols, depth, seed, kw = case
+    circ = I.random_grid_circuit(rows, cols, depth, seed)
+    plan = tnq_lib.Plan(circ, fuse_min_rank=0, **kw)
+    bits = I.random_bitstring(circ.n_qubits, 5)
+    n = min(8, plan.info()["n_slices"])
+    one = tnq_lib.contract_sliced(plan, bits, 0, n, per_slice=True)[1]
+    _steps(tnq_lib, plan)
+    _equal(one, tnq_lib.contract_sliced(plan, bits, 0, n, per_slice=True)[1])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("rows,cols,dim,p", [(3, 3, 2, 0), (4, 4, 3, 1), (4, 5, 5, 2), (5, 5, 3, 3)])
+def test_networks_have_the_launches_bits(cuda, tnq_lib, rows, cols, dim, p):
+    net = I.random_lattice_network(rows, cols, dim, 7)
+    plan = tnq_lib.Plan.from_network(net.dims, net.tensors, min_p=p, max_p=p, fuse_min_rank=0)
+    one = tnq_lib.contract_sliced(plan, None, per_slice=True)[1]
+    _steps(tnq_lib, plan)
+    _equal(one, tnq_lib.contract_sliced(plan, None, per_slice=True)[1])
