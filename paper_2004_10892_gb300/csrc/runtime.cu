@@ -4515,6 +4515,26 @@ static size_t noalloc_table_bytes(const tnq_plan& P, int B) {
          align_up(hoist * sizeof(HoistDev), 256) + align_up(vals * sizeof(float2), 256);
 }
 
+// The one-kernel form in the static scratch, B items a launch: the plan's tables
+// at its front (up again on each call: every call shares it), results, arenas.
+struct NoallocSmall {
+  size_t res, arena, total;
+};
+static NoallocSmall small_noalloc_places(const SmallPlan& S, int B) {
+  NoallocSmall at;
+  at.res = align_up(S.blob.size(), 256);
+  at.arena = align_up(at.res + 16 * (size_t)B, 256);
+  at.total = at.arena + 8 * (size_t)S.args.arena_elems * B;
+  return at;
+}
+
+// Most items (a power of two, at most cap) that fit it; 0: not even one.
+static int small_noalloc_batch(const SmallPlan& S, uint64_t cap) {
+  int B = 0;
+  for (uint64_t b = 1; b <= cap && small_noalloc_places(S, (int)b).total <= NOALLOC_SCRATCH_BYTES; b <<= 1) B = (int)b;
+  return B;
+}
+
 // Host-side configuration of the allocation-free path for batch B, built once
 // per (plan, B) on the plan's device and cached with its other configurations:
 // the same steps, launch shapes and early-bucket levels as the workspace path,
@@ -4596,6 +4616,15 @@ static tnq_status get_noalloc_config(const tnq_plan& P, uint64_t cap, char* scra
 
 extern "C" {
 
+// Internal test hook (not in include/tnq.h; host only): bytes of the static
+// scratch that the one-kernel form takes with `items` items a launch (0: the
+// plan has no such form), and in *batch how many the call runs at once.
+size_t tnq_internal_noalloc_small(const tnq_plan* plan, uint32_t items, uint64_t cap, int32_t* batch) {
+  const SmallPlan* S = small_plan(*plan);
+  *batch = S ? small_noalloc_batch(*S, cap) : 0;
+  return S ? small_noalloc_places(*S, (int)items).total : 0;
+}
+
 tnq_status tnq_contract_sliced_noalloc(const tnq_plan* plan, const uint8_t* bits, uint64_t slice_begin,
                                        uint64_t slice_end, void* stream, double* out_amp, double* out_slice_amps) {
   if (!plan || (!bits && plan->net.n_qubits > 0) || !out_amp) { set_error("NULL argument"); return TNQ_EINVAL; }
@@ -4612,22 +4641,18 @@ tnq_status tnq_contract_sliced_noalloc(const tnq_plan* plan, const uint8_t* bits
   const uint64_t n_items = slice_end - slice_begin;
   uint64_t cap = 1;
   while (cap < n_items && cap < (1ull << MAX_ITEM_BITS)) cap <<= 1;
-  if (const SmallPlan* S = small_plan(*plan)) {
-    // tables at the front of the scratch (up again on each call: every call shares it), results and arenas behind
+  const SmallPlan* S = small_plan(*plan);
+  // (a plan whose tables leave no room for one item goes on below, where it runs step by step or is refused)
+  if (const int B = S ? small_noalloc_batch(*S, cap) : 0) {
     std::lock_guard<std::mutex> lk(plan->dev_mu);
     DeviceState* D = nullptr;
     if ((st = device_state(*plan, &D)) != TNQ_OK || (st = small_occupancy(*S, *D)) != TNQ_OK) return st;
-    const size_t front = align_up(S->blob.size(), 256);
-    int B = 1;
-    while ((uint64_t)B * 2 <= cap &&
-           front + align_up(32 * (size_t)B, 256) + 16 * (size_t)S->args.arena_elems * B <= NOALLOC_SCRATCH_BYTES)
-      B *= 2;
+    const NoallocSmall at = small_noalloc_places(*S, B);
     char* base = reinterpret_cast<char*>(scratch);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     CU(cudaMemcpyAsync(base, S->blob.data(), S->blob.size(), cudaMemcpyHostToDevice, s));
-    return contract_small(*S, *plan, bits, slice_begin, slice_end, B, D->small_resident, base,
-                          base + front + align_up(16 * (size_t)B, 256), nullptr,
-                          reinterpret_cast<double2*>(base + front), s, out_amp, out_slice_amps);
+    return contract_small(*S, *plan, bits, slice_begin, slice_end, B, D->small_resident, base, base + at.arena, nullptr,
+                          reinterpret_cast<double2*>(base + at.res), s, out_amp, out_slice_amps);
   }
   NoallocConfig* NC = nullptr;
   if ((st = get_noalloc_config(*plan, cap, reinterpret_cast<char*>(scratch), &NC)) != TNQ_OK) return st;
