@@ -8,8 +8,9 @@
 namespace tnq {
 
 // Fold table entry e of one operand: the product of its small tensors at u_0 =
-// 0 and 1, starting from (f, 0).
-__device__ __forceinline__ float4 fold_entry(const PairParams& P, const PFold& F, int e, long long item, float f) {
+// 0 and 1, each times its scale, starting from (f, 0).
+__device__ __forceinline__ float4 fold_entry(const PairParams& P, const PFold& F, int e, long long item, float f,
+                                             const float* scale) {
   float2 p0 = make_float2(f, 0.f), p1 = p0;
   for (int j = 0; j < F.n; ++j) {
     const PIn& g = P.gin[F.gin[j]];
@@ -17,8 +18,10 @@ __device__ __forceinline__ float4 fold_entry(const PairParams& P, const PFold& F
 #pragma unroll
     for (int i = 0; i < PF_MAX; ++i)
       if (i < F.nf && ((e >> i) & 1)) q += F.fs[j][i];
-    p0 = cmul(p0, __ldg(q));
-    p1 = cmul(p1, __ldg(q + F.ustride[j]));
+    const float s = scale[F.gin[j]];
+    const float2 v0 = __ldg(q), v1 = __ldg(q + F.ustride[j]);
+    p0 = cmul(p0, make_float2(v0.x * s, v0.y * s));
+    p1 = cmul(p1, make_float2(v1.x * s, v1.y * s));
   }
   return make_float4(p0.x, p0.y, p1.x, p1.y);
 }
@@ -104,7 +107,9 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
   __shared__ const float2* s_src[RING][3];
   __shared__ float2* s_out[RING];
   __shared__ int s_fold[RING][2];
-  __shared__ float s_sc[PIN_MAX];
+  __shared__ float s_sc[PIN_MAX];  // scales of an item's inputs, and their exponents
+  __shared__ int s_m[PIN_MAX];
+  __shared__ float s_mul[2][4];    // per operand: scale of its staged entries; [3]: 1 when none is needed
   __shared__ int s_e[RING][PIN_MAX];
   __shared__ float s_red[PTPB / 32];
   constexpr int NX = 1 << RX, NY = 1 << RY;
@@ -203,7 +208,12 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
       s_fold[slot][w - 4] = v;
     }
   };
-  // exponents, scales and fold tables of an item (every input's power-of-two scale goes into B's table)
+  // Exponents, scales and fold tables of an item. Every input counts with its
+  // own power of two, as in k_bucket: their product would leave FP32's range at
+  // two inputs of 2^-64. A folded tensor's goes into its table, and an operand's
+  // into B's while it is below 2^PAIR_SCALE (no work then: three of them fit the
+  // table's range); beyond, the operand's staged entries are multiplied by it.
+  constexpr int PAIR_SCALE = 20;
   auto item_setup = [&](long long item, int n) {
     if (t < P.n_gin) {
       const PIn& g = P.gin[t];
@@ -215,15 +225,25 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
         e = P.meta_e[row] + m;
       }
       s_sc[t] = f;
+      s_m[t] = m;
       s_e[n % RING][t] = e;
     }
     __syncthreads();
-    if (t < (1 << P.fb.nf)) {
-      float f = 1.f;
-      for (int j = 0; j < P.n_gin; ++j) f *= s_sc[j];
-      s_fb[n & 1][t] = fold_entry(P, P.fb, t, item, f);
+    int in_table = 0;
+    float mul[3] = {1.f, 1.f, 1.f};
+#pragma unroll
+    for (int o = OP0; o < NOP; ++o) {
+      const int j = ops[o]->gin;
+      if (abs(s_m[j]) <= PAIR_SCALE) in_table += s_m[j];
+      else mul[o] = s_sc[j];
     }
-    if (fold_a && t < (1 << P.fa.nf)) s_fa[n & 1][t] = fold_entry(P, P.fa, t, item, 1.f);
+    if (t < (1 << P.fb.nf))
+      s_fb[n & 1][t] = fold_entry(P, P.fb, t, item, __int_as_float((127 - in_table) << 23), s_sc);
+    if (fold_a && t < (1 << P.fa.nf)) s_fa[n & 1][t] = fold_entry(P, P.fa, t, item, 1.f, s_sc);
+    if (t == 0) {
+      for (int o = 0; o < 3; ++o) s_mul[n & 1][o] = mul[o];
+      s_mul[n & 1][3] = mul[0] == 1.f && mul[1] == 1.f && mul[2] == 1.f ? 1.f : 0.f;
+    }
   };
   auto issue = [&](int slot, int chunk, int buf) {
 #pragma unroll
@@ -239,6 +259,23 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
         }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  // multiplies the pairs this thread copied by their operands' scales (out of the ordinary: see item_setup)
+  auto rescale = [&](int buf, int n) {
+#pragma unroll
+    for (int o = OP0; o < NOP; ++o) {
+      const POp& O = *ops[o];
+      const float f = s_mul[n & 1][o];
+      const int at = td[o] ^ (O.base + (buf ? O.size : 0));
+      const int nit = O.ebits > PTB ? 1 << (O.ebits - PTB) : 1;
+      if (f != 1.f && (O.ebits >= PTB || t < (1 << O.ebits))) {
+#pragma unroll 1
+        for (int it = 0; it < nit; ++it) {
+          float4& v = *reinterpret_cast<float4*>(smb + (at ^ s_it[o][it].y));
+          v = make_float4(v.x * f, v.y * f, v.z * f, v.w * f);
+        }
+      }
+    }
   };
   // multiplies the pairs this thread copied by the fold tables
   auto fold = [&](int slot, int chunk, int buf, int n) {
@@ -307,7 +344,9 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
         tile_setup(next, (slot + 1) % RING);
         if (new_item) item_setup(next >> P.n_h, n_item + 1);
       }
+      const bool odd = s_mul[n_item & 1][3] == 0.f;  // (fetched while the copies arrive)
       asm volatile("cp.async.wait_all;" ::: "memory");
+      if (odd) rescale(buf, n_item);
       if constexpr (!ONE) fold(slot, c, buf, n_item);
       __syncthreads();  // the chunk is staged, and every thread is done with the other stage
       if (!last) issue(slot, c + 1, buf ^ 1);
