@@ -214,7 +214,9 @@ tnq_status tnq_plan_buckets(const tnq_plan* plan, int32_t* bag, int32_t* k, int3
 
 /* ---- contraction (GPU) ------------------------------------------------
  * Device bytes of workspace that a call with `batch` items at once needs
- * (batch is rounded up to a power of two). */
+ * (batch is rounded up to a power of two). A small plan, which runs as one
+ * kernel, asks for up to 16 items' room there; in less it runs fewer at once,
+ * or step by step. */
 size_t tnq_plan_workspace_bytes(const tnq_plan* plan, uint32_t batch);
 
 /* tnq_contract_sliced: sum over slices s in [slice_begin, slice_end) of the

@@ -1322,10 +1322,25 @@ size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 constexpr size_t STATUS_OFF = 128;  // of the status word in every workspace
 static_assert(sizeof(BatchHdr) <= STATUS_OFF, "the status word overlaps the batch header");
 
-// What a batch of a small plan keeps in its workspace (below what make_layout
-// asks for): results after the status word, then the items' arenas.
+// What B items of a small plan at once keep in a workspace: results after the
+// status word, then the items' arenas.
 size_t small_res_off() { return 2 * STATUS_OFF; }
 size_t small_arena_off(int B) { return align_up(small_res_off() + 16 * (size_t)B, 256); }
+size_t small_bytes(const SmallPlan* S, int B) { return small_arena_off(B) + 8 * (size_t)small_arena(S) * B; }
+
+// Most items at once, at most cap, in a workspace of ws_bytes. 0 (the plan has
+// no such form, or not even one item fits): the plan runs step by step, which
+// fuses chains and stores what no slice changes once, so it needs less.
+int small_batch(const SmallPlan* S, size_t ws_bytes, uint64_t cap) {
+  if (!S || small_bytes(S, 1) > ws_bytes) return 0;
+  uint64_t lo = 1, hi = cap;
+  while (lo < hi) {
+    const uint64_t mid = (lo + hi + 1) / 2;
+    if (small_bytes(S, (int)mid) <= ws_bytes) lo = mid;
+    else hi = mid - 1;
+  }
+  return (int)lo;
+}
 
 bool tensor_dep(const PTensor& t, int mode) { return t.dep_slice || (mode == 1 && t.dep_bits); }
 
@@ -1436,7 +1451,6 @@ Layout make_layout(const tnq_plan& P, int mode, int B) {
   }
   L.gemm_off = (long long)align_up((size_t)L.arena_elems, 128);
   if (gemm_elems) L.arena_elems = L.gemm_off + gemm_elems;
-  if (const SmallPlan* S = small_plan(P)) L.arena_elems = std::max(L.arena_elems, small_arena(S) * B);
   L.n_words = (P.net.n_qubits + 31) / 32;
   L.n_rows = B + 1;
   size_t o = 0;
@@ -1648,6 +1662,9 @@ constexpr int SMALL_WIDE = 4096;             // a level of more entries is share
 constexpr int SMALL_TENSOR = 11;             // variables of a tensor in shared memory
 constexpr int SMALL_ELEMS = 64 * 1024 / 8;   // shared memory for tensors
 constexpr long long SMALL_ARENA = 1 << 20;   // elements per item in global memory
+// Items at once that a workspace is asked to hold: sixteen clusters of eight
+// fill the device; more items share it in turn, whichever launch they are in.
+constexpr int SMALL_AT_ONCE = 16;
 
 long long small_arena(const SmallPlan* S) { return S->args.arena_elems; }
 
@@ -3414,10 +3431,11 @@ static tnq_status small_tables(const SmallPlan& S, DeviceState& D, const char** 
 
 // tnq_contract_sliced of a small plan, B slices a launch: the header and the
 // bitstring go with the launch, the kernel writes each slice's value to
-// `host_res` (pinned) or, where that is null, to d_res, which is copied; the
-// slices are added here in increasing order. Caller holds dev_mu.
+// `host_res` (pinned) or, where that is null, to d_res, which is copied, N
+// slices (a multiple of B, or all) between two synchronisations; the slices are
+// added here in increasing order. Caller holds dev_mu.
 static tnq_status contract_small(const SmallPlan& S, const tnq_plan& P, const uint8_t* bits, uint64_t begin,
-                                 uint64_t end, int B, const int* resident, const char* tables, char* arena,
+                                 uint64_t end, int B, int N, const int* resident, const char* tables, char* arena,
                                  double2* host_res, double2* d_res, cudaStream_t s, double* out_amp,
                                  double* out_slice_amps) {
   double2* dst = d_res;
@@ -3425,13 +3443,17 @@ static tnq_status contract_small(const SmallPlan& S, const tnq_plan& P, const ui
   SmallArgs A = small_args(S, tables, arena, dst);
   for (int q = 0; q < P.net.n_qubits; ++q)
     if (bits[q]) A.words[q >> 5] |= 1u << (q & 31);
-  std::vector<double2> copy(host_res ? 0 : B);
+  std::vector<double2> copy(host_res ? 0 : N);
   const double2* res = host_res ? host_res : copy.data();
   double re = 0, im = 0;
-  for (uint64_t base = begin; base < end; base += B) {
-    const int n = (int)std::min<uint64_t>(B, end - base);
-    A.item_base = base;
-    CU(small_launch(A, n, small_cluster(S, resident, n), s));
+  for (uint64_t base = begin; base < end; base += N) {
+    const int n = (int)std::min<uint64_t>(N, end - base);
+    for (int i = 0; i < n; i += B) {  // (on one stream: the next launch may use the same arenas)
+      const int m = std::min(B, n - i);
+      A.item_base = base + i;
+      A.res = dst + i;
+      CU(small_launch(A, m, small_cluster(S, resident, m), s));
+    }
     if (!host_res) CU(cudaMemcpyAsync(copy.data(), d_res, (size_t)n * 16, cudaMemcpyDeviceToHost, s));
     CU(cudaStreamSynchronize(s));
     for (int i = 0; i < n; ++i) {
@@ -3534,10 +3556,6 @@ int tnq_internal_validate(const tnq_plan* plan, int mode, uint32_t batch, char* 
 // plan is shared, as tnq_plan_keep_chains.
 int tnq_internal_small(tnq_plan* plan, int use) {
   plan->small_mode = use == 0 ? SMALL_OFF : (use == 1 ? SMALL_ON : SMALL_RULE);
-  {
-    std::lock_guard<std::mutex> lk(plan->layout_mu);
-    plan->layout_bytes.clear();
-  }
   reset_device_state(*plan);
   return small_plan(*plan) ? 1 : 0;
 }
@@ -4134,7 +4152,10 @@ size_t tnq_plan_workspace_bytes(const tnq_plan* plan, uint32_t batch) {
   if (!plan) return 0;
   uint32_t B = 1;
   while (B < batch && B < (1u << MAX_ITEM_BITS)) B <<= 1;
-  return std::max(layout_bytes(*plan, 0, (int)B), layout_bytes(*plan, 1, (int)B));
+  // (a plan in its one-kernel form wants room for SMALL_AT_ONCE items at the most, and runs in less)
+  const SmallPlan* S = small_plan(*plan);
+  return std::max({layout_bytes(*plan, 0, (int)B), layout_bytes(*plan, 1, (int)B),
+                   S ? small_bytes(S, std::min<int>((int)B, SMALL_AT_ONCE)) : 0});
 }
 
 tnq_status tnq_contract_sliced(const tnq_plan* plan, const uint8_t* bits, uint64_t slice_begin, uint64_t slice_end,
@@ -4158,20 +4179,24 @@ tnq_status tnq_contract_sliced(const tnq_plan* plan, const uint8_t* bits, uint64
   if (B == 0) { set_error("workspace too small for one slice"); return TNQ_ENOMEM; }
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   char* ws = reinterpret_cast<char*>(workspace);
-  if (const SmallPlan* S = small_plan(*plan)) {
+  const SmallPlan* S = small_plan(*plan);
+  if (const int n = small_batch(S, ws_bytes, cap)) {
     std::lock_guard<std::mutex> lk(plan->dev_mu);  // the result buffer is the plan's
     DeviceState* D = nullptr;
     const char* tables = nullptr;
     if ((st = device_state(*plan, &D)) != TNQ_OK || (st = small_tables(*S, *D, &tables)) != TNQ_OK) return st;
-    if (D->h_res_n < B) {
+    // results of up to 2^16 slices (1 MiB) between two synchronisations
+    const int all = (int)std::min<uint64_t>(n_items, 1ull << MAX_ITEM_BITS), N = all <= n ? n : all / n * n;
+    if (D->h_res_n < N) {
       if (D->h_res) cudaFreeHost(D->h_res);
       D->h_res = nullptr;
       D->h_res_n = 0;
-      CU(cudaHostAlloc(reinterpret_cast<void**>(&D->h_res), (size_t)B * 16, cudaHostAllocMapped));
-      D->h_res_n = B;
+      const int room = std::min(1 << MAX_ITEM_BITS, 2 << ilog2_floor(N));
+      CU(cudaHostAlloc(reinterpret_cast<void**>(&D->h_res), (size_t)room * 16, cudaHostAllocMapped));
+      D->h_res_n = room;
     }
-    return contract_small(*S, *plan, bits, slice_begin, slice_end, B, D->small_resident, tables, ws, D->h_res,
-                          nullptr, s, out_amp, out_slice_amps);
+    return contract_small(*S, *plan, bits, slice_begin, slice_end, n, N, D->small_resident, tables,
+                          ws + small_arena_off(n), D->h_res, nullptr, s, out_amp, out_slice_amps);
   }
   ExecConfig* C = nullptr;
   if ((st = get_config(*plan, 0, B, &C)) != TNQ_OK) return st;
@@ -4264,13 +4289,17 @@ tnq_status tnq_amplitudes_batch(const tnq_plan* const* plans, size_t n_plans, co
   std::vector<Job> jobs;
   int n_lanes = 0;
   size_t region = 0;
-  // batch size of plan i in a lane of `reg` bytes, and the staging bytes
-  // (headers and bitstring words of every batch) that choice needs
-  auto batch_of = [&](size_t i, size_t reg) {
+  // batch size of plan i in a lane of `reg` bytes (its one-kernel form's if
+  // `one`), and the staging bytes (headers and bitstring words of every batch)
+  // that choice needs
+  bool one_kernel = true;
+  auto batch_of = [&](size_t i, size_t reg, bool* one = nullptr) {
     const uint64_t n_items = (uint64_t)(bits_offset[i + 1] - bits_offset[i]) << plans[i]->mu.size();
     uint64_t cap = 1;
     while (cap < n_items && cap < (1ull << MAX_ITEM_BITS)) cap <<= 1;
-    return pick_batch(*plans[i], 1, reg, cap);
+    const int n = one_kernel ? small_batch(small_plan(*plans[i]), reg, cap) : 0;
+    if (one) *one = n > 0;
+    return n ? n : pick_batch(*plans[i], 1, reg, cap);
   };
   auto staging = [&](size_t reg) {
     size_t nh = 0, nw = 0;
@@ -4284,23 +4313,27 @@ tnq_status tnq_amplitudes_batch(const tnq_plan* const* plans, size_t n_plans, co
     }
     return align_up(nh * sizeof(BatchHdr), 256) + align_up(nw * 4 + 4, 256);
   };
-  for (int K = std::min(N_LANES, n_distinct); K >= 1 && !n_lanes; --K) {
-    // the lanes take what the staging area and the accumulators leave; the
-    // staging area depends on the batch sizes, which depend on the lane size
-    size_t stage = 0;
-    for (int iter = 0; iter < 8; ++iter) {
-      if (ws_bytes < tail_bytes + stage + 256 * (size_t)K) break;
-      region = (ws_bytes - tail_bytes - stage) / K / 256 * 256;
-      bool fits = true;
-      for (size_t i = 0; i < n_plans && fits; ++i)
-        if (lane_of[i] >= 0 && batch_of(i, region) == 0) fits = false;
-      if (!fits) break;
-      const size_t need = staging(region);
-      if ((size_t)K * region + need + tail_bytes <= ws_bytes) {
-        n_lanes = K;
-        break;
+  // (at the last without the one-kernel form, whose smaller batches need more staging)
+  for (int pass = 0; pass < 2 && !n_lanes; ++pass) {
+    one_kernel = pass == 0;
+    for (int K = std::min(N_LANES, n_distinct); K >= 1 && !n_lanes; --K) {
+      // the lanes take what the staging area and the accumulators leave; the
+      // staging area depends on the batch sizes, which depend on the lane size
+      size_t stage = 0;
+      for (int iter = 0; iter < 8; ++iter) {
+        if (ws_bytes < tail_bytes + stage + 256 * (size_t)K) break;
+        region = (ws_bytes - tail_bytes - stage) / K / 256 * 256;
+        bool fits = true;
+        for (size_t i = 0; i < n_plans && fits; ++i)
+          if (lane_of[i] >= 0 && batch_of(i, region) == 0) fits = false;
+        if (!fits) break;
+        const size_t need = staging(region);
+        if ((size_t)K * region + need + tail_bytes <= ws_bytes) {
+          n_lanes = K;
+          break;
+        }
+        stage = need;
       }
-      stage = need;
     }
   }
   if (n_lanes == 0) { set_error("workspace too small for one item of some plan"); return TNQ_ENOMEM; }
@@ -4320,13 +4353,12 @@ tnq_status tnq_amplitudes_batch(const tnq_plan* const* plans, size_t n_plans, co
       if (nb == 0) continue;
       const int p = (int)P.mu.size();
       const uint64_t n_items = (uint64_t)nb << p;
-      uint64_t cap = 1;
-      while (cap < n_items && cap < (1ull << MAX_ITEM_BITS)) cap <<= 1;
-      const int B = pick_batch(P, 1, region, cap);
+      bool one = false;
+      const int B = batch_of(pi, region, &one);
       ExecConfig* C = nullptr;
       const char* tables = nullptr;
       const int* resident = nullptr;
-      const SmallPlan* S = small_plan(P);
+      const SmallPlan* S = one ? small_plan(P) : nullptr;
       if (S) {
         std::lock_guard<std::mutex> lk(P.dev_mu);
         DeviceState* D = nullptr;
@@ -4651,8 +4683,8 @@ tnq_status tnq_contract_sliced_noalloc(const tnq_plan* plan, const uint8_t* bits
     char* base = reinterpret_cast<char*>(scratch);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     CU(cudaMemcpyAsync(base, S->blob.data(), S->blob.size(), cudaMemcpyHostToDevice, s));
-    return contract_small(*S, *plan, bits, slice_begin, slice_end, B, D->small_resident, base, base + at.arena, nullptr,
-                          reinterpret_cast<double2*>(base + at.res), s, out_amp, out_slice_amps);
+    return contract_small(*S, *plan, bits, slice_begin, slice_end, B, B, D->small_resident, base, base + at.arena,
+                          nullptr, reinterpret_cast<double2*>(base + at.res), s, out_amp, out_slice_amps);
   }
   NoallocConfig* NC = nullptr;
   if ((st = get_noalloc_config(*plan, cap, reinterpret_cast<char*>(scratch), &NC)) != TNQ_OK) return st;
