@@ -1638,11 +1638,10 @@ static std::vector<int> bucket_inputs(const Program& prog, const PBucket& b, int
 // One-kernel form of a small plan (k_small, small.cuh): every bucket of the
 // program -- fused chains and GEMM chains bucket by bucket -- in levels.
 //
-// Which plans: those whose whole slice is a few ten million operations. Below
-// that the launches are what a slice costs (6x6 d1+24+1, 16 slices: 36
+// Which plans have it: those whose whole slice is a few ten million operations.
+// Below that the launches are what a slice costs (6x6 d1+24+1, 16 slices: 36
 // dependent launches, 0.28 ms for 0.06 GFLOP); above it a cluster of eight SMs
-// is slower than a launch on all of them. The rule looks at the plan alone, so
-// that a slice has the same value in a batch of any size.
+// is slower than a launch on all of them. Which of these take it: small_wanted.
 struct SmallPlan {
   bool ok = false;
   SmallArgs args;          // counts and scales; pointers are set per call
@@ -1656,7 +1655,7 @@ struct SmallPlan {
 // eight SMs then need 100 us and more for the arithmetic alone). Levels above
 // 2^10 or 2^14 entries over the cluster: 639 / 298 and 653 / 314, and 160 / 163
 // / 184 us (2^10, 2^12, 2^14) for 16 slices of 6x6 depth 24.
-constexpr double SMALL_FLOPS = 1 << 25;      // per slice
+constexpr double SMALL_FLOPS = 1 << 25;      // per slice, for plans that have this form
 constexpr int SMALL_BITS = 20;               // variables of a bucket's result
 constexpr int SMALL_WIDE = 4096;             // a level of more entries is shared by the cluster
 constexpr int SMALL_TENSOR = 11;             // variables of a tensor in shared memory
@@ -1847,11 +1846,34 @@ static void build_small(const tnq_plan& P, SmallPlan& S) {
   S.ok = small_smem(A) <= SMALL_SMEM_MAX && A.n_words <= SMALL_WORDS;
 }
 
-// Plans whose GEMM chains run in 3xBF16 keep their launches: a slice's value is
-// that of the precision asked for (13 such requests moved by 3e-6 to 1.6e-5
-// in FP32). 3xTF32 keeps all but two of FP32's bits: its values move by 1e-6.
+// Which plans take the one-kernel form. Few items at once are bound by latency,
+// where it wins; many by the arithmetic, which it does entry by entry, with
+// every item's arena out of L2, where the launches share what does not depend
+// on the item and tile their products. The rule looks at the plan alone, so
+// that a slice has the same value in every call: its slices are known, its
+// bitstrings are not, and a network has none. The lines lie where thousands of
+// items take as long as they did before there was this form. Microseconds of a
+// call, GB300, launches before k_pair / launches / one kernel (log2 flops a
+// slice, log2 slices; items are bitstrings times slices):
+//   20.6, 10   16 slices 295 / 259 / 139   256 441 / 369 / 243   1024 1022 / 797 / 713
+//   23.0, 6    64 slices 399 / 353 / 601
+//   23.4, 12   16 slices 324 / 283 / 216   1024 2943 / 1508 / 4088
+//   22.0, 0    16 items 285 / 293 / 201   128 553 / 506 / 388   1024 2542 / 2195 / 2285
+//   22.4, 1    64 items 367 / 330 / 257   1024 2115 / 1710 / 2022   4096 7588 / 5985 / 7496
+//   22.9, 1    64 items 389 / 333 / 286   1024 2030 / 1402 / 2504   4096 6975 / 4569 / 9480
+//   23.8, 4    64 items 517 / 381 / 371   1024 3186 / 1824 / 3647
+//   24.9, 2    a network's 4 slices 379 / 342 / 296
+constexpr int SMALL_P = 4;                    // few slices: at most 2^this
+constexpr double SMALL_FLOPS_BITS = 6e6;      // few slices, any number of bitstrings: 2^22.5
+constexpr double SMALL_FLOPS_MANY = 1 << 21;  // more slices
 static bool small_wanted(const tnq_plan& P) {
   if (P.small_mode != SMALL_RULE) return P.small_mode == SMALL_ON;
+  const double line =
+      (int)P.mu.size() > SMALL_P ? SMALL_FLOPS_MANY : (P.net.n_qubits > 0 ? SMALL_FLOPS_BITS : SMALL_FLOPS);
+  if (P.prog.flops_per_slice > line) return false;
+  // Plans whose GEMM chains run in 3xBF16 keep their launches: a slice's value
+  // is that of the precision asked for (13 such requests moved by 3e-6 to 1.6e-5
+  // in FP32). 3xTF32 keeps all but two of FP32's bits: its values move by 1e-6.
   if (P.opts.precision != TNQ_PREC_SPLIT_BF16) return true;
   return std::none_of(P.prog.groups.begin(), P.prog.groups.end(), [](const FusedGroup& g) { return g.gemm; });
 }

@@ -16,11 +16,11 @@ CIRCUITS = [
 ]
 
 
-def _steps(tnq_lib, plan):
+def _form(tnq_lib, plan, use):
+    """1: one kernel, 0: its launches."""
     f = tnq_lib.lib().tnq_internal_small
     f.argtypes = [ctypes.c_void_p, ctypes.c_int]
-    assert f(plan.handle, 2) == 1  # the rule takes the one-kernel form
-    assert f(plan.handle, 0) == 0
+    assert f(plan.handle, use) == use
 
 
 def _equal(a, b):
@@ -36,8 +36,9 @@ def test_circuits_have_the_launches_bits(cuda, tnq_lib, case):
     plan = tnq_lib.Plan(circ, fuse_min_rank=0, **kw)
     bits = I.random_bitstring(circ.n_qubits, 5)
     n = min(8, plan.info()["n_slices"])
+    _form(tnq_lib, plan, 1)
     one = tnq_lib.contract_sliced(plan, bits, 0, n, per_slice=True)[1]
-    _steps(tnq_lib, plan)
+    _form(tnq_lib, plan, 0)
     _equal(one, tnq_lib.contract_sliced(plan, bits, 0, n, per_slice=True)[1])
 
 
@@ -46,6 +47,7 @@ def test_circuits_have_the_launches_bits(cuda, tnq_lib, case):
 def test_networks_have_the_launches_bits(cuda, tnq_lib, rows, cols, dim, p):
     net = I.random_lattice_network(rows, cols, dim, 7)
     plan = tnq_lib.Plan.from_network(net.dims, net.tensors, min_p=p, max_p=p, fuse_min_rank=0)
+    _form(tnq_lib, plan, 1)
     one = tnq_lib.contract_sliced(plan, None, per_slice=True)[1]
-    _steps(tnq_lib, plan)
+    _form(tnq_lib, plan, 0)
     _equal(one, tnq_lib.contract_sliced(plan, None, per_slice=True)[1])

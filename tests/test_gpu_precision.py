@@ -26,6 +26,11 @@ def _small(tnq_lib, plan, use):
     return f(plan.handle, use)
 
 
+def _few(plan):
+    """What the rule takes in complex64."""
+    return plan.info()["flops_per_slice"] <= 6e6
+
+
 @pytest.mark.parametrize("case", SMALL, ids=str)
 def test_gemm_chains_in_bf16_keep_their_launches(tnq_lib, case):
     _, plan = _plan(tnq_lib, case, tnq_lib.PREC_SPLIT_BF16)
@@ -33,9 +38,9 @@ def test_gemm_chains_in_bf16_keep_their_launches(tnq_lib, case):
     assert _small(tnq_lib, plan, 1) == 1  # it has a one-kernel form,
     assert _small(tnq_lib, plan, 2) == 0  # which the rule does not take
     plan.keep_chains([])  # without GEMM chains every product is FP32
-    assert plan.info()["n_gemm_buckets"] == 0 and _small(tnq_lib, plan, 2) == 1
+    assert plan.info()["n_gemm_buckets"] == 0 and _small(tnq_lib, plan, 2) == _few(plan)
     _, plan = _plan(tnq_lib, case, tnq_lib.PREC_C64)
-    assert _small(tnq_lib, plan, 2) == 1
+    assert _small(tnq_lib, plan, 2) == _few(plan)
 
 
 @pytest.mark.gpu

@@ -19,7 +19,9 @@ CASES = [
 def _plan(tnq_lib, case):
     rows, cols, depth, seed, kw = case
     circ = I.random_grid_circuit(rows, cols, depth, seed)
-    return circ, tnq_lib.Plan(circ, **kw)
+    plan = tnq_lib.Plan(circ, **kw)
+    assert _small(tnq_lib, plan, 1) == 1
+    return circ, plan
 
 
 def _small(tnq_lib, plan, use):
@@ -37,7 +39,6 @@ def _steps_bytes(tnq_lib, case, batch):
 @pytest.mark.parametrize("case", CASES, ids=str)
 def test_sizes(tnq_lib, case):
     plan = _plan(tnq_lib, case)[1]
-    assert _small(tnq_lib, plan, 2) == 1
     for batch in (1, 2, 8, 16, 64, 512, 1 << 14):
         steps, got = _steps_bytes(tnq_lib, case, batch), plan.workspace_bytes(batch)
         assert steps <= got <= max(steps, min(batch, 16) * (8 * MB + 1024))
