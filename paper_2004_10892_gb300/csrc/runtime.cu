@@ -17,6 +17,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -1403,6 +1404,35 @@ Liveness layout_liveness(const Program& prog, const std::vector<int>& hoist) {
   return LV;
 }
 
+// Places tensors of given lifetimes in one address range: each at the lowest
+// offset where no placed one that is alive at the same time lies.
+class Places {
+  struct Tensor {
+    long long off, end;
+    int lo, hi;
+  };
+  std::vector<Tensor> by_off;
+
+ public:
+  long long used = 0;
+  // The tensor's offset; -1 (and nothing placed) if it would end above `most`.
+  long long put(long long size, int lo, int hi, long long most = LLONG_MAX) {
+    long long at = 0;
+    for (const Tensor& t : by_off) {
+      if (t.lo > hi || lo > t.hi) continue;
+      if (at + size <= t.off) break;
+      at = std::max(at, t.end);
+    }
+    if (at > most - size) return -1;
+    const Tensor t{at, at + size, lo, hi};
+    by_off.insert(std::upper_bound(by_off.begin(), by_off.end(), t,
+                                   [](const Tensor& a, const Tensor& b) { return a.off < b.off; }),
+                  t);
+    used = std::max(used, t.end);
+    return at;
+  }
+};
+
 Layout make_layout(const tnq_plan& P, int mode, int B) {
   const Program& prog = P.prog;
   Layout L;
@@ -1426,22 +1456,9 @@ Layout make_layout(const tnq_plan& P, int mode, int B) {
   for (int t = 0; t < T; ++t)
     if (!LV.internal[t]) idx.push_back(t);
   std::stable_sort(idx.begin(), idx.end(), [&](int a, int b) { return size[a] > size[b]; });
-  std::vector<int> placed;
-  for (int t : idx) {
-    // lowest offset not overlapping a placed tensor with an intersecting lifetime
-    std::vector<std::pair<long long, long long>> busy;
-    for (int o : placed)
-      if (lo[o] <= hi[t] && lo[t] <= hi[o]) busy.push_back({L.off[o], L.off[o] + size[o]});
-    std::sort(busy.begin(), busy.end());
-    long long cand = 0;
-    for (auto& iv : busy) {
-      if (cand + size[t] <= iv.first) break;
-      cand = std::max(cand, iv.second);
-    }
-    L.off[t] = cand;
-    L.arena_elems = std::max(L.arena_elems, cand + size[t]);
-    placed.push_back(t);
-  }
+  Places places;
+  for (int t : idx) L.off[t] = places.put(size[t], lo[t], hi[t]);
+  L.arena_elems = places.used;
   // GEMM operand scratch (shared by every GEMM step): hi/lo of both operands
   long long gemm_elems = 0;
   for (const FusedGroup& g : prog.groups) {
@@ -1706,25 +1723,12 @@ static void build_small(const tnq_plan& P, SmallPlan& S) {
   }
   std::stable_sort(idx.begin(), idx.end(),
                    [&](int a, int b) { return prog.tensors[a].rank() > prog.tensors[b].rank(); });
-  long long used[2] = {0, 0};
-  std::vector<int> placed[2];
+  Places places[2];
   auto place = [&](int t, int where) {
-    const long long size = std::max(4ll, 1ll << prog.tensors[t].rank());
-    std::vector<std::pair<long long, long long>> busy;
-    for (int o : placed[where])
-      if (lo[o] <= hi[t] && lo[t] <= hi[o])
-        busy.push_back({off[o], off[o] + std::max(4ll, 1ll << prog.tensors[o].rank())});
-    std::sort(busy.begin(), busy.end());
-    long long c = 0;
-    for (auto& iv : busy) {
-      if (c + size <= iv.first) break;
-      c = std::max(c, iv.second);
-    }
-    if (c + size > (where ? (long long)SMALL_ELEMS : SMALL_ARENA)) return false;
-    off[t] = (int)c;
-    used[where] = std::max(used[where], c + size);
-    placed[where].push_back(t);
-    return true;
+    const long long at = places[where].put(std::max(4ll, 1ll << prog.tensors[t].rank()), lo[t], hi[t],
+                                           where ? (long long)SMALL_ELEMS : SMALL_ARENA);
+    off[t] = (int)at;
+    return at >= 0;
   };
   for (int pass = 0; pass < 2; ++pass)  // the smallest tensors have the most readers per byte: shared memory first
     for (int i = 0; i < T; ++i) {
@@ -1836,8 +1840,8 @@ static void build_small(const tnq_plan& P, SmallPlan& S) {
   A.n_scalars = (int)scalars.size();
   A.n_inout = (int)P.net.inout_qubits.size();
   A.n_finals = (int)finals.size();
-  A.smem_elems = (int)align_up((size_t)used[1], 2);
-  A.arena_elems = (long long)align_up((size_t)used[0], 32);
+  A.smem_elems = (int)align_up((size_t)places[1].used, 2);
+  A.arena_elems = (long long)align_up((size_t)places[0].used, 32);
   A.p = (int)P.mu.size();
   A.n_words = (P.net.n_qubits + 31) / 32;
   const long long le = std::max<long long>(-100000, std::min<long long>(100000, P.net.leaf_exp));
