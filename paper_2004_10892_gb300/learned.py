@@ -16,6 +16,7 @@ import numpy as np
 from . import tnq
 
 HIDDEN = 128
+GATHER = 64  # batches whose rows train() gathers at once
 TRAINED = os.path.join(os.path.dirname(os.path.abspath(__file__)), "data", "proposer_h128.npy")
 
 
@@ -112,7 +113,9 @@ def train(X, y, epochs: int = 200, batch: int = 1024, lr: float = 0.05, mu: floa
     grads = torch.empty_like(params)
     n = Xd.shape[0]
     b = min(batch, n)
-    losses = torch.zeros(max(1, n // b), dtype=torch.float32, device="cuda")  # one per step, read once an epoch
+    steps = n // max(b, 1)
+    losses = torch.zeros(max(1, steps), dtype=torch.float32, device="cuda")  # one per step, read once an epoch
+    xp, yp = (torch.empty((min(steps, GATHER) * b,) + t.shape[1:], dtype=t.dtype, device="cuda") for t in (Xd, yd))
     work = torch.empty(L.tnq_mlp_workspace_floats(hidden, b), dtype=torch.float32, device="cuda")
     g = torch.Generator(device="cpu").manual_seed(seed)
     hist = []
@@ -120,11 +123,14 @@ def train(X, y, epochs: int = 200, batch: int = 1024, lr: float = 0.05, mu: floa
     pp, pg, pm, pw, count = _dptr(params), _dptr(grads), _dptr(mom), _dptr(work), params.numel()
     for ep in range(epochs):
         perm = torch.randperm(n, generator=g).cuda()
-        xp, yp = Xd.index_select(0, perm), yd.index_select(0, perm)  # the epoch's batches, one after the other
-        for k, i in enumerate(range(0, n - b + 1, b)):
-            tnq._check(L.tnq_mlp_backward(pp, hidden, _at(xp, i * xp.shape[1]), _at(yp, i), b, pg, _at(losses, k), pw,
-                                          st))
-            tnq._check(L.tnq_mlp_sgd(pp, pg, pm, count, lr, mu, st))
+        for first in range(0, n - b + 1, GATHER * b):  # the rows of the next batches, one after the other
+            rows = perm[first:min(first + GATHER * b, steps * b)]
+            torch.index_select(Xd, 0, rows, out=xp[:len(rows)])
+            torch.index_select(yd, 0, rows, out=yp[:len(rows)])
+            for k in range(len(rows) // b):
+                tnq._check(L.tnq_mlp_backward(pp, hidden, _at(xp, k * b * xp.shape[1]), _at(yp, k * b), b, pg,
+                                              _at(losses, first // b + k), pw, st))
+                tnq._check(L.tnq_mlp_sgd(pp, pg, pm, count, lr, mu, st))
         hist.append(sum(losses.tolist(), 0.0) / max(1, n // b))
     return params.cpu().numpy(), hist
 
