@@ -81,10 +81,14 @@ __device__ __forceinline__ float4 both(F f, float4 v, float sign = 1.f) {  // f 
 //  * two tensors: the FMA pipe (78 TFLOP/s measured). 5 buckets, bag 28, 32
 //    items: 12.9 -> 1.97 ms, 72 TFLOP/s.
 //  * three: issue slots (68 % busy, 62 % of them FMAs; 128 registers hold two
-//    blocks an SM) and the reads of C, each used once. 3 buckets, bag 28, 64
-//    items: 19.9 -> 5.53 ms, 36 TFLOP/s.
-//  * one: memory. A bucket of bag 23, 32 items: 4.0 -> 5.6 TB/s (k_bucket
-//    before); 5 buckets, bag 22: 3.5 -> 5.1 TB/s of a copy's 6.8.
+//    blocks an SM, and three of the 4 x 8 forms with C spill 5 to 41 words to
+//    fit them) and the reads of C, each used once. 3 buckets, bag 28, 64 items:
+//    19.9 -> 5.57 ms, 36 TFLOP/s.
+//  * one: memory. A bucket of bag 23, 32 items: 4.0 -> 5.5 TB/s (k_bucket
+//    before); 5 buckets, bag 22: 3.5 -> 5.2 TB/s of a copy's 6.8.
+//  * 3xBF16 chains of mostly padding: memory too; eight instructions a value
+//    for its low part. One row, 64 columns, K = 32, bag 25, 8 items: 4.11 (the
+//    padded GEMM) -> 0.66 ms, 0.49 in plain FP32.
 // Slower: register double buffering by halves of a pair (8-byte reads at a
 // 16-byte stride cost twice the cycles, 2.28 -> 2.85 ms on the first); no
 // faster: three or four stages.
@@ -213,7 +217,8 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
   // two inputs of 2^-64. A folded tensor's goes into its table, and an operand's
   // into B's while it is below 2^PAIR_SCALE (no work then: three of them fit the
   // table's range); beyond, the operand's staged entries are multiplied by it.
-  constexpr int PAIR_SCALE = 20;
+  // One operand alone keeps its scale in the table, up to 2^PAIR_ONE.
+  constexpr int PAIR_SCALE = 20, PAIR_ONE = 100;
   auto item_setup = [&](long long item, int n) {
     if (t < P.n_gin) {
       const PIn& g = P.gin[t];
@@ -222,6 +227,7 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
       if (g.meta >= 0) {
         const long long row = (long long)g.meta * P.B + (g.dep ? item : 0ll);
         f = scale_of_max(P.meta_m[row], &m);
+        if (ONE && t == P.b.gin) m = max(-PAIR_ONE, min(PAIR_ONE, m));
         e = P.meta_e[row] + m;
       }
       s_sc[t] = f;
@@ -234,7 +240,7 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
 #pragma unroll
     for (int o = OP0; o < NOP; ++o) {
       const int j = ops[o]->gin;
-      if (abs(s_m[j]) <= PAIR_SCALE) in_table += s_m[j];
+      if (ONE || abs(s_m[j]) <= PAIR_SCALE) in_table += s_m[j];
       else mul[o] = s_sc[j];
     }
     if (t < (1 << P.fb.nf))
@@ -344,7 +350,7 @@ __global__ void __launch_bounds__(PTPB, 2) k_pair(const __grid_constant__ PairPa
         tile_setup(next, (slot + 1) % RING);
         if (new_item) item_setup(next >> P.n_h, n_item + 1);
       }
-      const bool odd = s_mul[n_item & 1][3] == 0.f;  // (fetched while the copies arrive)
+      const bool odd = !ONE && s_mul[n_item & 1][3] == 0.f;  // (fetched while the copies arrive)
       asm volatile("cp.async.wait_all;" ::: "memory");
       if (odd) rescale(buf, n_item);
       if constexpr (!ONE) fold(slot, c, buf, n_item);

@@ -2659,8 +2659,8 @@ static bool gemm_as_pair(const ExecConfig& C, size_t i) {
 // the same sums on the FP32 pipe, 3xTF32 in FP32, which differs from it by 1e-6):
 // at one row an item (padded to 128 or 64 of the MMA tile) the tensor cores do
 // 128 times the work and the operands are packed for it. 8 items of such a
-// chain (25 variables, one row, 64 columns, K = 32; 2.2 GB): 3.96 -> 0.49 ms; 16
-// items of one with 4096 rows and 4 columns (padded to 64): 0.109 -> 0.039 ms.
+// chain (25 variables, one row, 64 columns, K = 32; 2.2 GB): 4.11 -> 0.66 ms; 16
+// items of one with 4096 rows and 4 columns (padded to 64): 0.109 -> 0.051 ms.
 // At a padding of 8 and below the two were not told apart.
 constexpr double PAIR_GEMM_PADDING = 16;
 static double gemm_padding(const FusedGroup& g, const GemmBucketArgs& G) {
