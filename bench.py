@@ -116,33 +116,37 @@ class ClockSampler:
                 "samples": len(sm), "samples_in_timed_region": len(inside)}
 
 
-# ncu DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of every
-# k_pair and k_group launch of a one-slice batch of this workload (capture
-# command in profiles/k_pair_7x7_d1+32+1.md), valid only while the chain kernels'
-# source (pair.cu, and runtime.cu between the "Fused chain of buckets" and "K4:
-# amplitude" comments) hashes to `kernel_sha1` and the plan has the recorded
-# tuning and number of chains (reported as null otherwise). Per launch at batch
-# B: bytes_one_slice x B / launches (traffic scales with the slices of a batch;
-# item-invariant operands are read once per batch, so this slightly overstates
-# it).
+# ncu DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of the chains'
+# launches (k_pair, k_group) of a one-slice batch of this workload (capture
+# command in profiles/k_pair_7x7_d1+32+1.md; the buckets that k_pair runs are not
+# among them), valid only while the source of these kernels and of the rules
+# that choose and shape their launches hashes to `kernel_sha1` and the plan has
+# the recorded tuning and number of chains (reported as null otherwise). Per
+# launch at batch B: bytes_one_slice x B / chains (traffic scales with the slices
+# of a batch; item-invariant operands are read once per batch, so this slightly
+# overstates it).
 MEASURED_TRAFFIC = [
-    {"kernel_sha1": "78232f70757bcf02e3642f6750eae68851d4e32c", "tuning": [4, 64], "chains": 12,
-     "bytes_one_slice": 158943744.0, "launches": 22,
-     "capture": "ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum -k regex:k_pair|k_group, the 22 k_pair "
-                "launches of a one-slice batch of the tuned default plan (tuning 2^4 / 64; 12 chains, 10 buckets)"},
+    {"kernel_sha1": "e259ca0a0b9db863210e8dc426704364deefd292", "tuning": [4, 64], "chains": 12, "bytes_one_slice": 104252928.0,
+     "capture": "ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum -k regex:k_pair|k_group, the 12 chains' "
+                "launches of a one-slice batch of the tuned default plan (tuning 2^4 / 64), without a graph"},
 ]
 
 
 def kernel_source_sha1():
-    """SHA-1 of the chain kernels' source: pair.cu and the region of runtime.cu."""
+    """SHA-1 of the chain kernels' source and of the rules that choose and shape their launches."""
     import hashlib
 
-    with open(os.path.join(ROOT, "paper_2004_10892_gb300", "csrc", "runtime.cu")) as f:
-        text = f.read()
-    a = text.index("// Fused chain of buckets")
-    b = text.index("// K4: amplitude")
-    with open(os.path.join(ROOT, "paper_2004_10892_gb300", "csrc", "pair.cu")) as f:
-        return hashlib.sha1((f.read() + text[a:b]).encode()).hexdigest()
+    def source(name):
+        with open(os.path.join(ROOT, "paper_2004_10892_gb300", "csrc", name)) as f:
+            return f.read()
+
+    text = source("runtime.cu")
+    parts = [source("pair.cu"), source("pair.cuh"), source("device_util.cuh")]
+    for first, last in (("// Fused chain of buckets", "// K4: amplitude"),
+                        ("// A fused chain as k_pair runs it", "// GEMM-step parameters of a GEMM group"),
+                        ("// A GEMM chain whose tiles are mostly padding", "// Host-side check of the one-kernel form")):
+        parts.append(text[text.index(first):text.index(last)])
+    return hashlib.sha1("".join(parts).encode()).hexdigest()
 
 
 # FP32 CUDA-core peak of GB300 from unit counts and clocks: 152 SMs x 128 FP32
@@ -233,8 +237,8 @@ def launch_roofline(L, plan, bits, ws, B, n_sl, stream, peaks, info):
         for mt in MEASURED_TRAFFIC:
             if (mt["kernel_sha1"] == kernel_source_sha1() and mt["tuning"] == list(plan.tuning())
                     and mt["chains"] == len(grp)):
-                out["traffic"] = mt["bytes_one_slice"] * b_out.value / mt["launches"]
-                out["traffic_source"] = mt["capture"] + ", x batch / those launches per batch"
+                out["traffic"] = mt["bytes_one_slice"] * b_out.value / mt["chains"]
+                out["traffic_source"] = mt["capture"] + ", x batch / chains"
     out["peak_source"] = dom.get("peak_source", "measured (MEASURED_PEAKS.json hbm_gbs)")
     out["batch"] = b_out.value
     out["other_kernel"] = other

@@ -1667,7 +1667,8 @@ struct SmallPlan {
   int widest = 1;          // most entries of a level that the whole cluster works on
 };
 // The lines, GB300, twelve small plans in one call / a 6x6 network of
-// three-valued indices (642 to 654 / 303 us): plans above 2^23 flops by
+// three-valued indices (642 to 654 / 303 us where every plan that has the form
+// takes it): plans above 2^23 flops by
 // launches 720 / 372; one kernel up to 2^27 650 / 305 (none lies between; its
 // eight SMs then need 100 us and more for the arithmetic alone). Levels above
 // 2^10 or 2^14 entries over the cluster: 639 / 298 and 653 / 314, and 160 / 163
