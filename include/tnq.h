@@ -89,8 +89,10 @@ typedef enum {
 
 typedef enum {
   TNQ_PREC_C64 = 0,         /* every bucket in complex64 */
-  TNQ_PREC_SPLIT_BF16 = 1,  /* merged GEMM buckets as 3xBF16 tensor-core GEMMs */
-  TNQ_PREC_SPLIT_TF32 = 2   /* merged GEMM buckets as 3xTF32 tensor-core GEMMs */
+  TNQ_PREC_SPLIT_BF16 = 1,  /* merged GEMM buckets as 3xBF16 tensor-core GEMMs (where these would be mostly
+                               padding, the same sums on the FP32 pipe) */
+  TNQ_PREC_SPLIT_TF32 = 2   /* merged GEMM buckets as 3xTF32 tensor-core GEMMs (in FP32, which is no less exact,
+                               where these would be mostly padding and in plans that run as one kernel) */
 } tnq_precision;
 
 typedef enum {
