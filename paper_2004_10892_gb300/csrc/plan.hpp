@@ -41,7 +41,7 @@ struct tnq_plan {
   mutable std::mutex small_mu;
   mutable std::shared_ptr<tnq::SmallPlan> small;  // built on first use, dropped with the program
   tnq::SmallMode small_mode = tnq::SMALL_RULE;    // the other two: internal test hook
-  bool pair_gemm = true;                          // false (internal test hook): every GEMM chain on the tensor cores
+  bool pair_chains = true, pair_gemm = true;      // false (internal test hook): k_pair runs no chain / no GEMM chain
   mutable std::mutex dev_mu;
   mutable tnq::DeviceState* dev = nullptr;
   ~tnq_plan() {

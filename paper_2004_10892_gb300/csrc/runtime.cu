@@ -1685,6 +1685,54 @@ constexpr int SMALL_AT_ONCE = 16;
 
 long long small_arena(const SmallPlan* S) { return S->args.arena_elems; }
 
+static GParams group_gparams(const tnq_plan& P, const Layout& L, const FusedGroup& g, bool* ok, int* smem);
+
+// How k_small multiplies a bucket: its inputs in order, and how many of the
+// first are a product of their own (SmallOp::split). The launches' order, so
+// that both give the same bits: k_bucket's, and k_group's in a chain that is
+// fused (whatever runs it now: k_pair sums a chain in another order).
+struct SmallOrder {
+  std::vector<int> ins;
+  int split = 0;
+};
+static std::vector<SmallOrder> small_orders(const tnq_plan& P) {
+  const Program& prog = P.prog;
+  std::vector<SmallOrder> R(prog.buckets.size());
+  for (size_t b = 0; b < prog.buckets.size(); ++b) {
+    int nv = 0;
+    R[b].ins = bucket_inputs(prog, prog.buckets[b], &nv);
+    std::rotate(R[b].ins.begin(), R[b].ins.begin() + nv, R[b].ins.end());
+  }
+  Layout L;  // (where tensors lie makes no difference)
+  L.off.assign(prog.tensors.size(), 0);
+  L.dep.assign(prog.tensors.size(), 0);
+  for (const FusedGroup& g : prog.groups) {
+    if (g.gemm) continue;
+    bool ok = false;
+    int smem = 0;
+    const GParams G = group_gparams(P, L, g, &ok, &smem);
+    if (!ok) continue;
+    for (int s = 0; s < G.n_st; ++s) {
+      const GSt& S = G.st[s];
+      SmallOrder& O = R[g.buckets[s]];
+      auto input = [&](int j) { return S.src[j] < 0 ? prog.buckets[g.buckets[s - 1]].output : g.ext_inputs[S.src[j]]; };
+      O.ins.clear();
+      if (G.tail && s > 0) {  // (previous stage [times an operand]) times the constants
+        O.split = S.n_var;
+        for (int j = 0; j < S.n_in; ++j) O.ins.push_back(input(j));
+        continue;
+      }
+      // (constants times the varying operands but the last) times the last
+      const int nv = S.n_var - (G.tail || G.lean2 ? S.n_tc : 0);
+      O.split = nv > 0 ? 1 : 0;
+      if (nv > 0) O.ins.push_back(input(nv - 1));
+      for (int j = nv; j < S.n_in; ++j) O.ins.push_back(input(j));
+      for (int j = 0; j + 1 < nv; ++j) O.ins.push_back(input(j));
+    }
+  }
+  return R;
+}
+
 static void build_small(const tnq_plan& P, SmallPlan& S) {
   const Program& prog = P.prog;
   const int nb = (int)prog.buckets.size(), T = (int)prog.tensors.size();
@@ -1743,6 +1791,7 @@ static void build_small(const tnq_plan& P, SmallPlan& S) {
   std::vector<SmallIn> ins;
   std::vector<SmallLevel> levels;
   std::vector<int> op_of(nb, -1);
+  const std::vector<SmallOrder> orders = small_orders(P);
   for (int l = 0; l < n_lv; ++l) {
     std::vector<int> bs;
     for (int b = 0; b < nb; ++b)
@@ -1755,12 +1804,9 @@ static void build_small(const tnq_plan& P, SmallPlan& S) {
       const PBucket& B = prog.buckets[b];
       const PTensor& o = prog.tensors[B.output];
       op_of[b] = (int)ops.size();
-      ops.push_back(SmallOp{where(B.output), V.entries, o.rank(), (int)ins.size(), B.k, B.sum ? 1 : 0});
+      ops.push_back(SmallOp{where(B.output), V.entries, o.rank(), (int)ins.size(), B.k, B.sum ? 1 : 0, orders[b].split});
       V.entries += 1 << o.rank();
-      int nv = 0;
-      std::vector<int> in_order = bucket_inputs(prog, B, &nv);
-      std::rotate(in_order.begin(), in_order.begin() + nv, in_order.end());  // as k_bucket multiplies them
-      for (int t : in_order) {
+      for (int t : orders[b].ins) {
         const PTensor& x = prog.tensors[t];
         SmallIn in;
         std::memset(&in, 0, sizeof(in));
@@ -2721,7 +2767,7 @@ static bool build_steps(const tnq_plan& P, const Layout& L, ExecConfig& C) {
       one.buckets = {(int)bi};
       one.output = prog.buckets[bi].output;
       one.ext_inputs = prog.buckets[bi].inputs;
-      pair_step(one, prog.buckets[bi].sum && !ever_early[bi]);
+      pair_step(one, P.pair_chains && prog.buckets[bi].sum && !ever_early[bi]);
     } else if ((int)bi == prog.groups[gi].buckets.back() && prog.groups[gi].gemm) {
       GemmBucketArgs G;
       GemmEpilogue E;
@@ -2748,7 +2794,7 @@ static bool build_steps(const tnq_plan& P, const Layout& L, ExecConfig& C) {
       C.step_hoist.push_back(0);
       C.gp.push_back(g);
       C.gsmem.push_back(smem);
-      pair_step(prog.groups[gi], true);
+      pair_step(prog.groups[gi], P.pair_chains);
       double by = tbytes(prog.groups[gi].output);
       for (int t : prog.groups[gi].ext_inputs) by += tbytes(t);
       C.step_bytes.push_back(by);
@@ -3587,10 +3633,12 @@ int tnq_internal_small(tnq_plan* plan, int use) {
   return small_plan(*plan) ? 1 : 0;
 }
 
-// Internal test hook (not in include/tnq.h): use = 0 runs GEMM chains of mostly
-// padding on the tensor cores, 1 undoes that. Before the plan is shared.
-void tnq_internal_pair_gemm(tnq_plan* plan, int use) {
-  plan->pair_gemm = use != 0;
+// Internal test hook (not in include/tnq.h): whether k_pair may run buckets and
+// chains (else k_bucket, k_group), and GEMM chains of mostly padding (else the
+// tensor cores). Before the plan is shared.
+void tnq_internal_pair(tnq_plan* plan, int chains, int gemms) {
+  plan->pair_chains = chains != 0;
+  plan->pair_gemm = gemms != 0;
   reset_device_state(*plan);
 }
 
@@ -3855,6 +3903,10 @@ void reset_device_state(const tnq_plan& P) {
       destroy_device_state(P.dev);
       P.dev = nullptr;
     }
+  }
+  {
+    std::lock_guard<std::mutex> lk(P.small_mu);
+    P.small.reset();  // (its products' order is the chains')
   }
   std::lock_guard<std::mutex> lk(P.layout_mu);
   P.layout_bytes.clear();

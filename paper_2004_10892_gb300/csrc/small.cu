@@ -41,12 +41,22 @@ __device__ __forceinline__ float part_max(float2 r) {  // (0 for NaN, as fmaxf a
   return fmaxf(fmaxf(fabsf(r.x), fabsf(r.y)), 0.f);
 }
 
+// sum over u of p_u v_u as k_group takes it
+__device__ __forceinline__ float2 sum_products(float2 p0, float2 p1, float2 v0, float2 v1) {
+  float x = __fmul_rn(p0.x, v0.x), y = __fmul_rn(p0.x, v0.y);
+  x = fmaf(-p0.y, v0.y, x);
+  y = fmaf(p0.y, v0.x, y);
+  x = fmaf(p1.x, v1.x, x);
+  y = fmaf(p1.x, v1.y, y);
+  return make_float2(fmaf(-p1.y, v1.y, x), fmaf(p1.y, v1.x, y));
+}
+
 // One bucket by all threads (t0 of step, a power of two): its inputs looked up
 // once, N entries in flight per thread. Entries b + i step of one b that is
 // aligned to N step differ in the bits of i alone, so their places in an input
 // are the first one's plus the places of those bits. Returns the thread's
 // largest part.
-template <int NIN>
+template <int NIN, int SPLIT>
 __device__ __noinline__ float small_bucket(const SmallOp& op, const SmallIn* ins, float2* out, const float2* sh,
                                               const float2* glob, const unsigned* s_max, unsigned t0, unsigned step) {
   constexpr int N = NIN <= 3 ? 4 : (NIN <= 5 ? 2 : 1);
@@ -64,11 +74,19 @@ __device__ __noinline__ float small_bucket(const SmallOp& op, const SmallIn* ins
   float mx = 0.f;
   auto product = [&](const float4* v) {
     float2 a0 = make_float2(v[0].x * f[0], v[0].y * f[0]), a1 = make_float2(v[0].z * f[0], v[0].w * f[0]);
+    float2 p0 = make_float2(1.f, 0.f), p1 = p0;
 #pragma unroll
     for (int j = 1; j < NIN; ++j) {
-      a0 = cmul(a0, make_float2(v[j].x * f[j], v[j].y * f[j]));
-      a1 = cmul(a1, make_float2(v[j].z * f[j], v[j].w * f[j]));
+      const float2 w0 = make_float2(v[j].x * f[j], v[j].y * f[j]), w1 = make_float2(v[j].z * f[j], v[j].w * f[j]);
+      if (!SPLIT || j < SPLIT) {
+        a0 = cmul(a0, w0);
+        a1 = cmul(a1, w1);
+      } else {
+        p0 = j == SPLIT ? w0 : cmul(p0, w0);
+        p1 = j == SPLIT ? w1 : cmul(p1, w1);
+      }
     }
+    if (SPLIT) return sum_products(p0, p1, a0, a1);
     return op.sum ? make_float2(a0.x + a1.x, a0.y + a1.y) : a0;
   };
   auto load = [&](int j, unsigned c) {
@@ -119,6 +137,7 @@ constexpr int SMALL_IN = 4;  // inputs of a prepared entry
 // up late.
 struct SmallEntry {
   int op, out, grp;                  // op < 0: none
+  int own;                           // inputs of the first product (SmallOp::split; all without one)
   int more;                          // first input that is not prepared (the number of inputs: none)
   int src[SMALL_IN], meta[SMALL_IN];  // tensor offset of the entry in each input, its bucket
 };
@@ -232,7 +251,11 @@ __global__ void __launch_bounds__(STPB, 1) k_small(const __grid_constant__ Small
       const SmallOp op = ops[o];
       float2* out = at(op.out);
       float mx;
-#define SMALL_RUN(n) mx = small_bucket<n>(op, ins, out, sh, glob, maxima, t0, step); break
+#define SMALL_RUN(n)                                                                       \
+  mx = op.split == 0   ? small_bucket<n, 0>(op, ins, out, sh, glob, maxima, t0, step)      \
+       : op.split == 1 ? small_bucket<n, 1>(op, ins, out, sh, glob, maxima, t0, step)      \
+                       : small_bucket<n, n == 1 ? 1 : 2>(op, ins, out, sh, glob, maxima, t0, step); \
+  break
       switch (op.nin) {
         case 1: SMALL_RUN(1);
         case 2: SMALL_RUN(2);
@@ -254,6 +277,7 @@ __global__ void __launch_bounds__(STPB, 1) k_small(const __grid_constant__ Small
     E.op = -1;
     E.out = 0;
     E.grp = 1;
+    E.own = KMAX;
     E.more = KMAX;
 #pragma unroll
     for (int j = 0; j < SMALL_IN; ++j) {
@@ -272,6 +296,7 @@ __global__ void __launch_bounds__(STPB, 1) k_small(const __grid_constant__ Small
     E.op = lo;
     E.out = op.out + (int)b;
     E.grp = 1 << min(op.bits, 5);
+    E.own = op.split ? op.split : KMAX;
     E.more = op.sum ? SMALL_IN : 0;
 #pragma unroll
     for (int j = 0; j < SMALL_IN; ++j)
@@ -293,11 +318,20 @@ __global__ void __launch_bounds__(STPB, 1) k_small(const __grid_constant__ Small
       f[j] = scale_of_max(maxima[E.meta[j]], &m);
     }
     float2 a0 = make_float2(v[0].x * f[0], v[0].y * f[0]), a1 = make_float2(v[0].z * f[0], v[0].w * f[0]);
+    const bool split = __any_sync(0xffffffffu, E.own < KMAX);  // (chains' buckets are mostly larger)
+    float2 p0 = make_float2(1.f, 0.f), p1 = p0;
+    auto times = [&](int j, float2 w0, float2 w1) {
+      if (!split || j < E.own) {
+        a0 = cmul(a0, w0);
+        a1 = cmul(a1, w1);
+      } else {
+        p0 = cmul(p0, w0);
+        p1 = cmul(p1, w1);
+      }
+    };
 #pragma unroll
-    for (int j = 1; j < SMALL_IN; ++j) {
-      a0 = cmul(a0, make_float2(v[j].x * f[j], v[j].y * f[j]));
-      a1 = cmul(a1, make_float2(v[j].z * f[j], v[j].w * f[j]));
-    }
+    for (int j = 1; j < SMALL_IN; ++j)
+      times(j, make_float2(v[j].x * f[j], v[j].y * f[j]), make_float2(v[j].z * f[j], v[j].w * f[j]));
     float mx = 0.f;
     if (E.op >= 0) {
       const SmallOp op = ops[E.op];
@@ -307,10 +341,10 @@ __global__ void __launch_bounds__(STPB, 1) k_small(const __grid_constant__ Small
         const float2* p = at(in.off) + (compress((unsigned)(E.out - op.out), in) << op.sum);
         int m;
         const float g = in.meta < 0 ? 1.f : scale_of_max(maxima[in.meta], &m);
-        a0 = cmul(a0, make_float2(p[0].x * g, p[0].y * g));
-        if (op.sum) a1 = cmul(a1, make_float2(p[1].x * g, p[1].y * g));
+        times(j, make_float2(p[0].x * g, p[0].y * g), op.sum ? make_float2(p[1].x * g, p[1].y * g) : p1);
       }
-      const float2 r = op.sum ? make_float2(a0.x + a1.x, a0.y + a1.y) : a0;
+      float2 r = op.sum ? make_float2(a0.x + a1.x, a0.y + a1.y) : a0;
+      if (split && op.split) r = sum_products(p0, p1, a0, a1);
       *at(E.out) = r;
       mx = part_max(r);
     }

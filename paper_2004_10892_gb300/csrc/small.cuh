@@ -53,8 +53,10 @@ struct SmallOp {
   int out;             // offset of the result
   int first;           // first entry within its level
   int bits;            // output variables
-  int in0, nin;        // inputs, in the order they are multiplied (k_bucket's, so that both give the same bits)
+  int in0, nin;        // inputs, in the order they are multiplied
   int sum;             // 1: sum over bit 0 of every input (Eq. 2), 0: product only
+  int split;           // 0: one product, added over the two values; else the first `split` inputs (one or two) are a
+                       // product of their own, times which the others' is summed by FMAs (k_group's arithmetic)
 };
 
 // Buckets that depend on earlier levels only.

@@ -42,6 +42,38 @@ def test_circuits_have_the_launches_bits(cuda, tnq_lib, case):
     _equal(one, tnq_lib.contract_sliced(plan, bits, 0, n, per_slice=True)[1])
 
 
+# plans whose chains are fused: in k_group's general form, with a register tail, with two lean stages
+CHAINS = [
+    (4, 4, 16, 21, dict(min_p=2, max_p=2, fuse_min_rank=1)),
+    (5, 5, 20, 21, dict(min_p=3, max_p=3, fuse_min_rank=4)),
+    (4, 5, 24, 22, dict(min_p=4, max_p=4, fuse_min_rank=8)),
+    (6, 6, 24, 0, dict(max_bag_log2=24, min_p=4, max_p=8)),
+    (6, 6, 24, 5, dict(max_bag_log2=18, max_p=20, reorder_every=1, fuse_min_rank=8)),
+    (5, 5, 28, 2, dict(min_p=2, max_p=2, reorder_every=1)),
+    (4, 7, 26, 3, dict(max_bag_log2=20, max_p=20, reorder_every=1, fuse_min_rank=6)),
+]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("case", CHAINS, ids=str)
+def test_chains_have_their_kernels_bits(cuda, tnq_lib, case):
+    """k_group's arithmetic, stage by stage (k_pair, off here, sums in another order)."""
+    rows, cols, depth, seed, kw = case
+    circ = I.random_grid_circuit(rows, cols, depth, seed)
+    plan = tnq_lib.Plan(circ, **kw)
+    assert plan.info()["n_fused_groups"] > 0
+    bits = I.random_bitstring(circ.n_qubits, 5)
+    n = min(8, plan.info()["n_slices"])
+    _form(tnq_lib, plan, 1)
+    one = tnq_lib.contract_sliced(plan, bits, 0, n, per_slice=True)[1]
+    _form(tnq_lib, plan, 0)
+    f = tnq_lib.lib().tnq_internal_pair
+    f.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_int]
+    f.restype = None
+    f(plan.handle, 0, 0)
+    _equal(one, tnq_lib.contract_sliced(plan, bits, 0, n, per_slice=True)[1])
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("rows,cols,dim,p", [(3, 3, 2, 0), (4, 4, 3, 1), (4, 5, 5, 2), (5, 5, 3, 3)])
 def test_networks_have_the_launches_bits(cuda, tnq_lib, rows, cols, dim, p):

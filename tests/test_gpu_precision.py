@@ -73,14 +73,14 @@ def test_padded_bf16_chains_give_the_gemm_values(cuda, tnq_lib, case):
     circ, plan = _plan(tnq_lib, case, tnq_lib.PREC_SPLIT_BF16)
     bits = I.random_bitstring(circ.n_qubits, 88)
     n = min(8, plan.info()["n_slices"])
-    f = tnq_lib.lib().tnq_internal_pair_gemm
-    f.argtypes = [ctypes.c_void_p, ctypes.c_int]
+    f = tnq_lib.lib().tnq_internal_pair
+    f.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_int]
     f.restype = None
     launches = tnq_lib.lib().tnq_internal_launches_per_batch
     launches.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_uint32]
     got = tnq_lib.contract_sliced(plan, bits, 0, n, per_slice=True)[1]
     fewer = launches(plan.handle, 0, 1)
-    f(plan.handle, 0)
+    f(plan.handle, 1, 0)
     assert launches(plan.handle, 0, 1) > fewer  # (a GEMM packs its operands first)
     gemm = tnq_lib.contract_sliced(plan, bits, 0, n, per_slice=True)[1]
     assert np.linalg.norm(got - gemm) <= 5e-6 * np.linalg.norm(gemm)
