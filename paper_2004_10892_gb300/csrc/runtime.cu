@@ -1913,7 +1913,7 @@ static void build_small(const tnq_plan& P, SmallPlan& S) {
 //   22.4, 1    64 items 367 / 330 / 257   1024 2115 / 1710 / 2022   4096 7588 / 5985 / 7496
 //   22.9, 1    64 items 389 / 333 / 286   1024 2030 / 1402 / 2504   4096 6975 / 4569 / 9480
 //   23.8, 4    64 items 517 / 381 / 371   1024 3186 / 1824 / 3647
-//   24.9, 2    a network's 4 slices 379 / 342 / 296
+//   24.9, 2    a network's 4 slices 379 / 342 / 287
 constexpr int SMALL_P = 4;                    // few slices: at most 2^this
 constexpr double SMALL_FLOPS_BITS = 6e6;      // few slices, any number of bitstrings: 2^22.5
 constexpr double SMALL_FLOPS_MANY = 1 << 21;  // more slices

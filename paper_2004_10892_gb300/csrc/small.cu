@@ -9,10 +9,10 @@
 // costs no latency.
 //
 // GB300, a whole call from the host, before (a captured graph, or direct
-// launches in the allocation-free call) and now: 4x4 depth 16 amplitude 138 ->
-// 53 us; 5x5 depth 20 without allocations 301 -> 98 us; 16 slices of 6x6 depth
-// 24 (6.3e7 flops) 275 -> 145 us; a 6x6 network of three-valued indices 379 ->
-// 293 us. What is left: about 1600 cycles for a level of one entry (index
+// launches in the allocation-free call) and now: 4x4 depth 16 amplitude 141 ->
+// 54 us; 5x5 depth 20 without allocations 305 -> 105 us; 16 slices of 6x6 depth
+// 24 (6.3e7 flops) 277 -> 148 us; a 6x6 network of three-valued indices 379 ->
+// 287 us. What is left: about 1600 cycles for a level of one entry (index
 // arithmetic, dependent loads, the barrier), and for levels of 2^16 entries
 // and more the 64 bytes a cycle that each of the cluster's SMs gets from L2.
 #include <cooperative_groups.h>
