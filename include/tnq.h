@@ -227,8 +227,8 @@ size_t tnq_plan_workspace_bytes(const tnq_plan* plan, uint32_t batch);
  *  bits: host, n_qubits bytes (0/1); may be NULL for a general network
  *    (tnq_plan_from_network), which has no qubits.
  *  workspace: device memory of ws_bytes >= tnq_plan_workspace_bytes(plan, 1);
- *    the call runs as many slices at once as the workspace holds (a power of
- *    two, at most max_batch if max_batch > 0).
+ *    the call runs as many slices at once as the workspace holds (at most
+ *    max_batch if max_batch > 0).
  *  stream: cudaStream_t or NULL.
  *  out_amp: host, 2 doubles (re, im): the partial sum in FP64.
  *  out_slice_amps: host, 2*(slice_end-slice_begin) doubles, or NULL: each sigma_s.
